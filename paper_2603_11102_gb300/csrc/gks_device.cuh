@@ -119,49 +119,54 @@ __device__ __forceinline__ void weno5_pair(const R q[5], R &right, R &left)
 }
 
 // erf(z), exp(-z^2) - 1 and exp(-z^2) of the half-space moments, z =
-// sqrt(lambda) U. For |z| <= 1/2 (|U| up to 7 U_ref at Ma 0.1) the Maclaurin
-// series
-//   erf z = (2/sqrt pi) sum_n (-1)^n z^(2n+1) / (n! (2n+1)),
-//   expm1 x = sum_n x^n / n!,
-// FP32: n = 0..6 and 1..7 (first dropped terms below 4e-10 and 2e-9
-// relative; within 2e-7 of the exact values after rounding); FP64: n = 0..12
-// and 1..13 (dropped terms below 1e-17; within 3e-16 of libm); exp = 1 +
-// expm1. Beyond 1/2 the library functions.
+// sqrt(lambda) U. For |z| <= 1/2 (|U| up to 7 U_ref at Ma 0.1), with t = z^2:
+//   erf z = z E(t),  exp(-t) - 1 = -t X(-t),
+// E and X as polynomials of least deviation on 0 <= t <= 1/4 (Chebyshev fits
+// of the two Maclaurin series): degree 4 in FP32 (within 1.5e-9 and 2.4e-9,
+// relative) and degree 8 in FP64 and double-single (within 4.3e-18 and
+// 7.3e-18), 4 and 8 multiply-adds less per pair than the truncated series of
+// the same accuracy. exp = 1 + expm1. Beyond 1/2 the library functions.
+template <typename T>
+__device__ __forceinline__ void half_space_polys(T t, T x, T &E, T &X)
+{
+    constexpr double ce[9] = {1.4725865480556743912e-6, -0.000014845849259707869768, 0.00012053335124353740746,
+                              -0.00085482977536749668828, 0.0052239773730214700169, -0.026866170632887929351,
+                              0.11283791670925353147, -0.37612638903183473544, 1.1283791670955125696};
+    constexpr double cx[9] = {2.4634585655528519648e-6, 0.000024667266113234713626, 0.00019837907206591588519,
+                              0.001388883962567040931, 0.0083333329084976221444, 0.041666666646060813782,
+                              0.166666666666165589, 0.49999999999999530577, 0.99999999999999999276};
+    E = T(ce[0]);
+    X = T(cx[0]);
+#pragma unroll
+    for (int k = 1; k < 9; ++k) {
+        E = fma(E, t, T(ce[k]));
+        X = fma(X, x, T(cx[k]));
+    }
+}
+template <typename T>
+__device__ __forceinline__ void half_space_polys32(T t, T x, T &E, T &X)
+{
+    constexpr double ce[5] = {0.0047190825672188138798, -0.026757732735015515622, 0.11282831428465861874,
+                              -0.37612609007469802928, 1.1283791656017914552};
+    constexpr double cx[5] = {0.0075136062215127308948, 0.04149065410396734984, 0.16665108206608517899,
+                              0.49999951482098960754, 0.99999999757585578433};
+    E = T(ce[0]);
+    X = T(cx[0]);
+#pragma unroll
+    for (int k = 1; k < 5; ++k) {
+        E = fma(E, t, T(ce[k]));
+        X = fma(X, x, T(cx[k]));
+    }
+}
 __device__ __forceinline__ void half_space_terms(double z, double &e, double &m1, double &ex)
 {
     const double t = z * z, x = -t;
     if (fabs(z) <= 0.5) {
-        constexpr double k = 1.1283791670955126;   // 2 / sqrt(pi)
-        // c_n = k (-1)^n / (n! (2n+1))
-        double p = k / (479001600.0 * 25.0);
-        p = fma(p, t, -k / (39916800.0 * 23.0));
-        p = fma(p, t, k / (3628800.0 * 21.0));
-        p = fma(p, t, -k / (362880.0 * 19.0));
-        p = fma(p, t, k / (40320.0 * 17.0));
-        p = fma(p, t, -k / (5040.0 * 15.0));
-        p = fma(p, t, k / (720.0 * 13.0));
-        p = fma(p, t, -k / (120.0 * 11.0));
-        p = fma(p, t, k / (24.0 * 9.0));
-        p = fma(p, t, -k / (6.0 * 7.0));
-        p = fma(p, t, k / (2.0 * 5.0));
-        p = fma(p, t, -k / 3.0);
-        p = fma(p, t, k);
-        e = p * z;
-        double q = 1.0 / 6227020800.0;   // 1/13!
-        q = fma(q, x, 1.0 / 479001600.0);
-        q = fma(q, x, 1.0 / 39916800.0);
-        q = fma(q, x, 1.0 / 3628800.0);
-        q = fma(q, x, 1.0 / 362880.0);
-        q = fma(q, x, 1.0 / 40320.0);
-        q = fma(q, x, 1.0 / 5040.0);
-        q = fma(q, x, 1.0 / 720.0);
-        q = fma(q, x, 1.0 / 120.0);
-        q = fma(q, x, 1.0 / 24.0);
-        q = fma(q, x, 1.0 / 6.0);
-        q = fma(q, x, 0.5);
-        q = fma(q, x, 1.0);
-        m1 = q * x;
-        ex = 1.0 + m1;
+        double E, X;
+        half_space_polys(t, x, E, X);
+        e = E * z;
+        m1 = X * x;
+        ex = fma(X, x, 1.0);
     } else {
         e = erf(z);
         m1 = expm1(x);
@@ -170,26 +175,13 @@ __device__ __forceinline__ void half_space_terms(double z, double &e, double &m1
 }
 __device__ __forceinline__ void half_space_terms(float z, float &e, float &m1, float &ex)
 {
-    const float t = z * z, x = -t;
+    const float t = __fmul_rn(z, z), x = -t;
     if (fabsf(z) <= 0.5f) {
-        constexpr double k = 1.1283791670955126;   // 2 / sqrt(pi)
-        float p = float(k / (720.0 * 13.0));
-        p = fmaf(p, t, float(-k / (120.0 * 11.0)));
-        p = fmaf(p, t, float(k / (24.0 * 9.0)));
-        p = fmaf(p, t, float(-k / (6.0 * 7.0)));
-        p = fmaf(p, t, float(k / (2.0 * 5.0)));
-        p = fmaf(p, t, float(-k / 3.0));
-        p = fmaf(p, t, float(k));
-        e = p * z;
-        float q = float(1.0 / 5040.0);
-        q = fmaf(q, x, float(1.0 / 720.0));
-        q = fmaf(q, x, float(1.0 / 120.0));
-        q = fmaf(q, x, float(1.0 / 24.0));
-        q = fmaf(q, x, float(1.0 / 6.0));
-        q = fmaf(q, x, 0.5f);
-        q = fmaf(q, x, 1.0f);
-        m1 = q * x;
-        ex = 1.0f + m1;
+        float E, X;
+        half_space_polys32(t, x, E, X);
+        e = __fmul_rn(E, z);
+        m1 = __fmul_rn(X, x);
+        ex = __fadd_rn(1.0f, m1);
     } else {
         e = erff(z);
         m1 = expm1f(x);
@@ -210,42 +202,16 @@ __device__ __forceinline__ T cvt(dsf x) { return (T)to_double(x); }
 template <>
 __device__ __forceinline__ dsf cvt<dsf>(dsf x) { return x; }
 
-// Double-single: the same Maclaurin series as the FP64 version (n = 0..12
-// and 1..13, dropped terms below 1e-17) in double-single arithmetic for
+// Double-single: the FP64 polynomials in double-single arithmetic for
 // |z| <= 1/2; beyond, the FP64 library functions.
 __device__ __forceinline__ void half_space_terms(dsf z, dsf &e, dsf &m1, dsf &ex)
 {
     if (fabsf(z.hi) <= 0.5f) {
         const dsf t = z * z, x = -t;
-        constexpr double k = 1.1283791670955126;   // 2 / sqrt(pi)
-        dsf p = dsf(k / (479001600.0 * 25.0));
-        p = fma(p, t, dsf(-k / (39916800.0 * 23.0)));
-        p = fma(p, t, dsf(k / (3628800.0 * 21.0)));
-        p = fma(p, t, dsf(-k / (362880.0 * 19.0)));
-        p = fma(p, t, dsf(k / (40320.0 * 17.0)));
-        p = fma(p, t, dsf(-k / (5040.0 * 15.0)));
-        p = fma(p, t, dsf(k / (720.0 * 13.0)));
-        p = fma(p, t, dsf(-k / (120.0 * 11.0)));
-        p = fma(p, t, dsf(k / (24.0 * 9.0)));
-        p = fma(p, t, dsf(-k / (6.0 * 7.0)));
-        p = fma(p, t, dsf(k / (2.0 * 5.0)));
-        p = fma(p, t, dsf(-k / 3.0));
-        p = fma(p, t, dsf(k));
-        e = p * z;
-        dsf q = dsf(1.0 / 6227020800.0);   // 1/13!
-        q = fma(q, x, dsf(1.0 / 479001600.0));
-        q = fma(q, x, dsf(1.0 / 39916800.0));
-        q = fma(q, x, dsf(1.0 / 3628800.0));
-        q = fma(q, x, dsf(1.0 / 362880.0));
-        q = fma(q, x, dsf(1.0 / 40320.0));
-        q = fma(q, x, dsf(1.0 / 5040.0));
-        q = fma(q, x, dsf(1.0 / 720.0));
-        q = fma(q, x, dsf(1.0 / 120.0));
-        q = fma(q, x, dsf(1.0 / 24.0));
-        q = fma(q, x, dsf(1.0 / 6.0));
-        q = fma(q, x, dsf(0.5));
-        q = fma(q, x, dsf(1.0));
-        m1 = q * x;
+        dsf E, X;
+        half_space_polys(t, x, E, X);
+        e = E * z;
+        m1 = X * x;
         ex = dsf(1.0) + m1;
     } else {
         double de, dm, dx;
@@ -256,23 +222,23 @@ __device__ __forceinline__ void half_space_terms(dsf z, dsf &e, dsf &m1, dsf &ex
     }
 }
 
-// Equilibrium state at a face (local frame, rho written as rho - off): the
-// u>0 half of the left Maxwellian plus the u<0 half of the right one.
-template <typename R>
-__device__ __forceinline__ void face_equilibrium(const Phys<R> &ph, const R Ql[4], const R Qr[4], R Q0[4])
+// Equilibrium state at a face (local frame) of an FP64 grid, where rho is
+// stored whole (ph.off = 0): the u>0 half of the left Maxwellian plus the u<0
+// half of the right one.
+__device__ __forceinline__ void face_equilibrium(const Phys<double> &ph, const double Ql[4], const double Qr[4],
+                                                 double Q0[4])
 {
-    const R rl = ph.off + Ql[0], rr = ph.off + Qr[0];
-    const R Ul = wdiv(Ql[1], rl), Ur = wdiv(Qr[1], rr);
-    R el, er, ml, mr, xl, xr;
+    const double Ul = Ql[1] / Ql[0], Ur = Qr[1] / Qr[0];
+    double el, er, ml, mr, xl, xr;
     half_space_terms(ph.sqlam * Ul, el, ml, xl);
     half_space_terms(ph.sqlam * Ur, er, mr, xr);
-    const R Pl = R(0.5) + R(0.5) * el;   // <u^0>_{u>0} of the left state
-    const R Pr = R(0.5) - R(0.5) * er;   // <u^0>_{u<0} of the right state
-    const R El = ph.kE * xl, Er = ph.kE * xr;
-    Q0[0] = Ql[0] * Pl + Qr[0] * Pr + ph.off * (R(0.5) * (el - er));
-    Q0[1] = Ql[1] * Pl + Qr[1] * Pr + (Ql[0] * El - Qr[0] * Er) + ph.off * (ph.kE * (ml - mr));
-    Q0[2] = Ql[2] * Pl + Qr[2] * Pr;
-    Q0[3] = Ql[3] * Pl + Qr[3] * Pr;
+    const double Pl = fma(0.5, el, 0.5);    // <u^0>_{u>0} of the left state
+    const double Pr = fma(-0.5, er, 0.5);   // <u^0>_{u<0} of the right state
+    const double El = ph.kE * xl, Er = ph.kE * xr;
+    Q0[0] = fma(Ql[0], Pl, Qr[0] * Pr);
+    Q0[1] = fma(Ql[1], Pl, Qr[1] * Pr) + fma(Ql[0], El, -(Qr[0] * Er));
+    Q0[2] = fma(Ql[2], Pl, Qr[2] * Pr);
+    Q0[3] = fma(Ql[3], Pl, Qr[3] * Pr);
 }
 
 // Quartic through 5 face averages q[-2..2], at the Gauss points -g, +g of
@@ -471,42 +437,17 @@ __device__ __forceinline__ dsf2 wdiv(dsf2 a, dsf2 b) { return a / b; }
 __device__ __forceinline__ dsf2 &operator*=(dsf2 &a, dsf2 b) { return a = a * b; }
 __device__ __forceinline__ dsf2 fma(dsf2 a, dsf2 b, dsf2 c) { return a * b + c; }
 
-// half_space_terms of two double-single arguments: the series of both lanes
+// half_space_terms of two double-single arguments: the polynomials of both lanes
 // as pairs when both lie in |z| <= 1/2, else lane by lane (the same bits as
 // the scalar double-single version either way).
 __device__ __forceinline__ void half_space_terms(dsf2 z, dsf2 &e, dsf2 &m1, dsf2 &ex)
 {
     if (fabsf(z.hi.v.x) <= 0.5f && fabsf(z.hi.v.y) <= 0.5f) {
         const dsf2 t = z * z, x = -t;
-        constexpr double k = 1.1283791670955126;   // 2 / sqrt(pi)
-        dsf2 p = dsf2(k / (479001600.0 * 25.0));
-        p = fma(p, t, dsf2(-k / (39916800.0 * 23.0)));
-        p = fma(p, t, dsf2(k / (3628800.0 * 21.0)));
-        p = fma(p, t, dsf2(-k / (362880.0 * 19.0)));
-        p = fma(p, t, dsf2(k / (40320.0 * 17.0)));
-        p = fma(p, t, dsf2(-k / (5040.0 * 15.0)));
-        p = fma(p, t, dsf2(k / (720.0 * 13.0)));
-        p = fma(p, t, dsf2(-k / (120.0 * 11.0)));
-        p = fma(p, t, dsf2(k / (24.0 * 9.0)));
-        p = fma(p, t, dsf2(-k / (6.0 * 7.0)));
-        p = fma(p, t, dsf2(k / (2.0 * 5.0)));
-        p = fma(p, t, dsf2(-k / 3.0));
-        p = fma(p, t, dsf2(k));
-        e = p * z;
-        dsf2 q = dsf2(1.0 / 6227020800.0);   // 1/13!
-        q = fma(q, x, dsf2(1.0 / 479001600.0));
-        q = fma(q, x, dsf2(1.0 / 39916800.0));
-        q = fma(q, x, dsf2(1.0 / 3628800.0));
-        q = fma(q, x, dsf2(1.0 / 362880.0));
-        q = fma(q, x, dsf2(1.0 / 40320.0));
-        q = fma(q, x, dsf2(1.0 / 5040.0));
-        q = fma(q, x, dsf2(1.0 / 720.0));
-        q = fma(q, x, dsf2(1.0 / 120.0));
-        q = fma(q, x, dsf2(1.0 / 24.0));
-        q = fma(q, x, dsf2(1.0 / 6.0));
-        q = fma(q, x, dsf2(0.5));
-        q = fma(q, x, dsf2(1.0));
-        m1 = q * x;
+        dsf2 E, X;
+        half_space_polys(t, x, E, X);
+        e = E * z;
+        m1 = X * x;
         ex = dsf2(1.0) + m1;
     } else {
         dsf e0, e1, m0, m1_, x0, x1;
@@ -518,103 +459,164 @@ __device__ __forceinline__ void half_space_terms(dsf2 z, dsf2 &e, dsf2 &m1, dsf2
     }
 }
 
-// face_equilibrium in double-single with the left and right half-space terms
-// evaluated as one pair (the same bits as face_equilibrium<dsf>).
-__device__ __forceinline__ void face_equilibrium_ds2(const Phys<dsf> &ph, const dsf Ql[4], const dsf Qr[4], dsf Q0[4])
+// face_equilibrium in double-single (an FP64 grid: ph.off = 0) with the left
+// and right half-space terms evaluated as one pair.
+__device__ __forceinline__ void face_equilibrium_ds2(const Phys<dsf> &ph, const dsf2 L[2], const dsf2 R[2], dsf2 Q0[2])
 {
-    const dsf2 r = dsf2(ph.off) + dsf2(Ql[0], Qr[0]);
-    const dsf2 U = wdiv(dsf2(Ql[1], Qr[1]), r);
+    // lanes (left, right) of rho and m_n
+    const dsf2 r(L[0].lane(0), R[0].lane(0));
+    const dsf2 U = wdiv(dsf2(L[0].lane(1), R[0].lane(1)), r);
     dsf2 e, m1, x;
     half_space_terms(dsf2(ph.sqlam) * U, e, m1, x);
-    const dsf el = e.lane(0), er = e.lane(1), ml = m1.lane(0), mr = m1.lane(1);
-    const dsf Pl = dsf(0.5) + dsf(0.5) * el;   // <u^0>_{u>0} of the left state
-    const dsf Pr = dsf(0.5) - dsf(0.5) * er;   // <u^0>_{u<0} of the right state
-    const dsf El = ph.kE * x.lane(0), Er = ph.kE * x.lane(1);
-    Q0[0] = Ql[0] * Pl + Qr[0] * Pr + ph.off * (dsf(0.5) * (el - er));
-    Q0[1] = Ql[1] * Pl + Qr[1] * Pr + (Ql[0] * El - Qr[0] * Er) + ph.off * (ph.kE * (ml - mr));
-    Q0[2] = Ql[2] * Pl + Qr[2] * Pr;
-    Q0[3] = Ql[3] * Pl + Qr[3] * Pr;
+    const dsf Pl = dsf(0.5) + scale_pow2(e.lane(0), 0.5f);   // <u^0>_{u>0} of the left state
+    const dsf Pr = dsf(0.5) - scale_pow2(e.lane(1), 0.5f);   // <u^0>_{u<0} of the right state
+    const dsf2 rE = r * (dsf2(ph.kE) * x);
+    Q0[0] = L[0] * dsf2(Pl) + R[0] * dsf2(Pr);
+    Q0[1] = L[1] * dsf2(Pl) + R[1] * dsf2(Pr);
+    const dsf mn = Q0[0].lane(1) + (rE.lane(0) - rE.lane(1));
+    Q0[0] = dsf2(Q0[0].lane(0), mn);
 }
 
 // ---- FP32 face state on packed pairs ----
 
-// Approximate reciprocal per lane (the scalar FP32 path's __fdividef(1, x)).
-__device__ __forceinline__ f2 wrcp(f2 x) { return f2(__fdividef(1.0f, x.v.x), __fdividef(1.0f, x.v.y)); }
-
-// weno5_pair of two components at once, every multiply-add fused explicitly
-// and the constant factors folded into the candidates:
-//  - the indicators are those of weno5_pair divided by 13/12 (the weights
-//    depend on their ratios only): s_k = (eps 12/13 + t_k^2 + (3/13) u_k^2)^2,
-//    with u_0 = t_0 + 2 (c - b) and u_2 = t_2 + 2 (c - d);
-//  - the right-face weights times 10 s0 s1 s2 / 3 are s1 s2 / 3, 2 s0 s2 and
-//    s0 s1 (mirrored for the left face), so with the candidates P_k = the
-//    integer-coefficient ones divided by 18, 3 and 6 the face value is
-//    (s12 P0 + s02 P1 + s01 P2) / (s12 / 3 + 2 s02 + s01).
-__device__ __forceinline__ void weno5_pair2(const f2 q[5], f2 &right, f2 &left)
+// Approximate reciprocal per lane (1 ulp; one instruction: the arguments, a
+// density or a sum of squared smoothness indicators of at least 1e-23, are
+// never subnormal, so the flush of subnormal inputs changes nothing).
+__device__ __forceinline__ float rcp_approx(float x)
 {
-    const f2 m2(-2.0f), two(2.0f), eps(float(12e-6 / 13.0)), k(float(3.0 / 13.0));
-    const f2 a = q[0], b = q[1], c = q[2], d = q[3], e = q[4];
-    f2 t = fma(b, m2, a) + c, u = fma(c - b, two, t);
-    f2 s0 = fma(t, t, fma(u * k, u, eps));
-    t = fma(c, m2, b) + d;
-    u = b - d;
-    f2 s1 = fma(t, t, fma(u * k, u, eps));
-    t = fma(d, m2, c) + e;
-    u = fma(c - d, two, t);
-    f2 s2 = fma(t, t, fma(u * k, u, eps));
-    s0 = s0 * s0;
-    s1 = s1 * s1;
-    s2 = s2 * s2;
-    const f2 s02 = s0 * s2, s01 = s0 * s1, s12 = s1 * s2;
-    const f2 third(float(1.0 / 3.0));
-    const f2 c3 = c * third, c53 = c * f2(float(5.0 / 3.0)), c1118 = c * f2(float(11.0 / 18.0));
-    const f2 k19(float(1.0 / 9.0)), k718(float(-7.0 / 18.0)), k23(float(2.0 / 3.0)), km13(float(-1.0 / 3.0));
-    const f2 k56(float(5.0 / 6.0)), km16(float(-1.0 / 6.0));
-    {
-        // right face: candidates on (a,b,c), (b,c,d), (c,d,e)
-        const f2 P0 = fma(a, k19, fma(b, k718, c1118));
-        const f2 P1 = fma(b, km13, fma(d, k23, c53));
-        const f2 P2 = fma(e, km16, fma(d, k56, c3));
-        right = fma(s12, P0, fma(s02, P1, s01 * P2)) * wrcp(fma(s12, third, fma(s02, two, s01)));
-    }
-    {
-        // left face: the mirrored candidates with indicators s2, s1, s0
-        const f2 P0 = fma(e, k19, fma(d, k718, c1118));
-        const f2 P1 = fma(d, km13, fma(b, k23, c53));
-        const f2 P2 = fma(a, km16, fma(b, k56, c3));
-        left = fma(s01, P0, fma(s02, P1, s12 * P2)) * wrcp(fma(s01, third, fma(s02, two, s12)));
-    }
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
+__device__ __forceinline__ f2 wrcp(f2 x) { return f2(rcp_approx(x.v.x), rcp_approx(x.v.y)); }
+__device__ __forceinline__ f2 wnrcp(f2 x) { return f2(rcp_approx(-x.v.x), rcp_approx(-x.v.y)); }
 
-// half_space_terms of two FP32 arguments: the series of both lanes as pairs
-// when both lie in |z| <= 1/2 (the same operations per lane as the scalar
-// series, so the same bits), else lane by lane.
+// half_space_terms of two FP32 arguments: the polynomials of both lanes as
+// pairs when both lie in |z| <= 1/2 (the same operations per lane as the
+// scalar version, so the same bits), else lane by lane.
 __device__ __forceinline__ void half_space_terms(f2 z, f2 &e, f2 &m1, f2 &ex)
 {
     if (fabsf(z.v.x) <= 0.5f && fabsf(z.v.y) <= 0.5f) {
         const f2 t = z * z, x = t * f2(-1.0f);
-        constexpr double k = 1.1283791670955126;   // 2 / sqrt(pi)
-        f2 p = f2(float(k / (720.0 * 13.0)));
-        p = fma(p, t, f2(float(-k / (120.0 * 11.0))));
-        p = fma(p, t, f2(float(k / (24.0 * 9.0))));
-        p = fma(p, t, f2(float(-k / (6.0 * 7.0))));
-        p = fma(p, t, f2(float(k / (2.0 * 5.0))));
-        p = fma(p, t, f2(float(-k / 3.0)));
-        p = fma(p, t, f2(float(k)));
-        e = p * z;
-        f2 q = f2(float(1.0 / 5040.0));
-        q = fma(q, x, f2(float(1.0 / 720.0)));
-        q = fma(q, x, f2(float(1.0 / 120.0)));
-        q = fma(q, x, f2(float(1.0 / 24.0)));
-        q = fma(q, x, f2(float(1.0 / 6.0)));
-        q = fma(q, x, f2(0.5f));
-        q = fma(q, x, f2(1.0f));
-        m1 = q * x;
+        f2 E, X;
+        half_space_polys32(t, x, E, X);
+        e = E * z;
+        m1 = X * x;
         ex = f2(1.0f) + m1;
     } else {
         half_space_terms(z.v.x, e.v.x, m1.v.x, ex.v.x);
         half_space_terms(z.v.y, e.v.y, m1.v.y, ex.v.y);
     }
+}
+
+// WENO5-JS along a march, in differences. With the first differences
+// D_{k+1/2} = q_{k+1} - q_k, the second ones S_k = D_{k+1/2} - D_{k-1/2} and
+// the third ones T_{k+1/2} = S_{k+1} - S_k, the face values of cell i are the
+// centre candidate plus what the outer two add to it,
+//   right = q_i + D_{i+1/2}/2 - S_i/6 - w0 T_{i-1/2}/3 - w2 T_{i+1/2}/6,
+//   left  = q_i - D_{i-1/2}/2 - S_i/6 + v0 T_{i+1/2}/3 + v2 T_{i-1/2}/6
+// (w0, w2 and, mirrored, v0, v2 the weights of the outer candidates), and the
+// indicators are those of weno5_pair over 13/12 (the weights depend on their
+// ratios only): beta = S^2 + (3/13) u^2 with u = S_{i-1} + 2 D_{i-1/2},
+// D_{i-1/2} + D_{i+1/2} and S_{i+1} - 2 D_{i+1/2}. A cell that enters the
+// march brings one new difference of each order and one new square, where
+// the 5-cell form redoes them for every cell: 33 operations per cell and
+// component against 53 (FP32 pairs) and 81 (FP64). The FP64 face state is
+// bound by the FP64 pipe and follows the count (6 launches of a 96^3 step:
+// 7.92 -> 4.67 ms), the double-single one too (2.38 -> 1.66 ms); the FP32 one
+// waits on its loads as well (a 384x256x256 step: 2.27 -> 2.15 ms). Written
+// without a product that feeds an addition, so that no contraction is left to
+// the compiler and a face's bits do not depend on its position in the march.
+template <typename T>
+struct WenoMarch {
+    T c, d;             // cells i, i + 1
+    T Dm, D0, Sm, S0;   // D_{i-1/2}, D_{i+1/2}, S_{i-1}, S_i
+    T Tm;               // T_{i-1/2}
+    T bm, b0;           // eps + S_{i-1}^2, eps + S_i^2
+
+    // cells i - 2 .. i + 1
+    __device__ __forceinline__ void start(T q0, T q1, T q2, T q3)
+    {
+        const T eps(12e-6 / 13.0);
+        c = q2;
+        d = q3;
+        Dm = q2 - q1;
+        D0 = q3 - q2;
+        Sm = Dm - (q1 - q0);
+        S0 = D0 - Dm;
+        Tm = S0 - Sm;
+        bm = fma(Sm, Sm, eps);
+        b0 = fma(S0, S0, eps);
+    }
+
+    // normal slope times the centre distance at the face between i - 1 and i
+    // (12 x the quartic's derivative is 15 D - (D_{-1} + D + D_{+1}) = 12 D - T)
+    __device__ __forceinline__ T slope() const { return fma(Tm, T(-1.0 / 12.0), Dm); }
+
+    // cell e = q_{i+2} enters: the right- and left-face values of cell i;
+    // then i + 1 becomes the centre
+    __device__ __forceinline__ void push(T e, T &right, T &left)
+    {
+        const T eps(12e-6 / 13.0), k(3.0 / 13.0), half(0.5), nhalf(-0.5);
+        const T D1 = e - d, S1 = D1 - D0, Tp = S1 - S0;
+        const T b1 = fma(S1, S1, eps);
+        const T u0 = fma(Dm, T(2.0), Sm), u1 = Dm + D0, u2 = fma(D0, T(-2.0), S1);
+        T s0 = fma(u0 * k, u0, bm), s1 = fma(u1 * k, u1, b0), s2 = fma(u2 * k, u2, b1);
+        s0 = s0 * s0;
+        s1 = s1 * s1;
+        s2 = s2 * s2;
+        const T s02 = s0 * s2, s01 = s0 * s1, s12 = s1 * s2;
+        // 3 x the sums of the weights (s12 : 6 s02 : 3 s01 and mirrored)
+        const T w1 = s02 * T(18.0);
+        const T dr = fma(s12, T(3.0), fma(s01, T(9.0), w1)), dl = fma(s01, T(3.0), fma(s12, T(9.0), w1));
+        const T a = s12 * Tm, b = s01 * Tp;
+        const T cs = fma(S0, T(-1.0 / 6.0), c);
+        sub_quotients(fma(b, T(1.5), a), dr, fma(D0, half, cs), right, fma(a, T(1.5), b), dl, fma(Dm, nhalf, cs), left);
+        c = d;
+        d = e;
+        Dm = D0;
+        D0 = D1;
+        Sm = S0;
+        S0 = S1;
+        Tm = Tp;
+        bm = b0;
+        b0 = b1;
+    }
+
+    // r = cr - nr / dr, l = cl + nl / dl
+    static __device__ __forceinline__ void sub_quotients(T nr, T dr, T cr, T &r, T nl, T dl, T cl, T &l);
+};
+template <>
+__device__ __forceinline__ void WenoMarch<f2>::sub_quotients(f2 nr, f2 dr, f2 cr, f2 &r, f2 nl, f2 dl, f2 cl, f2 &l)
+{
+    r = fma(nr, wnrcp(dr), cr);
+    l = fma(nl, wrcp(dl), cl);
+}
+// One FP64 division for both faces (the denominators are sums of 8th powers
+// of differences above 1e-23; where their product overflows, each by itself).
+template <>
+__device__ __forceinline__ void WenoMarch<double>::sub_quotients(double nr, double dr, double cr, double &r, double nl,
+                                                                 double dl, double cl, double &l)
+{
+    const double p = dr * dl;
+    double ir, il;
+    if (__double2hiint(p) < 0x7ff00000) {
+        const double ip = 1.0 / p;
+        ir = ip * dl;
+        il = ip * dr;
+    } else {
+        ir = 1.0 / dr;
+        il = 1.0 / dl;
+    }
+    r = fma(-nr, ir, cr);
+    l = fma(nl, il, cl);
+}
+template <>
+__device__ __forceinline__ void WenoMarch<dsf2>::sub_quotients(dsf2 nr, dsf2 dr, dsf2 cr, dsf2 &r, dsf2 nl, dsf2 dl,
+                                                               dsf2 cl, dsf2 &l)
+{
+    r = cr - nr / dr;
+    l = cl + nl / dl;
 }
 
 // face_equilibrium with the components paired as (rho, m_n) and (m_t1, m_t2)

@@ -181,14 +181,13 @@ struct FaceEqArgs {
 constexpr int kMarch32 = 32, kMarch = 16;
 
 // Marching variant: each thread walks K consecutive faces along d at one
-// tangential position of the extended face box, with the 5 cells around the
-// current cell in registers. Per cell it forms both face values of WENO5
-// from one set of smoothness indicators; face f takes the right-face value
-// of cell f-1 and the left-face value of cell f. Launched for FP64 grids in
-// FP64 arithmetic; FP32 grids and double-single arithmetic take the packed
-// variants below, which march the same way.
-template <typename R, typename C = R>
-__global__ void __launch_bounds__(256) face_eq_march_kernel(FaceEqArgs<R, C> A)
+// tangential position of the extended face box, with the differences around
+// the current cell in registers (WenoMarch). Per cell it forms both face
+// values of WENO5 from one set of smoothness indicators; face f takes the
+// right-face value of cell f-1 and the left-face value of cell f. Launched
+// for FP64 grids in FP64 arithmetic; FP32 grids and double-single arithmetic
+// take the packed variants below, which march the same way.
+__global__ void __launch_bounds__(256) face_eq_march_kernel(FaceEqArgs<double, double> A)
 {
     const int a = (int)(blockIdx.x * 32 + threadIdx.x) - 2;
     const int b = (int)(blockIdx.y * 8 + threadIdx.y) - 2;
@@ -201,54 +200,43 @@ __global__ void __launch_bounds__(256) face_eq_march_kernel(FaceEqArgs<R, C> A)
         !in_bounds(((long)f0 * (A.n2 + 4) + (b + 2)) * A.e1p + (a + 2), A.nfq) ||
         !in_bounds(((long)(f1 - 1) * (A.n2 + 4) + (b + 2)) * A.e1p + (a + 2), A.nfq))
         return;
-    const int comp[4] = {0, A.cn, A.c1, A.c2};
-    const Phys<C> &ph = A.ph;
-    // window w[v][k] = cell (c - 2 + k); start with c = f0 - 1
-    C w[4][5];
+    const double *pc[4] = {A.w + base, A.w + (long)A.cn * A.np + base, A.w + (long)A.c1 * A.np + base,
+                           A.w + (long)A.c2 * A.np + base};
+    // cells f0-3 .. f0 start the march at cell f0-1, cell f0+1 completes it
+    WenoMarch<double> w[4];
+    double Qprev[4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-        const R *p = A.w + comp[v] * A.np + base;
-#pragma unroll
-        for (int k = 0; k < 5; ++k) w[v][k] = cvt<C>(__ldg(p + (long)(f0 - 3 + k + G) * A.sd));
+        const double *p = pc[v] + (long)(f0 - 3 + G) * A.sd;
+        w[v].start(__ldg(p), __ldg(p + A.sd), __ldg(p + 2 * A.sd), __ldg(p + 3 * A.sd));
+        double l;
+        w[v].push(__ldg(p + 4 * A.sd), Qprev[v], l);
     }
-    C Qprev[4];
+    // the cell entering the march, loaded one face ahead
+    double nxt[4];
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        C l;
-        weno5_pair(w[v], Qprev[v], l);
-    }
-    // the cell entering the window, loaded one face ahead
-    R nxt[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) nxt[v] = __ldg(A.w + comp[v] * A.np + base + (long)(f0 + 2 + G) * A.sd);
+    for (int v = 0; v < 4; ++v) nxt[v] = __ldg(pc[v] + (long)(f0 + 2 + G) * A.sd);
     for (int f = f0; f < f1; ++f) {
-        C Ql[4], Qr[4];
+        const double ihf = A.ihf[f];
+        const long o = ((long)f * (A.n2 + 4) + (b + 2)) * A.e1p + (a + 2);
+        double e[4];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) w[v][k] = w[v][k + 1];
-            w[v][4] = cvt<C>(nxt[v]);
-        }
+        for (int v = 0; v < 4; ++v) e[v] = nxt[v];
         if (f + 1 < f1) {
             // cell f + 3 <= nf + 1 = n + 2: inside the ghost layers
 #pragma unroll
-            for (int v = 0; v < 4; ++v) nxt[v] = __ldg(A.w + comp[v] * A.np + base + (long)(f + 3 + G) * A.sd);
+            for (int v = 0; v < 4; ++v) nxt[v] = __ldg(pc[v] + (long)(f + 3 + G) * A.sd);
         }
+        double Ql[4], Qr[4], Q0[4];
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
+            A.fq[(4 + v) * A.nfq + o] = w[v].slope() * ihf;
             Ql[v] = Qprev[v];
-            weno5_pair(w[v], Qprev[v], Qr[v]);
+            w[v].push(e[v], Qprev[v], Qr[v]);
         }
-        C Q0[4];
-        face_equilibrium(ph, Ql, Qr, Q0);
-        const C s = cvt<C>(A.ihf[f]) * C(1.0 / 12.0);
-        const long o = ((long)f * (A.n2 + 4) + (b + 2)) * A.e1p + (a + 2);
+        face_equilibrium(A.ph, Ql, Qr, Q0);
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            A.fq[v * A.nfq + o] = cvt<Mid<R, C>>(Q0[v]);
-            // cells f-2 .. f+1 are w[v][0..3]
-            A.fq[(4 + v) * A.nfq + o] = cvt<Mid<R, C>>((C(15) * (w[v][2] - w[v][1]) - (w[v][3] - w[v][0])) * s);
-        }
+        for (int v = 0; v < 4; ++v) A.fq[v * A.nfq + o] = Q0[v];
     }
 }
 
@@ -279,32 +267,29 @@ __global__ void __launch_bounds__(256, 3) face_eq_f2_kernel(FaceEqArgs<float, fl
         return;
     const float *pc[4] = {A.w + base, A.w + (long)A.cn * A.np + base, A.w + (long)A.c1 * A.np + base,
                           A.w + (long)A.c2 * A.np + base};
-    // window w[p][k] = cell (c - 2 + k) of component pair p; start with c = f0 - 1
-    f2 w[2][5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        const long o = (long)(f0 - 3 + k + G) * A.sd;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) w[q][k] = f2(__ldg(pc[2 * q] + o), __ldg(pc[2 * q + 1] + o));
-    }
+    // cells f0-3 .. f0 start the march at cell f0-1, cell f0+1 completes it
+    WenoMarch<f2> w[2];
     f2 Qprev[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-        f2 l;
-        weno5_pair2(w[q], Qprev[q], l);
+        f2 v[5], l;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            const long o = (long)(f0 - 3 + k + G) * A.sd;
+            v[k] = f2(__ldg(pc[2 * q] + o), __ldg(pc[2 * q + 1] + o));
+        }
+        w[q].start(v[0], v[1], v[2], v[3]);
+        w[q].push(v[4], Qprev[q], l);
     }
-    // the cell entering the window, loaded one face ahead
+    // the cell entering the march, loaded one face ahead
     float nxt[4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) nxt[v] = __ldg(pc[v] + (long)(f0 + 2 + G) * A.sd);
 #pragma unroll 2
     for (int f = f0; f < f1; ++f) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) w[q][k] = w[q][k + 1];
-            w[q][4] = f2(nxt[2 * q], nxt[2 * q + 1]);
-        }
+        const f2 ihf(A.ihf[f]);
+        const long o = ((long)f * (A.n2 + 4) + (b + 2)) * A.e1p + (a + 2);
+        const f2 e[2] = {f2(nxt[0], nxt[1]), f2(nxt[2], nxt[3])};
         if (f + 1 < f1) {
             // cell f + 3 <= nf + 1 = n + 2: inside the ghost layers
 #pragma unroll
@@ -313,20 +298,17 @@ __global__ void __launch_bounds__(256, 3) face_eq_f2_kernel(FaceEqArgs<float, fl
         f2 Ql[2], Qr[2], Q0[2];
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-            Ql[q] = Qprev[q];
-            weno5_pair2(w[q], Qprev[q], Qr[q]);
-        }
-        face_equilibrium2(A.ph, Ql, Qr, Q0);
-        const f2 s(A.ihf[f] * float(1.0 / 12.0));
-        const long o = ((long)f * (A.n2 + 4) + (b + 2)) * A.e1p + (a + 2);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            // cells f-2 .. f+1 are w[q][0..3]
-            const f2 dq = fma(w[q][3] - w[q][0], f2(-1.0f), (w[q][2] - w[q][1]) * f2(15.0f)) * s;
-            A.fq[(2 * q) * A.nfq + o] = Q0[q].v.x;
-            A.fq[(2 * q + 1) * A.nfq + o] = Q0[q].v.y;
+            const f2 dq = w[q].slope() * ihf;
             A.fq[(4 + 2 * q) * A.nfq + o] = dq.v.x;
             A.fq[(5 + 2 * q) * A.nfq + o] = dq.v.y;
+            Ql[q] = Qprev[q];
+            w[q].push(e[q], Qprev[q], Qr[q]);
+        }
+        face_equilibrium2(A.ph, Ql, Qr, Q0);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            A.fq[(2 * q) * A.nfq + o] = Q0[q].v.x;
+            A.fq[(2 * q + 1) * A.nfq + o] = Q0[q].v.y;
         }
     }
 }
@@ -366,58 +348,49 @@ __global__ void __launch_bounds__(256, 2) face_eq_ds2_kernel(FaceEqArgs<double, 
         return;
     const double *pc[4] = {A.w + base, A.w + (long)A.cn * A.np + base, A.w + (long)A.c1 * A.np + base,
                            A.w + (long)A.c2 * A.np + base};
-    // window w[p][k] = cell (c - 2 + k) of component pair p; start with c = f0 - 1
-    dsf2 w[2][5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        const long o = (long)(f0 - 3 + k + G) * A.sd;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) w[q][k] = dsf2(to_ds(__ldg(pc[2 * q] + o)), to_ds(__ldg(pc[2 * q + 1] + o)));
-    }
+    // cells f0-3 .. f0 start the march at cell f0-1, cell f0+1 completes it
+    WenoMarch<dsf2> w[2];
     dsf2 Qprev[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-        dsf2 l;
-        weno5_pair(w[q], Qprev[q], l);
+        dsf2 v[5], l;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            const long o = (long)(f0 - 3 + k + G) * A.sd;
+            v[k] = dsf2(to_ds(__ldg(pc[2 * q] + o)), to_ds(__ldg(pc[2 * q + 1] + o)));
+        }
+        w[q].start(v[0], v[1], v[2], v[3]);
+        w[q].push(v[4], Qprev[q], l);
     }
-    // the cell entering the window, loaded one face ahead
+    // the cell entering the march, loaded one face ahead
     double nxt[4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) nxt[v] = __ldg(pc[v] + (long)(f0 + 2 + G) * A.sd);
     for (int f = f0; f < f1; ++f) {
+        const dsf2 ihf(to_ds(A.ihf[f]));
+        const long o = ((long)f * (A.n2 + 4) + (b + 2)) * A.e1p + (a + 2);
+        double e[4];
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) w[q][k] = w[q][k + 1];
-            w[q][4] = dsf2(to_ds(nxt[2 * q]), to_ds(nxt[2 * q + 1]));
-        }
+        for (int v = 0; v < 4; ++v) e[v] = nxt[v];
         if (f + 1 < f1) {
             // cell f + 3 <= nf + 1 = n + 2: inside the ghost layers
 #pragma unroll
             for (int v = 0; v < 4; ++v) nxt[v] = __ldg(pc[v] + (long)(f + 3 + G) * A.sd);
         }
-        dsf Ql[4], Qr[4];
+        dsf2 Ql[2], Qr[2], Q0[2];
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-            Ql[2 * q] = Qprev[q].lane(0);
-            Ql[2 * q + 1] = Qprev[q].lane(1);
-            dsf2 r;
-            weno5_pair(w[q], Qprev[q], r);
-            Qr[2 * q] = r.lane(0);
-            Qr[2 * q + 1] = r.lane(1);
-        }
-        dsf Q0[4];
-        face_equilibrium_ds2(A.ph, Ql, Qr, Q0);
-        const dsf2 s(to_ds(A.ihf[f]) * dsf(1.0 / 12.0));
-        const long o = ((long)f * (A.n2 + 4) + (b + 2)) * A.e1p + (a + 2);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            // cells f-2 .. f+1 are w[q][0..3]
-            const dsf2 dq = (dsf2(15) * (w[q][2] - w[q][1]) - (w[q][3] - w[q][0])) * s;
-            A.fq[(2 * q) * A.nfq + o] = Q0[2 * q];
-            A.fq[(2 * q + 1) * A.nfq + o] = Q0[2 * q + 1];
+            const dsf2 dq = w[q].slope() * ihf;
             A.fq[(4 + 2 * q) * A.nfq + o] = dq.lane(0);
             A.fq[(5 + 2 * q) * A.nfq + o] = dq.lane(1);
+            Ql[q] = Qprev[q];
+            w[q].push(dsf2(to_ds(e[2 * q]), to_ds(e[2 * q + 1])), Qprev[q], Qr[q]);
+        }
+        face_equilibrium_ds2(A.ph, Ql, Qr, Q0);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            A.fq[(2 * q) * A.nfq + o] = Q0[q].lane(0);
+            A.fq[(2 * q + 1) * A.nfq + o] = Q0[q].lane(1);
         }
     }
 }
@@ -1361,7 +1334,7 @@ void stage_impl(const Ctx &c)
         else if constexpr (std::is_same<C, float>::value)
             launch_face_eq_f2(E, d, c.stream);
         else
-            face_eq_march_kernel<R, C><<<ge, blk, 0, c.stream>>>(E);
+            face_eq_march_kernel<<<ge, blk, 0, c.stream>>>(E);
         mark(c, K_FACE_EQ, 0);
 
         FluxArgs<R, C> F;
