@@ -263,81 +263,41 @@ __device__ __forceinline__ void tan_val(R qm2, R qm1, R q0, R qp1, R qp2, R &vm,
 // The same values as tan_val as two 5-weight dot products (all on the FMA
 // pipe). Used for rows that vanish identically in a uniform state (normal
 // slopes, tangential derivatives), where the weights not summing exactly to
-// one in floating point is harmless.
-template <typename R>
+// one in floating point is harmless. NEG: the negated values (the density
+// slopes as gk_flux takes them), from negated weights.
+template <typename R, bool NEG = false>
 __device__ __forceinline__ void tan_val_direct(R qm2, R qm1, R q0, R qp1, R qp2, R &vm, R &vp)
 {
-    const R w0 = R(-1.0 / 4320.0 + 0.028065638085606807), w1 = R(1.0 / 1080.0 - 0.20046884346862007);
-    const R w2 = R(719.0 / 720.0);
-    const R w3 = R(1.0 / 1080.0 + 0.20046884346862007), w4 = R(-1.0 / 4320.0 - 0.028065638085606807);
+    constexpr double s = NEG ? -1.0 : 1.0;
+    const R w0 = R(s * (-1.0 / 4320.0 + 0.028065638085606807)), w1 = R(s * (1.0 / 1080.0 - 0.20046884346862007));
+    const R w2 = R(s * 719.0 / 720.0);
+    const R w3 = R(s * (1.0 / 1080.0 + 0.20046884346862007)), w4 = R(s * (-1.0 / 4320.0 - 0.028065638085606807));
     vp = fma(w4, qp2, fma(w3, qp1, fma(w2, q0, fma(w1, qm1, w0 * qm2))));
     vm = fma(w0, qp2, fma(w1, qp1, fma(w2, q0, fma(w3, qm1, w4 * qm2))));
 }
 
-template <typename R>
+// NEG: the derivatives negated.
+template <typename R, bool NEG = false>
 __device__ __forceinline__ void tan_val_der(R qm2, R qm1, R q0, R qp1, R qp2, R &vm, R &vp, R &dm,
                                             R &dp)
 {
+    constexpr double s = NEG ? -1.0 : 1.0;
     const R d1 = qp1 + qm1 - R(2) * q0, d2 = qp2 + qm2 - R(2) * q0;
     const R a1 = qp1 - qm1, a2 = qp2 - qm2;
     const R E = fma(d1, R(1.0 / 1080.0), fma(d2, R(-1.0 / 4320.0), q0));
     const R O = R(0.20046884346862007) * a1 - R(0.028065638085606807) * a2;
-    const R Do = R(2.0 / 3.0) * a1 - R(1.0 / 12.0) * a2;
-    const R De = R(0.41697519441472974) * d1 - R(0.032075014954979206) * d2;
+    const R Do = R(s * 2.0 / 3.0) * a1 - R(s * 1.0 / 12.0) * a2;
+    const R De = R(s * 0.41697519441472974) * d1 - R(s * 0.032075014954979206) * d2;
     vm = E - O;
     vp = E + O;
     dm = Do - De;
     dp = Do + De;
 }
 
-// Gas-kinetic flux at one Gauss point (local frame: index 0 normal, 1 and 2
-// tangential). The moments of f = g0 (1 - tau (a1 u + a2 v + a3 w + A) + A t)
-// with the coefficients solved from the slopes and compatibility (Appendix)
-// reduce to the closed form below (Chapman-Enskog structure, tau p = mu):
-//   a.u + A = (1/theta) d_i U_j (c_i c_j - theta delta_ij),   c = u - U,
-//   A = A0 + A_j c_j, A0 = -U.grad ln rho - div U,
-//   A_k = -d_k ln rho - 2 lambda U_i d_i U_k,
-//   F0 = (m_n, m_n U_k + p' delta_nk - mu (d_n U_k + d_k U_n)),
-//   F1 = rho (A0 U_n + theta A_n, A0 (U_n U_k + theta delta_nk) + theta (A_k U_n + A_n U_k)),
-// with p' = theta (rho - off): the constant theta off cancels in L.
-// D1 and D2 are index-space tangential slopes; ih1, ih2 turn them into
-// physical ones.
-template <typename R, bool NEED_F0>
-__device__ __forceinline__ void gk_flux(const Phys<R> &ph, const R q[4], const R Dn[4], const R D1[4],
-                                        const R D2[4], R ih1, R ih2, R F0[4], R F1[4])
-{
-    const R rho = ph.off + q[0];
-    const R inv = wdiv(R(1), rho);
-    const R inv1 = inv * ih1, inv2 = inv * ih2;
-    const R U0 = q[1] * inv, U1 = q[2] * inv, U2 = q[3] * inv;
-    const R g0 = Dn[0] * inv, g1 = D1[0] * inv1, g2 = D2[0] * inv2;
-    const R G00 = (Dn[1] - U0 * Dn[0]) * inv, G01 = (Dn[2] - U1 * Dn[0]) * inv,
-            G02 = (Dn[3] - U2 * Dn[0]) * inv;
-    const R G10 = (D1[1] - U0 * D1[0]) * inv1, G11 = (D1[2] - U1 * D1[0]) * inv1,
-            G12 = (D1[3] - U2 * D1[0]) * inv1;
-    const R G20 = (D2[1] - U0 * D2[0]) * inv2, G21 = (D2[2] - U1 * D2[0]) * inv2,
-            G22 = (D2[3] - U2 * D2[0]) * inv2;
-    const R th = ph.theta, tl = R(2) * ph.lambda;
-    const R A0 = -(U0 * g0 + U1 * g1 + U2 * g2) - (G00 + G11 + G22);
-    const R An = -g0 - tl * (U0 * G00 + U1 * G10 + U2 * G20);
-    const R A1 = -g1 - tl * (U0 * G01 + U1 * G11 + U2 * G21);
-    const R A2 = -g2 - tl * (U0 * G02 + U1 * G12 + U2 * G22);
-    if (NEED_F0) {
-        F0[0] = q[1];
-        F0[1] = q[1] * U0 + th * q[0] - ph.mu * (G00 + G00);
-        F0[2] = q[1] * U1 - ph.mu * (G01 + G10);
-        F0[3] = q[1] * U2 - ph.mu * (G02 + G20);
-    }
-    F1[0] = rho * (A0 * U0 + th * An);
-    F1[1] = rho * (A0 * (U0 * U0 + th) + th * (An * U0 + An * U0));
-    F1[2] = rho * (A0 * (U0 * U1) + th * (A1 * U0 + An * U1));
-    F1[3] = rho * (A0 * (U0 * U2) + th * (A2 * U0 + An * U2));
-}
-
 // ---- Packed FP32 pairs ----
 //
 // Two independent FP32 values that go through the same arithmetic (the two
-// t1 Gauss points of a face) as one float2: the FP32x2 add, multiply and
+// t2 Gauss points of a face) as one float2: the FP32x2 add, multiply and
 // fused multiply-add of sm_100 and later do both in one instruction, which
 // halves the issue slots of the arithmetic (the FP32 kernels are bound by
 // instruction issue, not by the FMA pipe). Every operation is rounded
@@ -638,52 +598,82 @@ __device__ __forceinline__ void face_equilibrium2(const Phys<float> &ph, const f
     Q0[1] = fma(R[1], Pr, L[1] * Pl);
 }
 
-__device__ __forceinline__ Phys<dsf2> pair_phys(const Phys<dsf> &p)
+// Gas-kinetic flux at one Gauss point (local frame: index 0 normal, 1 and 2
+// tangential), or at two at once (T = f2, dsf2). The moments of f = g0 (1 -
+// tau (a1 u + a2 v + a3 w + A) + A t) with the coefficients solved from the
+// slopes and compatibility (Appendix) reduce to a closed form (Chapman-Enskog
+// structure, tau p = mu):
+//   a.u + A = (1/theta) d_i U_j (c_i c_j - theta delta_ij),   c = u - U,
+//   A = A0 + A_j c_j, A0 = -U.grad ln rho - div U,
+//   A_k = -d_k ln rho - 2 lambda U_i d_i U_k,
+//   F0 = (m_n, m_n U_k + p' delta_nk - mu (d_n U_k + d_k U_n)),
+//   F1 = rho (A0 U_n + theta A_n, A0 (U_n U_k + theta delta_nk) + theta (A_k U_n + A_n U_k)),
+// with p' = theta (rho - off): the constant theta off cancels in L. It is
+// evaluated with rho multiplied through, so that a single reciprocal (for U)
+// is left and rho drops out of F1:
+//   H_ik = rho d_i U_k = d_i m_k - U_k d_i rho,
+//   B = -rho A0 = H_kk + U.grad rho,   C_k = -rho theta A_k = theta d_k rho + U_i H_ik,
+//   X = U_n B + C_n = -F1[0],
+//   -F1[k] = U_k X + U_n C_k + delta_nk theta B   (n: U_n X + C_n U_n + theta B),
+// 52 operations against the 77 of the form with G_ik = d_i U_k, A0 and A_k.
+// The density slopes Dn[0], D1[0] and D2[0] come negated (the t2 pass gives
+// them so for nothing), F1 is returned negated (nF1): no operation is spent
+// on a sign. D1 and D2 are index-space tangential slopes; ih1, ih2 turn them
+// into physical ones. What bounds the kernels that call it is the FMA pipe (FP32,
+// double-single) or the FP64 pipe, so operations are what counts.
+template <typename T>
+struct FluxPhys {
+    T off, th, nth, nmu;
+};
+template <typename T>
+__device__ __forceinline__ FluxPhys<T> flux_phys(const Phys<T> &p)
 {
-    Phys<dsf2> q;
-    q.lambda = dsf2(p.lambda);
-    q.theta = dsf2(p.theta);
-    q.mu = dsf2(p.mu);
-    q.off = dsf2(p.off);
-    q.sqlam = dsf2(p.sqlam);
-    q.kE = dsf2(p.kE);
-    return q;
+    return {p.off, p.theta, -p.theta, -p.mu};
 }
-
-// gk_flux at two Gauss points at once (the closed form above, every
-// multiply-add fused explicitly). ph holds the FP32 constants.
-template <bool NEED_F0>
-__device__ __forceinline__ void gk_flux2(const Phys<float> &ph, const f2 q[4], const f2 Dn[4], const f2 D1[4],
-                                         const f2 D2[4], f2 ih1, f2 ih2, f2 F0[4], f2 F1[4])
+__device__ __forceinline__ FluxPhys<f2> flux_phys_f2(const Phys<float> &p)
 {
-    const f2 m1(-1.0f);
-    const f2 rho = f2(ph.off) + q[0];
-    const f2 inv = wdiv(f2(1.0f), rho), ninv = inv * m1;
-    const f2 inv1 = inv * ih1, inv2 = inv * ih2, ninv1 = ninv * ih1, ninv2 = ninv * ih2;
-    const f2 U0 = q[1] * inv, U1 = q[2] * inv, U2 = q[3] * inv;
-    // the logarithmic density slopes, negated: -d_k ln rho
-    const f2 ng0 = Dn[0] * ninv, ng1 = D1[0] * ninv1, ng2 = D2[0] * ninv2;
-    // G_ik = d_i U_k = (d_i m_k) / rho - U_k d_i ln rho
-    const f2 G00 = fma(U0, ng0, Dn[1] * inv), G01 = fma(U1, ng0, Dn[2] * inv), G02 = fma(U2, ng0, Dn[3] * inv);
-    const f2 G10 = fma(U0, ng1, D1[1] * inv1), G11 = fma(U1, ng1, D1[2] * inv1), G12 = fma(U2, ng1, D1[3] * inv1);
-    const f2 G20 = fma(U0, ng2, D2[1] * inv2), G21 = fma(U1, ng2, D2[2] * inv2), G22 = fma(U2, ng2, D2[3] * inv2);
-    const f2 th(ph.theta), ntl(-2.0f * ph.lambda);
-    // A0 = -(U.g) - (G00 + G11 + G22); A_k = -g_k - 2 lambda U_i G_ik
-    const f2 A0 = fma(U2, ng2, fma(U1, ng1, U0 * ng0)) - ((G00 + G11) + G22);
-    const f2 An = fma(ntl, fma(U2, G20, fma(U1, G10, U0 * G00)), ng0);
-    const f2 A1 = fma(ntl, fma(U2, G21, fma(U1, G11, U0 * G01)), ng1);
-    const f2 A2 = fma(ntl, fma(U2, G22, fma(U1, G12, U0 * G02)), ng2);
+    return {f2(p.off), f2(p.theta), f2(-p.theta), f2(-p.mu)};
+}
+__device__ __forceinline__ FluxPhys<dsf2> flux_phys_ds2(const Phys<dsf> &p)
+{
+    return {dsf2(p.off), dsf2(p.theta), dsf2(-p.theta), dsf2(-p.mu)};
+}
+// rho and 1 / rho; FP64 grids store rho whole (off = 0)
+__device__ __forceinline__ f2 whole_rho(f2 off, f2 q) { return off + q; }
+__device__ __forceinline__ float whole_rho(float off, float q) { return __fadd_rn(off, q); }
+__device__ __forceinline__ double whole_rho(double, double q) { return q; }
+__device__ __forceinline__ dsf2 whole_rho(dsf2, dsf2 q) { return q; }
+__device__ __forceinline__ double inverse(double a) { return 1.0 / a; }
+__device__ __forceinline__ f2 inverse(f2 a) { return wrcp(a); }
+__device__ __forceinline__ dsf2 inverse(dsf2 a) { return dsf2(1.0) / a; }
+
+template <typename T, bool NEED_F0>
+__device__ __forceinline__ void gk_flux(const FluxPhys<T> &ph, const T q[4], const T Dn[4], const T D1[4],
+                                        const T D2[4], T ih1, T ih2, T F0[4], T nF1[4])
+{
+    const T inv = inverse(whole_rho(ph.off, q[0]));
+    const T U0 = q[1] * inv, U1 = q[2] * inv, U2 = q[3] * inv;
+    const T V1 = U1 * ih1, V2 = U2 * ih2;
+    const T H00 = fma(U0, Dn[0], Dn[1]), H01 = fma(U1, Dn[0], Dn[2]), H02 = fma(U2, Dn[0], Dn[3]);
+    const T H10 = fma(U0, D1[0], D1[1]), H11 = fma(U1, D1[0], D1[2]), H12 = fma(U2, D1[0], D1[3]);
+    const T H20 = fma(U0, D2[0], D2[1]), H21 = fma(U1, D2[0], D2[2]), H22 = fma(U2, D2[0], D2[3]);
+    const T S = fma(V2, D2[0], fma(V1, D1[0], U0 * Dn[0]));   // -U.grad rho
+    const T B = fma(ih2, H22, fma(ih1, H11, H00)) - S;
+    const T C0 = fma(ph.nth, Dn[0], fma(U0, H00, fma(V1, H10, V2 * H20)));
+    const T C1 = fma(ph.nth * ih1, D1[0], fma(U0, H01, fma(V1, H11, V2 * H21)));
+    const T C2 = fma(ph.nth * ih2, D2[0], fma(U0, H02, fma(V1, H12, V2 * H22)));
     if (NEED_F0) {
-        const f2 nmu(-ph.mu), n2mu(-2.0f * ph.mu);
+        const T nm = ph.nmu * inv;
         F0[0] = q[1];
-        F0[1] = fma(q[1], U0, fma(th, q[0], G00 * n2mu));
-        F0[2] = fma(q[1], U1, (G01 + G10) * nmu);
-        F0[3] = fma(q[1], U2, (G02 + G20) * nmu);
+        F0[1] = fma(q[1], U0, fma(ph.th, q[0], (H00 + H00) * nm));
+        F0[2] = fma(q[1], U1, fma(ih1, H10, H01) * nm);
+        F0[3] = fma(q[1], U2, fma(ih2, H20, H02) * nm);
     }
-    F1[0] = rho * fma(A0, U0, th * An);
-    F1[1] = rho * fma(A0, fma(U0, U0, th), f2(2.0f * ph.theta) * (An * U0));
-    F1[2] = rho * fma(A0, U0 * U1, th * fma(A1, U0, An * U1));
-    F1[3] = rho * fma(A0, U0 * U2, th * fma(A2, U0, An * U2));
+    const T X = fma(U0, B, C0);
+    nF1[0] = X;
+    nF1[1] = fma(U0, X, fma(C0, U0, ph.th * B));
+    nF1[2] = fma(U1, X, U0 * C1);
+    nF1[3] = fma(U2, X, U0 * C2);
 }
 
 constexpr int TX = 32, TY = 8;              // face tile

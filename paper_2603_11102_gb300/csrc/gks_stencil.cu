@@ -411,11 +411,14 @@ struct FluxArgs {
     Scalars *scal;
 };
 
-// The face average 1/4 sum of the Gauss-point fluxes in the storage type M.
-template <typename M, typename C>
-__device__ __forceinline__ M quarter(C acc) { return cvt<M>(acc) * M(0.25); }
-template <>
-__device__ __forceinline__ dsf quarter<dsf, dsf>(dsf acc) { return scale_pow2(acc, 0.25f); }
+// The face averages 1/4 sum of the Gauss-point fluxes: of F0, and of F1 from
+// the sum of -F1 (gk_flux).
+__device__ __forceinline__ double face_avg(double s) { return s * 0.25; }
+__device__ __forceinline__ float face_avg(float s) { return s * 0.25f; }
+__device__ __forceinline__ dsf face_avg(dsf s) { return scale_pow2(s, 0.25f); }
+__device__ __forceinline__ double face_avg_neg(double s) { return s * -0.25; }
+__device__ __forceinline__ float face_avg_neg(float s) { return s * -0.25f; }
+__device__ __forceinline__ dsf face_avg_neg(dsf s) { return scale_pow2(s, -0.25f); }
 
 // Tile t of the face box as (t1 tile, t2 tile, face): t = ta + NA (tb + NB f).
 struct TileIdx {
@@ -433,75 +436,71 @@ __device__ __forceinline__ TileIdx tile_add(TileIdx t, const TileIdx &g, int NA,
     return t;
 }
 
+// The t2 pass of component v at column (tx, ty) of the tile, t1 Gauss point
+// m: values and t2 slopes of Q0, values of the t1 slopes and of the normal
+// slope at the two t2 Gauss points -g, +g (k = 0, 1); the density's slopes
+// negated, as gk_flux takes them.
+template <typename R, int V>
+__device__ __forceinline__ void t2_pass(const R *st, int m, int tx, int ty, R q[2], R dn[2], R d1[2], R d2[2])
+{
+    constexpr bool NEG = V == 0;
+    const R *x = st + (V * 4 + m) * ST_ROWS + ty * TX + tx;
+    const R *y = st + (V * 4 + 2 + m) * ST_ROWS + ty * TX + tx;
+    const R *z = st + (16 + V * 2 + m) * ST_ROWS + ty * TX + tx;
+    tan_val_der<R, NEG>(x[0], x[TX], x[2 * TX], x[3 * TX], x[4 * TX], q[0], q[1], d2[0], d2[1]);
+    tan_val_direct<R, NEG>(y[0], y[TX], y[2 * TX], y[3 * TX], y[4 * TX], d1[0], d1[1]);
+    tan_val_direct<R, NEG>(z[0], z[TX], z[2 * TX], z[3 * TX], z[4 * TX], dn[0], dn[1]);
+}
+
 // t2 pass at each t1 Gauss point m, then the flux at (m, -g), (m, +g): the
-// sums of F0 and F1 over the 4 Gauss points of face (tx, ty) of the tile.
+// sums of F0 and of -F1 over the 4 Gauss points of face (tx, ty) of the tile.
 // GP (the recorded steps of the adjoint) with gp set: the inputs of Gauss
-// point g = 2m + n (Q0 with its density as rho, not rho - off; normal slope,
-// t1 and t2 slopes; 4 components each) go to gp[(16 g + k) ngp + face], as
-// double or (gp32) rounded to float (always float for R = float).
-template <typename R, bool NEED_F0, bool GP = false>
-__device__ __forceinline__ void tile_gauss_flux(const Phys<R> &ph, const R *st, int tx, int ty, R ih1, R ih2,
-                                                R acc0[4], R acc1[4], void *gp = nullptr, int gp32 = 0,
-                                                long ngp = 0, long face = 0)
+// point g = 2m + n (Q0 with its density as rho; normal slope, t1 and t2
+// slopes; 4 components each) go to gp[(16 g + k) ngp + face], as double or
+// (gp32) rounded to float.
+template <bool NEED_F0, bool GP = false>
+__device__ __forceinline__ void tile_gauss_flux(const FluxPhys<double> &ph, const double *st, int tx, int ty, double ih1,
+                                                double ih2, double acc0[4], double acc1[4], void *gp = nullptr,
+                                                int gp32 = 0, long ngp = 0, long face = 0)
 {
 #pragma unroll
-    for (int v = 0; v < 4; ++v) acc0[v] = acc1[v] = R(0);
+    for (int v = 0; v < 4; ++v) acc0[v] = acc1[v] = 0.0;
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
-        R Qv[2][4], Dn[2][4], D1[2][4], D2[2][4];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const R *x = st + (v * 4 + m) * ST_ROWS + ty * TX + tx;
-            const R *y = st + (v * 4 + 2 + m) * ST_ROWS + ty * TX + tx;
-            const R *z = st + (16 + v * 2 + m) * ST_ROWS + ty * TX + tx;
-            R vm, vp, dm, dp;
-            tan_val_der(x[0], x[TX], x[2 * TX], x[3 * TX], x[4 * TX], vm, vp, dm, dp);
-            Qv[0][v] = vm; Qv[1][v] = vp; D2[0][v] = dm; D2[1][v] = dp;
-            tan_val_direct(y[0], y[TX], y[2 * TX], y[3 * TX], y[4 * TX], vm, vp);
-            D1[0][v] = vm; D1[1][v] = vp;
-            tan_val_direct(z[0], z[TX], z[2 * TX], z[3 * TX], z[4 * TX], vm, vp);
-            Dn[0][v] = vm; Dn[1][v] = vp;
-        }
+        double t[4][4][2];   // [Q0, normal slope, t1 slope, t2 slope][component][t2 Gauss point]
+        t2_pass<double, 0>(st, m, tx, ty, t[0][0], t[1][0], t[2][0], t[3][0]);
+        t2_pass<double, 1>(st, m, tx, ty, t[0][1], t[1][1], t[2][1], t[3][1]);
+        t2_pass<double, 2>(st, m, tx, ty, t[0][2], t[1][2], t[2][2], t[3][2]);
+        t2_pass<double, 3>(st, m, tx, ty, t[0][3], t[1][3], t[2][3], t[3][3]);
         if constexpr (GP) {
-          if (gp) {
+            if (gp) {
 #pragma unroll
-            for (int nn = 0; nn < 2; ++nn) {
-                const long o = (long)(16 * (2 * m + nn)) * ngp + face;
-                const R q0 = Qv[nn][0] + ph.off;
-                if (sizeof(R) == 8 && !gp32) {
-                    R *p = (R *)gp + o;
-                    p[0] = q0;
+                for (int nn = 0; nn < 2; ++nn) {
+                    const long o = (long)(16 * (2 * m + nn)) * ngp + face;
 #pragma unroll
-                    for (int v = 1; v < 4; ++v) p[v * ngp] = Qv[nn][v];
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        p[(4 + v) * ngp] = Dn[nn][v];
-                        p[(8 + v) * ngp] = D1[nn][v];
-                        p[(12 + v) * ngp] = D2[nn][v];
-                    }
-                } else {
-                    float *p = (float *)gp + o;
-                    p[0] = (float)q0;
-#pragma unroll
-                    for (int v = 1; v < 4; ++v) p[v * ngp] = (float)Qv[nn][v];
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        p[(4 + v) * ngp] = (float)Dn[nn][v];
-                        p[(8 + v) * ngp] = (float)D1[nn][v];
-                        p[(12 + v) * ngp] = (float)D2[nn][v];
+                    for (int k = 0; k < 16; ++k) {
+                        // the density's slopes are recorded unnegated
+                        const double x = k >= 4 && k % 4 == 0 ? -t[k / 4][k % 4][nn] : t[k / 4][k % 4][nn];
+                        if (!gp32)
+                            ((double *)gp)[o + k * ngp] = x;
+                        else
+                            ((float *)gp)[o + k * ngp] = (float)x;
                     }
                 }
             }
-          }
         }
 #pragma unroll
         for (int nn = 0; nn < 2; ++nn) {
-            R F0[4], F1[4];
-            gk_flux<R, NEED_F0>(ph, Qv[nn], Dn[nn], D1[nn], D2[nn], ih1, ih2, F0, F1);
+            double q[4][4], F0[4], nF1[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) q[k][v] = t[k][v][nn];
+            gk_flux<double, NEED_F0>(ph, q[0], q[1], q[2], q[3], ih1, ih2, F0, nF1);
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
                 if (NEED_F0) acc0[v] += F0[v];
-                acc1[v] += F1[v];
+                acc1[v] += nF1[v];
             }
         }
     }
@@ -509,70 +508,80 @@ __device__ __forceinline__ void tile_gauss_flux(const Phys<R> &ph, const R *st, 
 
 // tile_gauss_flux for FP32 arithmetic: the same t2 pass, the flux at the two
 // t2 Gauss points of each t1 Gauss point as one packed evaluation.
+template <int V>
+__device__ __forceinline__ void t2_pass_f2(const float *st, int m, int tx, int ty, f2 &q, f2 &dn, f2 &d1, f2 &d2)
+{
+    float a[2], b[2], c[2], d[2];
+    t2_pass<float, V>(st, m, tx, ty, a, b, c, d);
+    q = f2(a[0], a[1]);
+    dn = f2(b[0], b[1]);
+    d1 = f2(c[0], c[1]);
+    d2 = f2(d[0], d[1]);
+}
 template <bool NEED_F0>
-__device__ __forceinline__ void tile_gauss_flux_f32(const Phys<float> &ph, const float *st, int tx, int ty, float ih1,
+__device__ __forceinline__ void tile_gauss_flux_f32(const FluxPhys<f2> &ph, const float *st, int tx, int ty, float ih1,
                                                     float ih2, float acc0[4], float acc1[4])
 {
-#pragma unroll
-    for (int v = 0; v < 4; ++v) acc0[v] = acc1[v] = 0.0f;
+    f2 s0[4], s1[4];   // the t2 Gauss points -g, +g in the lanes
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
-        f2 Qv[4], Dn[4], D1[4], D2[4];   // t2 Gauss points -g, +g in the lanes
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const float *x = st + (v * 4 + m) * ST_ROWS + ty * TX + tx;
-            const float *y = st + (v * 4 + 2 + m) * ST_ROWS + ty * TX + tx;
-            const float *z = st + (16 + v * 2 + m) * ST_ROWS + ty * TX + tx;
-            tan_val_der(x[0], x[TX], x[2 * TX], x[3 * TX], x[4 * TX], Qv[v].v.x, Qv[v].v.y, D2[v].v.x, D2[v].v.y);
-            tan_val_direct(y[0], y[TX], y[2 * TX], y[3 * TX], y[4 * TX], D1[v].v.x, D1[v].v.y);
-            tan_val_direct(z[0], z[TX], z[2 * TX], z[3 * TX], z[4 * TX], Dn[v].v.x, Dn[v].v.y);
-        }
+        f2 Qv[4], Dn[4], D1[4], D2[4];
+        t2_pass_f2<0>(st, m, tx, ty, Qv[0], Dn[0], D1[0], D2[0]);
+        t2_pass_f2<1>(st, m, tx, ty, Qv[1], Dn[1], D1[1], D2[1]);
+        t2_pass_f2<2>(st, m, tx, ty, Qv[2], Dn[2], D1[2], D2[2]);
+        t2_pass_f2<3>(st, m, tx, ty, Qv[3], Dn[3], D1[3], D2[3]);
         f2 F0[4], F1[4];
-        gk_flux2<NEED_F0>(ph, Qv, Dn, D1, D2, f2(ih1), f2(ih2), F0, F1);
+        gk_flux<f2, NEED_F0>(ph, Qv, Dn, D1, D2, f2(ih1), f2(ih2), F0, F1);
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            if (NEED_F0) acc0[v] += F0[v].v.x + F0[v].v.y;
-            acc1[v] += F1[v].v.x + F1[v].v.y;
+            if (NEED_F0) s0[v] = m == 0 ? F0[v] : s0[v] + F0[v];
+            s1[v] = m == 0 ? F1[v] : s1[v] + F1[v];
         }
+    }
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        if (NEED_F0) acc0[v] = s0[v].v.x + s0[v].v.y;
+        acc1[v] = s1[v].v.x + s1[v].v.y;
     }
 }
 
 // tile_gauss_flux for double-single arithmetic (no Gauss-point output): the
 // same t2 pass, the flux at the two t2 Gauss points of each t1 Gauss point
-// as one evaluation on packed double-single pairs, summed in the same order
-// (the same bits).
-template <bool NEED_F0>
-__device__ __forceinline__ void tile_gauss_flux_ds2(const Phys<dsf> &ph, const Phys<dsf2> &ph2, const dsf *st, int tx,
-                                                    int ty, dsf ih1, dsf ih2, dsf acc0[4], dsf acc1[4])
+// as one evaluation on packed double-single pairs.
+template <int V>
+__device__ __forceinline__ void t2_pass_ds2(const dsf *st, int m, int tx, int ty, dsf2 &q, dsf2 &dn, dsf2 &d1, dsf2 &d2)
 {
-#pragma unroll
-    for (int v = 0; v < 4; ++v) acc0[v] = acc1[v] = dsf(0);
+    dsf a[2], b[2], c[2], d[2];
+    t2_pass<dsf, V>(st, m, tx, ty, a, b, c, d);
+    q = dsf2(a[0], a[1]);
+    dn = dsf2(b[0], b[1]);
+    d1 = dsf2(c[0], c[1]);
+    d2 = dsf2(d[0], d[1]);
+}
+template <bool NEED_F0>
+__device__ __forceinline__ void tile_gauss_flux_ds2(const FluxPhys<dsf2> &ph, const dsf *st, int tx, int ty, dsf ih1,
+                                                    dsf ih2, dsf acc0[4], dsf acc1[4])
+{
+    dsf2 s0[4], s1[4];   // the t2 Gauss points -g, +g in the lanes
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
-        dsf2 Qv[4], Dn[4], D1[4], D2[4];   // t2 Gauss points -g, +g in the lanes
+        dsf2 Qv[4], Dn[4], D1[4], D2[4];
+        t2_pass_ds2<0>(st, m, tx, ty, Qv[0], Dn[0], D1[0], D2[0]);
+        t2_pass_ds2<1>(st, m, tx, ty, Qv[1], Dn[1], D1[1], D2[1]);
+        t2_pass_ds2<2>(st, m, tx, ty, Qv[2], Dn[2], D1[2], D2[2]);
+        t2_pass_ds2<3>(st, m, tx, ty, Qv[3], Dn[3], D1[3], D2[3]);
+        dsf2 F0[4], F1[4];
+        gk_flux<dsf2, NEED_F0>(ph, Qv, Dn, D1, D2, dsf2(ih1), dsf2(ih2), F0, F1);
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            const dsf *x = st + (v * 4 + m) * ST_ROWS + ty * TX + tx;
-            const dsf *y = st + (v * 4 + 2 + m) * ST_ROWS + ty * TX + tx;
-            const dsf *z = st + (16 + v * 2 + m) * ST_ROWS + ty * TX + tx;
-            dsf vm, vp, dm, dp;
-            tan_val_der(x[0], x[TX], x[2 * TX], x[3 * TX], x[4 * TX], vm, vp, dm, dp);
-            Qv[v] = dsf2(vm, vp);
-            D2[v] = dsf2(dm, dp);
-            tan_val_direct(y[0], y[TX], y[2 * TX], y[3 * TX], y[4 * TX], vm, vp);
-            D1[v] = dsf2(vm, vp);
-            tan_val_direct(z[0], z[TX], z[2 * TX], z[3 * TX], z[4 * TX], vm, vp);
-            Dn[v] = dsf2(vm, vp);
+            if (NEED_F0) s0[v] = m == 0 ? F0[v] : s0[v] + F0[v];
+            s1[v] = m == 0 ? F1[v] : s1[v] + F1[v];
         }
-        dsf2 F0[4], F1[4];
-        gk_flux<dsf2, NEED_F0>(ph2, Qv, Dn, D1, D2, dsf2(ih1), dsf2(ih2), F0, F1);
+    }
 #pragma unroll
-        for (int nn = 0; nn < 2; ++nn)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                if (NEED_F0) acc0[v] += F0[v].lane(nn);
-                acc1[v] += F1[v].lane(nn);
-            }
+    for (int v = 0; v < 4; ++v) {
+        if (NEED_F0) acc0[v] = s0[v].lane(0) + s0[v].lane(1);
+        acc1[v] = s1[v].lane(0) + s1[v].lane(1);
     }
 }
 
@@ -629,72 +638,84 @@ __global__ void __launch_bounds__(256, std::is_same<C, dsf>::value ? 2 : 1)
             const C ih1 = cvt<C>(__ldg(A.ih1 + a + G)), ih2 = cvt<C>(__ldg(A.ih2 + b + G));
             C acc0[4], acc1[4];
             const long o = ((long)f * A.n2 + b) * A.n1 + a;
-            if constexpr (std::is_same<C, dsf>::value && !GP)
-                tile_gauss_flux_ds2<NEED_F0>(A.ph, pair_phys(A.ph), st, tx, ty, ih1, ih2, acc0, acc1);
+            if constexpr (std::is_same<C, dsf>::value)
+                tile_gauss_flux_ds2<NEED_F0>(flux_phys_ds2(A.ph), st, tx, ty, ih1, ih2, acc0, acc1);
             else
-                tile_gauss_flux<C, NEED_F0, GP>(A.ph, st, tx, ty, ih1, ih2, acc0, acc1, A.gp, A.gp32, A.ngp, o);
+                tile_gauss_flux<NEED_F0, GP>(flux_phys(A.ph), st, tx, ty, ih1, ih2, acc0, acc1, A.gp, A.gp32, A.ngp, o);
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
                 if (!in_bounds(o, A.nff)) break;
-                if (NEED_F0) A.ff[A.gcomp[v] * A.nff + o] = quarter<M>(acc0[v]);
-                A.ff[(4 + A.gcomp[v]) * A.nff + o] = quarter<M>(acc1[v]);
+                if (NEED_F0) A.ff[A.gcomp[v] * A.nff + o] = face_avg(acc0[v]);
+                A.ff[(4 + A.gcomp[v]) * A.nff + o] = face_avg_neg(acc1[v]);
             }
         }
         __syncthreads();   // st and this buffer are free again
     }
 }
 
-// The t2 pass and the flux of the two faces (tx, r0) and (tx, r0 + 1) of a
-// tall tile (FP32C): each row array is read once over the 6 rows r0 .. r0+5
-// that the two 5-point stencils cover; the sums of F0 and F1 over the 4
-// Gauss points of each face, in the order of tile_gauss_flux.
+// The t2 pass of component V of the two faces (tx, r0) and (tx, r0 + 1) of a
+// tall tile (t2_pass, e = 0, 1): each row array is read once over the 6 rows
+// r0 .. r0+5 that the two 5-point stencils cover.
+template <int V>
+__device__ __forceinline__ void t2_pass_two(const float *st, int m, int tx, int r0, f2 q[2][4], f2 dn[2][4], f2 d1[2][4],
+                                            f2 d2[2][4])
+{
+    constexpr bool NEG = V == 0;
+    const float *x = st + (V * 4 + m) * ST_ROWS_T + r0 * TX + tx;
+    const float *y = st + (V * 4 + 2 + m) * ST_ROWS_T + r0 * TX + tx;
+    const float *z = st + (16 + V * 2 + m) * ST_ROWS_T + r0 * TX + tx;
+    float p[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) p[i] = x[i * TX];
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+        tan_val_der<float, NEG>(p[e], p[e + 1], p[e + 2], p[e + 3], p[e + 4], q[e][V].v.x, q[e][V].v.y, d2[e][V].v.x,
+                                d2[e][V].v.y);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) p[i] = y[i * TX];
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+        tan_val_direct<float, NEG>(p[e], p[e + 1], p[e + 2], p[e + 3], p[e + 4], d1[e][V].v.x, d1[e][V].v.y);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) p[i] = z[i * TX];
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+        tan_val_direct<float, NEG>(p[e], p[e + 1], p[e + 2], p[e + 3], p[e + 4], dn[e][V].v.x, dn[e][V].v.y);
+}
+
+// The flux of the two faces (tx, r0) and (tx, r0 + 1) of a tall tile (FP32C):
+// the sums of F0 and -F1 over the 4 Gauss points of each face.
 template <bool NEED_F0>
-__device__ __forceinline__ void tile_gauss_flux_pair(const Phys<float> &ph, const float *st, int tx, int r0,
+__device__ __forceinline__ void tile_gauss_flux_pair(const FluxPhys<f2> &ph, const float *st, int tx, int r0,
                                                      float ih1, const float ih2[2], float acc0[2][4],
                                                      float acc1[2][4])
 {
-#pragma unroll
-    for (int e = 0; e < 2; ++e)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc0[e][v] = acc1[e][v] = 0.0f;
+    f2 s0[2][4], s1[2][4];   // the two t2 Gauss points -g, +g in the lanes
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
-        // [face][component], the two t2 Gauss points -g, +g in the lanes of a pair
-        f2 Qv[2][4], Dn[2][4], D1[2][4], D2[2][4];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const float *x = st + (v * 4 + m) * ST_ROWS_T + r0 * TX + tx;
-            const float *y = st + (v * 4 + 2 + m) * ST_ROWS_T + r0 * TX + tx;
-            const float *z = st + (16 + v * 2 + m) * ST_ROWS_T + r0 * TX + tx;
-            float p[6];
-#pragma unroll
-            for (int i = 0; i < 6; ++i) p[i] = x[i * TX];
-#pragma unroll
-            for (int e = 0; e < 2; ++e)
-                tan_val_der(p[e], p[e + 1], p[e + 2], p[e + 3], p[e + 4], Qv[e][v].v.x, Qv[e][v].v.y, D2[e][v].v.x,
-                            D2[e][v].v.y);
-#pragma unroll
-            for (int i = 0; i < 6; ++i) p[i] = y[i * TX];
-#pragma unroll
-            for (int e = 0; e < 2; ++e)
-                tan_val_direct(p[e], p[e + 1], p[e + 2], p[e + 3], p[e + 4], D1[e][v].v.x, D1[e][v].v.y);
-#pragma unroll
-            for (int i = 0; i < 6; ++i) p[i] = z[i * TX];
-#pragma unroll
-            for (int e = 0; e < 2; ++e)
-                tan_val_direct(p[e], p[e + 1], p[e + 2], p[e + 3], p[e + 4], Dn[e][v].v.x, Dn[e][v].v.y);
-        }
+        f2 Qv[2][4], Dn[2][4], D1[2][4], D2[2][4];   // [face][component]
+        t2_pass_two<0>(st, m, tx, r0, Qv, Dn, D1, D2);
+        t2_pass_two<1>(st, m, tx, r0, Qv, Dn, D1, D2);
+        t2_pass_two<2>(st, m, tx, r0, Qv, Dn, D1, D2);
+        t2_pass_two<3>(st, m, tx, r0, Qv, Dn, D1, D2);
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             f2 F0[4], F1[4];
-            gk_flux2<NEED_F0>(ph, Qv[e], Dn[e], D1[e], D2[e], f2(ih1), f2(ih2[e]), F0, F1);
+            gk_flux<f2, NEED_F0>(ph, Qv[e], Dn[e], D1[e], D2[e], f2(ih1), f2(ih2[e]), F0, F1);
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
-                if (NEED_F0) acc0[e][v] += F0[v].v.x + F0[v].v.y;
-                acc1[e][v] += F1[v].v.x + F1[v].v.y;
+                if (NEED_F0) s0[e][v] = m == 0 ? F0[v] : s0[e][v] + F0[v];
+                s1[e][v] = m == 0 ? F1[v] : s1[e][v] + F1[v];
             }
         }
     }
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            if (NEED_F0) acc0[e][v] = s0[e][v].v.x + s0[e][v].v.y;
+            acc1[e][v] = s1[e][v].v.x + s1[e][v].v.y;
+        }
 }
 
 // face_flux_kernel on 32 x 16 tiles for FP32C grids (the same results bit
@@ -745,15 +766,15 @@ __global__ void __launch_bounds__(256, 2) face_flux_tall_kernel(const __grid_con
             const float ih1 = __ldg(A.ih1 + a + G);
             const float ih2[2] = {__ldg(A.ih2 + b + G), __ldg(A.ih2 + b + 1 + G)};
             float acc0[2][4], acc1[2][4];
-            tile_gauss_flux_pair<NEED_F0>(A.ph, st, tx, 2 * ty, ih1, ih2, acc0, acc1);
+            tile_gauss_flux_pair<NEED_F0>(flux_phys_f2(A.ph), st, tx, 2 * ty, ih1, ih2, acc0, acc1);
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 const long o = ((long)f * A.n2 + b + e) * A.n1 + a;
                 if (b + e >= A.n2 || !in_bounds(o, A.nff)) break;
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
-                    if (NEED_F0) A.ff[A.gcomp[v] * A.nff + o] = acc0[e][v] * 0.25f;
-                    A.ff[(4 + A.gcomp[v]) * A.nff + o] = acc1[e][v] * 0.25f;
+                    if (NEED_F0) A.ff[A.gcomp[v] * A.nff + o] = face_avg(acc0[e][v]);
+                    A.ff[(4 + A.gcomp[v]) * A.nff + o] = face_avg_neg(acc1[e][v]);
                 }
             }
         }
@@ -1050,15 +1071,15 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
         M F0[4], F1[4];
         if (in) {
             C G0[4], G1[4];
-            if constexpr (std::is_same<C, float>::value && !GP)
-                tile_gauss_flux_f32<NEED_F0>(A.ph, st, tx, ty, ih1, ih2, G0, G1);
+            if constexpr (std::is_same<C, float>::value)
+                tile_gauss_flux_f32<NEED_F0>(flux_phys_f2(A.ph), st, tx, ty, ih1, ih2, G0, G1);
             else
-                tile_gauss_flux<C, NEED_F0, GP>(A.ph, st, tx, ty, cvt<C>(ih1), cvt<C>(ih2), G0, G1, A.gp, A.gp32,
-                                                A.ngp, ((long)f * A.n2 + b) * A.n1 + a);
+                tile_gauss_flux<NEED_F0, GP>(flux_phys(A.ph), st, tx, ty, ih1, ih2, G0, G1, A.gp, A.gp32, A.ngp,
+                                             ((long)f * A.n2 + b) * A.n1 + a);
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
-                F0[v] = NEED_F0 ? quarter<M>(G0[v]) : M(0);
-                F1[v] = quarter<M>(G1[v]);
+                F0[v] = NEED_F0 ? face_avg(G0[v]) : M(0);
+                F1[v] = face_avg_neg(G1[v]);
             }
         }
         if (upd) {
@@ -1208,26 +1229,28 @@ int persistent_grid(K kernel, size_t smem)
 template <typename R, typename C, int STAGE>
 struct FluxGrids {
     int flux[2] = {0, 0}, flux_update[2] = {0, 0};   // without / with the Gauss-point output
-    int flux_tall = 0;                               // FP32C: 32 x 16 face tiles
 };
 
-// The Gauss-point output (recorded steps of the adjoint) exists only where the
-// arithmetic type is the storage type.
+// The Gauss-point output (recorded steps of the adjoint) exists only in FP64
+// arithmetic.
 template <typename R, typename C, int STAGE>
 const FluxGrids<R, C, STAGE> &flux_grids()
 {
     static FluxGrids<R, C, STAGE> g;
     if (!g.flux[0]) {
         constexpr size_t su = flux_update_smem_bytes<R>(STAGE == 1 ? 8 : 4);
-        g.flux[0] = persistent_grid(face_flux_kernel<R, C, STAGE == 1, false>, flux_smem_bytes<R>());
+        if constexpr (std::is_same<C, float>::value) {
+            // FP32C: 32 x 16 face tiles in x and y
+            g.flux[0] = persistent_grid(face_flux_tall_kernel<STAGE == 1>, flux_tall_smem_bytes());
+        } else {
+            g.flux[0] = persistent_grid(face_flux_kernel<R, C, STAGE == 1, false>, flux_smem_bytes<R>());
+        }
         if constexpr (!std::is_same<C, dsf>::value)   // double-single: separate z update
             g.flux_update[0] = persistent_grid(flux_update_kernel<R, C, STAGE, false>, su);
-        if constexpr (std::is_same<R, C>::value) {
+        if constexpr (std::is_same<C, double>::value) {
             g.flux[1] = persistent_grid(face_flux_kernel<R, C, STAGE == 1, true>, flux_smem_bytes<R>());
             g.flux_update[1] = persistent_grid(flux_update_kernel<R, C, STAGE, true>, su);
         }
-        if constexpr (std::is_same<R, float>::value && std::is_same<C, float>::value)
-            g.flux_tall = persistent_grid(face_flux_tall_kernel<STAGE == 1>, flux_tall_smem_bytes());
     }
     return g;
 }
@@ -1357,8 +1380,8 @@ void stage_impl(const Ctx &c)
         const long ntiles = (long)((F.n1 + TX - 1) / TX) * ((F.n2 + TY - 1) / TY) * F.nf;
         const int grp = d < 2 ? K_FACE_FLUX : K_FLUX_UPDATE;
         mark(c, grp, 1);
-        const int gpo = F.gp != nullptr;
-        if constexpr (!std::is_same<R, C>::value) F.gp = nullptr;
+        constexpr bool FP64A = std::is_same<C, double>::value;
+        const int gpo = FP64A && F.gp;
         if constexpr (std::is_same<C, dsf>::value) {
             if (d == 2) {
                 // double-single: z-face fluxes into their own buffer, then the update
@@ -1376,25 +1399,18 @@ void stage_impl(const Ctx &c)
             }
         }
         if (d < 2) {
-            const int grid = (int)(ntiles < grids.flux[gpo] ? ntiles : grids.flux[gpo]);
-            if constexpr (std::is_same<R, float>::value && std::is_same<C, float>::value) {
-                if (!gpo) {
-                    const long nt = (long)((F.n1 + TX - 1) / TX) * ((F.n2 + TYT - 1) / TYT) * F.nf;
-                    const int gt = (int)(nt < grids.flux_tall ? nt : grids.flux_tall);
-                    face_flux_tall_kernel<STAGE == 1><<<gt, blk, flux_tall_smem_bytes(), c.stream>>>(c.tmapT[d], F);
-                    mark(c, grp, 0);
-                    continue;
-                }
-            }
-            if constexpr (std::is_same<R, C>::value) {
-                if (gpo)
-                    face_flux_kernel<R, C, STAGE == 1, true><<<grid, blk, flux_smem_bytes<R>(), c.stream>>>(tmap, F);
+            if constexpr (std::is_same<C, float>::value) {
+                const long nt = (long)((F.n1 + TX - 1) / TX) * ((F.n2 + TYT - 1) / TYT) * F.nf;
+                const int gt = (int)(nt < grids.flux[0] ? nt : grids.flux[0]);
+                face_flux_tall_kernel<STAGE == 1><<<gt, blk, flux_tall_smem_bytes(), c.stream>>>(c.tmapT[d], F);
+            } else {
+                const int grid = (int)(ntiles < grids.flux[gpo] ? ntiles : grids.flux[gpo]);
+                if (FP64A && gpo)
+                    face_flux_kernel<R, C, STAGE == 1, FP64A><<<grid, blk, flux_smem_bytes<R>(), c.stream>>>(tmap, F);
                 else
                     face_flux_kernel<R, C, STAGE == 1, false><<<grid, blk, flux_smem_bytes<R>(), c.stream>>>(tmap, F);
-            } else {
-                face_flux_kernel<R, C, STAGE == 1, false><<<grid, blk, flux_smem_bytes<R>(), c.stream>>>(tmap, F);
             }
-        } else {
+        } else if constexpr (!std::is_same<C, dsf>::value) {
             // z faces: flux and the stage update of every cell
             UpdArgs<R, Mid<R, C>> U = update_args<R, C, STAGE>(c, F);
             const int ncol = ((F.n1 + TX - 1) / TX) * ((F.n2 + TY - 1) / TY);
@@ -1402,12 +1418,10 @@ void stage_impl(const Ctx &c)
             const long nitems = (long)ncol * ((F.nf + U.seg - 1) / U.seg);
             const int grid = (int)(nitems < grids.flux_update[gpo] ? nitems : grids.flux_update[gpo]);
             constexpr size_t su = flux_update_smem_bytes<R>(STAGE == 1 ? 8 : 4);
-            if constexpr (std::is_same<R, C>::value) {
-                if (gpo)
-                    flux_update_kernel<R, C, STAGE, true><<<grid, blk, su, c.stream>>>(tmap, F, U);
-                else
-                    flux_update_kernel<R, C, STAGE, false><<<grid, blk, su, c.stream>>>(tmap, F, U);
-            }
+            if (FP64A && gpo)
+                flux_update_kernel<R, C, STAGE, FP64A><<<grid, blk, su, c.stream>>>(tmap, F, U);
+            else
+                flux_update_kernel<R, C, STAGE, false><<<grid, blk, su, c.stream>>>(tmap, F, U);
         }
         mark(c, grp, 0);
     }
