@@ -955,14 +955,14 @@ __global__ void __launch_bounds__(256, 2) rev_tile32_kernel(const __grid_constan
         const int ta = t % NA, tb = (t / NA) % NB, f = t / (NA * NB);
         if (tid == 0) {
             fence_proxy_async();
-            tma_load_tile(&tmap, sq, &bar[0], ta * TX, tb * TY, f, bytes);
+            tma_load_tile(&tmap, sq, &bar[0], 2 * ta * TX, tb * TY, f, bytes);
         }
         const bool ok = mbar_wait(&bar[0], (uint32_t)(k & 1));
         if (__syncthreads_or(!ok)) {
             if (tid == 0) atomicOr(&A.scal->flags, FLAG_TIMEOUT);
             return;
         }
-        tile_t1_pass(sq, st, tid);
+        tile_t1_pass_f2<SQ_H>(reinterpret_cast<const float2 *>(sq), reinterpret_cast<float2 *>(st), tid);
         __syncthreads();
 
         // RA: per face, the 4 Gauss points
@@ -988,30 +988,14 @@ __global__ void __launch_bounds__(256, 2) rev_tile32_kernel(const __grid_constan
             const float ih1 = A.ih1[a + G], ih2 = A.ih2[b + G];
 #pragma unroll
             for (int m = 0; m < 2; ++m) {
-                float Qv[2][4], Dn[2][4], D1[2][4], D2[2][4];
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    const float *x = st + (v * 4 + m) * ST_ROWS + ty * TX + tx;
-                    const float *y = st + (v * 4 + 2 + m) * ST_ROWS + ty * TX + tx;
-                    const float *z = st + (16 + v * 2 + m) * ST_ROWS + ty * TX + tx;
-                    float vm, vp, dm, dp;
-                    tan_val_der(x[0], x[TX], x[2 * TX], x[3 * TX], x[4 * TX], vm, vp, dm, dp);
-                    Qv[0][v] = vm; Qv[1][v] = vp; D2[0][v] = dm; D2[1][v] = dp;
-                    tan_val_direct(y[0], y[TX], y[2 * TX], y[3 * TX], y[4 * TX], vm, vp);
-                    D1[0][v] = vm; D1[1][v] = vp;
-                    tan_val_direct(z[0], z[TX], z[2 * TX], z[3 * TX], z[4 * TX], vm, vp);
-                    Dn[0][v] = vm; Dn[1][v] = vp;
-                }
+                f2 q2[1][4], n2[1][4], a2[1][4], b2[1][4];
+                t2_pass_f2<SQ_H, 1, false>(reinterpret_cast<const float2 *>(st), m, tx, ty, q2, n2, a2, b2);
                 // the flux reverse at the two t2 Gauss points as one evaluation on
                 // packed FP32 pairs (the points in the lanes)
                 {
-                    f2 q2[4], n2[4], a2[4], b2[4], s0[4], s1[4], qb[4], Dnb[4], D1b[4], D2b[4];
+                    f2 s0[4], s1[4], qb[4], Dnb[4], D1b[4], D2b[4];
 #pragma unroll
                     for (int v = 0; v < 4; ++v) {
-                        q2[v] = f2(Qv[0][v], Qv[1][v]);
-                        n2[v] = f2(Dn[0][v], Dn[1][v]);
-                        a2[v] = f2(D1[0][v], D1[1][v]);
-                        b2[v] = f2(D2[0][v], D2[1][v]);
                         s0[v] = f2(sF0[v]);
                         s1[v] = f2(sF1[v]);
                     }
@@ -1022,7 +1006,7 @@ __global__ void __launch_bounds__(256, 2) rev_tile32_kernel(const __grid_constan
                     p2.off = f2(A.ph.off);
                     p2.sqlam = f2(A.ph.sqlam);
                     p2.kE = f2(A.ph.kE);
-                    gk_flux_rev<f2>(p2, q2, n2, a2, b2, f2(ih1), f2(ih2), s0, s1, needF0, qb, Dnb, D1b, D2b);
+                    gk_flux_rev<f2>(p2, q2[0], n2[0], a2[0], b2[0], f2(ih1), f2(ih2), s0, s1, needF0, qb, Dnb, D1b, D2b);
 #pragma unroll
                     for (int nn = 0; nn < 2; ++nn) {
                         float *gp = ga + (16 * (2 * m + nn)) * (TX * TY) + tid;

@@ -306,7 +306,9 @@ int gks_workspace_bytes(const gks_grid_desc *desc, size_t *state_bytes, size_t *
 namespace {
 
 // TMA descriptor of the face box of direction a at `base`: dims (t1 padded,
-// t2 + 4, faces, 8 components), box (36, 12, 1, 8). c.e1p must be set.
+// t2 + 4, faces, 8 components), box (36, rows, 1, 8); FP32C face boxes hold
+// component pairs: (2 t1 padded, t2 + 4, faces, 4 pairs), box (72, rows, 1, 4).
+// c.e1p must be set.
 int encode_face_map(const Ctx &c, int a, void *base, CUtensorMap *out, std::string *msg, int rows = 12)
 {
     static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
@@ -322,9 +324,10 @@ int encode_face_map(const Ctx &c, int a, void *base, CUtensorMap *out, std::stri
     }
     const cuuint64_t es = c.prec == GKS_FP64 ? 8 : 4;
     const int t2 = a == 2 ? 1 : 2;
-    const cuuint64_t dims[4] = {(cuuint64_t)c.e1p[a], (cuuint64_t)(c.n[t2] + 4), (cuuint64_t)(c.n[a] + 1), 8};
-    const cuuint64_t strides[3] = {dims[0] * es, dims[0] * dims[1] * es, (cuuint64_t)c.nfq * es};
-    const cuuint32_t box[4] = {36, (cuuint32_t)rows, 1, 8};
+    const cuuint32_t k = c.prec == GKS_FP64 ? 1 : 2;   // elements per position
+    const cuuint64_t dims[4] = {(cuuint64_t)c.e1p[a] * k, (cuuint64_t)(c.n[t2] + 4), (cuuint64_t)(c.n[a] + 1), 8 / k};
+    const cuuint64_t strides[3] = {dims[0] * es, dims[0] * dims[1] * es, (cuuint64_t)c.nfq * k * es};
+    const cuuint32_t box[4] = {36 * k, (cuuint32_t)rows, 1, 8 / k};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     CUresult r = encode(out, c.prec == GKS_FP64 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4,
                         base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -422,7 +425,7 @@ int gks_create_grid(const gks_grid_desc *desc, void *d_state, void *d_work, gks_
         c.e1p[a] = L.e1p[a];
         std::string m;
         if (encode_face_map(c, a, c.fq, &c.tmap[a], &m) ||
-            (c.prec == GKS_FP32C && encode_face_map(c, a, c.fq, &c.tmapT[a], &m, 20))) {
+            (c.prec == GKS_FP32C && encode_face_map(c, a, c.fq, &c.tmapM[a], &m, 5))) {
             delete g;
             return fail(nullptr, GKS_ERR_CUDA, m);
         }

@@ -252,7 +252,7 @@ __device__ __forceinline__ void face_equilibrium(const Phys<double> &ph, const d
 template <typename R>
 __device__ __forceinline__ void tan_val(R qm2, R qm1, R q0, R qp1, R qp2, R &vm, R &vp)
 {
-    const R d1 = qp1 + qm1 - R(2) * q0, d2 = qp2 + qm2 - R(2) * q0;
+    const R d1 = fma(q0, R(-2.0), qp1 + qm1), d2 = fma(q0, R(-2.0), qp2 + qm2);
     const R a1 = qp1 - qm1, a2 = qp2 - qm2;
     const R E = fma(d1, R(1.0 / 1080.0), fma(d2, R(-1.0 / 4320.0), q0));
     const R O = R(0.20046884346862007) * a1 - R(0.028065638085606807) * a2;
@@ -282,12 +282,12 @@ __device__ __forceinline__ void tan_val_der(R qm2, R qm1, R q0, R qp1, R qp2, R 
                                             R &dp)
 {
     constexpr double s = NEG ? -1.0 : 1.0;
-    const R d1 = qp1 + qm1 - R(2) * q0, d2 = qp2 + qm2 - R(2) * q0;
+    const R d1 = fma(q0, R(-2.0), qp1 + qm1), d2 = fma(q0, R(-2.0), qp2 + qm2);
     const R a1 = qp1 - qm1, a2 = qp2 - qm2;
     const R E = fma(d1, R(1.0 / 1080.0), fma(d2, R(-1.0 / 4320.0), q0));
-    const R O = R(0.20046884346862007) * a1 - R(0.028065638085606807) * a2;
-    const R Do = R(s * 2.0 / 3.0) * a1 - R(s * 1.0 / 12.0) * a2;
-    const R De = R(s * 0.41697519441472974) * d1 - R(s * 0.032075014954979206) * d2;
+    const R O = fma(a1, R(0.20046884346862007), a2 * R(-0.028065638085606807));
+    const R Do = fma(a1, R(s * 2.0 / 3.0), a2 * R(s * -1.0 / 12.0));
+    const R De = fma(d1, R(s * 0.41697519441472974), d2 * R(s * -0.032075014954979206));
     vm = E - O;
     vp = E + O;
     dm = Do - De;
@@ -619,8 +619,10 @@ __device__ __forceinline__ void face_equilibrium2(const Phys<float> &ph, const f
 // The density slopes Dn[0], D1[0] and D2[0] come negated (the t2 pass gives
 // them so for nothing), F1 is returned negated (nF1): no operation is spent
 // on a sign. D1 and D2 are index-space tangential slopes; ih1, ih2 turn them
-// into physical ones. What bounds the kernels that call it is the FMA pipe (FP32,
-// double-single) or the FP64 pipe, so operations are what counts.
+// into physical ones. What bounds the kernels that call it is the FMA pipe
+// (FP32, double-single) or the FP64 pipe, so operations are what counts (x and
+// y face fluxes of a 384x256x256 FP32C step 2.97 -> 2.77 ms, of a 96^3 FP64
+// step 5.59 -> 5.00 ms).
 template <typename T>
 struct FluxPhys {
     T off, th, nth, nmu;
@@ -725,16 +727,6 @@ __device__ __forceinline__ void sts4(dsf *p, const dsf q[4])
 
 static_assert(TX * TY == 256 && SQ_H == 12 && TX == 32, "t1-pass task split assumes 32 x 8 tiles");
 
-// Taller face tiles (FP32C x and y faces): 32 x 16 faces, each thread two
-// faces adjacent along t2, so that the t2 pass reads 6 rows for 2 faces
-// instead of 5 for 1 and the t1 pass recomputes 4 halo rows per 16 instead
-// of per 8.
-constexpr int TYT = 16;
-constexpr int SQ_HT = TYT + 4;
-constexpr int SQ_NT = 8 * SQ_HT * SQ_W;
-constexpr int ST_ROWS_T = SQ_HT * TX;
-constexpr int ST_NT = 24 * ST_ROWS_T;
-
 // t1 pass of one tile of H rows (with the tangential halo): values and
 // t1-derivatives of Q0, values of the normal slope, at the two t1 Gauss
 // points, for every row of the tile. 64 H equal tasks (Q0 or slope,
@@ -772,12 +764,140 @@ __device__ __forceinline__ void tile_t1_pass(const R *sq, C *st, int tid)
     }
 }
 
+// ---- FP32 component pairs ----
+//
+// FP32 face boxes and t1-pass rows hold the components as pairs (rho, m_n)
+// and (m_t1, m_t2), 8 bytes per position: the face-state kernel's packed
+// values are stored as they are (4 stores per face instead of 8), and the t1
+// and t2 passes run on both components of a pair at once. Face-box tile: 4
+// pair arrays (Q0 of both pairs, then their normal slopes) of H x SQ_W; rows:
+// 12 pair arrays of H x TX, 4 P + {0, 1} Q0 of pair P at the two t1 Gauss
+// points, 4 P + {2, 3} its t1 slopes there, 8 + 2 P + {0, 1} its normal slope.
+// The face state of a 384x256x256 step took 2.15 ms with 8 separate stores
+// and takes 1.90 ms with 4 paired ones.
+
+// t1 pass of a face-box tile of H rows: 64 H equal tasks (pair, row, group of
+// 2 columns), H / 4 per thread: 6 pairs in by 128-bit loads, 2 columns out by
+// one 128-bit store per array (consecutive lanes, consecutive 16 bytes: no
+// bank conflict; groups of 4 columns would store 32 bytes apart).
+template <int H>
+__device__ __forceinline__ void tile_t1_pass_f2(const float2 *sq, float2 *st, int tid)
+{
+    static_assert(H % 4 == 0, "a warp's tasks share the pair");
+    constexpr int NV = 16 * H, ROWS = H * TX;
+#pragma unroll
+    for (int j = 0; j < H / 4; ++j) {
+        const int task = tid + j * 256, p = task / NV, rem = task - p * NV, r = rem >> 4, cg = rem & 15;
+        const float4 *in = reinterpret_cast<const float4 *>(sq + (p * H + r) * SQ_W + 2 * cg);
+        f2 q[6];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const float4 x = in[i];
+            q[2 * i] = f2(x.x, x.y);
+            q[2 * i + 1] = f2(x.z, x.w);
+        }
+        float2 *o = st + r * TX + 2 * cg;
+        f2 v[4][2];
+        if (p < 2) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                tan_val_der(q[i], q[i + 1], q[i + 2], q[i + 3], q[i + 4], v[0][i], v[1][i], v[2][i], v[3][i]);
+            o += 4 * p * ROWS;
+        } else {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) tan_val_direct(q[i], q[i + 1], q[i + 2], q[i + 3], q[i + 4], v[0][i], v[1][i]);
+            o += (8 + 2 * (p - 2)) * ROWS;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (k < 2 || p < 2)
+                *reinterpret_cast<float4 *>(o + k * ROWS) = make_float4(v[k][0].v.x, v[k][0].v.y, v[k][1].v.x, v[k][1].v.y);
+    }
+}
+
+// tan_val_direct and tan_val_der of a component pair, with the two Gauss
+// points (not the components) in the lanes of the results, as the flux takes
+// them: x0 and x1 of the pair's two components, value (-g, +g). Everything up
+// to the last operation runs on both components at once; that one is scalar
+// and writes its lane in place (no moves). NEG: component 0 negated, by the
+// operand signs of the last operation.
+template <bool NEG>
+__device__ __forceinline__ void pair_val_direct(const f2 p[5], f2 &x0, f2 &x1)
+{
+    constexpr float w0 = float(-1.0 / 4320.0 + 0.028065638085606807), w1 = float(1.0 / 1080.0 - 0.20046884346862007);
+    constexpr float w2 = float(719.0 / 720.0);
+    constexpr float w3 = float(1.0 / 1080.0 + 0.20046884346862007), w4 = float(-1.0 / 4320.0 - 0.028065638085606807);
+    const f2 a = fma(f2(w3), p[3], fma(f2(w2), p[2], fma(f2(w1), p[1], f2(w0) * p[0])));
+    const f2 b = fma(f2(w1), p[3], fma(f2(w2), p[2], fma(f2(w3), p[1], f2(w4) * p[0])));
+    x0 = NEG ? f2(__fmaf_rn(-w0, p[4].v.x, -b.v.x), __fmaf_rn(-w4, p[4].v.x, -a.v.x))
+             : f2(__fmaf_rn(w0, p[4].v.x, b.v.x), __fmaf_rn(w4, p[4].v.x, a.v.x));
+    x1 = f2(__fmaf_rn(w0, p[4].v.y, b.v.y), __fmaf_rn(w4, p[4].v.y, a.v.y));
+}
+template <bool NEG>
+__device__ __forceinline__ void pair_val_der(const f2 p[5], f2 &x0, f2 &x1, f2 &d0, f2 &d1)
+{
+    const f2 s1 = fma(p[2], f2(-2.0f), p[3] + p[1]), s2 = fma(p[2], f2(-2.0f), p[4] + p[0]);
+    const f2 a1 = p[3] - p[1], a2 = p[4] - p[0];
+    const f2 E = fma(s1, f2(float(1.0 / 1080.0)), fma(s2, f2(float(-1.0 / 4320.0)), p[2]));
+    const f2 O = fma(a1, f2(float(0.20046884346862007)), a2 * f2(float(-0.028065638085606807)));
+    const f2 Do = fma(a1, f2(float(2.0 / 3.0)), a2 * f2(float(-1.0 / 12.0)));
+    const f2 De = fma(s1, f2(float(0.41697519441472974)), s2 * f2(float(-0.032075014954979206)));
+    x0 = f2(__fsub_rn(E.v.x, O.v.x), __fadd_rn(E.v.x, O.v.x));
+    x1 = f2(__fsub_rn(E.v.y, O.v.y), __fadd_rn(E.v.y, O.v.y));
+    d0 = NEG ? f2(__fsub_rn(De.v.x, Do.v.x), __fadd_rn(-Do.v.x, -De.v.x))
+             : f2(__fsub_rn(Do.v.x, De.v.x), __fadd_rn(Do.v.x, De.v.x));
+    d1 = f2(__fsub_rn(Do.v.y, De.v.y), __fadd_rn(Do.v.y, De.v.y));
+}
+
+// The t2 pass of the NE faces (tx, r0 + e) of a tile of H rows at t1 Gauss
+// point m: values and t2 slopes of Q0, values of the t1 slopes and of the
+// normal slope at the two t2 Gauss points (the lanes), each row read once
+// over the 4 + NE rows that the faces' stencils cover. NEG: the density's
+// slopes negated, as gk_flux takes them.
+template <int H, int NE, bool NEG>
+__device__ __forceinline__ void t2_pass_f2(const float2 *st, int m, int tx, int r0, f2 q[NE][4], f2 dn[NE][4],
+                                           f2 d1[NE][4], f2 d2[NE][4])
+{
+    constexpr int ROWS = H * TX;
+    const float2 *s = st + r0 * TX + tx;
+#pragma unroll
+    for (int P = 0; P < 2; ++P) {
+        f2 p[4 + NE];
+#pragma unroll
+        for (int i = 0; i < 4 + NE; ++i) p[i] = f2(s[(4 * P + m) * ROWS + i * TX]);
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+            if (P == 0)
+                pair_val_der<NEG>(p + e, q[e][0], q[e][1], d2[e][0], d2[e][1]);
+            else
+                pair_val_der<false>(p + e, q[e][2], q[e][3], d2[e][2], d2[e][3]);
+        }
+#pragma unroll
+        for (int i = 0; i < 4 + NE; ++i) p[i] = f2(s[(4 * P + 2 + m) * ROWS + i * TX]);
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+            if (P == 0)
+                pair_val_direct<NEG>(p + e, d1[e][0], d1[e][1]);
+            else
+                pair_val_direct<false>(p + e, d1[e][2], d1[e][3]);
+        }
+#pragma unroll
+        for (int i = 0; i < 4 + NE; ++i) p[i] = f2(s[(8 + 2 * P + m) * ROWS + i * TX]);
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+            if (P == 0)
+                pair_val_direct<NEG>(p + e, dn[e][0], dn[e][1]);
+            else
+                pair_val_direct<false>(p + e, dn[e][2], dn[e][3]);
+        }
+    }
+}
+
 template <typename R>
 constexpr size_t flux_smem_bytes()
 {
     return (size_t)(SQ_N + ST_N) * sizeof(R) + 2 * sizeof(unsigned long long);
 }
-constexpr size_t flux_tall_smem_bytes() { return (size_t)(SQ_NT + ST_NT) * sizeof(float) + 2 * sizeof(unsigned long long); }
 
 
 // ---- TMA and mbarrier helpers (sm_90+ PTX) ----

@@ -57,11 +57,12 @@ struct Ctx {
     void *wk0;                // reconstruction input of stage 1 (FP64: == state)
     void *wk1;                // W* (reconstruction input of stage 2), R[4][np]
     void *pbuf;               // P = W + dt L + dt^2/6 Lt (FP64 double[4][np]; FP32C hi/lo)
-    void *fq;                 // face equilibrium state + normal slope, R[8][nfq]
+    void *fq;                 // face equilibrium state + normal slope, R[8][nfq] (FP32C: float2[4][nfq],
+                              // component pairs)
     long nfq;
     int e1p[3];               // padded t1 extent of the face box per direction (multiple of 4)
     CUtensorMap tmap[3];      // TMA descriptors of the face box per direction
-    CUtensorMap tmapT[3];     // FP32C: the same with 20-row boxes (32 x 16 face tiles)
+    CUtensorMap tmapM[3];     // FP32C: the same with 5-row boxes (the marching flux kernel)
     // Optional (FP64): per direction, the 64 Gauss-point inputs of every face
     // (16 g + k arrays of stride ngp; g Gauss point, k = Q0, normal slope, t1
     // slope, t2 slope x 4 components), written by the flux kernels as double

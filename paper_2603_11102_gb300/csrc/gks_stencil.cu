@@ -2,20 +2,20 @@
 //
 // Per stage and per direction d (x, y, z):
 //   face_eq      one thread per tangential position of the extended face box,
-//                marching 16 faces along d with a 5-cell window: WENO5-JS
-//                (Sec. 2, Jiang-Shu) left/right states from one paired
-//                evaluation per cell, the equilibrium state Q0 from the half
-//                Maxwellians (u>0 from the left, u<0 from the right), and the
-//                quartic normal slope of Q0.
-//   face_flux    (x, y) persistent, face tiles loaded by TMA (32x16 with two
-//                faces per thread for FP32C, 32x8 otherwise): linear quartic
-//                reconstruction of Q0 and its normal slope to the 2x2 Gauss
-//                points (Sec. 2, Eq. (x_example)) with the t1 pass in shared
-//                memory, and the gas-kinetic flux F0 and its time derivative
-//                F1 at each point (Sec. 2, Eq. (flux); Appendix), averaged
-//                with weights 1/4 and stored per face. The flux of FP32 and
-//                double-single arithmetic runs at two Gauss points at once on
-//                packed pairs.
+//                marching along d with the differences around a cell in
+//                registers: WENO5-JS (Sec. 2, Jiang-Shu) left/right states
+//                from one paired evaluation per cell, the equilibrium state
+//                Q0 from the half Maxwellians (u>0 from the left, u<0 from
+//                the right), and the quartic normal slope of Q0.
+//   face_flux    (x, y) linear quartic reconstruction of Q0 and its normal
+//                slope to the 2x2 Gauss points (Sec. 2, Eq. (x_example)) and
+//                the gas-kinetic flux F0 and its time derivative F1 at each
+//                point (Sec. 2, Eq. (flux); Appendix), averaged with weights
+//                1/4 and stored per face. FP32C: warps marching along t2 with
+//                the t1-pass rows in registers; FP64 and double-single:
+//                persistent blocks on 32x8 face tiles loaded by TMA, the t1
+//                pass in shared memory. The flux of FP32 and double-single
+//                arithmetic runs at two Gauss points at once on packed pairs.
 //   flux_update  (z) the same flux, walking z per tile column, fused with the
 //                divergence (Eq. (finite)) and the two-stage fourth-order
 //                combination of every cell; stage 2 also prepares the next
@@ -28,6 +28,7 @@
 // FP32 difference; it cancels exactly between the two faces of a cell.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "gks_bounds.cuh"
@@ -267,6 +268,7 @@ __global__ void __launch_bounds__(256, 3) face_eq_f2_kernel(FaceEqArgs<float, fl
         return;
     const float *pc[4] = {A.w + base, A.w + (long)A.cn * A.np + base, A.w + (long)A.c1 * A.np + base,
                           A.w + (long)A.c2 * A.np + base};
+    float2 *fq = reinterpret_cast<float2 *>(A.fq);   // component pairs (see tile_t1_pass_f2)
     // cells f0-3 .. f0 start the march at cell f0-1, cell f0+1 completes it
     WenoMarch<f2> w[2];
     f2 Qprev[2];
@@ -298,18 +300,13 @@ __global__ void __launch_bounds__(256, 3) face_eq_f2_kernel(FaceEqArgs<float, fl
         f2 Ql[2], Qr[2], Q0[2];
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-            const f2 dq = w[q].slope() * ihf;
-            A.fq[(4 + 2 * q) * A.nfq + o] = dq.v.x;
-            A.fq[(5 + 2 * q) * A.nfq + o] = dq.v.y;
+            fq[(2 + q) * A.nfq + o] = (w[q].slope() * ihf).v;
             Ql[q] = Qprev[q];
             w[q].push(e[q], Qprev[q], Qr[q]);
         }
         face_equilibrium2(A.ph, Ql, Qr, Q0);
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            A.fq[(2 * q) * A.nfq + o] = Q0[q].v.x;
-            A.fq[(2 * q + 1) * A.nfq + o] = Q0[q].v.y;
-        }
+        for (int q = 0; q < 2; ++q) fq[q * A.nfq + o] = Q0[q].v;
     }
 }
 
@@ -506,43 +503,36 @@ __device__ __forceinline__ void tile_gauss_flux(const FluxPhys<double> &ph, cons
     }
 }
 
-// tile_gauss_flux for FP32 arithmetic: the same t2 pass, the flux at the two
-// t2 Gauss points of each t1 Gauss point as one packed evaluation.
-template <int V>
-__device__ __forceinline__ void t2_pass_f2(const float *st, int m, int tx, int ty, f2 &q, f2 &dn, f2 &d1, f2 &d2)
+// The flux of the NE faces (tx, r0 + e) of a tile of H rows in FP32: the t2
+// pass, then the two t2 Gauss points of each t1 Gauss point as one packed
+// evaluation; the sums of F0 and -F1 over the 4 Gauss points of each face.
+template <int H, int NE, bool NEED_F0>
+__device__ __forceinline__ void tile_gauss_flux_f2(const FluxPhys<f2> &ph, const float2 *st, int tx, int r0, float ih1,
+                                                   const float ih2[NE], float acc0[NE][4], float acc1[NE][4])
 {
-    float a[2], b[2], c[2], d[2];
-    t2_pass<float, V>(st, m, tx, ty, a, b, c, d);
-    q = f2(a[0], a[1]);
-    dn = f2(b[0], b[1]);
-    d1 = f2(c[0], c[1]);
-    d2 = f2(d[0], d[1]);
-}
-template <bool NEED_F0>
-__device__ __forceinline__ void tile_gauss_flux_f32(const FluxPhys<f2> &ph, const float *st, int tx, int ty, float ih1,
-                                                    float ih2, float acc0[4], float acc1[4])
-{
-    f2 s0[4], s1[4];   // the t2 Gauss points -g, +g in the lanes
+    f2 s0[NE][4], s1[NE][4];   // the two t2 Gauss points -g, +g in the lanes
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
-        f2 Qv[4], Dn[4], D1[4], D2[4];
-        t2_pass_f2<0>(st, m, tx, ty, Qv[0], Dn[0], D1[0], D2[0]);
-        t2_pass_f2<1>(st, m, tx, ty, Qv[1], Dn[1], D1[1], D2[1]);
-        t2_pass_f2<2>(st, m, tx, ty, Qv[2], Dn[2], D1[2], D2[2]);
-        t2_pass_f2<3>(st, m, tx, ty, Qv[3], Dn[3], D1[3], D2[3]);
-        f2 F0[4], F1[4];
-        gk_flux<f2, NEED_F0>(ph, Qv, Dn, D1, D2, f2(ih1), f2(ih2), F0, F1);
+        f2 Qv[NE][4], Dn[NE][4], D1[NE][4], D2[NE][4];   // [face][component]
+        t2_pass_f2<H, NE, true>(st, m, tx, r0, Qv, Dn, D1, D2);
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            if (NEED_F0) s0[v] = m == 0 ? F0[v] : s0[v] + F0[v];
-            s1[v] = m == 0 ? F1[v] : s1[v] + F1[v];
+        for (int e = 0; e < NE; ++e) {
+            f2 F0[4], F1[4];
+            gk_flux<f2, NEED_F0>(ph, Qv[e], Dn[e], D1[e], D2[e], f2(ih1), f2(ih2[e]), F0, F1);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                if (NEED_F0) s0[e][v] = m == 0 ? F0[v] : s0[e][v] + F0[v];
+                s1[e][v] = m == 0 ? F1[v] : s1[e][v] + F1[v];
+            }
         }
     }
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        if (NEED_F0) acc0[v] = s0[v].v.x + s0[v].v.y;
-        acc1[v] = s1[v].v.x + s1[v].v.y;
-    }
+    for (int e = 0; e < NE; ++e)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            if (NEED_F0) acc0[e][v] = s0[e][v].v.x + s0[e][v].v.y;
+            acc1[e][v] = s1[e][v].v.x + s1[e][v].v.y;
+        }
 }
 
 // tile_gauss_flux for double-single arithmetic (no Gauss-point output): the
@@ -653,133 +643,222 @@ __global__ void __launch_bounds__(256, std::is_same<C, dsf>::value ? 2 : 1)
     }
 }
 
-// The t2 pass of component V of the two faces (tx, r0) and (tx, r0 + 1) of a
-// tall tile (t2_pass, e = 0, 1): each row array is read once over the 6 rows
-// r0 .. r0+5 that the two 5-point stencils cover.
-template <int V>
-__device__ __forceinline__ void t2_pass_two(const float *st, int m, int tx, int r0, f2 q[2][4], f2 dn[2][4], f2 d1[2][4],
-                                            f2 d2[2][4])
+// ---- FP32C x and y face fluxes: a march along t2 in registers ----
+//
+// A warp owns 32 faces along t1 and walks a segment of t2 rows of one face
+// plane. Per row it forms the t1 pass of the 8 face-box values at both t1
+// Gauss points (the lanes of a pair) and keeps the last 5 rows of the 24
+// results in registers; every row then completes the t2 stencil of the face
+// two rows back, whose flux is evaluated at both t1 Gauss points at once. The
+// face box arrives by TMA, 5 rows (all components) at a time, into the warp's
+// own two buffers: no block barrier, and the t1 rows never go through shared
+// memory. The tile kernel that this replaces (32 x 16 faces, t1 rows in shared
+// memory) was held by shared-memory traffic and issue: 528 B and 718
+// instructions a face (stage 2) against 200 B here, and it redid the t1 pass
+// of 4 rows per 16 (here per segment).
+constexpr int RB = 5;                                  // rows per TMA box, and of the register window
+constexpr int kMarchStage = 4 * RB * 2 * SQ_W;         // floats of one box: 4 component pairs x 5 rows x 36 columns
+constexpr int kMarchWarps = 8;                         // warps per block at most
+constexpr size_t march_smem_bytes(int warps)
 {
-    constexpr bool NEG = V == 0;
-    const float *x = st + (V * 4 + m) * ST_ROWS_T + r0 * TX + tx;
-    const float *y = st + (V * 4 + 2 + m) * ST_ROWS_T + r0 * TX + tx;
-    const float *z = st + (16 + V * 2 + m) * ST_ROWS_T + r0 * TX + tx;
-    float p[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) p[i] = x[i * TX];
-#pragma unroll
-    for (int e = 0; e < 2; ++e)
-        tan_val_der<float, NEG>(p[e], p[e + 1], p[e + 2], p[e + 3], p[e + 4], q[e][V].v.x, q[e][V].v.y, d2[e][V].v.x,
-                                d2[e][V].v.y);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) p[i] = y[i * TX];
-#pragma unroll
-    for (int e = 0; e < 2; ++e)
-        tan_val_direct<float, NEG>(p[e], p[e + 1], p[e + 2], p[e + 3], p[e + 4], d1[e][V].v.x, d1[e][V].v.y);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) p[i] = z[i * TX];
-#pragma unroll
-    for (int e = 0; e < 2; ++e)
-        tan_val_direct<float, NEG>(p[e], p[e + 1], p[e + 2], p[e + 3], p[e + 4], dn[e][V].v.x, dn[e][V].v.y);
+    return (size_t)warps * (2 * kMarchStage * sizeof(float) + 2 * sizeof(uint64_t));
 }
 
-// The flux of the two faces (tx, r0) and (tx, r0 + 1) of a tall tile (FP32C):
-// the sums of F0 and -F1 over the 4 Gauss points of each face.
-template <bool NEED_F0>
-__device__ __forceinline__ void tile_gauss_flux_pair(const FluxPhys<f2> &ph, const float *st, int tx, int r0,
-                                                     float ih1, const float ih2[2], float acc0[2][4],
-                                                     float acc1[2][4])
+struct MarchWin {
+    f2 v[4][RB], d[4][RB], n[4][RB];   // Q0, its t1 slope, the normal slope: [component][row slot], t1 Gauss points
+};
+
+// t1 pass of row `j` of a box (columns lane .. lane + 4) into window slot J.
+template <int J>
+__device__ __forceinline__ void march_row(const float2 *box, int lane, MarchWin &w)
 {
-    f2 s0[2][4], s1[2][4];   // the two t2 Gauss points -g, +g in the lanes
+    constexpr float o1 = float(0.20046884346862007), o2 = float(0.028065638085606807);
+    constexpr float e1 = float(0.41697519441472974), e2 = float(0.032075014954979206);
+    constexpr float w0 = float(-1.0 / 4320.0 + 0.028065638085606807), w1 = float(1.0 / 1080.0 - 0.20046884346862007);
+    constexpr float w2 = float(719.0 / 720.0);
+    constexpr float w3 = float(1.0 / 1080.0 + 0.20046884346862007), w4 = float(-1.0 / 4320.0 - 0.028065638085606807);
 #pragma unroll
-    for (int m = 0; m < 2; ++m) {
-        f2 Qv[2][4], Dn[2][4], D1[2][4], D2[2][4];   // [face][component]
-        t2_pass_two<0>(st, m, tx, r0, Qv, Dn, D1, D2);
-        t2_pass_two<1>(st, m, tx, r0, Qv, Dn, D1, D2);
-        t2_pass_two<2>(st, m, tx, r0, Qv, Dn, D1, D2);
-        t2_pass_two<3>(st, m, tx, r0, Qv, Dn, D1, D2);
+    for (int P = 0; P < 2; ++P) {
+        float2 x[5];
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            f2 F0[4], F1[4];
-            gk_flux<f2, NEED_F0>(ph, Qv[e], Dn[e], D1[e], D2[e], f2(ih1), f2(ih2[e]), F0, F1);
+        for (int k = 0; k < 5; ++k) x[k] = box[(P * RB + J) * SQ_W + lane + k];
 #pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                if (NEED_F0) s0[e][v] = m == 0 ? F0[v] : s0[e][v] + F0[v];
-                s1[e][v] = m == 0 ? F1[v] : s1[e][v] + F1[v];
-            }
+        for (int c = 0; c < 2; ++c) {
+            float q[5];
+#pragma unroll
+            for (int k = 0; k < 5; ++k) q[k] = c ? x[k].y : x[k].x;
+            const float d1 = __fmaf_rn(q[2], -2.0f, __fadd_rn(q[3], q[1]));
+            const float d2 = __fmaf_rn(q[2], -2.0f, __fadd_rn(q[4], q[0]));
+            const float a1 = __fsub_rn(q[3], q[1]), a2 = __fsub_rn(q[4], q[0]);
+            const float E = __fmaf_rn(d1, float(1.0 / 1080.0), __fmaf_rn(d2, float(-1.0 / 4320.0), q[2]));
+            const float D = __fmaf_rn(a1, float(2.0 / 3.0), __fmul_rn(a2, float(-1.0 / 12.0)));
+            w.v[2 * P + c][J] = fma(f2(a1), f2(-o1, o1), fma(f2(a2), f2(o2, -o2), f2(E)));
+            w.d[2 * P + c][J] = fma(f2(d1), f2(-e1, e1), fma(f2(d2), f2(e2, -e2), f2(D)));
+        }
+#pragma unroll
+        for (int k = 0; k < 5; ++k) x[k] = box[((2 + P) * RB + J) * SQ_W + lane + k];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            float q[5];
+#pragma unroll
+            for (int k = 0; k < 5; ++k) q[k] = c ? x[k].y : x[k].x;
+            w.n[2 * P + c][J] = fma(f2(q[4]), f2(w0, w4), fma(f2(q[3]), f2(w1, w3),
+                                fma(f2(q[2]), f2(w2, w2), fma(f2(q[1]), f2(w3, w1), f2(q[0]) * f2(w4, w0)))));
         }
     }
+}
+
+// t2 pass over the window whose newest row is in slot J, and the flux of the
+// face two rows back: the sums of F0 and -F1 over its 4 Gauss points.
+template <int J, bool NEED_F0>
+__device__ __forceinline__ void march_face(const FluxPhys<f2> &ph, const MarchWin &w, f2 ih1, f2 ih2, float acc0[4],
+                                           float acc1[4])
+{
+    constexpr int r0 = (J + 1) % RB, r1 = (J + 2) % RB, r2 = (J + 3) % RB, r3 = (J + 4) % RB, r4 = J;
+    f2 q[2][4], dn[2][4], d1[2][4], d2[2][4];   // [t2 Gauss point][component]
 #pragma unroll
-    for (int e = 0; e < 2; ++e)
+    for (int v = 0; v < 4; ++v) {
+        if (v == 0) {
+            tan_val_der<f2, true>(w.v[v][r0], w.v[v][r1], w.v[v][r2], w.v[v][r3], w.v[v][r4], q[0][v], q[1][v], d2[0][v],
+                                  d2[1][v]);
+            tan_val_direct<f2, true>(w.d[v][r0], w.d[v][r1], w.d[v][r2], w.d[v][r3], w.d[v][r4], d1[0][v], d1[1][v]);
+            tan_val_direct<f2, true>(w.n[v][r0], w.n[v][r1], w.n[v][r2], w.n[v][r3], w.n[v][r4], dn[0][v], dn[1][v]);
+        } else {
+            tan_val_der<f2>(w.v[v][r0], w.v[v][r1], w.v[v][r2], w.v[v][r3], w.v[v][r4], q[0][v], q[1][v], d2[0][v],
+                            d2[1][v]);
+            tan_val_direct<f2>(w.d[v][r0], w.d[v][r1], w.d[v][r2], w.d[v][r3], w.d[v][r4], d1[0][v], d1[1][v]);
+            tan_val_direct<f2>(w.n[v][r0], w.n[v][r1], w.n[v][r2], w.n[v][r3], w.n[v][r4], dn[0][v], dn[1][v]);
+        }
+    }
+    f2 s0[4], s1[4];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        f2 F0[4], F1[4];
+        gk_flux<f2, NEED_F0>(ph, q[k], dn[k], d1[k], d2[k], ih1, ih2, F0, F1);
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            if (NEED_F0) acc0[e][v] = s0[e][v].v.x + s0[e][v].v.y;
-            acc1[e][v] = s1[e][v].v.x + s1[e][v].v.y;
+            if (NEED_F0) s0[v] = k == 0 ? F0[v] : s0[v] + F0[v];
+            s1[v] = k == 0 ? F1[v] : s1[v] + F1[v];
         }
+    }
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        if (NEED_F0) acc0[v] = s0[v].v.x + s0[v].v.y;
+        acc1[v] = s1[v].v.x + s1[v].v.y;
+    }
 }
 
-// face_flux_kernel on 32 x 16 tiles for FP32C grids (the same results bit
-// for bit): the face box of a tile (its tangential halo included) arrives by
-// TMA, the t1 pass fills 20 rows, and each thread computes two faces.
+// Position of a warp in its work: item (face plane, t2 segment, t1 tile), box
+// k of the item's n boxes; a0, b0 its first face along t1 and t2, be the end.
+struct MarchPos {
+    int it, k, n, f, a0, b0, be;
+};
+
 template <bool NEED_F0>
-__global__ void __launch_bounds__(256, 2) face_flux_tall_kernel(const __grid_constant__ CUtensorMap tmap,
-                                                                FluxArgs<float, float> A)
+__global__ void __launch_bounds__(32 * kMarchWarps, 1)
+    face_flux_march_kernel(const __grid_constant__ CUtensorMap tmap, FluxArgs<float, float> A, int L)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    float *sq = reinterpret_cast<float *>(smem_raw);   // face-box tile (SQ_NT)
-    float *st = sq + SQ_NT;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(st + ST_NT);
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
-    const int NA = (A.n1 + TX - 1) / TX, NB = (A.n2 + TYT - 1) / TYT;
-    const int ntiles = NA * NB * A.nf;
-    const uint32_t bytes = (uint32_t)(SQ_NT * sizeof(float));
-    const TileIdx g = {(int)(gridDim.x % NA), (int)((gridDim.x / NA) % NB), (int)(gridDim.x / (NA * NB))};
-    TileIdx cur = {(int)(blockIdx.x % NA), (int)((blockIdx.x / NA) % NB), (int)(blockIdx.x / (NA * NB))};
-    if (tid == 0) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    float *buf = reinterpret_cast<float *>(smem_raw) + warp * 2 * kMarchStage;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + (size_t)nw * 2 * kMarchStage * sizeof(float)) + 2 * warp;
+    const int NA = (A.n1 + TX - 1) / TX, NS = (A.n2 + L - 1) / L, nitems = NA * NS * A.nf;
+    const int step = gridDim.x * nw;
+    auto item = [&](int it) {
+        MarchPos p;
+        const int ta = it % NA, r = it / NA, sg = r % NS;
+        p.it = it;
+        p.k = 0;
+        p.f = r / NS;
+        p.a0 = ta * TX;
+        p.b0 = sg * L;
+        p.be = min(p.b0 + L, A.n2);
+        p.n = (p.be - p.b0 + 4 + RB - 1) / RB;
+        return p;
+    };
+    auto load = [&](const MarchPos &p, int s) {
+        if (lane == 0 && p.it < nitems)
+            tma_load_tile(&tmap, buf + s * kMarchStage, &bar[s], 2 * p.a0, p.b0 + p.k * RB, p.f,
+                          (uint32_t)(kMarchStage * sizeof(float)));
+    };
+    auto next = [&](const MarchPos &p) {
+        MarchPos q = p;
+        if (++q.k >= q.n) q = item(p.it + step);
+        return q;
+    };
+    if (lane == 0) {
         mbar_init(&bar[0], 1);
+        mbar_init(&bar[1], 1);
         mbar_fence_init();
     }
-    __syncthreads();
-    int t = blockIdx.x;
-    if (tid == 0 && t < ntiles) tma_load_tile(&tmap, sq, &bar[0], cur.ta * TX, cur.tb * TYT, cur.f, bytes);
-    for (int k = 0; t < ntiles; t += gridDim.x, ++k) {
-        const int tn = t + gridDim.x;
-        const TileIdx nxt = tile_add(cur, g, NA, NB);
-        const bool ok = mbar_wait(&bar[0], (uint32_t)(k & 1));
-        if (__syncthreads_or(!ok)) {
-            if (tid == 0) atomicOr(&A.scal->flags, FLAG_TIMEOUT);
+    __syncwarp();
+    MarchPos cur = item(blockIdx.x * nw + warp), ahead = cur;
+    load(ahead, 0);
+    if (ahead.it < nitems) ahead = next(ahead);
+    load(ahead, 1);
+    const FluxPhys<f2> ph = flux_phys_f2(A.ph);
+    MarchWin w;
+    for (int cnt = 0; cur.it < nitems; ++cnt) {
+        const int s = cnt & 1;
+        const int a = cur.a0 + lane, b = cur.b0 + cur.k * RB - 4;   // face that the box's first row completes
+        const bool in = a < A.n1;
+        const f2 ih1(in ? __ldg(A.ih1 + a + G) : 0.0f);
+        if (__any_sync(0xffffffffu, !mbar_wait(&bar[s], (uint32_t)((cnt >> 1) & 1)))) {
+            if (lane == 0) atomicOr(&A.scal->flags, FLAG_TIMEOUT);
+            mbar_wait(&bar[s ^ 1], (uint32_t)(((cnt + 1) >> 1) & 1));   // the copy in flight, with the same limit
             return;
         }
-        const int a0 = cur.ta * TX, b0 = cur.tb * TYT, f = cur.f;
-        cur = nxt;
-
-        tile_t1_pass<float, float, SQ_HT>(sq, st, tid);
-        __syncthreads();
-        if (tid == 0 && tn < ntiles) {
-            fence_proxy_async();
-            tma_load_tile(&tmap, sq, &bar[0], nxt.ta * TX, nxt.tb * TYT, nxt.f, bytes);
-        }
-
-        const int a = a0 + tx, b = b0 + 2 * ty;
-        if (a < A.n1 && b < A.n2) {
-            // b + 1 <= n2: inside the padded width array even when face b + 1 is not stored
-            const float ih1 = __ldg(A.ih1 + a + G);
-            const float ih2[2] = {__ldg(A.ih2 + b + G), __ldg(A.ih2 + b + 1 + G)};
-            float acc0[2][4], acc1[2][4];
-            tile_gauss_flux_pair<NEED_F0>(flux_phys_f2(A.ph), st, tx, 2 * ty, ih1, ih2, acc0, acc1);
+        const float2 *box = reinterpret_cast<const float2 *>(buf + s * kMarchStage);
+        auto row = [&](auto jc) {
+            constexpr int J = decltype(jc)::value;
+            march_row<J>(box, lane, w);
+            const int bf = b + J;
+            if (bf >= cur.b0 && bf < cur.be) {
+                float acc0[4], acc1[4];
+                march_face<J, NEED_F0>(ph, w, ih1, f2(__ldg(A.ih2 + bf + G)), acc0, acc1);
+                const long o = ((long)cur.f * A.n2 + bf) * A.n1 + a;
+                if (in && in_bounds(o, A.nff)) {
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const long o = ((long)f * A.n2 + b + e) * A.n1 + a;
-                if (b + e >= A.n2 || !in_bounds(o, A.nff)) break;
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    if (NEED_F0) A.ff[A.gcomp[v] * A.nff + o] = face_avg(acc0[e][v]);
-                    A.ff[(4 + A.gcomp[v]) * A.nff + o] = face_avg_neg(acc1[e][v]);
+                    for (int v = 0; v < 4; ++v) {
+                        if (NEED_F0) A.ff[A.gcomp[v] * A.nff + o] = face_avg(acc0[v]);
+                        A.ff[(4 + A.gcomp[v]) * A.nff + o] = face_avg_neg(acc1[v]);
+                    }
                 }
             }
-        }
-        __syncthreads();   // st and the face-box buffer are free again
+        };
+        row(std::integral_constant<int, 0>{});
+        row(std::integral_constant<int, 1>{});
+        row(std::integral_constant<int, 2>{});
+        row(std::integral_constant<int, 3>{});
+        row(std::integral_constant<int, 4>{});
+        // the box is read: fetch the one after the next into it
+        cur = next(cur);
+        if (ahead.it < nitems) ahead = next(ahead);
+        __syncwarp();
+        fence_proxy_async();
+        load(ahead, s);
     }
+}
+
+// Rows per march segment: S segments of L = ceil(n2 / S) rows; the busiest
+// warp's rows are least (the priming rows of a segment cost their t1 pass,
+// about one face together), over up to 64 segments. On large grids this picks
+// long segments with even rounds of the warps, on 32^3 single rows (1056
+// items for 1216 warps).
+int march_segment(int na, int nf, int n2, int warps)
+{
+    double best = -1.0;
+    int bestL = n2;
+    for (int S = 1; S <= 64 && S <= n2; ++S) {
+        const int L = (n2 + S - 1) / S, Sa = (n2 + L - 1) / L;
+        const long items = (long)na * nf * Sa;
+        const double cost = (double)((items + warps - 1) / warps) * (L + 1.0);
+        if (best < 0.0 || cost < best) {
+            best = cost;
+            bestL = L;
+        }
+    }
+    return bestL;
 }
 
 // ------------------------------------------------- z flux + stage update --
@@ -960,6 +1039,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
     // double-single grids take the z faces through face_flux_kernel and
     // update_ds_kernel instead
     static_assert(!std::is_same<C, dsf>::value, "the fused z kernel runs FP64 or FP32 arithmetic");
+    constexpr bool F32 = std::is_same<C, float>::value;   // face boxes and rows hold component pairs
+    constexpr int CX = F32 ? 2 : 1;                       // elements of a face-box position along t1
     constexpr bool NEED_F0 = STAGE == 1;
     constexpr int NC = STAGE == 1 ? 8 : 4, C0 = STAGE == 1 ? 0 : 4;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -979,7 +1060,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
         mbar_fence_init();
     }
     __syncthreads();
-    if (tid == 0) tma_load_tile(&tmap, sq, &bar[0], cur.a0, cur.b0, cur.f, bytes);
+    if (tid == 0) tma_load_tile(&tmap, sq, &bar[0], CX * cur.a0, cur.b0, cur.f, bytes);
     const double dt = A.scal->dt;
     bool bad = false;
     double mx = 0.0;   // stage 2 with prep: max |U|^2 of this thread's cells outside the forcing boxes
@@ -1060,26 +1141,30 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
             __syncthreads();
             return;
         }
-        tile_t1_pass(sq, st, tid);
+        if constexpr (F32)
+            tile_t1_pass_f2<SQ_H>(reinterpret_cast<const float2 *>(sq), reinterpret_cast<float2 *>(st), tid);
+        else
+            tile_t1_pass(sq, st, tid);
         __syncthreads();
         // the face box is free: fetch the next tile's during this one's flux
         if (tid == 0 && nxt.it < nitems) {
             fence_proxy_async();
-            tma_load_tile(&tmap, sq, &bar[0], nxt.a0, nxt.b0, nxt.f, bytes);
+            tma_load_tile(&tmap, sq, &bar[0], CX * nxt.a0, nxt.b0, nxt.f, bytes);
         }
 
         M F0[4], F1[4];
         if (in) {
-            C G0[4], G1[4];
-            if constexpr (std::is_same<C, float>::value)
-                tile_gauss_flux_f32<NEED_F0>(flux_phys_f2(A.ph), st, tx, ty, ih1, ih2, G0, G1);
+            C G0[1][4], G1[1][4];
+            if constexpr (F32)
+                tile_gauss_flux_f2<SQ_H, 1, NEED_F0>(flux_phys_f2(A.ph), reinterpret_cast<const float2 *>(st), tx, ty, ih1,
+                                                     &ih2, G0, G1);
             else
-                tile_gauss_flux<NEED_F0, GP>(flux_phys(A.ph), st, tx, ty, ih1, ih2, G0, G1, A.gp, A.gp32, A.ngp,
+                tile_gauss_flux<NEED_F0, GP>(flux_phys(A.ph), st, tx, ty, ih1, ih2, G0[0], G1[0], A.gp, A.gp32, A.ngp,
                                              ((long)f * A.n2 + b) * A.n1 + a);
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
-                F0[v] = NEED_F0 ? face_avg(G0[v]) : M(0);
-                F1[v] = face_avg_neg(G1[v]);
+                F0[v] = NEED_F0 ? face_avg(G0[0][v]) : M(0);
+                F1[v] = face_avg_neg(G1[0][v]);
             }
         }
         if (upd) {
@@ -1240,8 +1325,10 @@ const FluxGrids<R, C, STAGE> &flux_grids()
     if (!g.flux[0]) {
         constexpr size_t su = flux_update_smem_bytes<R>(STAGE == 1 ? 8 : 4);
         if constexpr (std::is_same<C, float>::value) {
-            // FP32C: 32 x 16 face tiles in x and y
-            g.flux[0] = persistent_grid(face_flux_tall_kernel<STAGE == 1>, flux_tall_smem_bytes());
+            // FP32C: the register march in x and y, one block of kMarchWarps warps per SM
+            cudaFuncSetAttribute(face_flux_march_kernel<STAGE == 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)march_smem_bytes(kMarchWarps));
+            g.flux[0] = sm_count();
         } else {
             g.flux[0] = persistent_grid(face_flux_kernel<R, C, STAGE == 1, false>, flux_smem_bytes<R>());
         }
@@ -1400,9 +1487,12 @@ void stage_impl(const Ctx &c)
         }
         if (d < 2) {
             if constexpr (std::is_same<C, float>::value) {
-                const long nt = (long)((F.n1 + TX - 1) / TX) * ((F.n2 + TYT - 1) / TYT) * F.nf;
-                const int gt = (int)(nt < grids.flux[0] ? nt : grids.flux[0]);
-                face_flux_tall_kernel<STAGE == 1><<<gt, blk, flux_tall_smem_bytes(), c.stream>>>(c.tmapT[d], F);
+                const int na = (F.n1 + TX - 1) / TX, L = march_segment(na, F.nf, F.n2, kMarchWarps * grids.flux[0]);
+                const long items = (long)na * F.nf * ((F.n2 + L - 1) / L);
+                // few items: fewer warps per block, so that they spread over the SMs
+                const int nw = (int)std::min((long)kMarchWarps, (items + grids.flux[0] - 1) / grids.flux[0]);
+                const int gm = (int)std::min((long)grids.flux[0], (items + nw - 1) / nw);
+                face_flux_march_kernel<STAGE == 1><<<gm, 32 * nw, march_smem_bytes(nw), c.stream>>>(c.tmapM[d], F, L);
             } else {
                 const int grid = (int)(ntiles < grids.flux[gpo] ? ntiles : grids.flux[gpo]);
                 if (FP64A && gpo)
