@@ -1558,19 +1558,6 @@ __global__ void __launch_bounds__(256) prep_cfl_kernel(const void *__restrict__ 
     block_max_to(mx, &scal->maxu2_bits);
 }
 
-__device__ __forceinline__ void load_cell(int prec, const void *S, long np, long lin, double q[4])
-{
-    if (prec == GKS_FP64) {
-        const double *W = (const double *)S;
-#pragma unroll
-        for (int v = 0; v < 4; ++v) q[v] = W[v * np + lin];
-    } else {
-        const float *W = (const float *)S;
-#pragma unroll
-        for (int v = 0; v < 4; ++v) q[v] = (double)W[v * np + lin] + (double)W[(4 + v) * np + lin];
-    }
-}
-
 __global__ void dt_kernel(Scalars *scal, double cfl, double dt_fixed, double hmin, double csound)
 {
     const double umax = sqrt(__longlong_as_double((long long)scal->maxu2_bits));
@@ -1646,44 +1633,208 @@ __global__ void __launch_bounds__(256) scatter_kernel(int prec, const double *__
     if (scal) block_max_to(prec == GKS_FP64 ? mx : (double)mxf, &scal->maxu2_bits);
 }
 
-__global__ void __launch_bounds__(256) gather_kernel(int prec, const void *S, double *dst, long np,
-                                                     int nx, int ny, int nz, int P0, int P1)
+template <int PREC>
+__global__ void __launch_bounds__(256) gather_kernel(const void *S, double *dst, long np, int nx, int ny, int nz,
+                                                     int P0, int P1)
 {
     const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y, k = blockIdx.z;
     if (i >= nx || j >= ny) return;
     const long N = (long)nx * ny * nz;
     const long ci = i + (long)nx * (j + (long)ny * k);
     const long lin = (long)(i + G) + (long)P0 * ((long)(j + G) + (long)P1 * (k + G));
-    double q[4];
-    load_cell(prec, S, np, lin, q);
+    if (PREC == GKS_FP64) {
+        const double *W = (const double *)S;
 #pragma unroll
-    for (int v = 0; v < 4; ++v) dst[v * N + ci] = q[v];
+        for (int v = 0; v < 4; ++v) dst[v * N + ci] = W[v * np + lin];
+    } else {
+        const float *W = (const float *)S;
+        float h[4], l[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            h[v] = W[v * np + lin];
+            l[v] = W[(4 + v) * np + lin];
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) dst[v * N + ci] = compose_hi_lo(h[v], l[v]);
+    }
 }
 
-// FP64 sums of mass, momentum and kinetic energy: per-block partial sums in
-// a fixed order, then one block adds the partials in order (deterministic).
-__global__ void __launch_bounds__(256) diag_partial_kernel(int prec, const void *S, long np, int nx,
-                                                           int ny, int nz, int P0, int P1,
-                                                           const double *hx, const double *hy,
+// a / b in FP64 from a double-single reciprocal r0 of b (within 2^-44): one
+// correction of the quotient by its remainder, 3 FP64 operations in place of
+// the library division's 9 or so (within one ulp of it).
+__device__ __forceinline__ double quotient(double a, double b, double r0)
+{
+    const double q = __dmul_rn(a, r0);
+    return fma(fma(-q, b, a), r0, q);
+}
+// Whether b and its reciprocal are far from the ends of the FP32 exponents.
+__device__ __forceinline__ bool rcp_range(unsigned int e) { return e >= 27u && e <= 227u; }
+
+// 1 / (h + l) as a double, within 2^-44, for h in the range of rcp_range.
+__device__ __forceinline__ double rcp_ds(float h, float l)
+{
+    const float r = rcp_approx(h);
+    const float e = __fmaf_rn(-l, r, __fmaf_rn(-h, r, 1.0f));
+    const float s = __fmul_rn(e, r);
+    const float rh = __fadd_rn(r, s);
+    return compose_hi_lo(rh, __fsub_rn(s, __fsub_rn(rh, r)));
+}
+
+// Sum of FP32 values with the rounding errors of the first two levels kept:
+// a + b + c holds the sum to about 2^-70 of its largest partial sum.
+struct Sum3 {
+    f2 a, b, c;
+    __device__ __forceinline__ void add(f2 x)
+    {
+        const dsf2 t = two_sum(a, x), u = two_sum(b, t.lo);
+        a = t.hi;
+        b = u.hi;
+        c += u.lo;
+    }
+    __device__ __forceinline__ void add_low(f2 x)
+    {
+        const dsf2 u = two_sum(b, x);
+        b = u.hi;
+        c += u.lo;
+    }
+};
+
+// FP64 sums of mass, momentum and kinetic energy: a block walks (32 x 8
+// columns) x (kDiagZ planes) pieces of the grid in a fixed order, a thread one
+// column of a piece; per-block partial sums, then one block adds the partials
+// in order (deterministic). GB300 runs FP64 at 1/64 of its FP32 rate, so what
+// counts is FP64 operations per cell (34 when every value was converted,
+// weighted by its cell volume and the energy divided out: 1.49 ms on 25.2M
+// cells against 0.12 ms of memory traffic). FP32C: the widths along z are
+// equal to 1e-12 (ZU), so mass and momentum are summed unweighted in FP32 with
+// their rounding errors kept (Sum3) and weighted once per column, the widths'
+// differences from the column's first one added as an FP32 correction; only
+// the energy stays FP64 per cell, 7 operations with a double-single
+// reciprocal of the density: 0.54 ms. A stretched z and FP64 grids weight each
+// value by its plane's width (a multiply-add each).
+constexpr int kDiagZ = 16;
+
+template <int PREC, bool ZU>
+__global__ void __launch_bounds__(256) diag_partial_kernel(const void *S, long np, int nx, int ny, int nz, int P0,
+                                                           int P1, const double *hx, const double *hy,
                                                            const double *hz, double *partials)
 {
     __shared__ double sh[5][256];
-    const long ncell = (long)nx * ny * nz;
+    __shared__ float dz[kDiagZ];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int NA = (nx + 31) / 32, NB = (ny + 7) / 8, NC = (nz + kDiagZ - 1) / kDiagZ;
+    const long nitems = (long)NA * NB * NC;
     double s[5] = {0, 0, 0, 0, 0};
-    for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < ncell;
-         c += (long)gridDim.x * blockDim.x) {
-        const int i = (int)(c % nx);
-        const long r = c / nx;
-        const int j = (int)(r % ny), k = (int)(r / ny);
-        const long lin = (long)(i + G) + (long)P0 * ((long)(j + G) + (long)P1 * (k + G));
-        double q[4];
-        load_cell(prec, S, np, lin, q);
-        const double vol = hx[i + G] * hy[j + G] * hz[k + G];
-        s[0] += q[0] * vol;
-        s[1] += q[1] * vol;
-        s[2] += q[2] * vol;
-        s[3] += q[3] * vol;
-        s[4] += 0.5 * (q[1] * q[1] + q[2] * q[2] + q[3] * q[3]) / q[0] * vol;
+    for (long it = blockIdx.x; it < nitems; it += gridDim.x) {
+        const long r = it / NA;
+        const int i = (int)(it - r * NA) * 32 + tx, j = (int)(r % NB) * 8 + ty;
+        const int k0 = (int)(r / NB) * kDiagZ, nk = min(kDiagZ, nz - k0);
+        if (ZU && PREC == GKS_FP32C) {
+            __syncthreads();
+            if ((int)threadIdx.x < nk) dz[threadIdx.x] = (float)(hz[k0 + threadIdx.x + G] - hz[k0 + G]);
+            __syncthreads();
+        }
+        if (i >= nx || j >= ny) continue;
+        const double area = hx[i + G] * hy[j + G], h0 = hz[k0 + G];
+        const long lin0 = (long)(i + G) + (long)P0 * ((long)(j + G) + (long)P1 * (k0 + G)), sz = (long)P0 * P1;
+        double t[5] = {0, 0, 0, 0, 0};   // the column's sums over z, times the widths
+        bool finite = true;
+        if (PREC == GKS_FP64) {
+            const double *W = (const double *)S;
+            for (int k = 0; k < nk; ++k) {
+                double q[4];
+#pragma unroll
+                for (int v = 0; v < 4; ++v) q[v] = W[v * np + lin0 + k * sz];
+                const double w = hz[k0 + k + G], m2 = fma(q[1], q[1], fma(q[2], q[2], q[3] * q[3]));
+                const int hw = __double2hiint(q[0]), e = ((hw >> 20) & 0x7ff) - 896;
+                double u;
+                if (e >= 27 && e <= 227) {
+                    // the top 24 bits of rho as a float, the rest as its low part
+                    const float f = __uint_as_float((hw & 0x80000000u) | ((unsigned int)e << 23) | ((hw & 0xfffffu) << 3) |
+                                                    ((unsigned int)__double2loint(q[0]) >> 29));
+                    const float g = __fmul_rn(__uint2float_rn((unsigned int)__double2loint(q[0]) & 0x1fffffffu),
+                                              __uint_as_float((unsigned int)(e > 52 ? e - 52 : 0) << 23));
+                    u = quotient(m2, q[0], rcp_ds(f, e > 52 ? copysignf(g, f) : 0.0f));
+                } else {
+                    u = m2 / q[0];
+                }
+#pragma unroll
+                for (int v = 0; v < 4; ++v) t[v] = fma(w, q[v], t[v]);
+                t[4] = fma(w, u, t[4]);
+            }
+        } else {
+            const float *W = (const float *)S;
+            const f2 z(0.0f);
+            Sum3 a[2] = {{z, z, z}, {z, z, z}};
+            f2 dc[2] = {z, z};
+            float de = 0.0f;
+#pragma unroll 2
+            for (int k = 0; k < nk; ++k) {
+                float h[4], l[4];
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    h[v] = W[v * np + lin0 + k * sz];
+                    l[v] = W[(4 + v) * np + lin0 + k * sz];
+                }
+                double m2 = 0.0;
+#pragma unroll
+                for (int v = 1; v < 4; ++v) {
+                    const double m = compose_hi_lo(h[v], l[v]);
+                    m2 = fma(m, m, m2);
+                }
+                const double rho = compose_hi_lo(h[0], l[0]);
+                const double u = rcp_range((__float_as_uint(h[0]) >> 23) & 0xffu) ? quotient(m2, rho, rcp_ds(h[0], l[0]))
+                                                                                  : m2 / rho;
+                if (ZU) {
+                    const f2 d(dz[k]);
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const f2 x(h[2 * q], h[2 * q + 1]);
+                        a[q].add(x);
+                        a[q].add_low(f2(l[2 * q], l[2 * q + 1]));
+                        dc[q] = fma(d, x, dc[q]);
+                    }
+                    de = __fmaf_rn(dz[k], __fmul_rn(__fmaf_rn(h[1], h[1], __fmaf_rn(h[2], h[2], h[3] * h[3])),
+                                                    rcp_approx(h[0])), de);
+                    t[4] += u;
+                } else {
+                    const double w = hz[k0 + k + G];
+                    t[0] = fma(w, rho, t[0]);
+#pragma unroll
+                    for (int v = 1; v < 4; ++v) t[v] = fma(w, compose_hi_lo(h[v], l[v]), t[v]);
+                    t[4] = fma(w, u, t[4]);
+                }
+            }
+            if (ZU) {
+                finite = isfinite(de) && isfinite(a[0].a.v.x) && isfinite(a[0].a.v.y) && isfinite(a[1].a.v.x) &&
+                         isfinite(a[1].a.v.y);
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    t[2 * q] = fma(h0, ((double)a[q].a.v.x + (double)a[q].b.v.x) + (double)a[q].c.v.x, (double)dc[q].v.x);
+                    t[2 * q + 1] =
+                        fma(h0, ((double)a[q].a.v.y + (double)a[q].b.v.y) + (double)a[q].c.v.y, (double)dc[q].v.y);
+                }
+                t[4] = fma(h0, t[4], (double)de);
+            }
+        }
+        if (!finite || !isfinite(t[4])) {
+            // an infinity, a NaN or an FP32 overflow: the column in plain FP64
+            for (int q = 0; q < 5; ++q) t[q] = 0.0;
+            for (int k = 0; k < nk; ++k) {
+                const double w = hz[k0 + k + G];
+                double q[4];
+                for (int v = 0; v < 4; ++v) {
+                    const long l = v * np + lin0 + k * sz;
+                    q[v] = PREC == GKS_FP64 ? ((const double *)S)[l]
+                                            : (double)((const float *)S)[l] + (double)((const float *)S)[4 * np + l];
+                    t[v] += w * q[v];
+                }
+                t[4] += w * ((q[1] * q[1] + q[2] * q[2] + q[3] * q[3]) / q[0]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s[q] = fma(area, t[q], s[q]);
+        s[4] = fma(0.5 * area, t[4], s[4]);
     }
 #pragma unroll
     for (int q = 0; q < 5; ++q) sh[q][threadIdx.x] = s[q];
@@ -1745,14 +1896,6 @@ __global__ void __launch_bounds__(256) raw_copy_kernel(T *S, T *cpt, int narr, l
         else
             S[a * np + lin] = cpt[a * N + ci];
     }
-}
-
-int reduce_blocks(long ncell)
-{
-    long b = (ncell + 255) / 256;
-    if (b > kMaxPartials) b = kMaxPartials;
-    if (b < 1) b = 1;
-    return (int)b;
 }
 
 }  // namespace
@@ -1895,8 +2038,10 @@ void launch_scatter_state_prep(const Ctx &c, const double *d_src)
 void launch_gather_state(const Ctx &c, double *d_dst)
 {
     dim3 blk(32, 8), g((c.n[0] + 31) / 32, (c.n[1] + 7) / 8, c.n[2]);
-    gather_kernel<<<g, blk, 0, c.stream>>>(c.prec, c.state, d_dst, c.np, c.n[0], c.n[1], c.n[2],
-                                           c.P[0], c.P[1]);
+    if (c.prec == GKS_FP64)
+        gather_kernel<GKS_FP64><<<g, blk, 0, c.stream>>>(c.state, d_dst, c.np, c.n[0], c.n[1], c.n[2], c.P[0], c.P[1]);
+    else
+        gather_kernel<GKS_FP32C><<<g, blk, 0, c.stream>>>(c.state, d_dst, c.np, c.n[0], c.n[1], c.n[2], c.P[0], c.P[1]);
 }
 
 void launch_fill_rest(const Ctx &c)
@@ -1941,10 +2086,13 @@ void launch_widen(const Ctx &c, const float *a, const float *b, double *out, lon
 
 void launch_diagnostics(const Ctx &c, double *d_out5)
 {
-    const int nb = reduce_blocks(c.ncell);
-    diag_partial_kernel<<<nb, 256, 0, c.stream>>>(c.prec, c.state, c.np, c.n[0], c.n[1], c.n[2],
-                                                  c.P[0], c.P[1], c.h64[0], c.h64[1], c.h64[2],
-                                                  c.partials);
+    const long items = (long)((c.n[0] + 31) / 32) * ((c.n[1] + 7) / 8) * ((c.n[2] + kDiagZ - 1) / kDiagZ);
+    const int nb = (int)std::min(items, (long)std::min(kMaxPartials, 4 * sm_count()));
+    auto kernel = c.prec == GKS_FP64 ? diag_partial_kernel<GKS_FP64, false>
+                  : c.uniform[2]     ? diag_partial_kernel<GKS_FP32C, true>
+                                     : diag_partial_kernel<GKS_FP32C, false>;
+    kernel<<<nb, 256, 0, c.stream>>>(c.state, c.np, c.n[0], c.n[1], c.n[2], c.P[0], c.P[1], c.h64[0], c.h64[1], c.h64[2],
+                                     c.partials);
     diag_final_kernel<<<1, 256, 0, c.stream>>>(c.partials, nb, d_out5);
 }
 
