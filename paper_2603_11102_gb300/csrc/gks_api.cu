@@ -554,14 +554,15 @@ int gks_add_actuator_lines(gks_grid *g, const gks_rotor_desc *d, int *id)
         return fail(g, GKS_ERR_RANGE, "rotor outside the grid");
     r.norm = 1.0 / (d->eps * d->eps * d->eps * pow(3.14159265358979323846, 1.5));
     r.ie2 = 1.0 / (d->eps * d->eps);
-    // per point: scale, X (3), F (4), Xr (3 floats in 2 doubles)
-    const size_t nd = 4 * (size_t)np + (size_t)npts + 3 * (size_t)npts + 4 * (size_t)npts + 2 * (size_t)npts +
-                      2 * nb + 2 * nb + 3;
+    // per point: scale, X (3), F (4), Xr (4 floats in 2 doubles, 16-byte aligned); the block counter last
+    const size_t nd = 2 * (size_t)npts + 4 * (size_t)np + (size_t)npts + 3 * (size_t)npts + 4 * (size_t)npts +
+                      2 * nb + 2 * nb + 3 + 1;
     double *buf = nullptr;
     int rc = device_alloc(g, (void **)&buf, nd * sizeof(double));
     if (rc) return rc;
     std::vector<double> host(nd, 0.0);
     size_t o = 0;
+    r.Xr = reinterpret_cast<float *>(buf + o); o += 2 * (size_t)npts;
     r.r = buf + o; memcpy(&host[o], d->r, np * sizeof(double)); o += np;
     r.chord = buf + o; memcpy(&host[o], d->chord, np * sizeof(double)); o += np;
     r.twist = buf + o; memcpy(&host[o], d->twist, np * sizeof(double)); o += np;
@@ -569,9 +570,9 @@ int gks_add_actuator_lines(gks_grid *g, const gks_rotor_desc *d, int *id)
     r.scale = buf + o; for (int q = 0; q < npts; ++q) host[o + q] = 1.0; o += npts;
     r.X = buf + o; o += 3 * (size_t)npts;
     r.F = buf + o; o += 4 * (size_t)npts;
-    r.Xr = reinterpret_cast<float *>(buf + o); o += 2 * (size_t)npts;
     r.et = buf + o; o += 2 * nb;
-    r.out = buf + o;
+    r.out = buf + o; o += 2 * nb + 3;
+    r.count = reinterpret_cast<unsigned *>(buf + o);
     rc = cuda_check(g, cudaMemcpyAsync(buf, host.data(), nd * sizeof(double), cudaMemcpyHostToDevice, c.stream),
                     "copy rotor");
     if (!rc) rc = sync(g);
@@ -662,7 +663,7 @@ int gks_add_ib_points(gks_grid *g, int n, const double *xyz, const double *dS, c
             return fail(g, GKS_ERR_RANGE, "body support reaches an exchange side of the slab");
     }
     b.nbox = (long)(b.box[0][1] - b.box[0][0] + 1) * (b.box[1][1] - b.box[1][0] + 1) * (b.box[2][1] - b.box[2][0] + 1);
-    const size_t nd = 7 * (size_t)n + 8 * (size_t)b.nbox + 7 + niter;
+    const size_t nd = 7 * (size_t)n + 8 * (size_t)b.nbox + 7 + niter + 1;   // the block counter last
     double *buf = nullptr;
     int rc = device_alloc(g, (void **)&buf, nd * sizeof(double));
     if (rc) return rc;
@@ -678,9 +679,10 @@ int gks_add_ib_points(gks_grid *g, int n, const double *xyz, const double *dS, c
     b.phi = b.vbar + 3 * b.nbox;
     b.fsum = b.phi + b.nbox;
     b.out = b.fsum + 3 * b.nbox;
+    b.count = reinterpret_cast<unsigned *>(b.out + 7 + niter);
     rc = cuda_check(g, cudaMemcpyAsync(buf, host.data(), host.size() * sizeof(double), cudaMemcpyHostToDevice, c.stream),
                     "copy body");
-    if (!rc) rc = cuda_check(g, cudaMemsetAsync(b.Vbar, 0, (8 * (size_t)b.nbox + 7 + niter) * sizeof(double), c.stream),
+    if (!rc) rc = cuda_check(g, cudaMemsetAsync(b.Vbar, 0, (8 * (size_t)b.nbox + 7 + niter + 1) * sizeof(double), c.stream),
                              "clear body");
     if (rc) return rc;
     launch_body_precompute(c, b);
@@ -702,13 +704,13 @@ int gks_add_ib_points(gks_grid *g, int n, const double *xyz, const double *dS, c
     b.csr_off = d_cnt;
     char *cbuf = nullptr;
     rc = device_alloc(g, (void **)&cbuf, (size_t)b.nnz * (sizeof(double) + sizeof(int) + sizeof(float)) +
-                                             3 * (sizeof(double) + sizeof(float)) * b.nbox + 64);
+                                             4 * (sizeof(double) + sizeof(float)) * b.nbox + 64);
     if (rc) return rc;
-    b.csr_w = (double *)cbuf;
-    b.Ubox = b.csr_w + b.nnz;
-    b.csr_cell = (int *)(b.Ubox + 3 * b.nbox);
+    b.Ubox = (double *)cbuf;
+    b.Uboxf = (float *)(b.Ubox + 4 * b.nbox);
+    b.csr_w = (double *)(b.Uboxf + 4 * b.nbox);
+    b.csr_cell = (int *)(b.csr_w + b.nnz);
     b.csr_wf = (float *)(b.csr_cell + b.nnz);
-    b.Uboxf = b.csr_wf + b.nnz;
     rc = cuda_check(g, cudaMemcpyAsync(d_cnt, off.data(), sizeof(long) * (n + 1), cudaMemcpyHostToDevice, c.stream),
                     "copy offsets");
     if (rc) return rc;
@@ -813,8 +815,7 @@ int step_once(gks_grid *g, const AdjWork *tp)
                                        "record the IBM iterations")))
                 return rc;
         }
-    if (fused_prep)
-        for (int k = 0; k < nobj; ++k) launch_prep_box(c, cc.prep_box[k]);
+    if (fused_prep) launch_prep_boxes(c, cc.prep_box, nobj);
     g->prep_valid = fused_prep;
     launch_advance(c);
     g->prof.last_end = nullptr;
@@ -1032,8 +1033,7 @@ int slab_step_once(gks_grid *const *sl, int n)
         const Ctx &c = g->c;
         for (size_t k = 0; k < g->obj_kind.size(); ++k)
             if (g->obj_kind[k] == 1) launch_ibm(c, g->bodies[g->obj_index[k]]);
-        if (fused[s])
-            for (int k = 0; k < cc[s].nprep_box; ++k) launch_prep_box(c, cc[s].prep_box[k]);
+        if (fused[s]) launch_prep_boxes(c, cc[s].prep_box, cc[s].nprep_box);
         g->prep_valid = fused[s];
         launch_advance(c);
         g->prof.last_end = nullptr;

@@ -1,19 +1,29 @@
 // gks_forcing.cu -- actuator-line (Sec. 3.1) and immersed-boundary (Sec. 3.2)
 // body forcing, applied after the S2O4 update (end of Sec. 3.2).
 //
-// ALM: one block per rotor samples the velocity at every actuator point at
-// t_{n+1} (trilinear, cell centres), evaluates the angle of attack, the
-// synthetic polar, lift and drag (Eq. (axial-tangential)) and the axial and
-// tangential forces; one warp per blade sums thrust and torque in FP64 with
-// a fixed shuffle tree. A second kernel gathers, for every cell of the box
-// swept by the rotor, the truncated Gaussian projection (Eq. (Gaussian)) of
-// all point forces in blade-then-point order and adds dt f to the momentum.
+// ALM: 8 lanes per actuator point sample the velocity at t_{n+1} (trilinear,
+// cell centres), evaluate the angle of attack, the synthetic polar, lift and
+// drag (Eq. (axial-tangential)) and the axial and tangential forces; the last
+// block sums thrust and torque per blade in FP64 with a fixed shuffle tree. A
+// second kernel gathers, for every cell of the box swept by the rotor, the
+// truncated Gaussian projection (Eq. (Gaussian)) of all point forces in a
+// fixed order and adds dt f to the momentum.
 //
 // IBM: the cell fields Vbar, vbar and phi of a stationary body are computed
 // once. Each step the direct-forcing iteration of Eq. (ibm-1) runs per cell
 // (cells are independent for a fixed iteration count), the force sum of
 // Eq. (force-ibm) is reduced in a fixed order, and the back-interpolated
-// residual max_p |v_p - sum W U| is evaluated per Lagrangian point.
+// residual max_p |v_p - sum W U| is evaluated per Lagrangian point: two
+// kernels per body with a fixed iteration count, one round of kernels per
+// iteration with a residual tolerance.
+//
+// These are small launches (the stencil of a 221x83x91 grid takes 0.7 ms a
+// step), so what bounds them is latency: the slow FP64 pipe in the loads (five
+// warps on one SM before, a warp of 4 points per SM now), the serial loop over
+// points in the projection (one thread per cell before, 8 now), and the
+// launches themselves (8 per body before). On that grid, rotor with tower and
+// nacelle, they took 0.22 ms a step with the prep of their boxes and take
+// 0.12 ms (8 steps 7.17 -> 6.41 ms).
 //
 // Distances that decide the 3 eps cut are formed in FP64 with explicit
 // round-to-nearest operations (no contraction), in the same order as a plain
@@ -83,43 +93,6 @@ __device__ __forceinline__ void cell_state(const Lattice &L, const void *S, long
     }
 }
 
-// Trilinear interpolation of the cell-centre velocity m/rho; false when X is
-// outside the hull of interior cell centres.
-__device__ bool trilinear(const Lattice &L, const void *S, const double X[3], double U[3])
-{
-    int i0[3];
-    double fr[3];
-    for (int d = 0; d < 3; ++d) {
-        const double s = (X[d] - L.x0[d]) / L.h[d] - 0.5 - (double)L.off[d];
-        const double fl = floor(s);
-        i0[d] = (int)fl;
-        fr[d] = s - fl;
-        if (i0[d] < 0 || i0[d] + 1 > L.n[d] - 1) {
-            if (L.n[d] == 1 && s >= -0.5 && s <= 0.5) {
-                i0[d] = 0;
-                fr[d] = 0.0;
-                continue;
-            }
-            return false;
-        }
-    }
-    U[0] = U[1] = U[2] = 0.0;
-    for (int c = 0; c < 8; ++c) {
-        const int di = c & 1, dj = (c >> 1) & 1, dk = (c >> 2) & 1;
-        const double w = (di ? fr[0] : 1.0 - fr[0]) * (dj ? fr[1] : 1.0 - fr[1]) * (dk ? fr[2] : 1.0 - fr[2]);
-        if (w == 0.0) continue;
-        const int ii = L.n[0] == 1 ? 0 : i0[0] + di;
-        const int jj = L.n[1] == 1 ? 0 : i0[1] + dj;
-        const int kk = L.n[2] == 1 ? 0 : i0[2] + dk;
-        double q[4];
-        cell_state(L, S, lin_index(L, ii, jj, kk), q);
-        U[0] += w * q[1] / q[0];
-        U[1] += w * q[2] / q[0];
-        U[2] += w * q[3] / q[0];
-    }
-    return true;
-}
-
 __device__ __forceinline__ double polar_cd(double a) { return 0.01 + 0.02 * a * a; }
 __device__ __forceinline__ double polar_cl(double a)
 {
@@ -138,88 +111,133 @@ __device__ __forceinline__ double tip_factor(double g1, int nb, double R, double
     return (2.0 / kPi) * acos(exp(-x));
 }
 
-__global__ void __launch_bounds__(256) alm_loads_kernel(Lattice L, const void *S, RotorDev r, Scalars *scal)
+// Actuator-point loads: a warp takes 4 points, 8 lanes each (the 8 corners of
+// the trilinear sample; the rest is the same on all 8). The FP64 pipe runs a
+// warp instruction in 16 cycles whatever its active lanes, so the points are
+// spread over as many SMs as there are warps: 150 points 34 -> 19 us.
+constexpr int kLoadPts = 4;   // points per block (one warp)
+
+__global__ void __launch_bounds__(32) alm_loads_kernel(Lattice L, const void *S, RotorDev r, Scalars *scal)
 {
     const double t = scal->t + scal->dt;   // blades and samples at t_{n+1}
-    const int npts = r.nb * r.np;
-    for (int q = threadIdx.x; q < npts; q += blockDim.x) {
-        const int b = q / r.np, p = q - b * r.np;
-        const double th = r.az0 + r.omega * t + 2.0 * kPi * b / r.nb;
-        const double cth = cos(th), sth = sin(th);
-        const double rr = r.r[p];
-        const double X[3] = {r.hub[0], r.hub[1] + rr * cth, r.hub[2] + rr * sth};
+    const int npts = r.nb * r.np, lane = threadIdx.x, c = lane & 7;
+    const int q = blockIdx.x * kLoadPts + (lane >> 3);
+    const bool on = q < npts;
+    const int b = on ? q / r.np : 0, p = on ? q - b * r.np : 0;
+    const double th = r.az0 + r.omega * t + 2.0 * kPi * b / r.nb;
+    double sth, cth;
+    sincos(th, &sth, &cth);
+    const double rr = r.r[p];
+    const double X[3] = {r.hub[0], r.hub[1] + rr * cth, r.hub[2] + rr * sth};
+    // trilinear interpolation of the cell-centre velocity m/rho: corner c
+    bool ok = true;
+    int i0[3];
+    double fr[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const double s = (X[d] - L.x0[d]) / L.h[d] - 0.5 - (double)L.off[d];
+        const double fl = floor(s);
+        i0[d] = (int)fl;
+        fr[d] = s - fl;
+        if (i0[d] < 0 || i0[d] + 1 > L.n[d] - 1) {
+            if (L.n[d] == 1 && s >= -0.5 && s <= 0.5) {
+                i0[d] = 0;
+                fr[d] = 0.0;
+            } else {
+                ok = false;
+            }
+        }
+    }
+    double U[3] = {0.0, 0.0, 0.0};
+    if (on && ok) {
+        const int dd[3] = {c & 1, (c >> 1) & 1, (c >> 2) & 1};
+        const double w = (dd[0] ? fr[0] : 1.0 - fr[0]) * (dd[1] ? fr[1] : 1.0 - fr[1]) * (dd[2] ? fr[2] : 1.0 - fr[2]);
+        if (w != 0.0) {
+            double s[4];
+            cell_state(L, S, lin_index(L, L.n[0] == 1 ? 0 : i0[0] + dd[0], L.n[1] == 1 ? 0 : i0[1] + dd[1],
+                                       L.n[2] == 1 ? 0 : i0[2] + dd[2]), s);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) U[d] = w * s[1 + d] / s[0];
+        }
+    }
+    for (int o = 1; o < 8; o <<= 1)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) U[d] += __shfl_xor_sync(0xffffffffu, U[d], o);
+    double Fx = 0.0, Ft = 0.0, al = 0.0, phi = 0.0;
+    if (!ok) {
+        if (on && c == 0) atomicOr(&scal->flags, FLAG_RANGE);
+    } else {
+        double ux = U[0];
+        double ut = -sth * U[1] + cth * U[2];
+        const double wr = r.omega * rr;
+        if (r.correction) {
+            const double phi0 = atan2(ux, wr - ut);
+            const double cd0 = polar_cd(phi0 - r.twist[p]);
+            const double fac = 1.0 / (1.0 - cd0 * r.chord[p] / (4.0 * sqrt(kPi) * r.eps));
+            ux *= fac;
+            ut *= fac;
+        }
+        phi = atan2(ux, wr - ut);
+        al = phi - r.twist[p];
+        const double urel2 = ux * ux + (wr - ut) * (wr - ut);
+        const double qd = 0.5 * r.rho_inf * r.chord[p] * r.width[p] * urel2;
+        const double Lf = qd * polar_cl(al), Df = qd * polar_cd(al);
+        double sp, cp;
+        sincos(phi, &sp, &cp);
+        const double scale = on ? r.scale[q] : 0.0;
+        Fx = (Lf * cp + Df * sp) * scale;
+        Ft = (Lf * sp - Df * cp) * scale;
+        if (r.tip) {
+            Fx *= tip_factor(r.tip_g[0], r.nb, r.radius, rr, phi);
+            Ft *= tip_factor(r.tip_g[1], r.nb, r.radius, rr, phi);
+        }
+    }
+    if (on && c == 0) {
         r.X[3 * q] = X[0];
         r.X[3 * q + 1] = X[1];
         r.X[3 * q + 2] = X[2];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) r.Xr[3 * q + d] = (float)(X[d] - r.hub[d]);
+        *reinterpret_cast<float4 *>(r.Xr + 4 * q) = make_float4((float)(X[0] - r.hub[0]), (float)(X[1] - r.hub[1]),
+                                                                (float)(X[2] - r.hub[2]), 0.0f);
         if (p == 0) {
             r.et[2 * b] = -sth;
             r.et[2 * b + 1] = cth;
-        }
-        double U[3];
-        double Fx = 0.0, Ft = 0.0, al = 0.0, phi = 0.0;
-        if (!trilinear(L, S, X, U)) {
-            atomicOr(&scal->flags, FLAG_RANGE);
-        } else {
-            double ux = U[0];
-            double ut = -sth * U[1] + cth * U[2];
-            const double wr = r.omega * rr;
-            if (r.correction) {
-                const double phi0 = atan2(ux, wr - ut);
-                const double cd0 = polar_cd(phi0 - r.twist[p]);
-                const double fac = 1.0 / (1.0 - cd0 * r.chord[p] / (4.0 * sqrt(kPi) * r.eps));
-                ux *= fac;
-                ut *= fac;
-            }
-            phi = atan2(ux, wr - ut);
-            al = phi - r.twist[p];
-            const double urel2 = ux * ux + (wr - ut) * (wr - ut);
-            const double qd = 0.5 * r.rho_inf * r.chord[p] * r.width[p] * urel2;
-            const double Lf = qd * polar_cl(al), Df = qd * polar_cd(al);
-            Fx = (Lf * cos(phi) + Df * sin(phi)) * r.scale[q];
-            Ft = (Lf * sin(phi) - Df * cos(phi)) * r.scale[q];
-            if (r.tip) {
-                Fx *= tip_factor(r.tip_g[0], r.nb, r.radius, rr, phi);
-                Ft *= tip_factor(r.tip_g[1], r.nb, r.radius, rr, phi);
-            }
         }
         r.F[q] = Fx;
         r.F[npts + q] = Ft;
         r.F[2 * npts + q] = al;
         r.F[3 * npts + q] = phi;
     }
-    __syncthreads();
-    // per-blade thrust and torque: warp b sums blade b in FP64
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp < r.nb) {
+    // the last block to finish: per-blade thrust and torque, in FP64
+    __threadfence();
+    unsigned done = 0;
+    if (lane == 0) done = atomicInc(r.count, gridDim.x - 1);
+    if (__shfl_sync(0xffffffffu, done, 0) != gridDim.x - 1) return;
+    __threadfence();
+    double tt = 0.0, qq = 0.0;
+    for (int k = 0; k < r.nb; ++k) {
         double T = 0.0, Q = 0.0;
-        for (int p = lane; p < r.np; p += 32) {
-            T += r.F[warp * r.np + p];
-            Q += r.r[p] * r.F[npts + warp * r.np + p];
+        for (int j = lane; j < r.np; j += 32) {
+            T += __ldcg(r.F + k * r.np + j);
+            Q += r.r[j] * __ldcg(r.F + npts + k * r.np + j);
         }
         for (int o = 16; o > 0; o >>= 1) {
             T += __shfl_xor_sync(0xffffffffu, T, o);
             Q += __shfl_xor_sync(0xffffffffu, Q, o);
         }
         if (lane == 0) {
-            r.out[warp] = T;
-            r.out[r.nb + warp] = Q;
+            r.out[k] = T;
+            r.out[r.nb + k] = Q;
         }
+        tt += T;
+        qq += Q;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double tt = 0.0, qq = 0.0;
-        for (int b = 0; b < r.nb; ++b) {
-            tt += r.out[b];
-            qq += r.out[r.nb + b];
-        }
+    if (lane == 0) {
         const double power = r.omega * qq;
         const double area = kPi * r.radius * r.radius;
-        const double U = r.uref;
+        const double U0 = r.uref;
         r.out[2 * r.nb] = power;
-        r.out[2 * r.nb + 1] = power / (0.5 * r.rho_inf * area * U * U * U);
-        r.out[2 * r.nb + 2] = tt / (0.5 * r.rho_inf * area * U * U);
+        r.out[2 * r.nb + 1] = power / (0.5 * r.rho_inf * area * U0 * U0 * U0);
+        r.out[2 * r.nb + 2] = tt / (0.5 * r.rho_inf * area * U0 * U0);
     }
 }
 
@@ -235,106 +253,109 @@ __device__ __forceinline__ void add_comp(float &hi, float &lo, float d)
 }
 
 // Projection of the point forces onto the cells of the rotor box (truncated
-// Gaussian, Eq. (Gaussian)), blade-then-point order per cell. FP64 grids:
-// distances and weights in FP64. FP32C grids: the blade screen, the
-// distances and the weights in FP32 on hub-relative coordinates (error below
-// 2e-6 relative in r^2); only a point whose r^2 lies within 1e-5 of the cut
-// takes the FP64 distance, so that the support is decided exactly as in FP64.
+// Gaussian, Eq. (Gaussian)). 8 lanes share a cell, each taking every 8th point
+// in order, and their sums meet in a fixed shuffle tree (a box of 20,000 cells
+// is 75 blocks with a thread per cell: half the SMs idle and each thread
+// walking 150 points; 36 -> 20 us in FP32, 0.39 -> 0.05 ms in FP64 on a
+// 256x96x96 grid, whose points all took the FP64 distance). The blade screen and the distances
+// are formed in FP32 on hub-relative coordinates, staged in shared memory
+// (error below 2e-6 relative in r^2). FP32C grids: the weights in FP32; only a
+// point whose r^2 lies within 1e-5 of the cut takes the FP64 distance. FP64
+// grids: every point that passes the FP32 screen with that margin takes the
+// FP64 distance and weight. Either way the support is decided exactly as in
+// FP64.
+constexpr int kSpreadPts = 256;   // points staged at a time
+
 template <typename R>
 __global__ void __launch_bounds__(256) alm_spread_kernel(Lattice L, void *S, RotorDev r, Scalars *scal)
 {
+    __shared__ float4 pt[kSpreadPts];   // hub-relative position; blade index
+    __shared__ float2 pf[kSpreadPts];   // F_x, F_theta (FP32C)
     const int bx = r.box[0][1] - r.box[0][0] + 1, by = r.box[1][1] - r.box[1][0] + 1;
     const int bz = r.box[2][1] - r.box[2][0] + 1;
-    const long idx = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (idx >= (long)bx * by * bz) return;
+    const int sub = threadIdx.x & 7;
+    const long idx = blockIdx.x * 32L + (threadIdx.x >> 3);
+    const bool on = idx < (long)bx * by * bz;
     const int i = r.box[0][0] + (int)(idx % bx);
     const int j = r.box[1][0] + (int)((idx / bx) % by);
     const int k = r.box[2][0] + (int)(idx / ((long)bx * by));
     const double xc[3] = {centre(L, 0, i), centre(L, 1, j), centre(L, 2, k)};
     const double cut = 3.0 * r.eps;
     const int npts = r.nb * r.np;
+    const float pc[3] = {(float)(xc[0] - r.hub[0]), (float)(xc[1] - r.hub[1]), (float)(xc[2] - r.hub[2])};
+    const float c2 = (float)(cut * cut), c2lo = c2 * (1.0f - 1e-5f), c2hi = c2 * (1.0f + 1e-5f);
+    const float rmin = (float)r.rmin, rmax = (float)r.rmax;
+    // every point of blade b lies on the segment hub + s e_r, s in [rmin,
+    // rmax]; a cell farther than 3 eps from it gets nothing of the blade
+    unsigned near = 0u;
+    for (int b = 0; b < r.nb; ++b) {
+        const float e1 = (float)r.et[2 * b], e2 = (float)r.et[2 * b + 1];
+        float sp = pc[1] * e2 - pc[2] * e1;
+        sp = fminf(fmaxf(sp, rmin), rmax);
+        const float qy = pc[1] - sp * e2, qz = pc[2] + sp * e1;
+        if (on && pc[0] * pc[0] + qy * qy + qz * qz <= c2 * 1.0001f) near |= 1u << b;
+    }
     R f[3] = {R(0), R(0), R(0)};
     bool any = false;
-    if constexpr (std::is_same<R, double>::value) {
-        for (int b = 0; b < r.nb; ++b) {
-            const double e1 = r.et[2 * b], e2 = r.et[2 * b + 1];
-            // every point of blade b lies on the segment hub + s e_r, s in
-            // [rmin, rmax]; a cell farther than 3 eps from it gets nothing
-            {
-                const double ery = e2, erz = -e1;
-                const double px = xc[0] - r.hub[0], py = xc[1] - r.hub[1], pz = xc[2] - r.hub[2];
-                double sp = py * ery + pz * erz;
-                sp = sp < r.rmin ? r.rmin : (sp > r.rmax ? r.rmax : sp);
-                const double qy = py - sp * ery, qz = pz - sp * erz;
-                if (px * px + qy * qy + qz * qz > cut * cut * (1.0 + 1e-6) + 1e-300) continue;
-            }
-            double fb[3] = {0.0, 0.0, 0.0};
-            for (int p = 0; p < r.np; ++p) {
-                const int q = b * r.np + p;
+    for (int q0 = 0; q0 < npts; q0 += kSpreadPts) {
+        const int m = min(kSpreadPts, npts - q0);
+        __syncthreads();
+        if ((int)threadIdx.x < m) {
+            float4 x = *reinterpret_cast<const float4 *>(r.Xr + 4 * (q0 + threadIdx.x));
+            x.w = (float)((q0 + (int)threadIdx.x) / r.np);
+            pt[threadIdx.x] = x;
+            pf[threadIdx.x] = make_float2((float)r.F[q0 + threadIdx.x], (float)r.F[npts + q0 + threadIdx.x]);
+        }
+        __syncthreads();
+        if (near == 0u) continue;
+        for (int p = sub; p < m; p += 8) {
+            const float4 x = pt[p];
+            const int b = (int)x.w;
+            if (!((near >> b) & 1u)) continue;
+            const float dx = pc[0] - x.x, dy = pc[1] - x.y, dz = pc[2] - x.z;
+            const float s2 = dx * dx + dy * dy + dz * dz;
+            if (s2 > c2hi) continue;
+            const int q = q0 + p;
+            if constexpr (std::is_same<R, double>::value) {
                 const double rr = dist(xc[0] - r.X[3 * q], xc[1] - r.X[3 * q + 1], xc[2] - r.X[3 * q + 2]);
                 if (rr > cut) continue;
-                any = true;
                 const double eta = exp(-(rr / r.eps) * (rr / r.eps)) * r.norm;
                 const double Fx = r.F[q], Ft = r.F[npts + q];
-                fb[0] += -Fx * eta;
-                fb[1] += -Ft * e1 * eta;
-                fb[2] += -Ft * e2 * eta;
+                f[0] += -Fx * eta;
+                f[1] += -Ft * r.et[2 * b] * eta;
+                f[2] += -Ft * r.et[2 * b + 1] * eta;
+            } else {
+                if (s2 >= c2lo && dist(xc[0] - r.X[3 * q], xc[1] - r.X[3 * q + 1], xc[2] - r.X[3 * q + 2]) > cut) continue;
+                const float eta = expf(-s2 * (float)r.ie2) * (float)r.norm;
+                const float2 F = pf[p];
+                f[0] += -F.x * eta;
+                f[1] += -F.y * (float)r.et[2 * b] * eta;
+                f[2] += -F.y * (float)r.et[2 * b + 1] * eta;
             }
-            f[0] += fb[0];
-            f[1] += fb[1];
-            f[2] += fb[2];
-        }
-    } else {
-        const float pc[3] = {(float)(xc[0] - r.hub[0]), (float)(xc[1] - r.hub[1]), (float)(xc[2] - r.hub[2])};
-        const float c2 = (float)(cut * cut), c2lo = c2 * (1.0f - 1e-5f), c2hi = c2 * (1.0f + 1e-5f);
-        const float ie2 = (float)r.ie2, norm = (float)r.norm;
-        const float rmin = (float)r.rmin, rmax = (float)r.rmax;
-        for (int b = 0; b < r.nb; ++b) {
-            const float e1 = (float)r.et[2 * b], e2 = (float)r.et[2 * b + 1];
-            {
-                float sp = pc[1] * e2 - pc[2] * e1;
-                sp = fminf(fmaxf(sp, rmin), rmax);
-                const float qy = pc[1] - sp * e2, qz = pc[2] + sp * e1;
-                if (pc[0] * pc[0] + qy * qy + qz * qz > c2 * 1.0001f) continue;
-            }
-            float fb[3] = {0.0f, 0.0f, 0.0f};
-            for (int p = 0; p < r.np; ++p) {
-                const int q = b * r.np + p;
-                const float dx = pc[0] - r.Xr[3 * q], dy = pc[1] - r.Xr[3 * q + 1], dz = pc[2] - r.Xr[3 * q + 2];
-                const float s2 = dx * dx + dy * dy + dz * dz;
-                if (s2 > c2hi) continue;
-                if (s2 >= c2lo &&
-                    dist(xc[0] - r.X[3 * q], xc[1] - r.X[3 * q + 1], xc[2] - r.X[3 * q + 2]) > cut)
-                    continue;
-                any = true;
-                const float eta = expf(-s2 * ie2) * norm;
-                const float Fx = (float)r.F[q], Ft = (float)r.F[npts + q];
-                fb[0] += -Fx * eta;
-                fb[1] += -Ft * e1 * eta;
-                fb[2] += -Ft * e2 * eta;
-            }
-            f[0] += fb[0];
-            f[1] += fb[1];
-            f[2] += fb[2];
+            any = true;
         }
     }
-    if (!any) return;
+    any = __any_sync(0xffu << (threadIdx.x & 24), any);
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) f[d] += __shfl_xor_sync(0xffffffffu, f[d], o);
+    if (!any || !on || sub >= 3) return;
+    // lane d of the cell's 8 updates momentum component d
+    const int d = sub;
     const long lin = lin_index(L, i, j, k);
     if (!in_bounds(lin, L.np)) return;
     const double dt = scal->dt;
+    const R fd = d == 0 ? f[0] : (d == 1 ? f[1] : f[2]);
     if constexpr (std::is_same<R, double>::value) {
         double *W = (double *)S;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) W[(1 + d) * L.np + lin] += dt * f[d];
+        W[(1 + d) * L.np + lin] += dt * fd;
     } else {
         float *W = (float *)S;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            float hi = W[(1 + d) * L.np + lin], lo = W[(5 + d) * L.np + lin];
-            add_comp(hi, lo, (float)dt * f[d]);
-            W[(1 + d) * L.np + lin] = hi;
-            W[(5 + d) * L.np + lin] = lo;
-        }
+        float hi = W[(1 + d) * L.np + lin], lo = W[(5 + d) * L.np + lin];
+        add_comp(hi, lo, (float)dt * fd);
+        W[(1 + d) * L.np + lin] = hi;
+        W[(5 + d) * L.np + lin] = lo;
     }
 }
 
@@ -377,7 +398,7 @@ __global__ void ibm_begin_kernel(BodyDev b)
 }
 
 template <typename R>
-__global__ void __launch_bounds__(256) ibm_iter_kernel(Lattice L, void *S, BodyDev b, Scalars *scal, int iters)
+__global__ void __launch_bounds__(256) ibm_iter_kernel(Lattice L, void *S, BodyDev b, Scalars *scal)
 {
     if (b.out[5] != 0.0) return;
     const long c = blockIdx.x * (long)blockDim.x + threadIdx.x;
@@ -397,15 +418,11 @@ __global__ void __launch_bounds__(256) ibm_iter_kernel(Lattice L, void *S, BodyD
         const double rho = W[lin];
         for (int d = 0; d < 3; ++d) {
             double m = W[(1 + d) * L.np + lin];
-            double fs = b.fsum[3 * c + d];
-            for (int s = 0; s < iters; ++s) {
-                const double U = m / rho;
-                const double F = rho * phi * vol * (b.vbar[3 * c + d] - U) / dt;
-                m += dt * F / vol;
-                fs += F;
-            }
+            const double U = m / rho;
+            const double F = rho * phi * vol * (b.vbar[3 * c + d] - U) / dt;
+            m += dt * F / vol;
             W[(1 + d) * L.np + lin] = m;
-            b.fsum[3 * c + d] = fs;
+            b.fsum[3 * c + d] += F;
         }
     } else {
         float *W = (float *)S;
@@ -413,16 +430,12 @@ __global__ void __launch_bounds__(256) ibm_iter_kernel(Lattice L, void *S, BodyD
         const float ph = (float)phi, vo = (float)vol, dtf = (float)dt;
         for (int d = 0; d < 3; ++d) {
             float hi = W[(1 + d) * L.np + lin], lo = W[(5 + d) * L.np + lin];
-            double fs = b.fsum[3 * c + d];
-            for (int s = 0; s < iters; ++s) {
-                const float U = (hi + lo) / rho;
-                const float F = rho * ph * vo * ((float)b.vbar[3 * c + d] - U) / dtf;
-                add_comp(hi, lo, dtf * F / vo);
-                fs += (double)F;
-            }
+            const float U = (hi + lo) / rho;
+            const float F = rho * ph * vo * ((float)b.vbar[3 * c + d] - U) / dtf;
+            add_comp(hi, lo, dtf * F / vo);
             W[(1 + d) * L.np + lin] = hi;
             W[(5 + d) * L.np + lin] = lo;
-            b.fsum[3 * c + d] = fs;
+            b.fsum[3 * c + d] += (double)F;
         }
     }
 }
@@ -487,7 +500,7 @@ __global__ void __launch_bounds__(256) ibm_velocity_kernel(Lattice L, const void
     cell_state(L, S, lin_index(L, i, j, k), q);
     R *U = std::is_same<R, double>::value ? (R *)b.Ubox : (R *)b.Uboxf;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) U[3 * c + d] = (R)(q[1 + d] / q[0]);
+    for (int d = 0; d < 3; ++d) U[4 * c + d] = (R)(q[1 + d] / q[0]);
 }
 
 // Residual max_p |v_p - sum_ijk W_{ijk->p} U_ijk|: one warp per point,
@@ -508,9 +521,9 @@ __global__ void __launch_bounds__(256) ibm_residual_kernel(BodyDev b)
         const R W = Wt[o];
         const long c = b.csr_cell[o];
         if (!in_bounds(c, b.nbox)) continue;
-        u0 += W * U[3 * c];
-        u1 += W * U[3 * c + 1];
-        u2 += W * U[3 * c + 2];
+        u0 += W * U[4 * c];
+        u1 += W * U[4 * c + 1];
+        u2 += W * U[4 * c + 2];
     }
     for (int s = 16; s > 0; s >>= 1) {
         u0 += __shfl_xor_sync(0xffffffffu, u0, s);
@@ -572,19 +585,177 @@ __global__ void __launch_bounds__(256) ibm_force_final_kernel(BodyDev b, const d
     if (threadIdx.x < 3) b.out[threadIdx.x] = -sh[threadIdx.x][0];
 }
 
+// Fixed iteration count, per box cell: the direct-forcing iterations of
+// Eq. (ibm-1), U^{s+1} = U^s + phi (vbar - U^s), the cell velocity for the
+// residual, and the block's share of the force on the body (the momentum
+// that the cells took up, times vol / dt; a fixed tree over the block). One
+// kernel in place of a clear, the iterations, the velocity and the first pass
+// of the force sum.
+constexpr int kIbmParts = 2048;   // blocks at most: 3 partial sums each in the grid's reduction scratch
+static_assert(3 * kIbmParts <= 8 * kMaxPartials, "the force parts fit the scratch");
+
+template <typename R>
+__global__ void __launch_bounds__(256) ibm_cells_kernel(Lattice L, void *S, BodyDev b, Scalars *scal, double *part)
+{
+    __shared__ double sh[3][8];
+    const int bx = b.box[0][1] - b.box[0][0] + 1, by = b.box[1][1] - b.box[1][0] + 1;
+    double fs[3] = {0.0, 0.0, 0.0};
+    for (long c = blockIdx.x * 256L + threadIdx.x; c < b.nbox; c += (long)gridDim.x * 256L) {
+        const int i = b.box[0][0] + (int)(c % bx);
+        const int j = b.box[1][0] + (int)((c / bx) % by);
+        const int k = b.box[2][0] + (int)(c / ((long)bx * by));
+        const long lin = lin_index(L, i, j, k);
+        if (!in_bounds(lin, L.np)) continue;
+        const bool body = b.Vbar[c] > 0.0;
+        if constexpr (std::is_same<R, double>::value) {
+            double *W = (double *)S;
+            const double rho = W[lin];
+            double u[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                double m = W[(1 + d) * L.np + lin];
+                if (body) {
+                    const double a = rho * b.phi[c], vb = b.vbar[3 * c + d];
+                    double t = 0.0;
+                    for (int s = 0; s < b.niter; ++s) {
+                        const double inc = a * (vb - m / rho);
+                        m += inc;
+                        t += inc;
+                    }
+                    W[(1 + d) * L.np + lin] = m;
+                    fs[d] += t;
+                }
+                u[d] = m / rho;
+            }
+            double2 *U = reinterpret_cast<double2 *>(b.Ubox) + 2 * c;
+            U[0] = make_double2(u[0], u[1]);
+            U[1] = make_double2(u[2], 0.0);
+        } else {
+            float *W = (float *)S;
+            const float rh = W[lin], rl = W[4 * L.np + lin], rho = rh + rl;
+            float u[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                float hi = W[(1 + d) * L.np + lin], lo = W[(5 + d) * L.np + lin];
+                if (body) {
+                    const float a = rho * (float)b.phi[c], vb = (float)b.vbar[3 * c + d];
+                    double t = 0.0;
+                    for (int s = 0; s < b.niter; ++s) {
+                        const float inc = a * (vb - (hi + lo) / rho);
+                        add_comp(hi, lo, inc);
+                        t += (double)inc;
+                    }
+                    W[(1 + d) * L.np + lin] = hi;
+                    W[(5 + d) * L.np + lin] = lo;
+                    fs[d] += t;
+                }
+                // (hi + lo) / (rh + rl) rounded once: quotient and remainder
+                const float q = hi / rh;
+                const float rem = __fmaf_rn(-q, rl, __fadd_rn(__fmaf_rn(-q, rh, hi), lo));
+                u[d] = isfinite(q) ? q + rem / rh : q;
+            }
+            reinterpret_cast<float4 *>(b.Uboxf)[c] = make_float4(u[0], u[1], u[2], 0.0f);
+        }
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        for (int o = 16; o > 0; o >>= 1) fs[d] += __shfl_xor_sync(0xffffffffu, fs[d], o);
+        if (lane == 0) sh[d][warp] = fs[d];
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        double s = 0.0;
+        for (int w = 0; w < 8; ++w) s += sh[threadIdx.x][w];
+        part[3 * blockIdx.x + threadIdx.x] = s;
+        if (blockIdx.x == 0 && threadIdx.x == 0) b.out[6] = 0.0;   // the residual maximum of the next kernel
+    }
+}
+
+// The residual of every point (as ibm_residual_kernel, the velocities by
+// 16-byte loads); the last block to finish writes the step's record: the
+// force on the body from the parts in order, the iterations, the residual.
+template <typename R>
+__global__ void __launch_bounds__(256) ibm_points_kernel(Lattice L, BodyDev b, Scalars *scal, const double *part,
+                                                         int nparts)
+{
+    __shared__ bool last;
+    __shared__ double sh[3][256];
+    const int warp = (int)((blockIdx.x * 256L + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (warp < b.n) {
+        const long o0 = b.csr_off[warp], o1 = b.csr_off[warp + 1];
+        R u[3] = {R(0), R(0), R(0)};
+        for (long o = o0 + lane; o < o1; o += 32) {
+            const long c = b.csr_cell[o];
+            if (!in_bounds(c, b.nbox)) continue;
+            if constexpr (std::is_same<R, double>::value) {
+                const double w = b.csr_w[o];
+                const double2 x = reinterpret_cast<const double2 *>(b.Ubox)[2 * c];
+                u[0] += w * x.x;
+                u[1] += w * x.y;
+                u[2] += w * b.Ubox[4 * c + 2];
+            } else {
+                const float w = b.csr_wf[o];
+                const float4 x = reinterpret_cast<const float4 *>(b.Uboxf)[c];
+                u[0] += w * x.x;
+                u[1] += w * x.y;
+                u[2] += w * x.z;
+            }
+        }
+        for (int s = 16; s > 0; s >>= 1)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) u[d] += __shfl_xor_sync(0xffffffffu, u[d], s);
+        if (lane == 0) {
+            const double e0 = b.vel[3 * warp] - (double)u[0], e1 = b.vel[3 * warp + 1] - (double)u[1],
+                         e2 = b.vel[3 * warp + 2] - (double)u[2];
+            const double e = sqrt(e0 * e0 + e1 * e1 + e2 * e2);
+            atomicMax((unsigned long long *)&b.out[6], (unsigned long long)__double_as_longlong(e));
+        }
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(b.count, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int k = threadIdx.x; k < nparts; k += 256)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) s[d] += part[3 * k + d];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) sh[d][threadIdx.x] = s[d];
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) sh[d][threadIdx.x] += sh[d][threadIdx.x + w];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        const double k = -(L.h[0] * L.h[1] * L.h[2]) / scal->dt;
+        for (int d = 0; d < 3; ++d) b.out[d] = k * sh[d][0];
+        const double res = __longlong_as_double((long long)__ldcg((const unsigned long long *)&b.out[6]));
+        b.out[3] = (double)b.niter;
+        b.out[4] = res;
+        b.out[5] = 0.0;
+        b.out[6] = 0.0;
+        b.out[7 + b.niter - 1] = res;   // the entries before it stay 0
+    }
+}
+
 }  // namespace
 
 void launch_alm_loads(const Ctx &c, const RotorDev &r)
 {
     const Lattice L = make_lattice(c);
-    alm_loads_kernel<<<1, 256, 0, c.stream>>>(L, c.state, r, c.scal);
+    const int blocks = (r.nb * r.np + kLoadPts - 1) / kLoadPts;
+    alm_loads_kernel<<<blocks, 32, 0, c.stream>>>(L, c.state, r, c.scal);
 }
 
 void launch_alm(const Ctx &c, const RotorDev &r)
 {
-    const Lattice L = make_lattice(c);
     mark(c, K_ALM, 1);
-    alm_loads_kernel<<<1, 256, 0, c.stream>>>(L, c.state, r, c.scal);
+    launch_alm_loads(c, r);
     mark(c, K_ALM, 0);
     launch_alm_spread(c, r);
 }
@@ -595,7 +766,7 @@ void launch_alm_spread(const Ctx &c, const RotorDev &r)
     const long nbox = (long)(r.box[0][1] - r.box[0][0] + 1) * (r.box[1][1] - r.box[1][0] + 1) *
                       (r.box[2][1] - r.box[2][0] + 1);
     if (nbox <= 0) return;
-    const int blocks = (int)((nbox + 255) / 256);
+    const int blocks = (int)((nbox + 31) / 32);
     mark(c, K_ALM, 1);
     if (c.prec == GKS_FP64)
         alm_spread_kernel<double><<<blocks, 256, 0, c.stream>>>(L, c.state, r, c.scal);
@@ -647,18 +818,33 @@ void launch_ibm(const Ctx &c, const BodyDev &b)
 {
     const Lattice L = make_lattice(c);
     const int cb = (int)((b.nbox + 255) / 256), pb = (int)(((long)b.n * 32 + 255) / 256);
+    if (!(b.tol > 0.0)) {
+        const int nparts = std::min(cb, kIbmParts);
+        mark(c, K_IBM, 1);
+        if (c.prec == GKS_FP64)
+            ibm_cells_kernel<double><<<nparts, 256, 0, c.stream>>>(L, c.state, b, c.scal, c.partials);
+        else
+            ibm_cells_kernel<float><<<nparts, 256, 0, c.stream>>>(L, c.state, b, c.scal, c.partials);
+        mark(c, K_IBM, 0);
+        mark(c, K_IBM, 1);
+        if (c.prec == GKS_FP64)
+            ibm_points_kernel<double><<<pb, 256, 0, c.stream>>>(L, b, c.scal, c.partials, nparts);
+        else
+            ibm_points_kernel<float><<<pb, 256, 0, c.stream>>>(L, b, c.scal, c.partials, nparts);
+        mark(c, K_IBM, 0);
+        return;
+    }
+    // residual tolerance: one iteration per round, stopped on the device
     mark(c, K_IBM, 1);
     ibm_begin_kernel<<<1, 256, 0, c.stream>>>(b);
     mark(c, K_IBM, 0);
     cudaMemsetAsync(b.fsum, 0, sizeof(double) * 3 * b.nbox, c.stream);
-    const int rounds = b.tol > 0.0 ? b.niter : 1;
-    const int per = b.tol > 0.0 ? 1 : b.niter;
-    for (int s = 0; s < rounds; ++s) {
+    for (int s = 0; s < b.niter; ++s) {
         mark(c, K_IBM, 1);
         if (c.prec == GKS_FP64)
-            ibm_iter_kernel<double><<<cb, 256, 0, c.stream>>>(L, c.state, b, c.scal, per);
+            ibm_iter_kernel<double><<<cb, 256, 0, c.stream>>>(L, c.state, b, c.scal);
         else
-            ibm_iter_kernel<float><<<cb, 256, 0, c.stream>>>(L, c.state, b, c.scal, per);
+            ibm_iter_kernel<float><<<cb, 256, 0, c.stream>>>(L, c.state, b, c.scal);
         mark(c, K_IBM, 0);
         mark(c, K_IBM, 1);
         if (c.prec == GKS_FP64) {
@@ -670,7 +856,7 @@ void launch_ibm(const Ctx &c, const BodyDev &b)
         }
         mark(c, K_IBM, 0);
         mark(c, K_IBM, 1);
-        ibm_check_kernel<<<1, 1, 0, c.stream>>>(b, b.tol > 0.0 ? s : b.niter - 1, b.tol);
+        ibm_check_kernel<<<1, 1, 0, c.stream>>>(b, s, b.tol);
         mark(c, K_IBM, 0);
     }
     // the grid's reduction scratch holds kMaxPartials x 8 doubles

@@ -108,7 +108,7 @@ int bounds_flag_adjoint();
 
 // Launchers of the stencil path (gks_stencil.cu).
 void launch_prep(const Ctx &c);                        // max |U|^2 into scal; FP32C: state -> wk0
-void launch_prep_box(const Ctx &c, const int box[3][2]);   // the same over the interior cells of a box
+void launch_prep_boxes(const Ctx &c, const int (*box)[3][2], int n);   // the same over the interior cells of n boxes
 void launch_ghost(const Ctx &c, void *w);              // 3 ghost layers of w (working type)
 void launch_stage(const Ctx &c, int stage);            // face kernels + update
 void launch_cfl(const Ctx &c);                          // dt from max |U| (after launch_prep)
@@ -142,6 +142,7 @@ struct RotorDev {
     double *F;          // 4 nb np: F_x, F_th, alpha, phi
     double *et;         // 2 nb: -sin th_b, cos th_b
     double *out;        // thrust[nb], torque[nb], power, cp, ct
+    unsigned *count;    // blocks of the loads kernel that are done (the last one sums and clears it)
     int box[3][2];      // interior cell box swept by the 3 eps supports
     int shared = 0;     // a slab's share of a neighbouring slab's rotor: its point buffers are the
                         // owner's, the owner computes the loads, this grid only spreads them
@@ -209,7 +210,7 @@ struct BodyDev {
     int box[3][2];
     long nbox;
     double *Vbar, *vbar, *phi;  // per box cell (vbar: 3 per cell)
-    double *fsum;               // 3 per box cell
+    double *fsum;               // 3 per box cell (residual-tolerance mode)
     double *out;                // force[3], iters, residual, residual history[niter]
     // back-interpolation weights W_{ijk->p} (static): CSR over points, columns
     // are box-local cell indices in (k, j, i) order
@@ -217,8 +218,9 @@ struct BodyDev {
     int *csr_cell;              // nnz
     double *csr_w;              // nnz
     long nnz;
-    double *Ubox;               // 3 per box cell: cell velocity of the residual
+    double *Ubox;               // 4 per box cell (3 used): cell velocity of the residual, 16-byte aligned
     float *csr_wf, *Uboxf;      // FP32 copies of csr_w and Ubox (FP32C grids)
+    unsigned *count;            // blocks of the residual kernel that are done (the last one finishes the step)
 };
 void launch_body_csr_count(const Ctx &c, const BodyDev &b, long *d_counts);
 void launch_body_csr_fill(const Ctx &c, const BodyDev &b);
