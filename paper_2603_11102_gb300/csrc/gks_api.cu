@@ -86,11 +86,20 @@ int cuda_check(gks_grid *g, cudaError_t e, const char *what)
 
 struct Layout {
     size_t state = 0, work = 0;
-    size_t o_wk0 = 0, o_wk1 = 0, o_p = 0, o_fq = 0, o_ff[3] = {0, 0, 0};
+    size_t o_wk0 = 0, o_wk1 = 0, o_p = 0, o_fq[3] = {0, 0, 0}, o_ff[3] = {0, 0, 0};
+    int small = 0;
     size_t o_ih[3], o_ihf[3], o_h64[3], o_part = 0, o_scal = 0, o_diag = 0;
     long np = 0, nfq = 0, nff[3] = {0, 0, 0};
     int P[3], e1p[3];
 };
+
+// Face boxes of all three directions up to this size are kept apart and the
+// directions run together: they stay in the 129 MB L2 next to the state, and a
+// grid of that size is bound by its launches and by half-filled ones (FP32C up
+// to about 75^3 cells, FP64 59^3: 32^3 steps replayed from a graph 69 -> 48 us
+// with 8 launches instead of 20, FP64 1.04 -> 0.73 ms). Beyond it the launches
+// are long enough and one box at a time stays in L2 between its two kernels.
+constexpr size_t kSmallBoxBytes = (size_t)48 << 20;
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -132,18 +141,24 @@ void plan(const gks_grid_desc *d, Layout *L)
         L->e1p[a] = (d->n[t1] + 4 + 3) / 4 * 4;
         const long nfq = (long)(d->n[a] + 1) * (d->n[t2] + 4) * L->e1p[a];
         if (nfq > L->nfq) L->nfq = nfq;
-        // face fluxes are kept for x and y only: the z-face kernel applies
-        // the stage update itself (FP64 grids keep the z faces too, for the
-        // separate update of their double-single arithmetic)
-        L->nff[a] = a == 2 && d->precision != GKS_FP64 ? 0 : (long)(d->n[a] + 1) * d->n[t1] * d->n[t2];
+        L->nff[a] = (long)(d->n[a] + 1) * d->n[t1] * d->n[t2];
     }
     L->nfq = (L->nfq + 63) / 64 * 64;
+    // a small grid keeps the three face boxes apart, so that all directions
+    // of a stage run in one launch
+    L->small = 3 * 8 * (size_t)L->nfq * R <= kSmallBoxBytes;
+    // large FP32C grids keep no z-face fluxes: the z-face kernel applies the
+    // stage update itself
+    if (d->precision == GKS_FP32C && !L->small) L->nff[2] = 0;
     size_t o = 0;
     L->o_wk0 = o;
     if (d->precision == GKS_FP32C) o = align256(o + 4 * (size_t)L->np * 4);
     L->o_wk1 = o; o = align256(o + 4 * (size_t)L->np * R);
     L->o_p = o; o = align256(o + (d->precision == GKS_FP64 ? 4 : 8) * (size_t)L->np * R);
-    L->o_fq = o; o = align256(o + 8 * (size_t)L->nfq * R);
+    for (int a = 0; a < 3; ++a) {
+        L->o_fq[a] = a > 0 && !L->small ? L->o_fq[0] : o;
+        if (a == 0 || L->small) o = align256(o + 8 * (size_t)L->nfq * R);
+    }
     for (int a = 0; a < 3; ++a) { L->o_ff[a] = o; o = align256(o + 8 * (size_t)L->nff[a] * R); }
     for (int a = 0; a < 3; ++a) { L->o_ih[a] = o; o = align256(o + (size_t)L->P[a] * R); }
     for (int a = 0; a < 3; ++a) { L->o_ihf[a] = o; o = align256(o + (size_t)(d->n[a] + 1) * R); }
@@ -379,9 +394,10 @@ int gks_create_grid(const gks_grid_desc *desc, void *d_state, void *d_work, gks_
     c.wk0 = c.prec == GKS_FP32C ? (void *)(w + L.o_wk0) : d_state;
     c.wk1 = w + L.o_wk1;
     c.pbuf = w + L.o_p;
-    c.fq = w + L.o_fq;
+    c.small = L.small;
     c.nfq = L.nfq;
     for (int a = 0; a < 3; ++a) {
+        c.fq[a] = w + L.o_fq[a];
         c.ff[a] = w + L.o_ff[a];
         c.nff[a] = L.nff[a];
         c.ih[a] = w + L.o_ih[a];
@@ -424,8 +440,8 @@ int gks_create_grid(const gks_grid_desc *desc, void *d_state, void *d_work, gks_
     for (int a = 0; a < 3; ++a) {
         c.e1p[a] = L.e1p[a];
         std::string m;
-        if (encode_face_map(c, a, c.fq, &c.tmap[a], &m) ||
-            (c.prec == GKS_FP32C && encode_face_map(c, a, c.fq, &c.tmapM[a], &m, 5))) {
+        if (encode_face_map(c, a, c.fq[a], &c.tmap[a], &m) ||
+            (c.prec == GKS_FP32C && encode_face_map(c, a, c.fq[a], &c.tmapM[a], &m, 5))) {
             delete g;
             return fail(nullptr, GKS_ERR_CUDA, m);
         }
@@ -751,8 +767,7 @@ int step_once(gks_grid *g, const AdjWork *tp)
     int rc = GKS_OK;
     g->prof.last_end = nullptr;   // launch boundaries are shared inside a step only
     if (!g->prep_valid) launch_prep(c);
-    launch_ghost(c, c.wk0);
-    launch_cfl(c);   // dt from max |U|^2, which it clears
+    launch_ghost(c, c.wk0, true);   // and dt from max |U|^2, which it clears
     if (tp) {
         rc = cuda_check(g, cudaMemcpyAsync(tp->hdr + 1, &c.scal->t, 2 * sizeof(double), cudaMemcpyDeviceToDevice,
                                            c.stream), "record time");
@@ -776,7 +791,7 @@ int step_once(gks_grid *g, const AdjWork *tp)
         if (c.prec == GKS_FP64) use_tape_gauss(cc, *tp, 0);
     }
     launch_stage(cc, 1);
-    launch_ghost(cc, cc.wk1);
+    launch_ghost(cc, cc.wk1, false);
     if (tp) {
         if (c.prec == GKS_FP32C) {
             rc = cuda_check(g, cudaMemcpyAsync(tp->Wsf, c.wk1, sizeof(float) * 4 * c.np, cudaMemcpyDeviceToDevice,
@@ -797,6 +812,7 @@ int step_once(gks_grid *g, const AdjWork *tp)
             memcpy(cc.prep_box[k], box, sizeof(int) * 6);
         }
     }
+    cc.advance = nobj == 0;
     launch_stage(cc, 2);
     if (tp && c.prec == GKS_FP64 &&
         (rc = cuda_check(g, cudaMemcpyAsync(tp->Wp, c.state, bytes4, cudaMemcpyDeviceToDevice, c.stream),
@@ -815,9 +831,9 @@ int step_once(gks_grid *g, const AdjWork *tp)
                                        "record the IBM iterations")))
                 return rc;
         }
-    if (fused_prep) launch_prep_boxes(c, cc.prep_box, nobj);
+    const bool advanced = fused_prep && launch_prep_boxes(c, cc.prep_box, nobj, true);
     g->prep_valid = fused_prep;
-    launch_advance(c);
+    if (!advanced && nobj) launch_advance(c);
     g->prof.last_end = nullptr;
     rc = check_launch(g, "step");
     if (rc) return rc;
@@ -988,7 +1004,7 @@ int slab_step_once(gks_grid *const *sl, int n)
         g->prof.last_end = nullptr;
         g->stepped = true;
         if (!g->prep_valid) launch_prep(g->c);
-        launch_ghost(g->c, g->c.wk0);
+        launch_ghost(g->c, g->c.wk0, false);
     }
     slab_exchange(sl, n, 0);
     Scalars *scal[64];
@@ -999,7 +1015,7 @@ int slab_step_once(gks_grid *const *sl, int n)
     for (int s = 0; s < n; ++s) {
         cc[s] = sl[s]->c;
         launch_stage(cc[s], 1);
-        launch_ghost(cc[s], cc[s].wk1);
+        launch_ghost(cc[s], cc[s].wk1, false);
     }
     slab_exchange(sl, n, 1);
     std::vector<int> fused(n);
@@ -1033,7 +1049,7 @@ int slab_step_once(gks_grid *const *sl, int n)
         const Ctx &c = g->c;
         for (size_t k = 0; k < g->obj_kind.size(); ++k)
             if (g->obj_kind[k] == 1) launch_ibm(c, g->bodies[g->obj_index[k]]);
-        if (fused[s]) launch_prep_boxes(c, cc[s].prep_box, cc[s].nprep_box);
+        if (fused[s]) launch_prep_boxes(c, cc[s].prep_box, cc[s].nprep_box, false);
         g->prep_valid = fused[s];
         launch_advance(c);
         g->prof.last_end = nullptr;
@@ -1574,10 +1590,10 @@ int gks_step_adjoint(gks_grid *g, void *d_adj_work, double t_n, const double *d_
         cc.pbuf = w.Ws;
         cc.prep_next = 0;
         launch_scatter_state_prep(cc, d_state_n);
-        launch_ghost(cc, cc.wk0);
+        launch_ghost(cc, cc.wk0, false);
         launch_widen(cc, w.A0f, nullptr, w.A0, 4 * c.np, c.np, c.off);
         launch_stage(cc, 1);
-        launch_ghost(cc, cc.wk1);
+        launch_ghost(cc, cc.wk1, false);
         launch_stage(cc, 2);
         launch_widen(cc, w.Wsf, nullptr, w.Ws, 4 * c.np, c.np, c.off);
         launch_widen(cc, (const float *)w.lamA, (const float *)w.lamA + 4 * c.np, w.Wp, 4 * c.np, 0, 0.0);
@@ -1586,10 +1602,10 @@ int gks_step_adjoint(gks_grid *g, void *d_adj_work, double t_n, const double *d_
         cc.wk0 = w.A0;
         cc.wk1 = w.Ws;
         launch_scatter_state(cc, d_state_n);
-        launch_ghost(cc, w.A0);
+        launch_ghost(cc, w.A0, false);
         use_tape_gauss(cc, w, 0);
         launch_stage(cc, 1);
-        launch_ghost(cc, cc.wk1);
+        launch_ghost(cc, cc.wk1, false);
         cc.state = w.Wp;
         use_tape_gauss(cc, w, 1);
         launch_stage(cc, 2);

@@ -59,7 +59,8 @@ __device__ __forceinline__ double max_u2(double a, double b) { return (b > a || 
 __device__ __forceinline__ float max_u2f(float a, float b) { return (b > a || b != b) ? b : a; }
 
 // Block-wide max of v (blockDim.x * blockDim.y threads, a multiple of 32,
-// at most 1024) folded into *bits (a non-negative double) by one atomicMax.
+// at most 1024) folded into *bits (a non-negative double) by one atomicMax,
+// left out when *bits is already no smaller (it only grows during the launch).
 __device__ __forceinline__ void block_max_to(double v, unsigned long long *bits)
 {
     __shared__ double red[32];
@@ -69,7 +70,8 @@ __device__ __forceinline__ void block_max_to(double v, unsigned long long *bits)
     __syncthreads();
     if (tid == 0) {
         for (int w = 1; w < nw; ++w) v = max_u2(v, red[w]);
-        atomicMax(bits, (unsigned long long)__double_as_longlong(v));
+        const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+        if (b > *(volatile unsigned long long *)bits) atomicMax(bits, b);
     }
 }
 
@@ -776,6 +778,22 @@ __device__ __forceinline__ void tile_t1_pass(const R *sq, C *st, int tid)
 // The face state of a 384x256x256 step took 2.15 ms with 8 separate stores
 // and takes 1.90 ms with 4 paired ones.
 
+// tan_val_der of a component pair, with the operations of the marching flux
+// kernel (the same bits): E -+ O and Do -+ De with the last terms fused.
+__device__ __forceinline__ void pair_t1(const f2 q[5], f2 &vm, f2 &vp, f2 &dm, f2 &dp)
+{
+    constexpr float o1 = float(0.20046884346862007), o2 = float(0.028065638085606807);
+    constexpr float e1 = float(0.41697519441472974), e2 = float(0.032075014954979206);
+    const f2 d1 = fma(q[2], f2(-2.0f), q[3] + q[1]), d2 = fma(q[2], f2(-2.0f), q[4] + q[0]);
+    const f2 a1 = q[3] - q[1], a2 = q[4] - q[0];
+    const f2 E = fma(d1, f2(float(1.0 / 1080.0)), fma(d2, f2(float(-1.0 / 4320.0)), q[2]));
+    const f2 D = fma(a1, f2(float(2.0 / 3.0)), a2 * f2(float(-1.0 / 12.0)));
+    vm = fma(a1, f2(-o1), fma(a2, f2(o2), E));
+    vp = fma(a1, f2(o1), fma(a2, f2(-o2), E));
+    dm = fma(d1, f2(-e1), fma(d2, f2(e2), D));
+    dp = fma(d1, f2(e1), fma(d2, f2(-e2), D));
+}
+
 // t1 pass of a face-box tile of H rows: 64 H equal tasks (pair, row, group of
 // 2 columns), H / 4 per thread: 6 pairs in by 128-bit loads, 2 columns out by
 // one 128-bit store per array (consecutive lanes, consecutive 16 bytes: no
@@ -800,8 +818,7 @@ __device__ __forceinline__ void tile_t1_pass_f2(const float2 *sq, float2 *st, in
         f2 v[4][2];
         if (p < 2) {
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
-                tan_val_der(q[i], q[i + 1], q[i + 2], q[i + 3], q[i + 4], v[0][i], v[1][i], v[2][i], v[3][i]);
+            for (int i = 0; i < 2; ++i) pair_t1(q + i, v[0][i], v[1][i], v[2][i], v[3][i]);
             o += 4 * p * ROWS;
         } else {
 #pragma unroll

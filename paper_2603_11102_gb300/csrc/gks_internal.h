@@ -57,8 +57,10 @@ struct Ctx {
     void *wk0;                // reconstruction input of stage 1 (FP64: == state)
     void *wk1;                // W* (reconstruction input of stage 2), R[4][np]
     void *pbuf;               // P = W + dt L + dt^2/6 Lt (FP64 double[4][np]; FP32C hi/lo)
-    void *fq;                 // face equilibrium state + normal slope, R[8][nfq] (FP32C: float2[4][nfq],
-                              // component pairs)
+    void *fq[3];              // face equilibrium state + normal slope, R[8][nfq] (FP32C: float2[4][nfq],
+                              // component pairs); one buffer for all directions unless the grid is small
+    int small = 0;            // the directions of a stage run in one launch each (small_grid)
+    int advance = 0;          // stage 2 also moves the time on (a step without forcing)
     long nfq;
     int e1p[3];               // padded t1 extent of the face box per direction (multiple of 4)
     CUtensorMap tmap[3];      // TMA descriptors of the face box per direction
@@ -75,7 +77,7 @@ struct Ctx {
     int prep_next = 0;
     int nprep_box = 0;
     int prep_box[8][3][2];
-    void *ff[3];              // face-averaged F0 and F1 of x and y faces, R[8][nff] (none for z)
+    void *ff[3];              // face-averaged F0 and F1, R[8][nff] (no z faces on large FP32C grids)
     long nff[3];
     void *ih[3];              // R: inverse cell widths, padded index i + 3
     void *ihf[3];             // R: inverse centre distance at faces, f = 0..n
@@ -108,8 +110,9 @@ int bounds_flag_adjoint();
 
 // Launchers of the stencil path (gks_stencil.cu).
 void launch_prep(const Ctx &c);                        // max |U|^2 into scal; FP32C: state -> wk0
-void launch_prep_boxes(const Ctx &c, const int (*box)[3][2], int n);   // the same over the interior cells of n boxes
-void launch_ghost(const Ctx &c, void *w);              // 3 ghost layers of w (working type)
+// the same over the interior cells of n boxes, and with `advance` t += dt; false when nothing was launched
+bool launch_prep_boxes(const Ctx &c, const int (*box)[3][2], int n, bool advance);
+void launch_ghost(const Ctx &c, void *w, bool with_dt);   // 3 ghost layers of w (working type); dt of the step
 void launch_stage(const Ctx &c, int stage);            // face kernels + update
 void launch_cfl(const Ctx &c);                          // dt from max |U| (after launch_prep)
 void launch_advance(const Ctx &c);                      // t += dt

@@ -16,11 +16,14 @@
 //                persistent blocks on 32x8 face tiles loaded by TMA, the t1
 //                pass in shared memory. The flux of FP32 and double-single
 //                arithmetic runs at two Gauss points at once on packed pairs.
-//   flux_update  (z) the same flux, walking z per tile column, fused with the
-//                divergence (Eq. (finite)) and the two-stage fourth-order
-//                combination of every cell; stage 2 also prepares the next
-//                step (FP32 input, max |U|^2 for the CFL step). Double-single
-//                grids store the z-face fluxes and update in update_ds_kernel.
+//   flux_update  FP32C: the z-face flux, walking z per tile column, fused with
+//                the divergence (Eq. (finite)) and the two-stage fourth-order
+//                combination of every cell; FP64: the z-face flux like the
+//                others, then the update over the stored fluxes. Stage 2 also
+//                prepares the next step (FP32 input, max |U|^2 for the CFL
+//                step).
+// Small grids run the three directions of face_eq and of face_flux as one
+// launch each and the update over stored fluxes.
 //
 // All arithmetic runs in the working type R: double for GKS_FP64, float for
 // GKS_FP32C. The reconstruction works on rho - off (off = rho_ref in FP32C,
@@ -47,65 +50,64 @@ struct GhostArgs {
     R *w;
     long np;
     int n[3], P[3];
-    int d, e1, e2, lo1, lo2, len1, len2;
-    int bc0, bc1;
+    int bc[3][2];
     R off, csound;
     R uin[3];
-    int rows;   // x ghosts (d = 0): one thread per ghost of a (y, z) row, rows x 2G threads
+    long nz, ny, nx;   // ghosts of the z, y and x layers (in that order of thread ranges)
+    // dt of the step (first launch of a step), by the first thread
+    Scalars *scal;
+    double cfl, dt_fixed, hmin, cs64;
 };
 
-template <typename R>
-__global__ void __launch_bounds__(256) ghost_kernel(GhostArgs<R> A)
+// dt from the largest |U|^2, which it clears.
+__device__ __forceinline__ void set_dt(Scalars *scal, double cfl, double dt_fixed, double hmin, double csound)
 {
-    int a, b, s, l;
-    if (A.rows) {
-        // x ghosts: consecutive threads take the 2G ghosts of one row, whose
-        // cells are contiguous in memory (the lanes of a warp cover ~5 rows)
-        const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
-        const long r = t / (2 * G);
-        if (r >= A.rows) return;
-        const int k = (int)(t - r * 2 * G);
-        s = k / G;
-        l = k % G + 1;
-        a = A.lo1 + (int)(r % A.len1);
-        b = A.lo2 + (int)(r / A.len1);
+    const double umax = sqrt(__longlong_as_double((long long)scal->maxu2_bits));
+    double dt;
+    if (dt_fixed > 0.0) {
+        dt = dt_fixed;
+        const double num = dt * (umax + csound) / hmin;
+        scal->cfl_number = num;
+        if (cfl > 0.0 && !(num <= cfl)) atomicOr(&scal->flags, FLAG_CFL);
     } else {
-        a = A.lo1 + (int)(blockIdx.x * blockDim.x + threadIdx.x);
-        b = A.lo2 + (int)(blockIdx.y * blockDim.y + threadIdx.y);
-        if (a >= A.lo1 + A.len1 || b >= A.lo2 + A.len2) return;
-        s = blockIdx.z / G;
-        l = blockIdx.z % G + 1;
+        dt = cfl * hmin / (umax + csound);
+        scal->cfl_number = cfl;
+        if (!isfinite(dt)) atomicOr(&scal->flags, FLAG_NONFINITE);
     }
-    const int d = A.d, nd = A.n[d];
-    const int bc = s == 0 ? A.bc0 : A.bc1;
-    if (bc == GKS_BC_EXCHANGE) return;   // filled from the neighbouring slab
-    const int gi = s == 0 ? -l : nd - 1 + l;
-    int src;
+    scal->dt = dt;
+    scal->maxu2_bits = 0ull;
+}
+
+// The ghosts of axis d at index g (inside [0, n) for an interior index): the
+// source index and the change of the source's value that the boundary makes.
+template <typename R>
+__device__ __forceinline__ int ghost_source(const GhostArgs<R> &A, int d, int g)
+{
+    const int n = A.n[d];
+    if (g >= 0 && g < n) return g;
+    const int bc = A.bc[d][g < 0 ? 0 : 1];
     if (bc == GKS_BC_PERIODIC) {
-        src = gi % nd;
-        if (src < 0) src += nd;
-    } else if (bc == GKS_BC_NOSLIP || bc == GKS_BC_SLIP) {
-        src = s == 0 ? l - 1 : nd - l;
-    } else {
-        src = s == 0 ? 0 : nd - 1;
+        const int r = g % n;
+        return r < 0 ? r + n : r;
     }
-    int cg[3], cs[3];
-    cg[d] = gi; cg[A.e1] = a; cg[A.e2] = b;
-    cs[d] = src; cs[A.e1] = a; cs[A.e2] = b;
-    const long ig = (long)(cg[0] + G) + (long)A.P[0] * ((long)(cg[1] + G) + (long)A.P[1] * (cg[2] + G));
-    const long is = (long)(cs[0] + G) + (long)A.P[0] * ((long)(cs[1] + G) + (long)A.P[1] * (cs[2] + G));
-    if (!in_bounds(ig, A.np) || !in_bounds(is, A.np)) return;
-    R q[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) q[v] = A.w[v * A.np + is];
+    if (bc == GKS_BC_NOSLIP || bc == GKS_BC_SLIP) return g < 0 ? -1 - g : 2 * n - 1 - g;
+    return g < 0 ? 0 : n - 1;
+}
+template <typename R>
+__device__ __forceinline__ void ghost_value(const GhostArgs<R> &A, int d, int g, R q[4])
+{
+    if (g >= 0 && g < A.n[d]) return;
+    const int s = g < 0 ? 0 : 1, bc = A.bc[d][s];
     if (bc == GKS_BC_NOSLIP) {
         q[1] = -q[1]; q[2] = -q[2]; q[3] = -q[3];
     } else if (bc == GKS_BC_SLIP) {
-        q[1 + d] = -q[1 + d];
+        if (d == 0) q[1] = -q[1];
+        else if (d == 1) q[2] = -q[2];
+        else q[3] = -q[3];
     } else if (bc == GKS_BC_INFLOW) {
         // density from the outgoing isothermal Riemann invariant of cell 1
         const R r1 = A.off + q[0];
-        const R un1 = q[1 + d] / r1;
+        const R un1 = (d == 0 ? q[1] : (d == 1 ? q[2] : q[3])) / r1;
         const R x = (s == 0 ? R(1) : R(-1)) * (A.uin[d] - un1) / A.csound;
         const R ex = exp(x);
         const R rg = r1 * ex;
@@ -114,43 +116,85 @@ __global__ void __launch_bounds__(256) ghost_kernel(GhostArgs<R> A)
         q[2] = rg * A.uin[1];
         q[3] = rg * A.uin[2];
     }
+}
+
+// All ghost cells in one launch. The fill is defined axis by axis (x, then y
+// and z over the ghosts of the axes before, which gives the edges and
+// corners); a ghost of several axes is the interior source cell of all of them
+// with each axis's change applied in that order, so no ghost waits for
+// another one. Consecutive threads take cells that are contiguous in memory (a
+// row of the z or y layers, the 2G x ghosts of a row). One launch in place of
+// three, and the step's dt with the first: 384x256x256 121 -> 48 us a step,
+// 128^3 54 -> 21, 32^3 37 -> 14. An exchange side's ghosts are left to the
+// copy from the neighbouring slab.
+template <typename R>
+__global__ void __launch_bounds__(256) ghost_kernel(const __grid_constant__ GhostArgs<R> A)
+{
+    long t = blockIdx.x * 256L + threadIdx.x;
+    if (t == 0 && A.scal) set_dt(A.scal, A.cfl, A.dt_fixed, A.hmin, A.cs64);
+    int i, j, k;
+    if (t < A.nz) {
+        const long r = t / A.P[0];
+        i = (int)(t - r * A.P[0]) - G;
+        const long l = r / A.P[1];
+        j = (int)(r - l * A.P[1]) - G;
+        k = l < G ? (int)l - G : A.n[2] + (int)l - G;
+    } else if ((t -= A.nz) < A.ny) {
+        const long r = t / A.P[0];
+        i = (int)(t - r * A.P[0]) - G;
+        const int l = (int)(r % (2 * G));
+        k = (int)(r / (2 * G));
+        j = l < G ? l - G : A.n[1] + l - G;
+    } else if ((t -= A.ny) < A.nx) {
+        const long r = t / (2 * G);
+        const int l = (int)(t - r * 2 * G);
+        i = l < G ? l - G : A.n[0] + l - G;
+        j = (int)(r % A.n[1]);
+        k = (int)(r / A.n[1]);
+    } else {
+        return;
+    }
+    if ((i < 0 && A.bc[0][0] == GKS_BC_EXCHANGE) || (i >= A.n[0] && A.bc[0][1] == GKS_BC_EXCHANGE)) return;
+    const int is = ghost_source(A, 0, i), js = ghost_source(A, 1, j), ks = ghost_source(A, 2, k);
+    const long lg = (long)(i + G) + (long)A.P[0] * ((long)(j + G) + (long)A.P[1] * (k + G));
+    const long ls = (long)(is + G) + (long)A.P[0] * ((long)(js + G) + (long)A.P[1] * (ks + G));
+    if (!in_bounds(lg, A.np) || !in_bounds(ls, A.np)) return;
+    R q[4];
 #pragma unroll
-    for (int v = 0; v < 4; ++v) A.w[v * A.np + ig] = q[v];
+    for (int v = 0; v < 4; ++v) q[v] = A.w[v * A.np + ls];
+    ghost_value(A, 0, i, q);
+    ghost_value(A, 1, j, q);
+    ghost_value(A, 2, k, q);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) A.w[v * A.np + lg] = q[v];
 }
 
 template <typename R>
-void ghost_impl(const Ctx &c, R *w)
+void ghost_impl(const Ctx &c, R *w, bool with_dt)
 {
-    for (int d = 0; d < 3; ++d) {
-        GhostArgs<R> A;
-        A.w = w;
-        A.np = c.np;
-        for (int e = 0; e < 3; ++e) { A.n[e] = c.n[e]; A.P[e] = c.P[e]; }
-        A.d = d;
-        A.e1 = tan1(d);
-        A.e2 = tan2(d);
-        // axes swept before d include their ghosts (edges and corners)
-        A.lo1 = A.e1 < d ? -G : 0;
-        A.len1 = A.e1 < d ? c.n[A.e1] + 2 * G : c.n[A.e1];
-        A.lo2 = A.e2 < d ? -G : 0;
-        A.len2 = A.e2 < d ? c.n[A.e2] + 2 * G : c.n[A.e2];
-        A.bc0 = c.bc[d][0];
-        A.bc1 = c.bc[d][1];
-        A.off = (R)c.off;
-        A.csound = (R)c.csound;
-        for (int e = 0; e < 3; ++e) A.uin[e] = (R)c.inflow[1 + e];
-        mark(c, K_GHOST, 1);
-        if (d == 0) {
-            A.rows = A.len1 * A.len2;
-            const long nt = (long)A.rows * 2 * G;
-            ghost_kernel<R><<<(int)((nt + 255) / 256), 256, 0, c.stream>>>(A);
-        } else {
-            A.rows = 0;
-            dim3 blk(32, 8), grd((A.len1 + 31) / 32, (A.len2 + 7) / 8, 2 * G);
-            ghost_kernel<R><<<grd, blk, 0, c.stream>>>(A);
-        }
-        mark(c, K_GHOST, 0);
+    GhostArgs<R> A;
+    A.w = w;
+    A.np = c.np;
+    for (int e = 0; e < 3; ++e) {
+        A.n[e] = c.n[e];
+        A.P[e] = c.P[e];
+        A.bc[e][0] = c.bc[e][0];
+        A.bc[e][1] = c.bc[e][1];
+        A.uin[e] = (R)c.inflow[1 + e];
     }
+    A.off = (R)c.off;
+    A.csound = (R)c.csound;
+    A.nz = 2L * G * c.P[0] * c.P[1];
+    A.ny = 2L * G * c.P[0] * c.n[2];
+    A.nx = 2L * G * c.n[1] * c.n[2];
+    A.scal = with_dt ? c.scal : nullptr;
+    A.cfl = c.cfl;
+    A.dt_fixed = c.dt_fixed;
+    A.hmin = c.hmin;
+    A.cs64 = c.csound;
+    mark(c, K_GHOST, 1);
+    ghost_kernel<R><<<(unsigned)((A.nz + A.ny + A.nx + 255) / 256), 256, 0, c.stream>>>(A);
+    mark(c, K_GHOST, 0);
 }
 
 // ------------------------------------------------------------ face state --
@@ -188,11 +232,11 @@ constexpr int kMarch32 = 32, kMarch = 16;
 // right-face value of cell f-1 and the left-face value of cell f. Launched
 // for FP64 grids in FP64 arithmetic; FP32 grids and double-single arithmetic
 // take the packed variants below, which march the same way.
-__global__ void __launch_bounds__(256) face_eq_march_kernel(FaceEqArgs<double, double> A)
+__device__ __forceinline__ void face_eq_march(const FaceEqArgs<double, double> &A, int3 blk)
 {
-    const int a = (int)(blockIdx.x * 32 + threadIdx.x) - 2;
-    const int b = (int)(blockIdx.y * 8 + threadIdx.y) - 2;
-    const int f0 = blockIdx.z * A.K;
+    const int a = (int)(blk.x * 32 + threadIdx.x) - 2;
+    const int b = (int)(blk.y * 8 + threadIdx.y) - 2;
+    const int f0 = blk.z * A.K;
     if (a >= A.n1 + 2 || b >= A.n2 + 2 || f0 >= A.nf) return;
     const int f1 = min(f0 + A.K, A.nf);
     const long base = (long)(a + G) * A.s1 + (long)(b + G) * A.s2;   // cell index along d = -G
@@ -241,7 +285,7 @@ __global__ void __launch_bounds__(256) face_eq_march_kernel(FaceEqArgs<double, d
     }
 }
 
-// face_eq_march_kernel for FP32 grids on packed pairs: WENO5 of the
+// face_eq_march for FP32 grids on packed pairs: WENO5 of the
 // components paired as (rho, m_n) and (m_t1, m_t2), the half-space terms of
 // the left and right states as one pair, the normal slopes paired like the
 // components. Unrolled by two so that the window shifts cost no moves.
@@ -253,11 +297,11 @@ __global__ void __launch_bounds__(256) face_eq_march_kernel(FaceEqArgs<double, d
 // a store of the face box still writes 4 whole sectors (8 rows of 4
 // segments).
 template <bool SEG>
-__global__ void __launch_bounds__(256, 3) face_eq_f2_kernel(FaceEqArgs<float, float> A)
+__device__ __forceinline__ void face_eq_f2(const FaceEqArgs<float, float> &A, int3 blk)
 {
-    const int a = SEG ? (int)(blockIdx.x * 8 + (threadIdx.x & 7)) - 2 : (int)(blockIdx.x * 32 + threadIdx.x) - 2;
-    const int b = (int)(blockIdx.y * 8 + threadIdx.y) - 2;
-    const int f0 = SEG ? (int)(blockIdx.z * 4 + (threadIdx.x >> 3)) * A.K : (int)blockIdx.z * A.K;
+    const int a = SEG ? (int)(blk.x * 8 + (threadIdx.x & 7)) - 2 : (int)(blk.x * 32 + threadIdx.x) - 2;
+    const int b = (int)(blk.y * 8 + threadIdx.y) - 2;
+    const int f0 = SEG ? (int)(blk.z * 4 + (threadIdx.x >> 3)) * A.K : blk.z * A.K;
     if (a >= A.n1 + 2 || b >= A.n2 + 2 || f0 >= A.nf) return;
     const int f1 = min(f0 + A.K, A.nf);
     const long base = (long)(a + G) * A.s1 + (long)(b + G) * A.s2;   // cell index along d = -G
@@ -310,31 +354,16 @@ __global__ void __launch_bounds__(256, 3) face_eq_f2_kernel(FaceEqArgs<float, fl
     }
 }
 
-// FP32 face state of direction d: the x faces (unit stride along the
-// normal) by march segments of at most 8 faces, 4 per warp.
-void launch_face_eq_f2(FaceEqArgs<float, float> E, int d, cudaStream_t stream)
-{
-    const dim3 blk(TX, TY);
-    if (d == 0 && E.sd == 1) {
-        E.K = std::min(E.K, 8);
-        const dim3 g((E.n1 + 4 + 7) / 8, (E.n2 + 4 + 7) / 8, (E.nf + 4 * E.K - 1) / (4 * E.K));
-        face_eq_f2_kernel<true><<<g, blk, 0, stream>>>(E);
-    } else {
-        const dim3 g((E.n1 + 4 + 31) / 32, (E.n2 + 4 + 7) / 8, (E.nf + E.K - 1) / E.K);
-        face_eq_f2_kernel<false><<<g, blk, 0, stream>>>(E);
-    }
-}
-
-// face_eq_march_kernel for FP64 grids in double-single arithmetic on packed
+// face_eq_march for FP64 grids in double-single arithmetic on packed
 // pairs: WENO5 of the components paired as (rho, m_n) and (m_t1, m_t2), the
 // half-space terms of the left and right states as one pair, the normal
 // slopes paired like the components. Every lane takes the operations of the
 // scalar double-single kernel, so the face boxes have the same bits.
-__global__ void __launch_bounds__(256, 2) face_eq_ds2_kernel(FaceEqArgs<double, dsf> A)
+__device__ __forceinline__ void face_eq_ds2(const FaceEqArgs<double, dsf> &A, int3 blk)
 {
-    const int a = (int)(blockIdx.x * 32 + threadIdx.x) - 2;
-    const int b = (int)(blockIdx.y * 8 + threadIdx.y) - 2;
-    const int f0 = blockIdx.z * A.K;
+    const int a = (int)(blk.x * 32 + threadIdx.x) - 2;
+    const int b = (int)(blk.y * 8 + threadIdx.y) - 2;
+    const int f0 = blk.z * A.K;
     if (a >= A.n1 + 2 || b >= A.n2 + 2 || f0 >= A.nf) return;
     const int f1 = min(f0 + A.K, A.nf);
     const long base = (long)(a + G) * A.s1 + (long)(b + G) * A.s2;   // cell index along d = -G
@@ -392,6 +421,76 @@ __global__ void __launch_bounds__(256, 2) face_eq_ds2_kernel(FaceEqArgs<double, 
     }
 }
 
+// Blocks of the face-state launch of one direction: FP32 x faces (unit stride
+// along the normal) by march segments of at most 8 faces, 4 per warp.
+template <typename R, typename C>
+dim3 face_eq_blocks(FaceEqArgs<R, C> &E, int d)
+{
+    if (std::is_same<C, float>::value && d == 0) {
+        E.K = std::min(E.K, 8);
+        return dim3((E.n1 + 4 + 7) / 8, (E.n2 + 4 + 7) / 8, (E.nf + 4 * E.K - 1) / (4 * E.K));
+    }
+    return dim3((E.n1 + 4 + 31) / 32, (E.n2 + 4 + 7) / 8, (E.nf + E.K - 1) / E.K);
+}
+
+template <bool SEG>
+__global__ void __launch_bounds__(256, 3) face_eq_f2_kernel(FaceEqArgs<float, float> A)
+{
+    face_eq_f2<SEG>(A, make_int3(blockIdx.x, blockIdx.y, blockIdx.z));
+}
+template <typename C>
+__global__ void __launch_bounds__(256, std::is_same<C, dsf>::value ? 2 : 1)
+    face_eq_kernel(const __grid_constant__ FaceEqArgs<double, C> A)
+{
+    const int3 blk = make_int3(blockIdx.x, blockIdx.y, blockIdx.z);
+    if constexpr (std::is_same<C, dsf>::value)
+        face_eq_ds2(A, blk);
+    else
+        face_eq_march(A, blk);
+}
+
+template <typename R, typename C>
+void launch_face_eq(FaceEqArgs<R, C> E, int d, cudaStream_t stream)
+{
+    const dim3 g = face_eq_blocks(E, d), blk(TX, TY);
+    if constexpr (std::is_same<C, float>::value) {
+        if (d == 0)
+            face_eq_f2_kernel<true><<<g, blk, 0, stream>>>(E);
+        else
+            face_eq_f2_kernel<false><<<g, blk, 0, stream>>>(E);
+    } else {
+        face_eq_kernel<C><<<g, blk, 0, stream>>>(E);
+    }
+}
+
+// The face states of all three directions in one launch (small grids, whose
+// three face boxes are kept apart): blocks of x, then y, then z.
+template <typename R, typename C>
+struct FaceEq3 {
+    FaceEqArgs<R, C> d[3];
+    int gx[3], gy[3], first[4];   // blocks along t1 and t2 of each direction, its first block
+};
+template <typename R, typename C>
+__global__ void __launch_bounds__(256, std::is_same<C, double>::value ? 1 : 2)
+    face_eq_all_kernel(const __grid_constant__ FaceEq3<R, C> E)
+{
+    int b = blockIdx.x;
+    const int d = b < E.first[1] ? 0 : (b < E.first[2] ? 1 : 2);
+    b -= E.first[d];
+    const int r = b / E.gx[d];
+    const int3 blk = make_int3(b - r * E.gx[d], r % E.gy[d], r / E.gy[d]);
+    if constexpr (std::is_same<C, float>::value) {
+        if (d == 0)
+            face_eq_f2<true>(E.d[0], blk);
+        else
+            face_eq_f2<false>(E.d[d], blk);
+    } else if constexpr (std::is_same<C, dsf>::value) {
+        face_eq_ds2(E.d[d], blk);
+    } else {
+        face_eq_march(E.d[d], blk);
+    }
+}
+
 // ------------------------------------------------------------- face flux --
 
 template <typename R, typename C = R>
@@ -408,6 +507,18 @@ struct FluxArgs {
     Scalars *scal;
 };
 
+// The launch of ND directions: one (index 0), or all three of a small grid.
+template <int ND>
+struct FluxMaps {
+    CUtensorMap d[ND];
+};
+template <typename R, typename C, int ND>
+struct FluxLaunch {
+    FluxArgs<R, C> A[ND];
+    int L[ND];          // t2 rows per segment (march), unused by the tile kernel
+    int first[ND + 1];  // first work item of each direction
+};
+
 // The face averages 1/4 sum of the Gauss-point fluxes: of F0, and of F1 from
 // the sum of -F1 (gk_flux).
 __device__ __forceinline__ double face_avg(double s) { return s * 0.25; }
@@ -416,22 +527,6 @@ __device__ __forceinline__ dsf face_avg(dsf s) { return scale_pow2(s, 0.25f); }
 __device__ __forceinline__ double face_avg_neg(double s) { return s * -0.25; }
 __device__ __forceinline__ float face_avg_neg(float s) { return s * -0.25f; }
 __device__ __forceinline__ dsf face_avg_neg(dsf s) { return scale_pow2(s, -0.25f); }
-
-// Tile t of the face box as (t1 tile, t2 tile, face): t = ta + NA (tb + NB f).
-struct TileIdx {
-    int ta, tb, f;
-};
-
-// t + g for a step g given in the same mixed radix (ga < NA, gb < NB).
-__device__ __forceinline__ TileIdx tile_add(TileIdx t, const TileIdx &g, int NA, int NB)
-{
-    t.ta += g.ta;
-    t.tb += g.tb;
-    t.f += g.f;
-    if (t.ta >= NA) { t.ta -= NA; t.tb += 1; }
-    if (t.tb >= NB) { t.tb -= NB; t.f += 1; }
-    return t;
-}
 
 // The t2 pass of component v at column (tx, ty) of the tile, t1 Gauss point
 // m: values and t2 slopes of Q0, values of the t1 slopes and of the normal
@@ -503,36 +598,30 @@ __device__ __forceinline__ void tile_gauss_flux(const FluxPhys<double> &ph, cons
     }
 }
 
-// The flux of the NE faces (tx, r0 + e) of a tile of H rows in FP32: the t2
-// pass, then the two t2 Gauss points of each t1 Gauss point as one packed
-// evaluation; the sums of F0 and -F1 over the 4 Gauss points of each face.
-template <int H, int NE, bool NEED_F0>
-__device__ __forceinline__ void tile_gauss_flux_f2(const FluxPhys<f2> &ph, const float2 *st, int tx, int r0, float ih1,
-                                                   const float ih2[NE], float acc0[NE][4], float acc1[NE][4])
+// The flux of face (tx, ty) of a 32 x 8 tile in FP32 (the fused z kernel): the
+// t2 pass, then the two t2 Gauss points of each t1 Gauss point as one packed
+// evaluation; the sums of F0 and -F1 over the 4 Gauss points, in the order of
+// march_face (the same bits).
+template <bool NEED_F0>
+__device__ __forceinline__ void tile_gauss_flux_f2(const FluxPhys<f2> &ph, const float2 *st, int tx, int ty, float ih1,
+                                                   float ih2, float acc0[4], float acc1[4])
 {
-    f2 s0[NE][4], s1[NE][4];   // the two t2 Gauss points -g, +g in the lanes
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
-        f2 Qv[NE][4], Dn[NE][4], D1[NE][4], D2[NE][4];   // [face][component]
-        t2_pass_f2<H, NE, true>(st, m, tx, r0, Qv, Dn, D1, D2);
-#pragma unroll
-        for (int e = 0; e < NE; ++e) {
-            f2 F0[4], F1[4];
-            gk_flux<f2, NEED_F0>(ph, Qv[e], Dn[e], D1[e], D2[e], f2(ih1), f2(ih2[e]), F0, F1);
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                if (NEED_F0) s0[e][v] = m == 0 ? F0[v] : s0[e][v] + F0[v];
-                s1[e][v] = m == 0 ? F1[v] : s1[e][v] + F1[v];
-            }
-        }
-    }
-#pragma unroll
-    for (int e = 0; e < NE; ++e)
+        f2 Qv[1][4], Dn[1][4], D1[1][4], D2[1][4];   // the two t2 Gauss points -g, +g in the lanes
+        t2_pass_f2<SQ_H, 1, true>(st, m, tx, ty, Qv, Dn, D1, D2);
+        f2 F0[4], F1[4];
+        gk_flux<f2, NEED_F0>(ph, Qv[0], Dn[0], D1[0], D2[0], f2(ih1), f2(ih2), F0, F1);
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            if (NEED_F0) acc0[e][v] = s0[e][v].v.x + s0[e][v].v.y;
-            acc1[e][v] = s1[e][v].v.x + s1[e][v].v.y;
+            if (NEED_F0) {
+                const float s = F0[v].v.x + F0[v].v.y;
+                acc0[v] = m == 0 ? s : acc0[v] + s;
+            }
+            const float s = F1[v].v.x + F1[v].v.y;
+            acc1[v] = m == 0 ? s : acc1[v] + s;
         }
+    }
 }
 
 // tile_gauss_flux for double-single arithmetic (no Gauss-point output): the
@@ -579,9 +668,13 @@ __device__ __forceinline__ void tile_gauss_flux_ds2(const FluxPhys<dsf2> &ph, co
 // box of a tile is dead once its t1 pass is in shared memory, so the next
 // tile's face box is fetched by TMA into the same buffer while the Gauss
 // points of the current one are computed (one buffer: more blocks per SM).
-template <typename R, typename C, bool NEED_F0, bool GP>
+struct TilePos {
+    int t, d, f, a0, b0;   // tile, direction, face plane, first face along t1 and t2
+};
+
+template <typename R, typename C, bool NEED_F0, bool GP, int ND>
 __global__ void __launch_bounds__(256, std::is_same<C, dsf>::value ? 2 : 1)
-    face_flux_kernel(const __grid_constant__ CUtensorMap tmap, FluxArgs<R, C> A)
+    face_flux_kernel(const __grid_constant__ FluxMaps<ND> maps, FluxLaunch<R, C, ND> F)
 {
     static_assert(sizeof(C) == sizeof(R), "the t1-pass rows share the storage size");
     using M = Mid<R, C>;
@@ -590,48 +683,56 @@ __global__ void __launch_bounds__(256, std::is_same<C, dsf>::value ? 2 : 1)
     C *st = reinterpret_cast<C *>(sq + SQ_N);
     uint64_t *bar = reinterpret_cast<uint64_t *>(st + ST_N);
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
-    const int NA = (A.n1 + TX - 1) / TX, NB = (A.n2 + TY - 1) / TY;
-    const int ntiles = NA * NB * A.nf;
+    const int ntiles = F.first[ND];
     const uint32_t bytes = (uint32_t)(SQ_N * sizeof(R));
-    // the block's first tile and its stride, in (ta, tb, f)
-    const TileIdx g = {(int)(gridDim.x % NA), (int)((gridDim.x / NA) % NB), (int)(gridDim.x / (NA * NB))};
-    TileIdx cur = {(int)(blockIdx.x % NA), (int)((blockIdx.x / NA) % NB), (int)(blockIdx.x / (NA * NB))};
+    auto tile = [&](int t) {
+        TilePos p;
+        p.t = t;
+        p.d = ND == 1 ? 0 : (t < F.first[1] ? 0 : (t < F.first[ND - 1] ? 1 : ND - 1));
+        const FluxArgs<R, C> &A = F.A[p.d];
+        const int NA = (A.n1 + TX - 1) / TX, NB = (A.n2 + TY - 1) / TY;
+        const int l = t - F.first[p.d], r = l / NA;
+        p.a0 = (l - r * NA) * TX;
+        p.f = r / NB;
+        p.b0 = (r - p.f * NB) * TY;
+        return p;
+    };
+    auto load = [&](const TilePos &p) {
+        if (tid == 0 && p.t < ntiles)
+            tma_load_tile(&maps.d[p.d], sq, &bar[0], p.a0, p.b0, p.f, bytes);
+    };
     if (tid == 0) {
         mbar_init(&bar[0], 1);
         mbar_fence_init();
     }
     __syncthreads();
-    int t = blockIdx.x;
-    if (tid == 0 && t < ntiles) tma_load_tile(&tmap, sq, &bar[0], cur.ta * TX, cur.tb * TY, cur.f, bytes);
-    for (int k = 0; t < ntiles; t += gridDim.x, ++k) {
-        const int tn = t + gridDim.x;
-        const TileIdx nxt = tile_add(cur, g, NA, NB);
+    TilePos cur = tile(blockIdx.x);
+    load(cur);
+    for (int k = 0; cur.t < ntiles; ++k) {
+        const TilePos nxt = tile(cur.t + gridDim.x);
+        const FluxArgs<R, C> &A = F.A[cur.d];
         const bool ok = mbar_wait(&bar[0], (uint32_t)(k & 1));
         if (__syncthreads_or(!ok)) {
             if (tid == 0) atomicOr(&A.scal->flags, FLAG_TIMEOUT);
             return;
         }
-        const int a0 = cur.ta * TX, b0 = cur.tb * TY, f = cur.f;
-        cur = nxt;
-
         tile_t1_pass(sq, st, tid);
         __syncthreads();
         // the face box is free: fetch the next tile's while this one's Gauss
         // points are computed
-        if (tid == 0 && tn < ntiles) {
-            fence_proxy_async();
-            tma_load_tile(&tmap, sq, &bar[0], nxt.ta * TX, nxt.tb * TY, nxt.f, bytes);
-        }
+        if (tid == 0) fence_proxy_async();
+        load(nxt);
 
-        const int a = a0 + tx, b = b0 + ty;
+        const int a = cur.a0 + tx, b = cur.b0 + ty;
         if (a < A.n1 && b < A.n2) {
             const C ih1 = cvt<C>(__ldg(A.ih1 + a + G)), ih2 = cvt<C>(__ldg(A.ih2 + b + G));
             C acc0[4], acc1[4];
-            const long o = ((long)f * A.n2 + b) * A.n1 + a;
+            const long o = ((long)cur.f * A.n2 + b) * A.n1 + a;
             if constexpr (std::is_same<C, dsf>::value)
                 tile_gauss_flux_ds2<NEED_F0>(flux_phys_ds2(A.ph), st, tx, ty, ih1, ih2, acc0, acc1);
             else
-                tile_gauss_flux<NEED_F0, GP>(flux_phys(A.ph), st, tx, ty, ih1, ih2, acc0, acc1, A.gp, A.gp32, A.ngp, o);
+                tile_gauss_flux<NEED_F0, GP>(flux_phys(A.ph), st, tx, ty, ih1, ih2, acc0, acc1, A.gp, A.gp32, A.ngp,
+                                             o);
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
                 if (!in_bounds(o, A.nff)) break;
@@ -639,11 +740,12 @@ __global__ void __launch_bounds__(256, std::is_same<C, dsf>::value ? 2 : 1)
                 A.ff[(4 + A.gcomp[v]) * A.nff + o] = face_avg_neg(acc1[v]);
             }
         }
+        cur = nxt;
         __syncthreads();   // st and this buffer are free again
     }
 }
 
-// ---- FP32C x and y face fluxes: a march along t2 in registers ----
+// ---- FP32C face fluxes: a march along t2 in registers ----
 //
 // A warp owns 32 faces along t1 and walks a segment of t2 rows of one face
 // plane. Per row it forms the t1 pass of the 8 face-box values at both t1
@@ -748,29 +850,32 @@ __device__ __forceinline__ void march_face(const FluxPhys<f2> &ph, const MarchWi
     }
 }
 
-// Position of a warp in its work: item (face plane, t2 segment, t1 tile), box
-// k of the item's n boxes; a0, b0 its first face along t1 and t2, be the end.
+// Position of a warp in its work: item (direction, face plane, t2 segment, t1
+// tile), box k of the item's n boxes; a0, b0 its first face along t1 and t2,
+// be the end.
 struct MarchPos {
-    int it, k, n, f, a0, b0, be;
+    int it, d, k, n, f, a0, b0, be;
 };
 
-template <bool NEED_F0>
+template <bool NEED_F0, int ND>
 __global__ void __launch_bounds__(32 * kMarchWarps, 1)
-    face_flux_march_kernel(const __grid_constant__ CUtensorMap tmap, FluxArgs<float, float> A, int L)
+    face_flux_march_kernel(const __grid_constant__ FluxMaps<ND> maps, FluxLaunch<float, float, ND> F)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     float *buf = reinterpret_cast<float *>(smem_raw) + warp * 2 * kMarchStage;
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + (size_t)nw * 2 * kMarchStage * sizeof(float)) + 2 * warp;
-    const int NA = (A.n1 + TX - 1) / TX, NS = (A.n2 + L - 1) / L, nitems = NA * NS * A.nf;
-    const int step = gridDim.x * nw;
+    const int nitems = F.first[ND], step = gridDim.x * nw;
     auto item = [&](int it) {
         MarchPos p;
-        const int ta = it % NA, r = it / NA, sg = r % NS;
+        p.d = ND == 1 ? 0 : (it < F.first[1] ? 0 : (it < F.first[ND - 1] ? 1 : ND - 1));
+        const FluxArgs<float, float> &A = F.A[p.d];
+        const int L = F.L[p.d], NA = (A.n1 + TX - 1) / TX, NS = (A.n2 + L - 1) / L;
+        const int l = it - F.first[p.d], r = l / NA, sg = r % NS;
         p.it = it;
         p.k = 0;
         p.f = r / NS;
-        p.a0 = ta * TX;
+        p.a0 = (l - r * NA) * TX;
         p.b0 = sg * L;
         p.be = min(p.b0 + L, A.n2);
         p.n = (p.be - p.b0 + 4 + RB - 1) / RB;
@@ -778,7 +883,7 @@ __global__ void __launch_bounds__(32 * kMarchWarps, 1)
     };
     auto load = [&](const MarchPos &p, int s) {
         if (lane == 0 && p.it < nitems)
-            tma_load_tile(&tmap, buf + s * kMarchStage, &bar[s], 2 * p.a0, p.b0 + p.k * RB, p.f,
+            tma_load_tile(&maps.d[p.d], buf + s * kMarchStage, &bar[s], 2 * p.a0, p.b0 + p.k * RB, p.f,
                           (uint32_t)(kMarchStage * sizeof(float)));
     };
     auto next = [&](const MarchPos &p) {
@@ -796,9 +901,10 @@ __global__ void __launch_bounds__(32 * kMarchWarps, 1)
     load(ahead, 0);
     if (ahead.it < nitems) ahead = next(ahead);
     load(ahead, 1);
-    const FluxPhys<f2> ph = flux_phys_f2(A.ph);
+    const FluxPhys<f2> ph = flux_phys_f2(F.A[0].ph);
     MarchWin w;
     for (int cnt = 0; cur.it < nitems; ++cnt) {
+        const FluxArgs<float, float> &A = F.A[cur.d];
         const int s = cnt & 1;
         const int a = cur.a0 + lane, b = cur.b0 + cur.k * RB - 4;   // face that the box's first row completes
         const bool in = a < A.n1;
@@ -864,17 +970,13 @@ int march_segment(int na, int nf, int n2, int warps)
 // ------------------------------------------------- z flux + stage update --
 
 constexpr int kMaxPrepBoxes = 8;   // forcing boxes the fused prep can leave out
-
-
+constexpr int kUpdZ = 4;           // planes per block of the stage update
 
 template <typename R, typename M = R>
 struct UpdArgs {
-    const M *ffx, *ffy;   // face fluxes of the x and y directions (8 arrays each)
-    long nffx, nffy;
-    const M *ffz;         // z face fluxes (the separate update of double-single FP64 grids)
-    long nffz;
-    const R *ihx, *ihy;   // inverse cell widths along x, y (separate update)
-    const R *ihz;         // inverse cell widths along z (padded index)
+    const M *ffx, *ffy, *ffz;     // face fluxes of the x, y and z directions (8 arrays each; no z in the fused kernel)
+    long nffx, nffy, nffz;
+    const R *ihx, *ihy, *ihz;     // inverse cell widths (padded index)
     int nx, ny, nz, P0, P1;
     long np;
     const void *w0;   // stage 1: state (FP64 W / FP32C hi,lo)
@@ -883,13 +985,14 @@ struct UpdArgs {
     void *state;      // stage 2 output
     R off;
     R fb[3];
-    int seg;          // z-faces per segment of the fused z kernel
     // stage 2, optional: the next step's prep (FP32C: the FP32 input into
     // wk0n; max |U|^2 over the cells outside the forcing boxes into scal)
     int prep;
     float *wk0n;
     int nbox;
     int box[kMaxPrepBoxes][3][2];
+    int advance;      // stage 2: t += dt (the last launch of a step without forcing)
+    Scalars *scal;
 };
 
 __device__ __forceinline__ void add_comp(float &hi, float &lo, float d)
@@ -950,32 +1053,32 @@ __device__ __forceinline__ bool update_cell(const UpdArgs<R> &A, long lin, doubl
     bool bad = false;
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-        const R Lt = -(dx[4 + v] * ihx + dy[4 + v] * ihy + dz[4 + v] * ihz);
+        const R Lt = -fma(dz[4 + v], ihz, fma(dy[4 + v], ihy, dx[4 + v] * ihx));
         if (STAGE == 1) {
-            const R L = -(dx[v] * ihx + dy[v] * ihy + dz[v] * ihz);
+            const R L = -fma(dz[v], ihz, fma(dy[v], ihy, dx[v] * ihx));
             if constexpr (std::is_same<R, double>::value) {
                 const double w = s0[v];
-                ((double *)A.wk1)[v * A.np + lin] = w + 0.5 * dt * L + 0.125 * dt * dt * Lt;
-                ((double *)A.pbuf)[v * A.np + lin] = w + dt * L + dt * dt / 6.0 * Lt;
+                ((double *)A.wk1)[v * A.np + lin] = w + fma(0.5 * dt, L, 0.125 * dt * dt * Lt);
+                ((double *)A.pbuf)[v * A.np + lin] = w + fma(dt, L, dt * dt / 6.0 * Lt);
             } else {
                 float hi = s0[v], lo = s1[v];
                 const float offv = v == 0 ? A.off : 0.0f;
-                ((float *)A.wk1)[v * A.np + lin] = ((hi - offv) + lo) + (0.5f * dtr * L + 0.125f * dtr * dtr * Lt);
-                add_comp(hi, lo, dtr * L + dtr * dtr * (1.0f / 6.0f) * Lt);
+                ((float *)A.wk1)[v * A.np + lin] = ((hi - offv) + lo) + fma(0.5f * dtr, L, 0.125f * dtr * dtr * Lt);
+                add_comp(hi, lo, fma(dtr, L, dtr * dtr * (1.0f / 6.0f) * Lt));
                 ((float *)A.pbuf)[v * A.np + lin] = hi;
                 ((float *)A.pbuf)[(4 + v) * A.np + lin] = lo;
             }
         } else {
             if constexpr (std::is_same<R, double>::value) {
-                double w = s0[v] + dt * dt / 3.0 * Lt;
-                if (v > 0) w += dt * (double)A.fb[v - 1];
+                double w = fma(dt * dt / 3.0, Lt, s0[v]);
+                if (v > 0) w = fma(dt, (double)A.fb[v - 1], w);
                 ((double *)A.state)[v * A.np + lin] = w;
                 bad |= !isfinite(w);
                 o0[v] = w;
             } else {
                 float hi = s0[v], lo = s1[v];
                 float inc = dtr * dtr * (1.0f / 3.0f) * Lt;
-                if (v > 0) inc += dtr * A.fb[v - 1];
+                if (v > 0) inc = fma(dtr, A.fb[v - 1], inc);
                 add_comp(hi, lo, inc);
                 ((float *)A.state)[v * A.np + lin] = hi;
                 ((float *)A.state)[(4 + v) * A.np + lin] = lo;
@@ -992,13 +1095,12 @@ constexpr int SX_H = TX + 1, SX_W = TY + 1;   // x-face slab of a tile in shared
 
 constexpr int SY_H = TY + 1;                  // y-face slab of a tile: the TY + 1 face rows of its cells
 
-template <typename R>
 constexpr size_t flux_update_smem_bytes(int nc)
 {
-    return flux_smem_bytes<R>() + (size_t)nc * (SX_H * SX_W + SY_H * TX) * sizeof(R);
+    return flux_smem_bytes<float>() + (size_t)nc * (SX_H * SX_W + SY_H * TX) * sizeof(float);
 }
 
-// z-direction face flux fused with the stage update. Work items are
+// z-direction face flux fused with the stage update (FP32C). Work items are
 // (z segment, tile column) pairs, segment-major, taken round-robin by the
 // persistent blocks, so that the blocks resident at one time march through
 // the same z range of neighbouring columns (their tile halos and the x-face
@@ -1030,27 +1132,22 @@ __device__ __forceinline__ ZWalk zwalk_item(int it, int ncol, int NA, int L, int
     return z;
 }
 
-template <typename R, typename C, int STAGE, bool GP>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
-    flux_update_kernel(const __grid_constant__ CUtensorMap tmap, FluxArgs<R, C> A, UpdArgs<R, Mid<R, C>> U)
+template <int STAGE>
+__global__ void __launch_bounds__(256, 2)
+    flux_update_kernel(const __grid_constant__ CUtensorMap tmap, FluxArgs<float, float> A, UpdArgs<float> U, int seg)
 {
-    static_assert(sizeof(C) == sizeof(R), "the t1-pass rows share the storage size");
-    using M = Mid<R, C>;                       // face boxes, face fluxes and their differences
-    // double-single grids take the z faces through face_flux_kernel and
-    // update_ds_kernel instead
-    static_assert(!std::is_same<C, dsf>::value, "the fused z kernel runs FP64 or FP32 arithmetic");
-    constexpr bool F32 = std::is_same<C, float>::value;   // face boxes and rows hold component pairs
-    constexpr int CX = F32 ? 2 : 1;                       // elements of a face-box position along t1
+    using R = float;
+    using M = float;
     constexpr bool NEED_F0 = STAGE == 1;
     constexpr int NC = STAGE == 1 ? 8 : 4, C0 = STAGE == 1 ? 0 : 4;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    M *sq = reinterpret_cast<M *>(smem_raw);             // face-box tile (SQ_N), refilled after its t1 pass
-    C *st = reinterpret_cast<C *>(sq + SQ_N);
-    uint64_t *bar = reinterpret_cast<uint64_t *>(st + ST_N);
+    float2 *sq = reinterpret_cast<float2 *>(smem_raw);   // face-box tile (SQ_N floats), refilled after its t1 pass
+    float2 *st = sq + SQ_N / 2;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(st + ST_N / 2);
     M *sx = reinterpret_cast<M *>(bar + 2);               // [NC][SX_H][SX_W]
     M *sy = sx + NC * SX_H * SX_W;                        // [NC][SY_H][TX]
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
-    const int NA = (A.n1 + TX - 1) / TX, NB = (A.n2 + TY - 1) / TY, nf = A.nf, L = U.seg;
+    const int NA = (A.n1 + TX - 1) / TX, NB = (A.n2 + TY - 1) / TY, nf = A.nf, L = seg;
     const int ncol = NA * NB, nitems = ncol * ((nf + L - 1) / L);
     if ((int)blockIdx.x >= nitems) return;
     const uint32_t bytes = (uint32_t)(SQ_N * sizeof(R));
@@ -1060,10 +1157,10 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
         mbar_fence_init();
     }
     __syncthreads();
-    if (tid == 0) tma_load_tile(&tmap, sq, &bar[0], CX * cur.a0, cur.b0, cur.f, bytes);
+    if (tid == 0) tma_load_tile(&tmap, sq, &bar[0], 2 * cur.a0, cur.b0, cur.f, bytes);
     const double dt = A.scal->dt;
     bool bad = false;
-    double mx = 0.0;   // stage 2 with prep: max |U|^2 of this thread's cells outside the forcing boxes
+    float mx = 0.0f;   // stage 2 with prep: max |U|^2 of this thread's cells outside the forcing boxes
     M P0[4], P1[4];   // F0, F1 of the previous face of this column (storage type: the
                       // differences of neighbouring faces telescope exactly)
     for (int k = 0; cur.it < nitems; ++k) {
@@ -1130,7 +1227,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
                     s0[v] = __ldg(src + v * U.np + lin);
-                    s1[v] = std::is_same<R, double>::value ? R(0) : __ldg(src + (4 + v) * U.np + lin);
+                    s1[v] = __ldg(src + (4 + v) * U.np + lin);
                 }
             }
         }
@@ -1141,30 +1238,22 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
             __syncthreads();
             return;
         }
-        if constexpr (F32)
-            tile_t1_pass_f2<SQ_H>(reinterpret_cast<const float2 *>(sq), reinterpret_cast<float2 *>(st), tid);
-        else
-            tile_t1_pass(sq, st, tid);
+        tile_t1_pass_f2<SQ_H>(sq, st, tid);
         __syncthreads();
         // the face box is free: fetch the next tile's during this one's flux
         if (tid == 0 && nxt.it < nitems) {
             fence_proxy_async();
-            tma_load_tile(&tmap, sq, &bar[0], CX * nxt.a0, nxt.b0, nxt.f, bytes);
+            tma_load_tile(&tmap, sq, &bar[0], 2 * nxt.a0, nxt.b0, nxt.f, bytes);
         }
 
         M F0[4], F1[4];
         if (in) {
-            C G0[1][4], G1[1][4];
-            if constexpr (F32)
-                tile_gauss_flux_f2<SQ_H, 1, NEED_F0>(flux_phys_f2(A.ph), reinterpret_cast<const float2 *>(st), tx, ty, ih1,
-                                                     &ih2, G0, G1);
-            else
-                tile_gauss_flux<NEED_F0, GP>(flux_phys(A.ph), st, tx, ty, ih1, ih2, G0[0], G1[0], A.gp, A.gp32, A.ngp,
-                                             ((long)f * A.n2 + b) * A.n1 + a);
+            float G0[4], G1[4];
+            tile_gauss_flux_f2<NEED_F0>(flux_phys_f2(A.ph), st, tx, ty, ih1, ih2, G0, G1);
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
-                F0[v] = NEED_F0 ? face_avg(G0[0][v]) : M(0);
-                F1[v] = face_avg_neg(G1[0][v]);
+                F0[v] = NEED_F0 ? face_avg(G0[v]) : 0.0f;
+                F1[v] = face_avg_neg(G1[v]);
             }
         }
         if (upd) {
@@ -1192,13 +1281,9 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
                     for (int q = 0; q < U.nbox; ++q)
                         boxed |= a >= U.box[q][0][0] && a <= U.box[q][0][1] && b >= U.box[q][1][0] &&
                                  b <= U.box[q][1][1] && z >= U.box[q][2][0] && z <= U.box[q][2][1];
-                    if constexpr (std::is_same<R, double>::value) {
-                        if (!boxed) mx = max_u2(mx, cell_u2(o0));
-                    } else {
 #pragma unroll
-                        for (int v = 0; v < 4; ++v) U.wk0n[v * U.np + lin] = (o0[v] - (v == 0 ? U.off : 0.0f)) + o1[v];
-                        if (!boxed) mx = max_u2(mx, cell_u2(o0, o1));
-                    }
+                    for (int v = 0; v < 4; ++v) U.wk0n[v * U.np + lin] = (o0[v] - (v == 0 ? U.off : 0.0f)) + o1[v];
+                    if (!boxed) mx = max_u2f(mx, cell_u2f(o0, o1));
                 }
             }
         }
@@ -1213,76 +1298,109 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
         __syncthreads();   // st, the face buffer and the slabs are free again
     }
     if (STAGE == 2 && bad) atomicOr(&A.scal->flags, FLAG_NONFINITE);
-    if (STAGE == 2 && U.prep) block_max_to(mx, &A.scal->maxu2_bits);
+    if (STAGE == 2 && U.prep) block_max_to((double)mx, &A.scal->maxu2_bits);
+    if (STAGE == 2 && U.advance && blockIdx.x == 0 && tid == 0) U.scal->t = U.scal->t + dt;
 }
 
-
-// Stage update of every cell from stored x, y and z face fluxes, for FP64
-// grids in double-single arithmetic: there the fused z kernel needs about 220
-// registers (one block per SM) while the face-flux kernel runs two blocks per
-// SM, so the z faces go through face_flux_kernel into their own buffer and
-// this kernel applies update_cell_ds (the same operations as the fused
-// kernel, the same bits). One thread per cell of a 32 x 8 x 1 block; the
-// x-face fluxes of the block's cells (y-fastest) arrive through a padded
-// shared slab.
-template <int STAGE>
-__global__ void __launch_bounds__(256) update_ds_kernel(UpdArgs<double, dsf> U, Scalars *scal)
+// Stage update of every cell from the stored fluxes of all its faces (FP64
+// grids, and the small FP32C grids whose directions run together). A block
+// takes 32 x 8 columns of kUpdZ planes, a thread one cell per plane; the
+// x-face fluxes (y fastest in memory) arrive through a padded shared slab, the
+// y- and z-face fluxes and the state straight from memory: bound by memory.
+// FP64 kernels: the fused form needs 218 registers and recomputes the first
+// face of each z segment (z faces and update of a 96^3 step 2.89 -> 2.70 ms
+// apart). Large FP32C grids stay fused: 2.75 ms apart against 2.44 ms on
+// 384x256x256, where the z-face fluxes' way through memory costs more than the
+// tile kernel's shared memory.
+template <typename R, typename C, int STAGE>
+__global__ void __launch_bounds__(256) update_kernel(const __grid_constant__ UpdArgs<R, Mid<R, C>> U, int planes)
 {
+    using M = Mid<R, C>;
     constexpr int NC = STAGE == 1 ? 8 : 4, C0 = STAGE == 1 ? 0 : 4;
-    __shared__ dsf sx[NC][SX_H][SX_W];
+    __shared__ M sx[2][NC][SX_H][SX_W];
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
-    const int a0 = blockIdx.x * TX, b0 = blockIdx.y * TY, z = blockIdx.z;
-    {
-        // x faces a0 .. a0+32 of rows b0 .. b0+7: thread row b0 + (tid & 7),
-        // face a0 + tid/8; the 8 threads with tid/8 = 0 also take face a0 + 32
+    const int a0 = blockIdx.x * TX, b0 = blockIdx.y * TY, zb = blockIdx.z * planes, ze = min(zb + planes, U.nz);
+    const int a = a0 + tx, b = b0 + ty;
+    const bool in = a < U.nx && b < U.ny;
+    const double dt = U.scal->dt;
+    R ihx = R(0), ihy = R(0);
+    if (in) {
+        ihx = __ldg(U.ihx + a + G);
+        ihy = __ldg(U.ihy + b + G);
+    }
+    // x faces a0 .. a0+32 of rows b0 .. b0+7 of plane z: thread row b0 + (tid &
+    // 7), face a0 + tid/8; the 8 threads with tid/8 = 0 also take face a0 + 32
+    auto slab = [&](int z, int s) {
         const int yy = tid & 7, xf = tid >> 3;
         if (b0 + yy < U.ny) {
             const long sxf = (long)U.nz * U.ny;
             const long g0 = ((long)(a0 + xf) * U.nz + z) * U.ny + b0 + yy;
             if (a0 + xf <= U.nx && in_bounds(g0, U.nffx)) {
 #pragma unroll
-                for (int c = 0; c < NC; ++c) sx[c][xf][yy] = U.ffx[(C0 + c) * U.nffx + g0];
+                for (int c = 0; c < NC; ++c) cp_async(&sx[s][c][xf][yy], U.ffx + (C0 + c) * U.nffx + g0);
             }
             if (xf == 0 && a0 + 32 <= U.nx && in_bounds(g0 + 32 * sxf, U.nffx)) {
 #pragma unroll
-                for (int c = 0; c < NC; ++c) sx[c][32][yy] = U.ffx[(C0 + c) * U.nffx + g0 + 32 * sxf];
+                for (int c = 0; c < NC; ++c) cp_async(&sx[s][c][32][yy], U.ffx + (C0 + c) * U.nffx + g0 + 32 * sxf);
             }
         }
-    }
-    __syncthreads();
-    const int a = a0 + tx, b = b0 + ty;
+        cp_async_commit();
+    };
     bool bad = false;
     double mx = 0.0;
-    if (a < U.nx && b < U.ny) {
+    float mxf = 0.0f;
+    slab(zb, 0);
+    for (int z = zb, s = 0; z < ze; ++z, s ^= 1) {
         const long lin = (long)(a + G) + (long)U.P0 * ((long)(b + G) + (long)U.P1 * (z + G));
         const long iy = ((long)b * U.nz + z) * U.nx + a, sy = (long)U.nz * U.nx;
         const long iz = ((long)z * U.ny + b) * U.nx + a, sz = (long)U.ny * U.nx;
-        if (in_bounds(lin, U.np) && in_bounds(iy + sy, U.nffy) && in_bounds(iz + sz, U.nffz)) {
-            dsf dx[8], dy[8], dz[8];
+        const bool ok = in && in_bounds(lin, U.np) && in_bounds(iy + sy, U.nffy) && in_bounds(iz + sz, U.nffz);
+        M dx[8], dy[8], dz[8];
+        R s0[4], s1[4];
+        if (ok) {
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 const int k = C0 + c;
-                dx[k] = sx[c][tx + 1][ty] - sx[c][tx][ty];
                 dy[k] = U.ffy[k * U.nffy + iy + sy] - U.ffy[k * U.nffy + iy];
                 dz[k] = U.ffz[k * U.nffz + iz + sz] - U.ffz[k * U.nffz + iz];
             }
-            const double *src = (const double *)(STAGE == 1 ? U.w0 : U.pbuf);
-            double s0[4], o0[4];
+            const R *src = (const R *)(STAGE == 1 ? U.w0 : U.pbuf);
 #pragma unroll
-            for (int v = 0; v < 4; ++v) s0[v] = src[v * U.np + lin];
-            bad = !update_cell_ds<STAGE>(U, lin, scal->dt, dx, dy, dz, to_ds(__ldg(U.ihx + a + G)),
-                                         to_ds(__ldg(U.ihy + b + G)), to_ds(__ldg(U.ihz + z + G)), s0, o0);
-            if (STAGE == 2 && U.prep) {
-                bool boxed = false;
-                for (int q = 0; q < U.nbox; ++q)
-                    boxed |= a >= U.box[q][0][0] && a <= U.box[q][0][1] && b >= U.box[q][1][0] &&
-                             b <= U.box[q][1][1] && z >= U.box[q][2][0] && z <= U.box[q][2][1];
+            for (int v = 0; v < 4; ++v) {
+                s0[v] = src[v * U.np + lin];
+                s1[v] = std::is_same<R, double>::value ? R(0) : src[(4 + v) * U.np + lin];
+            }
+        }
+        cp_async_wait_all();
+        __syncthreads();   // the slab of plane z is in place, that of z - 1 has been read
+        if (z + 1 < ze) slab(z + 1, s ^ 1);
+        if (!ok) continue;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) dx[C0 + c] = sx[s][c][tx + 1][ty] - sx[s][c][tx][ty];
+        const R ihz = __ldg(U.ihz + z + G);
+        R o0[4], o1[4];
+        if constexpr (std::is_same<C, dsf>::value)
+            bad |= !update_cell_ds<STAGE>(U, lin, dt, dx, dy, dz, to_ds(ihx), to_ds(ihy), to_ds(ihz), s0, o0);
+        else
+            bad |= !update_cell<R, STAGE>(U, lin, dt, dx, dy, dz, ihx, ihy, ihz, s0, s1, o0, o1);
+        if (STAGE == 2 && U.prep) {
+            bool boxed = false;
+            for (int q = 0; q < U.nbox; ++q)
+                boxed |= a >= U.box[q][0][0] && a <= U.box[q][0][1] && b >= U.box[q][1][0] && b <= U.box[q][1][1] &&
+                         z >= U.box[q][2][0] && z <= U.box[q][2][1];
+            if constexpr (std::is_same<R, double>::value) {
                 if (!boxed) mx = max_u2(mx, cell_u2(o0));
+            } else {
+#pragma unroll
+                for (int v = 0; v < 4; ++v) U.wk0n[v * U.np + lin] = (o0[v] - (v == 0 ? U.off : 0.0f)) + o1[v];
+                if (!boxed) mxf = max_u2f(mxf, cell_u2f(o0, o1));
             }
         }
     }
-    if (STAGE == 2 && bad) atomicOr(&scal->flags, FLAG_NONFINITE);
-    if (STAGE == 2 && U.prep) block_max_to(mx, &scal->maxu2_bits);
+    if (STAGE == 2 && bad) atomicOr(&U.scal->flags, FLAG_NONFINITE);
+    if (STAGE == 2 && U.prep) block_max_to(std::is_same<R, double>::value ? mx : (double)mxf, &U.scal->maxu2_bits);
+    if (STAGE == 2 && U.advance && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && tid == 0)
+        U.scal->t = U.scal->t + dt;
 }
 
 // Faces per thread of the marching face-state kernel: k0 (kMarch32 or
@@ -1311,35 +1429,22 @@ int persistent_grid(K kernel, size_t smem)
     return (per > 0 ? per : 1) * (sms > 0 ? sms : 1);
 }
 
-template <typename R, typename C, int STAGE>
-struct FluxGrids {
-    int flux[2] = {0, 0}, flux_update[2] = {0, 0};   // without / with the Gauss-point output
-};
-
-// The Gauss-point output (recorded steps of the adjoint) exists only in FP64
-// arithmetic.
-template <typename R, typename C, int STAGE>
-const FluxGrids<R, C, STAGE> &flux_grids()
+// Blocks of the persistent face-flux kernels (FP32C: one block per SM), found
+// once per kernel; GP (the Gauss-point output of the adjoint's recorded steps)
+// exists in FP64 arithmetic only.
+template <typename R, typename C, int STAGE, bool GP, int ND>
+int flux_blocks()
 {
-    static FluxGrids<R, C, STAGE> g;
-    if (!g.flux[0]) {
-        constexpr size_t su = flux_update_smem_bytes<R>(STAGE == 1 ? 8 : 4);
+    static const int n = [] {
         if constexpr (std::is_same<C, float>::value) {
-            // FP32C: the register march in x and y, one block of kMarchWarps warps per SM
-            cudaFuncSetAttribute(face_flux_march_kernel<STAGE == 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            cudaFuncSetAttribute(face_flux_march_kernel<STAGE == 1, ND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)march_smem_bytes(kMarchWarps));
-            g.flux[0] = sm_count();
+            return sm_count();
         } else {
-            g.flux[0] = persistent_grid(face_flux_kernel<R, C, STAGE == 1, false>, flux_smem_bytes<R>());
+            return persistent_grid(face_flux_kernel<R, C, STAGE == 1, GP, ND>, flux_smem_bytes<R>());
         }
-        if constexpr (!std::is_same<C, dsf>::value)   // double-single: separate z update
-            g.flux_update[0] = persistent_grid(flux_update_kernel<R, C, STAGE, false>, su);
-        if constexpr (std::is_same<C, double>::value) {
-            g.flux[1] = persistent_grid(face_flux_kernel<R, C, STAGE == 1, true>, flux_smem_bytes<R>());
-            g.flux_update[1] = persistent_grid(flux_update_kernel<R, C, STAGE, true>, su);
-        }
-    }
-    return g;
+    }();
+    return n;
 }
 
 // z-faces per segment of the fused z kernel: the length L that minimises the
@@ -1370,7 +1475,7 @@ FaceEqArgs<R, C> face_eq_args(const Ctx &c, int d, const R *w, const Phys<C> &ph
     FaceEqArgs<R, C> E;
     E.w = w;
     E.np = c.np;
-    E.fq = (Mid<R, C> *)c.fq;
+    E.fq = (Mid<R, C> *)c.fq[d];
     E.nfq = c.nfq;
     E.ihf = (const R *)c.ihf[d];
     E.n1 = c.n[t1];
@@ -1390,19 +1495,70 @@ FaceEqArgs<R, C> face_eq_args(const Ctx &c, int d, const R *w, const Phys<C> &ph
     return E;
 }
 
-// Arguments of the stage update of the z-face kernels (the fused one and the
-// separate double-single one).
+// Arguments of the face flux of direction d.
+template <typename R, typename C>
+FluxArgs<R, C> flux_args(const Ctx &c, int d, const Phys<C> &ph)
+{
+    const int t1 = tan1(d), t2 = tan2(d);
+    FluxArgs<R, C> F;
+    F.ff = (Mid<R, C> *)c.ff[d];
+    F.nff = c.nff[d];
+    F.ih1 = (const R *)c.ih[t1];
+    F.ih2 = (const R *)c.ih[t2];
+    F.n1 = c.n[t1];
+    F.n2 = c.n[t2];
+    F.nf = c.n[d] + 1;
+    F.gcomp[0] = 0;
+    F.gcomp[1] = 1 + d;
+    F.gcomp[2] = 1 + t1;
+    F.gcomp[3] = 1 + t2;
+    F.ph = ph;
+    F.scal = c.scal;
+    F.gp = std::is_same<C, double>::value ? c.gp_dir[d] : nullptr;
+    F.ngp = c.ngp;
+    F.gp32 = c.gp_bytes == 4;
+    return F;
+}
+
+// The face fluxes of ND directions (their arguments in F.A).
+template <typename R, typename C, int STAGE, bool GP, int ND>
+void launch_flux(const FluxMaps<ND> &maps, FluxLaunch<R, C, ND> &F, cudaStream_t stream)
+{
+    const int G1 = flux_blocks<R, C, STAGE, GP, ND>();
+    F.first[0] = 0;
+    for (int k = 0; k < ND; ++k) {
+        const FluxArgs<R, C> &A = F.A[k];
+        const int na = (A.n1 + TX - 1) / TX;
+        if (std::is_same<C, float>::value) {
+            F.L[k] = march_segment(na, A.nf, A.n2, kMarchWarps * G1 / ND);
+            F.first[k + 1] = F.first[k] + na * A.nf * ((A.n2 + F.L[k] - 1) / F.L[k]);
+        } else {
+            F.first[k + 1] = F.first[k] + na * ((A.n2 + TY - 1) / TY) * A.nf;
+        }
+    }
+    const int items = F.first[ND];
+    if constexpr (std::is_same<C, float>::value) {
+        // few items: fewer warps per block, so that they spread over the SMs
+        const int nw = std::min(kMarchWarps, (items + G1 - 1) / G1), g = std::min(G1, (items + nw - 1) / nw);
+        face_flux_march_kernel<STAGE == 1, ND><<<g, 32 * nw, march_smem_bytes(nw), stream>>>(maps, F);
+    } else {
+        face_flux_kernel<R, C, STAGE == 1, GP, ND>
+            <<<std::min(items, G1), dim3(TX, TY), flux_smem_bytes<R>(), stream>>>(maps, F);
+    }
+}
+
 template <typename R, typename C, int STAGE>
-UpdArgs<R, Mid<R, C>> update_args(const Ctx &c, const FluxArgs<R, C> &F)
+UpdArgs<R, Mid<R, C>> update_args(const Ctx &c)
 {
     UpdArgs<R, Mid<R, C>> U;
     U.ffx = (const Mid<R, C> *)c.ff[0];
     U.ffy = (const Mid<R, C> *)c.ff[1];
+    U.ffz = (const Mid<R, C> *)c.ff[2];
     U.nffx = c.nff[0];
     U.nffy = c.nff[1];
-    U.ffz = nullptr;
-    U.nffz = 0;
-    U.ihx = U.ihy = nullptr;
+    U.nffz = c.nff[2];
+    U.ihx = (const R *)c.ih[0];
+    U.ihy = (const R *)c.ih[1];
     U.ihz = (const R *)c.ih[2];
     U.nx = c.n[0];
     U.ny = c.n[1];
@@ -1416,105 +1572,100 @@ UpdArgs<R, Mid<R, C>> update_args(const Ctx &c, const FluxArgs<R, C> &F)
     U.state = c.state;
     U.off = (R)c.off;
     for (int a = 0; a < 3; ++a) U.fb[a] = (R)c.fbody[a];
-    U.seg = 0;
     U.prep = STAGE == 2 && c.prep_next && c.nprep_box <= kMaxPrepBoxes;
     U.wk0n = c.prec == GKS_FP32C ? (float *)c.wk0 : nullptr;
     U.nbox = U.prep ? c.nprep_box : 0;
     for (int q = 0; q < U.nbox; ++q)
         for (int e = 0; e < 3; ++e)
             for (int k = 0; k < 2; ++k) U.box[q][e][k] = c.prep_box[q][e][k];
+    U.advance = STAGE == 2 && c.advance;
+    U.scal = c.scal;
     return U;
 }
 
 template <typename R, typename C, int STAGE>
+void launch_update(const Ctx &c)
+{
+    // planes per block: the grid's z extent stays within its 65535 blocks
+    int planes = kUpdZ;
+    while ((c.n[2] + planes - 1) / planes > 65535) planes *= 2;
+    const dim3 g((c.n[0] + TX - 1) / TX, (c.n[1] + TY - 1) / TY, (c.n[2] + planes - 1) / planes);
+    mark(c, K_FLUX_UPDATE, 1);
+    update_kernel<R, C, STAGE><<<g, dim3(TX, TY), 0, c.stream>>>(update_args<R, C, STAGE>(c), planes);
+    mark(c, K_FLUX_UPDATE, 0);
+}
+
+// z faces of a large FP32C grid: flux and the stage update of every cell.
+template <int STAGE>
+void launch_flux_update(const Ctx &c, const FluxArgs<float, float> &F)
+{
+    constexpr size_t su = flux_update_smem_bytes(STAGE == 1 ? 8 : 4);
+    static const int G1 = persistent_grid(flux_update_kernel<STAGE>, su);
+    const int ncol = ((F.n1 + TX - 1) / TX) * ((F.n2 + TY - 1) / TY), seg = z_segment(ncol, F.nf, G1);
+    const long nitems = (long)ncol * ((F.nf + seg - 1) / seg);
+    mark(c, K_FLUX_UPDATE, 1);
+    flux_update_kernel<STAGE><<<(int)std::min(nitems, (long)G1), dim3(TX, TY), su, c.stream>>>(
+        c.tmap[2], F, update_args<float, float, STAGE>(c), seg);
+    mark(c, K_FLUX_UPDATE, 0);
+}
+
+template <typename R, typename C, int STAGE, bool GP>
 void stage_impl(const Ctx &c)
 {
     const Phys<C> ph = make_phys<C>(c);
     const R *w = (const R *)(STAGE == 1 ? c.wk0 : c.wk1);
-    const FluxGrids<R, C, STAGE> &grids = flux_grids<R, C, STAGE>();
-    const dim3 blk(TX, TY);
-    for (int d = 0; d < 3; ++d) {
-        const int t1 = tan1(d), t2 = tan2(d);
-        const FaceEqArgs<R, C> E = face_eq_args<R, C>(c, d, w, ph);
-        const CUtensorMap &tmap = c.tmap[d];
-        dim3 ge((E.n1 + 4 + 31) / 32, (E.n2 + 4 + 7) / 8, (E.nf + E.K - 1) / E.K);
+    auto map = [&](int d) -> const CUtensorMap & { return std::is_same<C, float>::value ? c.tmapM[d] : c.tmap[d]; };
+    if (c.small) {
+        // all directions at once: their face boxes have buffers of their own
+        FaceEq3<R, C> E;
+        long blocks = 0;
+        for (int d = 0; d < 3; ++d) {
+            E.d[d] = face_eq_args<R, C>(c, d, w, ph);
+            blocks += (long)((E.d[d].n1 + 4 + 31) / 32) * ((E.d[d].n2 + 4 + 7) / 8);
+        }
+        E.first[0] = 0;
+        for (int d = 0; d < 3; ++d) {
+            constexpr bool F32 = std::is_same<C, float>::value;
+            E.d[d].K = march_faces(blocks, E.d[d].nf, F32 ? kMarch32 : kMarch, F32 ? 9 : 2);
+            const dim3 g = face_eq_blocks(E.d[d], d);
+            E.gx[d] = g.x;
+            E.gy[d] = g.y;
+            E.first[d + 1] = E.first[d] + g.x * g.y * g.z;
+        }
         mark(c, K_FACE_EQ, 1);
-        if constexpr (std::is_same<C, dsf>::value)
-            face_eq_ds2_kernel<<<ge, blk, 0, c.stream>>>(E);
-        else if constexpr (std::is_same<C, float>::value)
-            launch_face_eq_f2(E, d, c.stream);
-        else
-            face_eq_march_kernel<<<ge, blk, 0, c.stream>>>(E);
+        face_eq_all_kernel<R, C><<<E.first[3], dim3(TX, TY), 0, c.stream>>>(E);
         mark(c, K_FACE_EQ, 0);
-
-        FluxArgs<R, C> F;
-        F.ff = (Mid<R, C> *)c.ff[d];
-        F.nff = c.nff[d];
-        F.ih1 = (const R *)c.ih[t1];
-        F.ih2 = (const R *)c.ih[t2];
-        F.n1 = c.n[t1];
-        F.n2 = c.n[t2];
-        F.nf = c.n[d] + 1;
-        F.gcomp[0] = 0;
-        F.gcomp[1] = 1 + d;
-        F.gcomp[2] = 1 + t1;
-        F.gcomp[3] = 1 + t2;
-        F.ph = ph;
-        F.scal = c.scal;
-        F.gp = c.gp_dir[d];
-        F.ngp = c.ngp;
-        F.gp32 = c.gp_bytes == 4;
-        const long ntiles = (long)((F.n1 + TX - 1) / TX) * ((F.n2 + TY - 1) / TY) * F.nf;
+        FluxMaps<3> maps;
+        FluxLaunch<R, C, 3> F;
+        for (int d = 0; d < 3; ++d) {
+            maps.d[d] = map(d);
+            F.A[d] = flux_args<R, C>(c, d, ph);
+        }
+        mark(c, K_FACE_FLUX, 1);
+        launch_flux<R, C, STAGE, GP, 3>(maps, F, c.stream);
+        mark(c, K_FACE_FLUX, 0);
+        launch_update<R, C, STAGE>(c);
+        return;
+    }
+    for (int d = 0; d < 3; ++d) {
+        mark(c, K_FACE_EQ, 1);
+        launch_face_eq(face_eq_args<R, C>(c, d, w, ph), d, c.stream);
+        mark(c, K_FACE_EQ, 0);
+        FluxMaps<1> maps;
+        FluxLaunch<R, C, 1> F;
+        maps.d[0] = map(d);
+        F.A[0] = flux_args<R, C>(c, d, ph);
+        if constexpr (std::is_same<C, float>::value)
+            if (d == 2) {
+                launch_flux_update<STAGE>(c, F.A[0]);
+                return;
+            }
         const int grp = d < 2 ? K_FACE_FLUX : K_FLUX_UPDATE;
         mark(c, grp, 1);
-        constexpr bool FP64A = std::is_same<C, double>::value;
-        const int gpo = FP64A && F.gp;
-        if constexpr (std::is_same<C, dsf>::value) {
-            if (d == 2) {
-                // double-single: z-face fluxes into their own buffer, then the update
-                const int grid = (int)(ntiles < grids.flux[0] ? ntiles : grids.flux[0]);
-                face_flux_kernel<R, C, STAGE == 1, false><<<grid, blk, flux_smem_bytes<R>(), c.stream>>>(tmap, F);
-                UpdArgs<R, Mid<R, C>> U = update_args<R, C, STAGE>(c, F);
-                U.ffz = (const Mid<R, C> *)c.ff[2];
-                U.nffz = c.nff[2];
-                U.ihx = (const R *)c.ih[0];
-                U.ihy = (const R *)c.ih[1];
-                const dim3 gu((c.n[0] + TX - 1) / TX, (c.n[1] + TY - 1) / TY, c.n[2]);
-                update_ds_kernel<STAGE><<<gu, blk, 0, c.stream>>>(U, c.scal);
-                mark(c, grp, 0);
-                continue;
-            }
-        }
-        if (d < 2) {
-            if constexpr (std::is_same<C, float>::value) {
-                const int na = (F.n1 + TX - 1) / TX, L = march_segment(na, F.nf, F.n2, kMarchWarps * grids.flux[0]);
-                const long items = (long)na * F.nf * ((F.n2 + L - 1) / L);
-                // few items: fewer warps per block, so that they spread over the SMs
-                const int nw = (int)std::min((long)kMarchWarps, (items + grids.flux[0] - 1) / grids.flux[0]);
-                const int gm = (int)std::min((long)grids.flux[0], (items + nw - 1) / nw);
-                face_flux_march_kernel<STAGE == 1><<<gm, 32 * nw, march_smem_bytes(nw), c.stream>>>(c.tmapM[d], F, L);
-            } else {
-                const int grid = (int)(ntiles < grids.flux[gpo] ? ntiles : grids.flux[gpo]);
-                if (FP64A && gpo)
-                    face_flux_kernel<R, C, STAGE == 1, FP64A><<<grid, blk, flux_smem_bytes<R>(), c.stream>>>(tmap, F);
-                else
-                    face_flux_kernel<R, C, STAGE == 1, false><<<grid, blk, flux_smem_bytes<R>(), c.stream>>>(tmap, F);
-            }
-        } else if constexpr (!std::is_same<C, dsf>::value) {
-            // z faces: flux and the stage update of every cell
-            UpdArgs<R, Mid<R, C>> U = update_args<R, C, STAGE>(c, F);
-            const int ncol = ((F.n1 + TX - 1) / TX) * ((F.n2 + TY - 1) / TY);
-            U.seg = z_segment(ncol, F.nf, grids.flux_update[gpo]);
-            const long nitems = (long)ncol * ((F.nf + U.seg - 1) / U.seg);
-            const int grid = (int)(nitems < grids.flux_update[gpo] ? nitems : grids.flux_update[gpo]);
-            constexpr size_t su = flux_update_smem_bytes<R>(STAGE == 1 ? 8 : 4);
-            if (FP64A && gpo)
-                flux_update_kernel<R, C, STAGE, FP64A><<<grid, blk, su, c.stream>>>(tmap, F, U);
-            else
-                flux_update_kernel<R, C, STAGE, false><<<grid, blk, su, c.stream>>>(tmap, F, U);
-        }
+        launch_flux<R, C, STAGE, GP, 1>(maps, F, c.stream);
         mark(c, grp, 0);
     }
+    launch_update<R, C, STAGE>(c);
 }
 
 // ----------------------------------------------------- prep, CFL, misc --
@@ -1539,8 +1690,10 @@ struct PrepBoxes {
 template <int PREC>
 __global__ void __launch_bounds__(256) prep_cfl_kernel(const void *__restrict__ S, float *__restrict__ wk, long np,
                                                        const __grid_constant__ PrepBoxes B, int planes, int P0, int P1,
-                                                       float off, Scalars *scal)
+                                                       float off, Scalars *scal, int advance)
 {
+    if (advance && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0 && threadIdx.y == 0)
+        scal->t = scal->t + scal->dt;   // the last launch of a step with forcing
     const int q = blockIdx.z / B.nz;
     const int3 lo = B.lo[q], hi = B.hi[q];
     const int i = lo.x + blockIdx.x * 32 + threadIdx.x, j = lo.y + blockIdx.y * 8 + threadIdx.y;
@@ -1576,20 +1729,7 @@ __global__ void __launch_bounds__(256) prep_cfl_kernel(const void *__restrict__ 
 
 __global__ void dt_kernel(Scalars *scal, double cfl, double dt_fixed, double hmin, double csound)
 {
-    const double umax = sqrt(__longlong_as_double((long long)scal->maxu2_bits));
-    double dt;
-    if (dt_fixed > 0.0) {
-        dt = dt_fixed;
-        const double num = dt * (umax + csound) / hmin;
-        scal->cfl_number = num;
-        if (cfl > 0.0 && !(num <= cfl)) atomicOr(&scal->flags, FLAG_CFL);
-    } else {
-        dt = cfl * hmin / (umax + csound);
-        scal->cfl_number = cfl;
-        if (!isfinite(dt)) atomicOr(&scal->flags, FLAG_NONFINITE);
-    }
-    scal->dt = dt;
-    scal->maxu2_bits = 0ull;
+    set_dt(scal, cfl, dt_fixed, hmin, csound);
 }
 
 __global__ void advance_kernel(Scalars *scal) { scal->t = scal->t + scal->dt; }
@@ -1917,7 +2057,7 @@ __global__ void __launch_bounds__(256) raw_copy_kernel(T *S, T *cpt, int narr, l
 }  // namespace
 
 namespace {
-void prep_boxes(const Ctx &c, const int (*box)[3][2], int n, int planes)
+bool prep_boxes(const Ctx &c, const int (*box)[3][2], int n, int planes, int advance)
 {
     PrepBoxes B;
     int nb = 0, gx = 0, gy = 0;
@@ -1932,26 +2072,27 @@ void prep_boxes(const Ctx &c, const int (*box)[3][2], int n, int planes)
         gy = std::max(gy, (hi.y - lo.y + 7) / 8);
         B.nz = std::max(B.nz, (hi.z - lo.z + planes - 1) / planes);
     }
-    if (!nb) return;
+    if (!nb) return false;
     const dim3 blk(32, 8), g(gx, gy, B.nz * nb);
     const int grp = c.prec == GKS_FP32C ? K_PREP : K_CFL;
     mark(c, grp, 1);
     if (c.prec == GKS_FP32C)
         prep_cfl_kernel<GKS_FP32C><<<g, blk, 0, c.stream>>>(c.state, (float *)c.wk0, c.np, B, planes, c.P[0], c.P[1],
-                                                           (float)c.off, c.scal);
+                                                           (float)c.off, c.scal, advance);
     else
         prep_cfl_kernel<GKS_FP64><<<g, blk, 0, c.stream>>>(c.state, nullptr, c.np, B, planes, c.P[0], c.P[1], 0.0f,
-                                                          c.scal);
+                                                          c.scal, advance);
     mark(c, grp, 0);
+    return true;
 }
 }  // namespace
 
-void launch_prep_boxes(const Ctx &c, const int (*box)[3][2], int n)
+bool launch_prep_boxes(const Ctx &c, const int (*box)[3][2], int n, bool advance)
 {
     // planes per block: the grid's z extent stays within its 65535 blocks
     int planes = kPrepBoxZ;
     while ((long)((c.n[2] + planes - 1) / planes) * kMaxPrepBoxes > 65535) planes *= 2;
-    prep_boxes(c, box, n, planes);
+    return prep_boxes(c, box, n, planes, advance);
 }
 
 void launch_prep(const Ctx &c)
@@ -1959,15 +2100,15 @@ void launch_prep(const Ctx &c)
     const int box[1][3][2] = {{{0, c.n[0] - 1}, {0, c.n[1] - 1}, {0, c.n[2] - 1}}};
     int planes = kPrepZ;
     while ((c.n[2] + planes - 1) / planes > 65535) planes *= 2;
-    prep_boxes(c, box, 1, planes);
+    prep_boxes(c, box, 1, planes, 0);
 }
 
-void launch_ghost(const Ctx &c, void *w)
+void launch_ghost(const Ctx &c, void *w, bool with_dt)
 {
     if (c.prec == GKS_FP64)
-        ghost_impl<double>(c, (double *)w);
+        ghost_impl<double>(c, (double *)w, with_dt);
     else
-        ghost_impl<float>(c, (float *)w);
+        ghost_impl<float>(c, (float *)w, with_dt);
 }
 
 // ------------------------------------------------------------ slab groups --
@@ -2032,17 +2173,19 @@ void launch_group_max_u2(Scalars *const *scal, int n, cudaStream_t stream)
 // w into the face box c.fq (the reverse recomputes it instead of storing it).
 void launch_face_state32(const Ctx &c, int d, const float *w)
 {
-    launch_face_eq_f2(face_eq_args<float, float>(c, d, w, make_phys<float>(c)), d, c.stream);
+    launch_face_eq(face_eq_args<float, float>(c, d, w, make_phys<float>(c)), d, c.stream);
 }
 
 void launch_stage(const Ctx &c, int stage)
 {
-    if (c.prec == GKS_FP64 && c.fp64_ds && !c.gp_dir[0])
-        stage == 1 ? stage_impl<double, dsf, 1>(c) : stage_impl<double, dsf, 2>(c);
+    if (c.prec == GKS_FP64 && c.gp_dir[0])
+        stage == 1 ? stage_impl<double, double, 1, true>(c) : stage_impl<double, double, 2, true>(c);
+    else if (c.prec == GKS_FP64 && c.fp64_ds)
+        stage == 1 ? stage_impl<double, dsf, 1, false>(c) : stage_impl<double, dsf, 2, false>(c);
     else if (c.prec == GKS_FP64)
-        stage == 1 ? stage_impl<double, double, 1>(c) : stage_impl<double, double, 2>(c);
+        stage == 1 ? stage_impl<double, double, 1, false>(c) : stage_impl<double, double, 2, false>(c);
     else
-        stage == 1 ? stage_impl<float, float, 1>(c) : stage_impl<float, float, 2>(c);
+        stage == 1 ? stage_impl<float, float, 1, false>(c) : stage_impl<float, float, 2, false>(c);
 }
 
 void launch_cfl(const Ctx &c)

@@ -170,3 +170,20 @@ def test_body_box_larger_than_one_pass(gks, precision):
     assert rel_linf(a["force"], np.asarray(b["force"])) <= 10 * TOL[precision]
     assert a["iters"] == 2 and abs(a["residual"] - b["residual"]) <= 10 * TOL[precision]
     g.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32c", "fp64"])
+def test_small_and_large_launch_paths_give_the_same_bits(gks, precision):
+    # 96 x 80 x 80 runs one direction after the other (FP32C: z faces fused
+    # with the update), its thirds run all directions in one launch
+    n = (96, 80, 80)
+    w = smooth_workload(n, [(3, 4), (0, 0), (2, 1)], seed=11)
+    w.inflow = (1.0, 0.3, 0.0, 0.0)
+    w.body_force = (0.01, 0.0, 0.0)
+    g = grid(gks, w, precision)
+    t = g.step(3)
+    s = gks.SlabGroup(w, [32, 64], precision=precision)
+    assert s.step(3) == t
+    assert np.array_equal(g.get_state(), s.get_state())
+    g.close()
+    s.close()
