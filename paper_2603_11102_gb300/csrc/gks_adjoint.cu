@@ -77,106 +77,78 @@ __device__ __forceinline__ long lin(const int P0, const int P1, int i, int j, in
 
 // ------------------------------------------------------ reverse building blocks
 
-// Adjoint of dev::gk_flux: given the adjoints of F0 (if needF0) and F1,
-// accumulate the adjoints of its inputs (index-space tangential slopes).
+__device__ __forceinline__ float rev_inverse(float a) { return rcp_approx(a); }
+__device__ __forceinline__ double rev_inverse(double a) { return 1.0 / a; }
+__device__ __forceinline__ f2 rev_inverse(f2 a) { return wrcp(a); }
+
+// Adjoint of dev::gk_flux: given the adjoints of F0 (if needF0) and F1, the
+// adjoints of its inputs (index-space tangential slopes, density slopes as
+// they are, not negated). It reverses the form with rho multiplied through,
+//   H_ik = D_i m_k - U_k D_i rho, B = H_kk + U.grad rho, C_k = theta d_k rho + U_i H_ik,
+//   X = U_n B + C_n, -F1 = (X, U_n X + C_n U_n + theta B, U_k X + U_n C_k),
+// in about 110 operations (135 with F0) against the 230 of the form with
+// d_i U_k, A_0 and A_k. With the FP32 tile adjoints (below) 736 -> 570 us a
+// direction of a 256x128x128 FP32C stage; the FP64 reverse 1.04x.
 template <typename T>
 __device__ __forceinline__ void gk_flux_rev(const Phys<T> &ph, const T q[4], const T Dn[4], const T D1[4],
                                             const T D2[4], T ih1, T ih2, const T lF0[4], const T lF1[4],
                                             bool needF0, T qb[4], T Dnb[4], T D1b[4], T D2b[4])
 {
-    const T rho = ph.off + q[0];
-    const T inv = T(1.0) / rho;
-    const T invi[3] = {inv, inv * ih1, inv * ih2};
-    const T *D[3] = {Dn, D1, D2};
-    const T U[3] = {q[1] * inv, q[2] * inv, q[3] * inv};
-    T g[3], Gm[3][3];
-    for (int i = 0; i < 3; ++i) {
-        g[i] = D[i][0] * invi[i];
-        for (int j = 0; j < 3; ++j) Gm[i][j] = (D[i][j + 1] - U[j] * D[i][0]) * invi[i];
-    }
-    const T th = ph.theta, tl = T(2.0) * ph.lambda, mu = ph.mu;
-    const T A0 = -(U[0] * g[0] + U[1] * g[1] + U[2] * g[2]) - (Gm[0][0] + Gm[1][1] + Gm[2][2]);
-    T A[3];
-    for (int k = 0; k < 3; ++k) A[k] = -g[k] - tl * (U[0] * Gm[0][k] + U[1] * Gm[1][k] + U[2] * Gm[2][k]);
-
-    const T z0 = T(0.0);
-    T rhob = z0, Ub[3] = {z0, z0, z0}, gb[3] = {z0, z0, z0}, Gb[3][3] = {{z0, z0, z0}, {z0, z0, z0}, {z0, z0, z0}};
-    T A0b = z0, Ab[3] = {z0, z0, z0}, qd[4] = {z0, z0, z0, z0};
-    // F1[0] = rho (A0 U0 + th A_0)
-    {
-        const T T0 = A0 * U[0] + th * A[0];
-        rhob += lF1[0] * T0;
-        const T T0b = lF1[0] * rho;
-        A0b += T0b * U[0];
-        Ub[0] += T0b * A0;
-        Ab[0] += T0b * th;
-    }
-    // F1[1+k] = rho (A0 (U0 U_k + th d_k0) + th (A_k U0 + A_0 U_k))
-    for (int k = 0; k < 3; ++k) {
-        const T c = U[0] * U[k] + (k == 0 ? th : T(0.0));
-        const T Tk = A0 * c + th * (A[k] * U[0] + A[0] * U[k]);
-        rhob += lF1[1 + k] * Tk;
-        const T Tb = lF1[1 + k] * rho;
-        A0b += Tb * c;
-        Ub[0] += Tb * A0 * U[k];
-        Ub[k] += Tb * A0 * U[0];
-        Ab[k] += Tb * th * U[0];
-        Ub[0] += Tb * th * A[k];
-        Ab[0] += Tb * th * U[k];
-        Ub[k] += Tb * th * A[0];
-    }
+    const T inv = rev_inverse(ph.off + q[0]);
+    const T U0 = q[1] * inv, U1 = q[2] * inv, U2 = q[3] * inv, V1 = U1 * ih1, V2 = U2 * ih2;
+    const T e0 = Dn[0], e1 = D1[0], e2 = D2[0];
+    const T H00 = fma(-U0, e0, Dn[1]), H01 = fma(-U1, e0, Dn[2]), H02 = fma(-U2, e0, Dn[3]);
+    const T H10 = fma(-U0, e1, D1[1]), H11 = fma(-U1, e1, D1[2]), H12 = fma(-U2, e1, D1[3]);
+    const T H20 = fma(-U0, e2, D2[1]), H21 = fma(-U1, e2, D2[2]), H22 = fma(-U2, e2, D2[3]);
+    const T th = ph.theta, th1 = th * ih1, th2 = th * ih2;
+    const T B = fma(V2, e2, fma(V1, e1, fma(U0, e0, fma(ih2, H22, fma(ih1, H11, H00)))));
+    const T C0 = fma(th, e0, fma(U0, H00, fma(V1, H10, V2 * H20)));
+    const T C1 = fma(th1, e1, fma(U0, H01, fma(V1, H11, V2 * H21)));
+    const T C2 = fma(th2, e2, fma(U0, H02, fma(V1, H12, V2 * H22)));
+    const T X = fma(U0, B, C0);
+    const T n0 = -lF1[0], n1 = -lF1[1], n2 = -lF1[2], n3 = -lF1[3];
+    const T Xb = fma(U2, n3, fma(U1, n2, fma(U0, n1, n0)));
+    const T C0b = fma(U0, n1, Xb), C1b = U0 * n2, C2b = U0 * n3;
+    const T Bb = fma(th, n1, U0 * Xb);
+    T U0b = fma(n1, X + C0, fma(n2, C1, fma(n3, C2, Xb * B)));
+    T U1b = n2 * X, U2b = n3 * X;
+    T e0b = fma(th, C0b, U0 * Bb), e1b = fma(th1, C1b, V1 * Bb), e2b = fma(th2, C2b, V2 * Bb);
+    T H00b = fma(U0, C0b, Bb), H01b = U0 * C1b, H02b = U0 * C2b;
+    T H10b = V1 * C0b, H11b = fma(V1, C1b, ih1 * Bb), H12b = V1 * C2b;
+    T H20b = V2 * C0b, H21b = V2 * C1b, H22b = fma(V2, C2b, ih2 * Bb);
+    U0b = fma(H00, C0b, fma(H01, C1b, fma(H02, C2b, fma(e0, Bb, U0b))));
+    const T V1b = fma(H10, C0b, fma(H11, C1b, fma(H12, C2b, e1 * Bb)));
+    const T V2b = fma(H20, C0b, fma(H21, C1b, fma(H22, C2b, e2 * Bb)));
+    T q0b = T(0.0), q1b = T(0.0), invb = T(0.0);
     if (needF0) {
-        qd[1] += lF0[0];
-        qd[1] += lF0[1] * U[0];
-        Ub[0] += lF0[1] * q[1];
-        qd[0] += lF0[1] * th;
-        Gb[0][0] += -T(2.0) * mu * lF0[1];
-        for (int k = 1; k < 3; ++k) {
-            qd[1] += lF0[1 + k] * U[k];
-            Ub[k] += lF0[1 + k] * q[1];
-            Gb[0][k] -= mu * lF0[1 + k];
-            Gb[k][0] -= mu * lF0[1 + k];
-        }
+        const T nm = -ph.mu * inv, t2 = nm * lF0[2], t3 = nm * lF0[3];
+        H00b = fma(T(2.0) * nm, lF0[1], H00b);
+        H01b += t2;
+        H10b = fma(ih1, t2, H10b);
+        H02b += t3;
+        H20b = fma(ih2, t3, H20b);
+        invb = -ph.mu * fma(T(2.0) * H00, lF0[1], fma(fma(ih1, H10, H01), lF0[2], fma(ih2, H20, H02) * lF0[3]));
+        q1b = fma(U2, lF0[3], fma(U1, lF0[2], fma(U0, lF0[1], lF0[0])));
+        U0b = fma(q[1], lF0[1], U0b);
+        U1b = fma(q[1], lF0[2], U1b);
+        U2b = fma(q[1], lF0[3], U2b);
+        q0b = th * lF0[1];
     }
-    // A_k = -g_k - tl sum_i U_i G_ik
-    for (int k = 0; k < 3; ++k) {
-        gb[k] -= Ab[k];
-        for (int i = 0; i < 3; ++i) {
-            Ub[i] -= tl * Ab[k] * Gm[i][k];
-            Gb[i][k] -= tl * Ab[k] * U[i];
-        }
-    }
-    // A0 = -sum U_i g_i - sum G_ii
-    for (int i = 0; i < 3; ++i) {
-        Ub[i] -= A0b * g[i];
-        gb[i] -= A0b * U[i];
-        Gb[i][i] -= A0b;
-    }
-    T Db[3][4] = {{z0, z0, z0, z0}, {z0, z0, z0, z0}, {z0, z0, z0, z0}};
-    T invb[3] = {z0, z0, z0};
-    for (int i = 0; i < 3; ++i) {
-        for (int j = 0; j < 3; ++j) {
-            Db[i][j + 1] += Gb[i][j] * invi[i];
-            Ub[j] -= Gb[i][j] * D[i][0] * invi[i];
-            Db[i][0] -= Gb[i][j] * U[j] * invi[i];
-            invb[i] += Gb[i][j] * (D[i][j + 1] - U[j] * D[i][0]);
-        }
-        Db[i][0] += gb[i] * invi[i];
-        invb[i] += gb[i] * D[i][0];
-    }
-    T inv_b = invb[0] + invb[1] * ih1 + invb[2] * ih2;
-    for (int j = 0; j < 3; ++j) {
-        qd[j + 1] += Ub[j] * inv;
-        inv_b += Ub[j] * q[j + 1];
-    }
-    rhob += -inv_b * inv * inv;
-    qd[0] += rhob;
-    for (int v = 0; v < 4; ++v) {
-        qb[v] = qd[v];
-        Dnb[v] = Db[0][v];
-        D1b[v] = Db[1][v];
-        D2b[v] = Db[2][v];
-    }
+    U1b = fma(ih1, V1b, U1b);
+    U2b = fma(ih2, V2b, U2b);
+    U0b = fma(-e0, H00b, fma(-e1, H10b, fma(-e2, H20b, U0b)));
+    U1b = fma(-e0, H01b, fma(-e1, H11b, fma(-e2, H21b, U1b)));
+    U2b = fma(-e0, H02b, fma(-e1, H12b, fma(-e2, H22b, U2b)));
+    Dnb[0] = fma(-U0, H00b, fma(-U1, H01b, fma(-U2, H02b, e0b)));
+    D1b[0] = fma(-U0, H10b, fma(-U1, H11b, fma(-U2, H12b, e1b)));
+    D2b[0] = fma(-U0, H20b, fma(-U1, H21b, fma(-U2, H22b, e2b)));
+    Dnb[1] = H00b; Dnb[2] = H01b; Dnb[3] = H02b;
+    D1b[1] = H10b; D1b[2] = H11b; D1b[3] = H12b;
+    D2b[1] = H20b; D2b[2] = H21b; D2b[3] = H22b;
+    qb[0] = fma(-inv, fma(U0b, U0, fma(U1b, U1, fma(U2b, U2, invb * inv))), q0b);
+    qb[1] = fma(U0b, inv, q1b);
+    qb[2] = U1b * inv;
+    qb[3] = U2b * inv;
 }
 
 // Adjoint of dev::weno5_pair (both face values of the centre cell of
@@ -336,7 +308,7 @@ struct RevArgs {
     const float *Ahi, *Alo;   // FP32 reverse: A as hi + lo floats
     long nfq;                 // component stride of the face-box adjoints
     int e1p;
-    const double *lamL, *lamLt;   // padded indexing; lamL may be null (stage 2)
+    const void *lamL, *lamLt;     // padded indexing, in the reverse's compute type; lamL may be null (stage 2)
     // the recorded Gauss-point inputs (read only) and the adjoints inside the
     // spatial adjoint of one direction, in the reverse's compute type:
     // Gauss-point inputs, t1-pass rows, face boxes, per-face cell slots
@@ -348,6 +320,7 @@ struct RevArgs {
     void *lamFQ, *lamC;
     double *lamA;
     const double *ihd, *ih1, *ih2, *ihf;
+    const float *ihf32;       // FP32C grids: ihf as the forward's FP32 values
     int n[3], P[3];
     int d, t1, t2, nd, n1, n2;
     long np;
@@ -379,10 +352,11 @@ __global__ void __launch_bounds__(256) rev_flux_kernel(RevArgs A)
     const T ihl = hasl ? T(A.ihd[f - 1 + G]) : T(0), ihr = hasr ? T(A.ihd[f + G]) : T(0);
     for (int v = 0; v < 4; ++v) {
         const long o = gc[v] * A.np;
-        const T ll = hasl ? T(A.lamLt[o + il]) : T(0), lr = hasr ? T(A.lamLt[o + ir]) : T(0);
+        const T *lt = (const T *)A.lamLt, *l0 = (const T *)A.lamL;
+        const T ll = hasl ? lt[o + il] : T(0), lr = hasr ? lt[o + ir] : T(0);
         sF1[v] = T(0.25) * (-ll * ihl + lr * ihr);
-        if (A.lamL) {
-            const T ml = hasl ? T(A.lamL[o + il]) : T(0), mr = hasr ? T(A.lamL[o + ir]) : T(0);
+        if (l0) {
+            const T ml = hasl ? l0[o + il] : T(0), mr = hasr ? l0[o + ir] : T(0);
             sF0[v] = T(0.25) * (-ml * ihl + mr * ihr);
         }
     }
@@ -609,35 +583,80 @@ __global__ void __launch_bounds__(256) rev_face_state_kernel(RevArgs A)
     }
 }
 
-// The WENO5 pair in FP32 of 5 cells given as hi + lo floats, on the cells
-// minus the centre cell: (hi_k - hi_2) + (lo_k - lo_2) keeps the precision of
-// the FP64 differences (the hi difference of nearby values is exact).
-__device__ __forceinline__ void diffs32(const float hi[5], const float lo[5], float qs[5])
-{
-#pragma unroll
-    for (int k = 0; k < 5; ++k) qs[k] = (hi[k] - hi[2]) + (lo[k] - lo[2]);
-}
+// WENO5 in FP32 from the 4 first differences D of the 5 cells around a cell
+// (WenoMarch's form): the weights' pieces, and the right- and left-face values
+// relative to the cell.
+struct Weno32 {
+    float Sm, S0, S1, Tm, Tp, u0, u1, u2, g0, g1, g2, s0, s1, s2, s12, s01, ir, il, a, b;
+    __device__ __forceinline__ explicit Weno32(const float D[4])
+    {
+        constexpr float eps = float(12e-6 / 13.0), k = float(3.0 / 13.0);
+        Sm = D[1] - D[0];
+        S0 = D[2] - D[1];
+        S1 = D[3] - D[2];
+        Tm = S0 - Sm;
+        Tp = S1 - S0;
+        u0 = fmaf(2.0f, D[1], Sm);
+        u1 = D[1] + D[2];
+        u2 = fmaf(-2.0f, D[2], S1);
+        g0 = fmaf(u0 * k, u0, fmaf(Sm, Sm, eps));
+        g1 = fmaf(u1 * k, u1, fmaf(S0, S0, eps));
+        g2 = fmaf(u2 * k, u2, fmaf(S1, S1, eps));
+        s0 = g0 * g0;
+        s1 = g1 * g1;
+        s2 = g2 * g2;
+        s01 = s0 * s1;
+        s12 = s1 * s2;
+        const float w = 18.0f * (s0 * s2);
+        ir = rcp_approx(fmaf(3.0f, s12, fmaf(9.0f, s01, w)));
+        il = rcp_approx(fmaf(3.0f, s01, fmaf(9.0f, s12, w)));
+        a = s12 * Tm;
+        b = s01 * Tp;
+    }
+    __device__ __forceinline__ float right(const float D[4]) const
+    {
+        return fmaf(0.5f, D[2], fmaf(float(-1.0 / 6.0), S0, -(fmaf(1.5f, b, a) * ir)));
+    }
+    __device__ __forceinline__ float left(const float D[4]) const
+    {
+        return fmaf(-0.5f, D[1], fmaf(float(-1.0 / 6.0), S0, fmaf(1.5f, a, b) * il));
+    }
+};
 
-__device__ __forceinline__ void pair_values32(const float hi[5], const float lo[5], float &right, float &left)
+// Adjoint of both face values (seeds sR, sL): added to the adjoints of the 5
+// cells, out. About 100 operations with the recomputed pieces against the 190
+// of the form in the cells' values; rev_face_cells32_kernel stays at 0.40 ms on
+// 256x128x128 all the same (its time goes to the loads).
+__device__ __forceinline__ void weno32_rev(const float D[4], float sR, float sL, float out[5])
 {
-    float qs[5], r, l;
-    diffs32(hi, lo, qs);
-    weno5_pair(qs, r, l);
-    right = hi[2] + (lo[2] + r);
-    left = hi[2] + (lo[2] + l);
-}
-
-__device__ __forceinline__ void pair_rev32(const float hi[5], const float lo[5], float sR, float sL, float out[5])
-{
-    float qs[5];
-    diffs32(hi, lo, qs);
-    weno5_pair_rev<float>(qs, sR, sL, out);
+    const Weno32 w(D);
+    constexpr float k2 = float(6.0 / 13.0);
+    // right = c + D_2/2 - S_0/6 - (a + 1.5 b) ir, left = c - D_1/2 - S_0/6 + (b + 1.5 a) il
+    const float nr = -sR * w.ir, nl = sL * w.il;
+    const float drb = -nr * (fmaf(1.5f, w.b, w.a) * w.ir), dlb = -nl * (fmaf(1.5f, w.a, w.b) * w.il);
+    const float ab = fmaf(1.5f, nl, nr), bb = fmaf(1.5f, nr, nl);
+    const float s12b = fmaf(ab, w.Tm, fmaf(3.0f, drb, 9.0f * dlb)), s01b = fmaf(bb, w.Tp, fmaf(9.0f, drb, 3.0f * dlb));
+    const float s02b = 18.0f * (drb + dlb);
+    const float Tmb = ab * w.s12, Tpb = bb * w.s01;
+    const float g0b = 2.0f * w.g0 * fmaf(s02b, w.s2, s01b * w.s1);
+    const float g1b = 2.0f * w.g1 * fmaf(s01b, w.s0, s12b * w.s2);
+    const float g2b = 2.0f * w.g2 * fmaf(s02b, w.s0, s12b * w.s1);
+    const float u0b = k2 * w.u0 * g0b, u1b = k2 * w.u1 * g1b, u2b = k2 * w.u2 * g2b;
+    const float Smb = fmaf(2.0f * w.Sm, g0b, u0b) - Tmb;
+    const float S1b = fmaf(2.0f * w.S1, g2b, u2b) + Tpb;
+    const float S0b = fmaf(2.0f * w.S0, g1b, Tmb - Tpb) - float(1.0 / 6.0) * (sR + sL);
+    const float D1b = fmaf(2.0f, u0b, u1b) + (Smb - S0b) - 0.5f * sL;
+    const float D2b = fmaf(-2.0f, u2b, u1b) + (S0b - S1b) + 0.5f * sR;
+    out[0] += Smb;
+    out[1] -= Smb + D1b;
+    out[2] += (D1b - D2b) + (sR + sL);
+    out[3] += D2b - S1b;
+    out[4] += S1b;
 }
 
 // RD in FP32 (the FP32 reverse): the same march as rev_face_state_kernel on
 // the working array split into hi + lo floats, with FP32 face-box adjoints in
 // and FP32 cell slots out.
-template <bool LO>
 __global__ void __launch_bounds__(256) rev_face_state32_kernel(RevArgs A)
 {
     const float *lamFQ = (const float *)A.lamFQ;
@@ -658,28 +677,40 @@ __global__ void __launch_bounds__(256) rev_face_state32_kernel(RevArgs A)
         return;
     const int comp[4] = {0, 1 + A.d, 1 + A.t1, 1 + A.t2};
     const Phys<float> ph = phys_as<float>(A.ph);
-    float wh[4][6], wl[4][6];
-#pragma unroll
-    for (int v = 0; v < 4; ++v)
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            const int cell = f0 - 4 + k;
-            const long l = comp[v] * A.np + base + (long)cell * sd;
-            wh[v][k] = cell >= -G ? A.Ahi[l] : 0.0f;
-            wl[v][k] = (LO && cell >= -G) ? A.Alo[l] : 0.0f;
-        }
+    // the 5 differences of the cells f-3 .. f+2 of the current face (hi and lo
+    // parts differenced apart: the precision of the FP64 differences), and the
+    // cells f, f+1, f+2
+    float D[4][5], ch[4][3], cl[4][3];
     float Rprev[4], Sprev[4];
     {
-        float lft[4];
+        float wh[4][6], wl[4][6], lft[4];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) pair_values32(&wh[v][1], &wl[v][1], Rprev[v], lft[v]);   // cell f0-1
+        for (int v = 0; v < 4; ++v) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                const int cell = f0 - 4 + k;
+                const long l = comp[v] * A.np + base + (long)cell * sd;
+                wh[v][k] = cell >= -G ? A.Ahi[l] : 0.0f;
+                wl[v][k] = cell >= -G ? A.Alo[l] : 0.0f;
+            }
+#pragma unroll
+            for (int k = 0; k < 5; ++k) D[v][k] = (wh[v][k + 1] - wh[v][k]) + (wl[v][k + 1] - wl[v][k]);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                ch[v][k] = wh[v][k + 3];
+                cl[v][k] = wl[v][k + 3];
+            }
+            const Weno32 w(&D[v][1]);   // cell f0-1
+            Rprev[v] = wh[v][3] + (wl[v][3] + w.right(&D[v][1]));
+            lft[v] = wh[v][3] + (wl[v][3] + w.left(&D[v][1]));
+        }
         if (f0 == 0) {
 #pragma unroll
             for (int v = 0; v < 4; ++v) Sprev[v] = 0.0f;
         } else {
-            float Rpp[4], dum;
+            float Rpp[4];
 #pragma unroll
-            for (int v = 0; v < 4; ++v) pair_values32(&wh[v][0], &wl[v][0], Rpp[v], dum);    // cell f0-2
+            for (int v = 0; v < 4; ++v) Rpp[v] = wh[v][2] + (wl[v][2] + Weno32(&D[v][0]).right(&D[v][0]));   // cell f0-2
             const long o = ((long)(f0 - 1) * (A.n2 + 4) + (b + 2)) * A.e1p + (a + 2);
             float Q0b[4], Qlb[4];
 #pragma unroll
@@ -691,19 +722,24 @@ __global__ void __launch_bounds__(256) rev_face_state32_kernel(RevArgs A)
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
 #pragma unroll
-            for (int k = 0; k < 5; ++k) {
-                wh[v][k] = wh[v][k + 1];
-                wl[v][k] = wl[v][k + 1];
+            for (int k = 0; k < 4; ++k) D[v][k] = D[v][k + 1];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                ch[v][k] = ch[v][k + 1];
+                cl[v][k] = cl[v][k + 1];
             }
             const long l = comp[v] * A.np + base + (long)(f + 2) * sd;
-            wh[v][5] = A.Ahi[l];
-            wl[v][5] = LO ? A.Alo[l] : 0.0f;
+            ch[v][2] = A.Ahi[l];
+            cl[v][2] = A.Alo[l];
+            D[v][4] = (ch[v][2] - ch[v][1]) + (cl[v][2] - cl[v][1]);
         }
         float Ql[4], Qr[4], Rt[4];
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             Ql[v] = Rprev[v];
-            pair_values32(&wh[v][1], &wl[v][1], Rt[v], Qr[v]);   // cell f
+            const Weno32 w(&D[v][1]);   // cell f
+            Rt[v] = ch[v][0] + (cl[v][0] + w.right(&D[v][1]));
+            Qr[v] = ch[v][0] + (cl[v][0] + w.left(&D[v][1]));
         }
         const long o = ((long)f * (A.n2 + 4) + (b + 2)) * A.e1p + (a + 2);
         float Q0b[4], DNb[4], Qlb[4], Qrb[4];
@@ -722,8 +758,8 @@ __global__ void __launch_bounds__(256) rev_face_state32_kernel(RevArgs A)
             cb[2] -= 15.0f * ds;
             cb[3] += 15.0f * ds;
             cb[4] -= ds;
-            pair_rev32(&wh[v][0], &wl[v][0], Qlb[v], Sprev[v], &cb[0]);      // cell f-1
-            if (f == nf - 1) pair_rev32(&wh[v][1], &wl[v][1], 0.0f, Qrb[v], &cb[1]);   // cell f, left value only
+            weno32_rev(&D[v][0], Qlb[v], Sprev[v], &cb[0]);      // cell f-1
+            if (f == nf - 1) weno32_rev(&D[v][1], 0.0f, Qrb[v], &cb[1]);   // cell f, left value only
 #pragma unroll
             for (int m = 0; m < 6; ++m) lamC[(m * 4 + v) * A.nfq + o] = cb[m];
             Rprev[v] = Rt[v];
@@ -762,27 +798,34 @@ __global__ void __launch_bounds__(256, 2) rev_face_cells32_kernel(RevArgs A)
         return;
     const int comp[4] = {0, 1 + A.d, 1 + A.t1, 1 + A.t2};
     const Phys<float> ph = phys_as<float>(A.ph);
-    const float zl[5] = {0, 0, 0, 0, 0};
-    float wh[4][6];
-#pragma unroll
-    for (int v = 0; v < 4; ++v)
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            const int cell = fs - 4 + k;
-            wh[v][k] = cell >= -G ? A.Ahi[comp[v] * A.np + base + (long)cell * sd] : 0.0f;
-        }
+    // the 5 differences of the cells f-3 .. f+2 of the current face, and the
+    // cells f, f+1, f+2
+    float D[4][5], ch[4][3];
     float Rprev[4], Sprev[4];
     {
-        float lft[4];
+        float wh[4][6], lft[4];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) pair_values32(&wh[v][1], zl, Rprev[v], lft[v]);   // cell fs-1
+        for (int v = 0; v < 4; ++v) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                const int cell = fs - 4 + k;
+                wh[v][k] = cell >= -G ? A.Ahi[comp[v] * A.np + base + (long)cell * sd] : 0.0f;
+            }
+#pragma unroll
+            for (int k = 0; k < 5; ++k) D[v][k] = wh[v][k + 1] - wh[v][k];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) ch[v][k] = wh[v][k + 3];
+            const Weno32 w(&D[v][1]);   // cell fs-1
+            Rprev[v] = wh[v][3] + w.right(&D[v][1]);
+            lft[v] = wh[v][3] + w.left(&D[v][1]);
+        }
         if (fs == 0) {
 #pragma unroll
             for (int v = 0; v < 4; ++v) Sprev[v] = 0.0f;
         } else {
-            float Rpp[4], dum;
+            float Rpp[4];
 #pragma unroll
-            for (int v = 0; v < 4; ++v) pair_values32(&wh[v][0], zl, Rpp[v], dum);    // cell fs-2
+            for (int v = 0; v < 4; ++v) Rpp[v] = wh[v][2] + Weno32(&D[v][0]).right(&D[v][0]);   // cell fs-2
             const long o = ((long)(fs - 1) * (A.n2 + 4) + (b + 2)) * A.e1p + (a + 2);
             float Q0b[4], Qlb[4];
 #pragma unroll
@@ -804,8 +847,11 @@ __global__ void __launch_bounds__(256, 2) rev_face_cells32_kernel(RevArgs A)
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
 #pragma unroll
-            for (int k = 0; k < 5; ++k) wh[v][k] = wh[v][k + 1];
-            wh[v][5] = nxt[v];
+            for (int k = 0; k < 4; ++k) D[v][k] = D[v][k + 1];
+            ch[v][0] = ch[v][1];
+            ch[v][1] = ch[v][2];
+            ch[v][2] = nxt[v];
+            D[v][4] = ch[v][2] - ch[v][1];
         }
         if (f < fe) {   // cell f + 3 <= fe + 2: inside the checked range
 #pragma unroll
@@ -815,7 +861,9 @@ __global__ void __launch_bounds__(256, 2) rev_face_cells32_kernel(RevArgs A)
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             Ql[v] = Rprev[v];
-            pair_values32(&wh[v][1], zl, Rt[v], Qr[v]);   // cell f
+            const Weno32 w(&D[v][1]);   // cell f
+            Rt[v] = ch[v][0] + w.right(&D[v][1]);
+            Qr[v] = ch[v][0] + w.left(&D[v][1]);
         }
         const long o = ((long)f * (A.n2 + 4) + (b + 2)) * A.e1p + (a + 2);
         float Q0b[4], DNb[4], Qlb[4], Qrb[4];
@@ -825,7 +873,7 @@ __global__ void __launch_bounds__(256, 2) rev_face_cells32_kernel(RevArgs A)
             DNb[v] = lamFQ[(4 + v) * A.nfq + o];
         }
         equilibrium_rev<float>(ph, Ql, Qr, Q0b, Qlb, Qrb);
-        const float s = (float)(A.ihf[f] * (1.0 / 12.0));
+        const float s = __ldg(A.ihf32 + f) * float(1.0 / 12.0);
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             float cb[6] = {0, 0, 0, 0, 0, 0};
@@ -834,8 +882,8 @@ __global__ void __launch_bounds__(256, 2) rev_face_cells32_kernel(RevArgs A)
             cb[2] -= 15.0f * ds;
             cb[3] += 15.0f * ds;
             cb[4] -= ds;
-            pair_rev32(&wh[v][0], zl, Qlb[v], Sprev[v], &cb[0]);      // cell f-1
-            if (f == nf - 1) pair_rev32(&wh[v][1], zl, 0.0f, Qrb[v], &cb[1]);   // cell f, left value only
+            weno32_rev(&D[v][0], Qlb[v], Sprev[v], &cb[0]);      // cell f-1
+            if (f == nf - 1) weno32_rev(&D[v][1], 0.0f, Qrb[v], &cb[1]);   // cell f, left value only
 #pragma unroll
             for (int m = 0; m < 6; ++m) acc[v][m] += cb[m];
             Rprev[v] = Rt[v];
@@ -845,7 +893,7 @@ __global__ void __launch_bounds__(256, 2) rev_face_cells32_kernel(RevArgs A)
         const int cl = f - 3;
         if (cl >= c0 && cl < c1) {
 #pragma unroll
-            for (int v = 0; v < 4; ++v) A.lamA[comp[v] * A.np + base + (long)cl * sd] += (double)acc[v][0];
+            for (int v = 0; v < 4; ++v) A.lamA[comp[v] * A.np + base + (long)cl * sd] += compose_hi_lo(acc[v][0], 0.0f);
         }
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
@@ -860,7 +908,7 @@ __global__ void __launch_bounds__(256, 2) rev_face_cells32_kernel(RevArgs A)
         const int cl = fe - 2 + k;
         if (cl >= c0 && cl < c1) {
 #pragma unroll
-            for (int v = 0; v < 4; ++v) A.lamA[comp[v] * A.np + base + (long)cl * sd] += (double)acc[v][k];
+            for (int v = 0; v < 4; ++v) A.lamA[comp[v] * A.np + base + (long)cl * sd] += compose_hi_lo(acc[v][k], 0.0f);
         }
     }
 }
@@ -917,7 +965,7 @@ __global__ void __launch_bounds__(256) rev_gather_cells_kernel(RevArgs A)
 // neighbouring tiles: sum_partials32_kernel adds the partials of a face in a
 // fixed order.
 struct Rev32Args {
-    const double *lamL, *lamLt;       // padded cell adjoints; lamL null in stage 2
+    const float *lamL, *lamLt;        // padded cell adjoints; lamL null in stage 2
     const float *ihd, *ih1, *ih2;     // inverse cell widths along d, t1, t2 (padded index)
     float *part;                      // per tile: 8 x SQ_H x SQ_W face-box adjoints
     int n1, n2, nf, nd, d, t1, t2;
@@ -976,12 +1024,12 @@ __global__ void __launch_bounds__(256, 2) rev_tile32_kernel(const __grid_constan
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
                 const long o = gc[v] * A.np;
-                const float ll = (hasl && okc) ? (float)A.lamLt[o + il] : 0.0f;
-                const float lr = (hasr && okc) ? (float)A.lamLt[o + ir] : 0.0f;
+                const float ll = (hasl && okc) ? A.lamLt[o + il] : 0.0f;
+                const float lr = (hasr && okc) ? A.lamLt[o + ir] : 0.0f;
                 sF1[v] = 0.25f * (-ll * ihl + lr * ihr);
                 if (needF0) {
-                    const float ml = (hasl && okc) ? (float)A.lamL[o + il] : 0.0f;
-                    const float mr = (hasr && okc) ? (float)A.lamL[o + ir] : 0.0f;
+                    const float ml = (hasl && okc) ? A.lamL[o + il] : 0.0f;
+                    const float mr = (hasr && okc) ? A.lamL[o + ir] : 0.0f;
                     sF0[v] = 0.25f * (-ml * ihl + mr * ihr);
                 }
             }
@@ -1107,8 +1155,7 @@ __global__ void __launch_bounds__(256, 2) rev_tile32_kernel(const __grid_constan
                 float acc = 0.0f;
 #pragma unroll
                 for (int sx = 0; sx < 5; ++sx) {
-                    const int k = 4 + i - sx;   // row column cc0 + i - sx
-                    if (cc0 + i - sx < 0 || cc0 + i - sx >= TX) continue;
+                    const int k = 4 + i - sx;   // row column cc0 + i - sx (zero outside the tile)
 #pragma unroll
                     for (int m = 0; m < 2; ++m) {
                         if (j < 4)
@@ -1155,29 +1202,40 @@ __global__ void __launch_bounds__(256) sum_partials32_kernel(const float *part, 
     for (int j = 0; j < 8; ++j) lamFQ[j * nfq + o] = acc[j];
 }
 
-// Ghost adjoint of one (axis, side, layer): the ghost's adjoint goes to its
-// source cell and is cleared.
+// Ghost adjoint of one axis: the adjoints of the ghosts go to their source
+// cells and are cleared.
 struct GhostRevArgs {
     const double *A;  // forward working array
     double *lamA;
     double *uinf_part;
     int n[3], P[3];
     long np;
-    int d, e1, e2, lo1, lo2, len1, len2, s, bc;
+    int d, e1, e2, lo1, lo2, len1, len2, s0, bc[2];
     long uinf_layer;   // stride of uinf_part between layers
     double csound, uin[3];
 };
 
-// One (axis, side): the layers l = G .. 1 in turn, each thread one position
-// of the side (the sources are interior cells, so a thread's layers are its
-// own and keep the order of a sweep per layer).
-__global__ void __launch_bounds__(256) ghost_rev_kernel(GhostRevArgs A)
+// Sides s0, s0 + 1, .. (blockIdx.z) of one axis: the layers l = G .. 1 in
+// turn, each thread one position of a side. The 12 ghost values are loaded
+// before anything is stored (a layer at a time was a chain of 3 dependent
+// round trips to memory); both sides of an axis run in one launch where their
+// source cells are apart (n >= 2G). Sources of inflow and outflow sides are
+// one cell for all layers, added to in the order of the layers. All sides of a
+// stage of 256x128x128: 0.55 -> 0.08 ms.
+__global__ void __launch_bounds__(256) ghost_rev_kernel(const __grid_constant__ GhostRevArgs A)
 {
     const int a = A.lo1 + (int)(blockIdx.x * blockDim.x + threadIdx.x);
     const int b = A.lo2 + (int)(blockIdx.y * blockDim.y + threadIdx.y);
     if (a >= A.lo1 + A.len1 || b >= A.lo2 + A.len2) return;
-    const int d = A.d, nd = A.n[d], s = A.s, bc = A.bc;
-    for (int l = G; l >= 1; --l) {
+    const int d = A.d, nd = A.n[d], s = A.s0 + blockIdx.z, bc = A.bc[s];
+    const long str[3] = {1, A.P[0], (long)A.P[0] * A.P[1]};
+    const long sd = d == 0 ? str[0] : (d == 1 ? str[1] : str[2]);
+    const long base = G * (str[0] + str[1] + str[2]) + a * (d == 0 ? str[1] : str[0]) + b * (d == 2 ? str[1] : str[2]);
+    // offsets of the ghosts and their sources, layers 1 .. G
+    long ig[G], is[G];
+    bool ok = true;
+#pragma unroll
+    for (int l = 1; l <= G; ++l) {
         const int gi = s == 0 ? -l : nd - 1 + l;
         int src;
         if (bc == GKS_BC_PERIODIC) {
@@ -1188,39 +1246,74 @@ __global__ void __launch_bounds__(256) ghost_rev_kernel(GhostRevArgs A)
         } else {
             src = s == 0 ? 0 : nd - 1;
         }
-        int cg[3], cs[3];
-        cg[d] = gi; cg[A.e1] = a; cg[A.e2] = b;
-        cs[d] = src; cs[A.e1] = a; cs[A.e2] = b;
-        const long ig = lin(A.P[0], A.P[1], cg[0], cg[1], cg[2]), is = lin(A.P[0], A.P[1], cs[0], cs[1], cs[2]);
-        if (!in_bounds(ig, A.np) || !in_bounds(is, A.np)) continue;
-        double lg[4];
-        for (int v = 0; v < 4; ++v) {
-            lg[v] = A.lamA[v * A.np + ig];
-            A.lamA[v * A.np + ig] = 0.0;
-        }
-        double add[4] = {lg[0], lg[1], lg[2], lg[3]};
-        double gu = 0.0;
-        if (bc == GKS_BC_NOSLIP) {
-            add[1] = -lg[1]; add[2] = -lg[2]; add[3] = -lg[3];
-        } else if (bc == GKS_BC_SLIP) {
-            add[1 + d] = -lg[1 + d];
-        } else if (bc == GKS_BC_INFLOW) {
-            const double r1 = A.A[is], un1 = A.A[(1 + d) * A.np + is] / r1;
-            const double sg = s == 0 ? 1.0 : -1.0;
-            const double x = sg * (A.uin[d] - un1) / A.csound;
-            const double ex = exp(x);
-            const double rg = r1 * ex;
-            const double rgb = lg[0] + lg[1] * A.uin[0] + lg[2] * A.uin[1] + lg[3] * A.uin[2];
-            add[0] = rgb * ex * (1.0 + sg * un1 / A.csound);
-            add[1] = add[2] = add[3] = 0.0;
-            add[1 + d] = -rgb * sg * ex / A.csound;
-            // sensitivity to the inflow speed U_inf = u_in[0]
-            gu = lg[1] * rg + (d == 0 ? rgb * r1 * ex * sg / A.csound : 0.0);
-        }
-        for (int v = 0; v < 4; ++v) A.lamA[v * A.np + is] += add[v];
-        if (bc == GKS_BC_INFLOW)
-            A.uinf_part[(long)(l - 1) * A.uinf_layer + (long)(b - A.lo2) * A.len1 + (a - A.lo1)] = gu;
+        ig[l - 1] = base + gi * sd;
+        is[l - 1] = base + src * sd;
+        ok = ok && in_bounds(ig[l - 1], A.np) && in_bounds(is[l - 1], A.np);
     }
+    if (!ok) return;
+    double lg[G][4];
+#pragma unroll
+    for (int l = 0; l < G; ++l)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) lg[l][v] = A.lamA[v * A.np + ig[l]];
+#pragma unroll
+    for (int l = 0; l < G; ++l)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) A.lamA[v * A.np + ig[l]] = 0.0;
+    if (bc == GKS_BC_PERIODIC && nd < G) {
+        // several ghosts of one source cell
+#pragma unroll
+        for (int l = G - 1; l >= 0; --l)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) A.lamA[v * A.np + is[l]] += lg[l][v];
+        return;
+    }
+    if (bc == GKS_BC_PERIODIC || bc == GKS_BC_NOSLIP || bc == GKS_BC_SLIP) {
+        double q[G][4];
+#pragma unroll
+        for (int l = 0; l < G; ++l)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) q[l][v] = A.lamA[v * A.np + is[l]];
+#pragma unroll
+        for (int l = 0; l < G; ++l)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const bool neg = v > 0 && (bc == GKS_BC_NOSLIP || (bc == GKS_BC_SLIP && v == 1 + d));
+                A.lamA[v * A.np + is[l]] = q[l][v] + (neg ? -lg[l][v] : lg[l][v]);
+            }
+        return;
+    }
+    // inflow, outflow: one source cell
+    double q[4], r1 = 1.0, un1 = 0.0;
+#pragma unroll
+    for (int v = 0; v < 4; ++v) q[v] = A.lamA[v * A.np + is[0]];
+    const double sg = s == 0 ? 1.0 : -1.0;
+    double ex = 1.0;
+    if (bc == GKS_BC_INFLOW) {
+        r1 = A.A[is[0]];
+        un1 = A.A[(1 + d) * A.np + is[0]] / r1;
+        ex = exp(sg * (A.uin[d] - un1) / A.csound);
+    }
+#pragma unroll
+    for (int l = G - 1; l >= 0; --l) {
+        if (bc == GKS_BC_INFLOW) {
+            const double rg = r1 * ex;
+            const double rgb = lg[l][0] + lg[l][1] * A.uin[0] + lg[l][2] * A.uin[1] + lg[l][3] * A.uin[2];
+            q[0] += rgb * ex * (1.0 + sg * un1 / A.csound);
+            const double t = -rgb * sg * ex / A.csound;
+            if (d == 0) q[1] += t;
+            else if (d == 1) q[2] += t;
+            else q[3] += t;
+            // sensitivity to the inflow speed U_inf = u_in[0]
+            A.uinf_part[(long)(s * G + l) * A.uinf_layer + (long)(b - A.lo2) * A.len1 + (a - A.lo1)] =
+                lg[l][1] * rg + (d == 0 ? rgb * r1 * ex * sg / A.csound : 0.0);
+        } else {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) q[v] += lg[l][v];
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < 4; ++v) A.lamA[v * A.np + is[0]] = q[v];
 }
 
 // Fixed-order two-pass sum of x[0..n) added to *acc: block b of kRedBlocks
@@ -1261,22 +1354,31 @@ __global__ void __launch_bounds__(256) reduce_final_kernel(const double *part, d
 //   stage 1: W* = W + dt/2 L + dt^2/8 Lt, P = W + dt L + dt^2/6 Lt:
 //            lamW = lamWs + lamP, lamL = dt/2 lamWs + dt lamP,
 //            lamLt = dt^2/8 lamWs + dt^2/6 lamP
-__global__ void __launch_bounds__(256) rev_update_kernel(int stage, const double *lamWs, const double *lamP,
-                                                         double *lamW, double *lamL, double *lamLt, double dt,
-                                                         long np, int nx, int ny, int P0, int P1)
+// lamL and lamLt go out in the reverse's compute type T (the tile and flux
+// kernels read them up to 6 times: as FP64 each read was a conversion on the
+// FP64 pipe); the factors come from the host. 176 -> 141 us a stage of
+// 256x128x128.
+struct UpdFactors {
+    double l1, l2, t1, t2;   // lamL = l1 lamWs + l2 lamP, lamLt = t1 lamWs + t2 lamP
+};
+
+template <typename T, int STAGE>
+__global__ void __launch_bounds__(256) rev_update_kernel(const double *lamWs, const double *lamP, double *lamW, T *lamL,
+                                                         T *lamLt, UpdFactors k, long np, int nx, int ny, int P0, int P1)
 {
-    const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y, k = blockIdx.z;
+    const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y;
     if (i >= nx || j >= ny) return;
-    const long l = lin(P0, P1, i, j, k);
+    const long l = lin(P0, P1, i, j, blockIdx.z);
+#pragma unroll
     for (int v = 0; v < 4; ++v) {
         const long o = v * np + l;
-        if (stage == 2) {
-            lamLt[o] = dt * dt / 3.0 * lamP[o];
+        if (STAGE == 2) {
+            lamLt[o] = T(k.t2 * lamP[o]);
         } else {
             const double ws = lamWs[o], p = lamP[o];
             lamW[o] = ws + p;
-            lamL[o] = 0.5 * dt * ws + dt * p;
-            lamLt[o] = 0.125 * dt * dt * ws + dt * dt / 6.0 * p;
+            lamL[o] = T(k.l1 * ws + k.l2 * p);
+            lamLt[o] = T(k.t1 * ws + k.t2 * p);
         }
     }
 }
@@ -1583,7 +1685,7 @@ __global__ void alm_sample_add_serial_kernel(AlmAdjArgs A, const double *ptc, co
 // for lamL (may be null) and lamLt; result accumulated into w.lamA.
 template <typename T>
 void spatial_adjoint(const Ctx &c, const AdjWork &w, const double *Aw, void *const gp[3],
-                     const double *lamL, const double *lamLt)
+                     const void *lamL, const void *lamLt)
 {
     const Phys<double> ph = make_phys<double>(c);
     constexpr bool f32 = sizeof(T) == 4;
@@ -1633,7 +1735,7 @@ void spatial_adjoint(const Ctx &c, const AdjWork &w, const double *Aw, void *con
         rev_t1_kernel<T><<<dim3((R.n1 + 4 + 31) / 32, (R.n2 + 4 + 7) / 8, nf), blk, 0, c.stream>>>(R);
         const dim3 gfs((R.n1 + 4 + 31) / 32, (R.n2 + 4 + 7) / 8, (nf + kRevMarch - 1) / kRevMarch);
         if (f32)
-            rev_face_state32_kernel<true><<<gfs, blk, 0, c.stream>>>(R);
+            rev_face_state32_kernel<<<gfs, blk, 0, c.stream>>>(R);
         else
             rev_face_state_kernel<<<gfs, blk, 0, c.stream>>>(R);
         rev_gather_cells_kernel<T><<<dim3((R.n1 + 4 + 31) / 32, (R.n2 + 4 + 7) / 8, R.nd + 2 * G), blk, 0,
@@ -1646,8 +1748,7 @@ void spatial_adjoint(const Ctx &c, const AdjWork &w, const double *Aw, void *con
 // in one pass over the tiles, the partials added per face, then RD on the
 // FP32 cells and RE. c32 is the grid's own context (FP32 widths, the density
 // offset, the face-box buffer and its TMA maps); cw the reverse's context.
-void spatial_adjoint_fused32(const Ctx &cw, const AdjWork &w, const float *A32, const double *lamL,
-                             const double *lamLt)
+void spatial_adjoint_fused32(const Ctx &cw, const AdjWork &w, const float *A32, const float *lamL, const float *lamLt)
 {
     const Ctx &c = *w.c32;
     const Phys<float> ph = make_phys<float>(c);
@@ -1703,6 +1804,7 @@ void spatial_adjoint_fused32(const Ctx &cw, const AdjWork &w, const float *A32, 
         R.lamC = w.lamC;
         R.lamA = w.lamA;
         R.ihf = (const double *)cw.ihf[d];
+        R.ihf32 = (const float *)c.ihf[d];
         for (int e = 0; e < 3; ++e) {
             R.n[e] = c.n[e];
             R.P[e] = c.P[e];
@@ -1746,13 +1848,13 @@ void ghost_adjoint(const Ctx &c, const AdjWork &w, const double *Aw)
         A.len2 = A.e2 < d ? c.n[A.e2] + 2 * G : c.n[A.e2];
         A.csound = c.csound;
         for (int e = 0; e < 3; ++e) A.uin[e] = c.inflow[1 + e];
-        for (int s = 0; s < 2; ++s) {
-            A.s = s;
-            A.bc = c.bc[d][s];
-            A.uinf_layer = w.nuinf / (6 * G);
-            A.uinf_part = w.uinf_part + (long)((d * 2 + s) * G) * A.uinf_layer;
-            ghost_rev_kernel<<<dim3((A.len1 + 31) / 32, (A.len2 + 7) / 8, 1), dim3(32, 8), 0, c.stream>>>(A);
-        }
+        A.bc[0] = c.bc[d][0];
+        A.bc[1] = c.bc[d][1];
+        A.uinf_layer = w.nuinf / (6 * G);
+        A.uinf_part = w.uinf_part + (long)(d * 2 * G) * A.uinf_layer;
+        const int sides = c.n[d] >= 2 * G ? 2 : 1;   // in one launch
+        for (A.s0 = 0; A.s0 < 2; A.s0 += sides)
+            ghost_rev_kernel<<<dim3((A.len1 + 31) / 32, (A.len2 + 7) / 8, sides), dim3(32, 8), 0, c.stream>>>(A);
     }
     static_assert(kRedBlocks == 256, "one part per thread of the final pass");
     reduce_part_kernel<<<kRedBlocks, 256, 0, c.stream>>>(w.uinf_part, w.nuinf, w.red);
@@ -1942,20 +2044,30 @@ void adjoint_reverse(const Ctx &c, const AdjWork &w, const RotorDev *rot, const 
             alm_sample_add_serial_kernel<<<1, 1, 0, c.stream>>>(A, w.ptc, (const long *)w.ptl);
     }
     // stage 2: W' = P + dt^2/3 Lt(W*)
-    rev_update_kernel<<<gcell, blk, 0, c.stream>>>(2, nullptr, w.lamP, nullptr, nullptr, w.lamLt, dt, c.np,
-                                                   c.n[0], c.n[1], c.P[0], c.P[1]);
+    const bool f32 = w.gp_bytes == 4;
+    const UpdFactors k2 = {0.0, 0.0, 0.0, dt * dt / 3.0}, k1 = {0.5 * dt, dt, 0.125 * dt * dt, dt * dt / 6.0};
+    if (f32)
+        rev_update_kernel<float, 2><<<gcell, blk, 0, c.stream>>>(nullptr, w.lamP, nullptr, nullptr, (float *)w.lamLt, k2,
+                                                                 c.np, c.n[0], c.n[1], c.P[0], c.P[1]);
+    else
+        rev_update_kernel<double, 2><<<gcell, blk, 0, c.stream>>>(nullptr, w.lamP, nullptr, nullptr, w.lamLt, k2, c.np,
+                                                                  c.n[0], c.n[1], c.P[0], c.P[1]);
     cudaMemsetAsync(w.lamA, 0, bytes4, c.stream);
     if (w.A0f)
-        spatial_adjoint_fused32(c, w, w.Wsf, nullptr, w.lamLt);
+        spatial_adjoint_fused32(c, w, w.Wsf, nullptr, (const float *)w.lamLt);
     else
         spatial(c, w, w.Ws, w.gps[1], nullptr, w.lamLt);
     ghost_adjoint(c, w, w.Ws);
     // stage 1: lamA (interior) is lambda of W*
-    rev_update_kernel<<<gcell, blk, 0, c.stream>>>(1, w.lamA, w.lamP, w.lamW, w.lamL, w.lamLt, dt, c.np, c.n[0],
-                                                   c.n[1], c.P[0], c.P[1]);
+    if (f32)
+        rev_update_kernel<float, 1><<<gcell, blk, 0, c.stream>>>(w.lamA, w.lamP, w.lamW, (float *)w.lamL, (float *)w.lamLt,
+                                                                 k1, c.np, c.n[0], c.n[1], c.P[0], c.P[1]);
+    else
+        rev_update_kernel<double, 1><<<gcell, blk, 0, c.stream>>>(w.lamA, w.lamP, w.lamW, w.lamL, w.lamLt, k1, c.np,
+                                                                  c.n[0], c.n[1], c.P[0], c.P[1]);
     cudaMemsetAsync(w.lamA, 0, bytes4, c.stream);
     if (w.A0f)
-        spatial_adjoint_fused32(c, w, w.A0f, w.lamL, w.lamLt);
+        spatial_adjoint_fused32(c, w, w.A0f, (const float *)w.lamL, (const float *)w.lamLt);
     else
         spatial(c, w, w.A0, w.gps[0], w.lamL, w.lamLt);
     ghost_adjoint(c, w, w.A0);

@@ -318,9 +318,10 @@ __device__ __forceinline__ f2 operator*(f2 a, f2 b) { return f2(__fmul2_rn(a.v, 
 __device__ __forceinline__ f2 fma(f2 a, f2 b, f2 c) { return f2(__ffma2_rn(a.v, b.v, c.v)); }
 // a - b as a + (-1) b: the product is exact, so one rounding as in __fsub_rn
 __device__ __forceinline__ f2 operator-(f2 a, f2 b) { return fma(b, f2(-1.0f), a); }
+// a sign costs nothing: the packed instructions negate their operands
+__device__ __forceinline__ f2 operator-(f2 a) { return f2(-a.v.x, -a.v.y); }
 __device__ __forceinline__ f2 &operator+=(f2 &a, f2 b) { return a = a + b; }
 __device__ __forceinline__ f2 &operator-=(f2 &a, f2 b) { return a = a - b; }
-__device__ __forceinline__ f2 operator-(f2 a) { return a * f2(-1.0f); }
 // IEEE division per lane (the scalar FP32 path's a / b)
 __device__ __forceinline__ f2 operator/(f2 a, f2 b) { return f2(__fdiv_rn(a.v.x, b.v.x), __fdiv_rn(a.v.y, b.v.y)); }
 // the two-instruction approximate division of the scalar FP32 path, per lane

@@ -2246,13 +2246,13 @@ void launch_raw_copy(const Ctx &c, void *compact, int to_compact)
                                                         to_compact);
 }
 
-// FP32 values as FP64: out[i] = a[i] (+ b[i]) (+ off0 for i < n0), i < n.
+// FP32 values as FP64: out[i] = a[i] (+ b[i]) (+ off0 for i < n0), i < n; in
+// integer operations (4 x 4.6M hi and lo: 35 -> 20 us).
 __global__ void __launch_bounds__(256) widen_kernel(const float *a, const float *b, double *out, long n, long n0,
                                                      double off0)
 {
     for (long i = blockIdx.x * 256L + threadIdx.x; i < n; i += (long)gridDim.x * 256L) {
-        double v = (double)a[i];
-        if (b) v += (double)b[i];
+        double v = compose_hi_lo(a[i], b ? b[i] : 0.0f);
         if (i < n0) v += off0;
         out[i] = v;
     }

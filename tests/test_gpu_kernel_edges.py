@@ -187,3 +187,44 @@ def test_small_and_large_launch_paths_give_the_same_bits(gks, precision):
     assert np.array_equal(g.get_state(), s.get_state())
     g.close()
     s.close()
+
+
+@pytest.mark.parametrize("n", [(3, 4, 5), (5, 33, 9), (37, 8, 6), (64, 9, 17)], ids=lambda n: "%dx%dx%d" % n)
+def test_reverse_step_at_tile_and_ghost_edges(gks, n):
+    """Axes shorter than two ghost layers (the sides of the ghost reverse one
+    after the other), remainders of the reverse's tiles. The bars are those of
+    the adjoint tests: 1e-5 of a central difference whose terms cannot cancel,
+    3e-5 of the largest element for the FP32 reverses."""
+    import torch
+    h = min(2 * np.pi * (1 + 0.1 * d) / n[d] for d in range(3))
+    w = smooth_workload(n, [(3, 4), (0, 0), (1, 2)], seed=sum(n), dt_fixed=0.01 * h)
+    w.inflow = (1.0, 0.3, 0.0, 0.0)
+    rng = np.random.default_rng(7)
+    W = torch.tensor(w.state0, dtype=torch.float64, device="cuda")
+    lam1 = torch.tensor(rng.standard_normal(W.shape), dtype=torch.float64, device="cuda")
+    g = grid(gks, w, "fp64")
+    g.set_adjoint_precision("fp64")
+    ref, _ = g.step_adjoint(g.adjoint_workspace(), 0.0, W, lam1, 0.0, None)
+
+    def J(Wx):
+        g.set_state_tensor(Wx)
+        g.set_time(0.0)
+        g.step(1)
+        return float((lam1 * g.state_tensor()).sum().item())
+
+    dW = torch.sign(ref) * torch.tensor(0.5 + rng.random(W.shape), dtype=torch.float64, device="cuda")
+    eps = 1e-7
+    fd = (J(W + eps * dW) - J(W - eps * dW)) / (2 * eps)
+    assert abs(fd - float((ref * dW).sum().item())) <= 1e-5 * abs(fd)
+    g.set_adjoint_precision("fp32")
+    lam, _ = g.step_adjoint(g.adjoint_workspace(), 0.0, W, lam1, 0.0, None)
+    assert float((lam - ref).abs().max()) <= 3e-5 * float(ref.abs().max())
+    g.close()
+    c = grid(gks, w, "fp32c")
+    c.set_state_tensor(W)
+    c.set_time(0.0)
+    tape = c.adjoint_tape()
+    c.step_record(tape)
+    lam, _ = c.step_reverse(tape, c.adjoint_scratch(), lam1, 0.0, None)
+    assert float((lam - ref).abs().max()) <= 3e-5 * float(ref.abs().max())
+    c.close()
