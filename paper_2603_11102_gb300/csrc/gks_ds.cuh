@@ -152,7 +152,17 @@ __device__ __forceinline__ dsf &operator-=(dsf &a, dsf b) { return a = a - b; }
 __device__ __forceinline__ dsf &operator*=(dsf &a, dsf b) { return a = a * b; }
 
 using ::fma;
-__device__ __forceinline__ dsf fma(dsf a, dsf b, dsf c) { return a * b + c; }
+// a b + c with the product left unnormalised (see the pair version)
+__device__ __forceinline__ dsf fma(dsf a, dsf b, dsf c)
+{
+    const float p = __fmul_rn(a.hi, b.hi);
+    float e = __fmaf_rn(a.hi, b.hi, -p);
+    e = __fmaf_rn(a.hi, b.lo, e);
+    e = __fmaf_rn(a.lo, b.hi, e);
+    const dsf s = two_sum(p, c.hi), t = two_sum(e, c.lo);
+    const dsf r = fast_two_sum(s.hi, __fadd_rn(s.lo, t.hi));
+    return dsf(r.hi, __fadd_rn(r.lo, t.lo));
+}
 __device__ __forceinline__ dsf wdiv(dsf a, dsf b) { return a / b; }
 // exact scaling by a power of two
 __device__ __forceinline__ dsf scale_pow2(dsf a, float p) { return dsf(__fmul_rn(a.hi, p), __fmul_rn(a.lo, p)); }

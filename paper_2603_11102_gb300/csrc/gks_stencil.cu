@@ -532,9 +532,11 @@ __device__ __forceinline__ dsf face_avg_neg(dsf s) { return scale_pow2(s, -0.25f
 // m: values and t2 slopes of Q0, values of the t1 slopes and of the normal
 // slope at the two t2 Gauss points -g, +g (k = 0, 1); the density's slopes
 // negated, as gk_flux takes them.
-template <typename R, int V>
-__device__ __forceinline__ void t2_pass(const R *st, int m, int tx, int ty, R q[2], R dn[2], R d1[2], R d2[2])
+template <int V>
+__device__ __forceinline__ void t2_pass(const double *st, int m, int tx, int ty, double q[2], double dn[2], double d1[2],
+                                        double d2[2])
 {
+    using R = double;
     constexpr bool NEG = V == 0;
     const R *x = st + (V * 4 + m) * ST_ROWS + ty * TX + tx;
     const R *y = st + (V * 4 + 2 + m) * ST_ROWS + ty * TX + tx;
@@ -560,10 +562,10 @@ __device__ __forceinline__ void tile_gauss_flux(const FluxPhys<double> &ph, cons
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
         double t[4][4][2];   // [Q0, normal slope, t1 slope, t2 slope][component][t2 Gauss point]
-        t2_pass<double, 0>(st, m, tx, ty, t[0][0], t[1][0], t[2][0], t[3][0]);
-        t2_pass<double, 1>(st, m, tx, ty, t[0][1], t[1][1], t[2][1], t[3][1]);
-        t2_pass<double, 2>(st, m, tx, ty, t[0][2], t[1][2], t[2][2], t[3][2]);
-        t2_pass<double, 3>(st, m, tx, ty, t[0][3], t[1][3], t[2][3], t[3][3]);
+        t2_pass<0>(st, m, tx, ty, t[0][0], t[1][0], t[2][0], t[3][0]);
+        t2_pass<1>(st, m, tx, ty, t[0][1], t[1][1], t[2][1], t[3][1]);
+        t2_pass<2>(st, m, tx, ty, t[0][2], t[1][2], t[2][2], t[3][2]);
+        t2_pass<3>(st, m, tx, ty, t[0][3], t[1][3], t[2][3], t[3][3]);
         if constexpr (GP) {
             if (gp) {
 #pragma unroll
@@ -630,12 +632,22 @@ __device__ __forceinline__ void tile_gauss_flux_f2(const FluxPhys<f2> &ph, const
 template <int V>
 __device__ __forceinline__ void t2_pass_ds2(const dsf *st, int m, int tx, int ty, dsf2 &q, dsf2 &dn, dsf2 &d1, dsf2 &d2)
 {
-    dsf a[2], b[2], c[2], d[2];
-    t2_pass<dsf, V>(st, m, tx, ty, a, b, c, d);
-    q = dsf2(a[0], a[1]);
-    dn = dsf2(b[0], b[1]);
-    d1 = dsf2(c[0], c[1]);
-    d2 = dsf2(d[0], d[1]);
+    constexpr bool NEG = V == 0;
+    const dsf *x = st + (V * 4 + m) * ST_ROWS + ty * TX + tx;
+    const dsf *y = st + (V * 4 + 2 + m) * ST_ROWS + ty * TX + tx;
+    const dsf *z = st + (16 + V * 2 + m) * ST_ROWS + ty * TX + tx;
+    dsf p[5], D[4];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) p[i] = x[i * TX];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) D[i] = p[i + 1] - p[i];
+    ds_val_der<NEG>(p[2], D, q, d2);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) p[i] = y[i * TX];
+    d1 = ds_val_direct<NEG>(p);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) p[i] = z[i * TX];
+    dn = ds_val_direct<NEG>(p);
 }
 template <bool NEED_F0>
 __device__ __forceinline__ void tile_gauss_flux_ds2(const FluxPhys<dsf2> &ph, const dsf *st, int tx, int ty, dsf ih1,
