@@ -87,7 +87,7 @@ __device__ __forceinline__ f2 rev_inverse(f2 a) { return wrcp(a); }
 //   H_ik = D_i m_k - U_k D_i rho, B = H_kk + U.grad rho, C_k = theta d_k rho + U_i H_ik,
 //   X = U_n B + C_n, -F1 = (X, U_n X + C_n U_n + theta B, U_k X + U_n C_k),
 // in about 110 operations (135 with F0) against the 230 of the form with
-// d_i U_k, A_0 and A_k. With the FP32 tile adjoints (below) 736 -> 570 us a
+// d_i U_k, A_0 and A_k. The FP32 tile adjoints (below) took 736 -> 570 us a
 // direction of a 256x128x128 FP32C stage; the FP64 reverse 1.04x.
 template <typename T>
 __device__ __forceinline__ void gk_flux_rev(const Phys<T> &ph, const T q[4], const T Dn[4], const T D1[4],
@@ -625,8 +625,8 @@ struct Weno32 {
 
 // Adjoint of both face values (seeds sR, sL): added to the adjoints of the 5
 // cells, out. About 100 operations with the recomputed pieces against the 190
-// of the form in the cells' values; rev_face_cells32_kernel stays at 0.40 ms on
-// 256x128x128 all the same (its time goes to the loads).
+// of the form in the cells' values (no gain by itself: the loads bounded
+// rev_face_cells32_kernel).
 __device__ __forceinline__ void weno32_rev(const float D[4], float sR, float sL, float out[5])
 {
     const Weno32 w(D);
@@ -768,23 +768,40 @@ __global__ void __launch_bounds__(256) rev_face_state32_kernel(RevArgs A)
     }
 }
 
-// RD and RE of an FP32C grid in one march: a thread owns the cells
-// [c0, c0 + kRevCells) of one line along d (ghost cells included) and walks
-// the faces c0 - 2 .. c0 + kRevCells + 2 that read them, with the 6 cells of
-// the current face's stencil in registers (FP32 cells as the forward read
-// them, density as rho - off) and their adjoints in a rolling window; a cell
-// leaves the window after its last face (f = c + 3) and its adjoint, summed
-// over its faces in face order as RE sums them, is added to lamA. Each cell
-// is written by one thread. The face reverse is rev_face_state32_kernel's.
-constexpr int kRevCells = 24;
+// RD and RE of an FP32C grid in one march: a thread owns the cells [c0, c1) of
+// one line along d (ghost cells included) and walks the faces c0 - 2 .. c1 + 2
+// that read them, with the differences of the current face's 6 cells in
+// registers (FP32 cells as the forward read them, density as rho - off) and
+// their adjoints in a rolling window; a cell leaves the window after its last
+// face (f = c + 3) and its adjoint, summed over its faces in face order as RE
+// sums them, is added to lamA. Each cell is written by one thread. The face
+// reverse is rev_face_state32_kernel's.
+//
+// What the next face takes from memory (its 8 adjoints, the entering cell and
+// lamA of the leaving one, RevSlot) is copied to shared memory a face ahead:
+// 5 to 6 lines in flight a thread without registers. The positions of the
+// extended face plane are dealt out to the threads in one row (a block of 32 x 8
+// leaves a quarter of the threads of 132 x 132 positions idle), and a line is
+// cut so that the blocks fill whole waves (rev_cells; 918 blocks on 304 places
+// took 4 waves): 0.37 -> 0.22 ms for the y and z faces of 256x128x128, 0.48 ->
+// 0.37 ms for the x faces, whose cells lie a row apart across the lanes.
+struct RevSlot {
+    double lam[4][256];
+    float q[8][256], w[4][256];
+};
+constexpr size_t rev_cells_smem_bytes() { return 2 * sizeof(RevSlot); }
 
-__global__ void __launch_bounds__(256, 2) rev_face_cells32_kernel(RevArgs A)
+__global__ void __launch_bounds__(256, 2) rev_face_cells32_kernel(RevArgs A, int cells)
 {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    RevSlot *ring = reinterpret_cast<RevSlot *>(smem_raw);
     const float *lamFQ = (const float *)A.lamFQ;
-    const int a = (int)(blockIdx.x * 32 + threadIdx.x) - 2, b = (int)(blockIdx.y * 8 + threadIdx.y) - 2;
+    const int tid = threadIdx.x;
+    const long pos = blockIdx.x * 256L + tid;
+    const int a = (int)(pos % (A.n1 + 4)) - 2, b = (int)(pos / (A.n1 + 4)) - 2;
     const int nf = A.nd + 1;
-    const int c0 = (int)blockIdx.z * kRevCells - G, c1 = min(c0 + kRevCells, A.nd + G);
-    if (a >= A.n1 + 2 || b >= A.n2 + 2 || c0 >= A.nd + G) return;
+    const int c0 = (int)blockIdx.y * cells - G, c1 = min(c0 + cells, A.nd + G);
+    if (b >= A.n2 + 2 || c0 >= A.nd + G) return;
     const int fs = max(0, c0 - 2), fe = min(nf - 1, c1 + 2);   // faces [fs, fe]
     if (fs > fe) return;
     // padded strides by axis (selects, not an indexed local array)
@@ -838,24 +855,34 @@ __global__ void __launch_bounds__(256, 2) rev_face_cells32_kernel(RevArgs A)
     for (int v = 0; v < 4; ++v)
 #pragma unroll
         for (int k = 0; k < 6; ++k) acc[v][k] = 0.0f;
-    // the cell entering the window, loaded one face ahead
-    float nxt[4];
+    auto request = [&](int f) {   // f <= fe: inside the checked range
+        RevSlot &r = ring[f & 1];
+        const long o = ((long)f * (A.n2 + 4) + (b + 2)) * A.e1p + (a + 2);
 #pragma unroll
-    for (int v = 0; v < 4; ++v) nxt[v] = A.Ahi[comp[v] * A.np + base + (long)(fs + 2) * sd];
+        for (int v = 0; v < 8; ++v) cp_async(&r.q[v][tid], lamFQ + v * A.nfq + o);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) cp_async(&r.w[v][tid], A.Ahi + comp[v] * A.np + base + (long)(f + 2) * sd);
+        if (f - 3 >= c0 && f - 3 < c1) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+                cp_async(&r.lam[v][tid], (const double *)A.lamA + comp[v] * A.np + base + (long)(f - 3) * sd);
+        }
+        cp_async_commit();
+    };
+    request(fs);
 #pragma unroll 1
     for (int f = fs; f <= fe; ++f) {
+        cp_async_wait_all();
+        if (f < fe) request(f + 1);
+        const RevSlot &r = ring[f & 1];
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) D[v][k] = D[v][k + 1];
             ch[v][0] = ch[v][1];
             ch[v][1] = ch[v][2];
-            ch[v][2] = nxt[v];
+            ch[v][2] = r.w[v][tid];
             D[v][4] = ch[v][2] - ch[v][1];
-        }
-        if (f < fe) {   // cell f + 3 <= fe + 2: inside the checked range
-#pragma unroll
-            for (int v = 0; v < 4; ++v) nxt[v] = A.Ahi[comp[v] * A.np + base + (long)(f + 3) * sd];
         }
         float Ql[4], Qr[4], Rt[4];
 #pragma unroll
@@ -865,12 +892,11 @@ __global__ void __launch_bounds__(256, 2) rev_face_cells32_kernel(RevArgs A)
             Rt[v] = ch[v][0] + w.right(&D[v][1]);
             Qr[v] = ch[v][0] + w.left(&D[v][1]);
         }
-        const long o = ((long)f * (A.n2 + 4) + (b + 2)) * A.e1p + (a + 2);
         float Q0b[4], DNb[4], Qlb[4], Qrb[4];
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            Q0b[v] = lamFQ[v * A.nfq + o];
-            DNb[v] = lamFQ[(4 + v) * A.nfq + o];
+            Q0b[v] = r.q[v][tid];
+            DNb[v] = r.q[4 + v][tid];
         }
         equilibrium_rev<float>(ph, Ql, Qr, Q0b, Qlb, Qrb);
         const float s = __ldg(A.ihf32 + f) * float(1.0 / 12.0);
@@ -893,7 +919,8 @@ __global__ void __launch_bounds__(256, 2) rev_face_cells32_kernel(RevArgs A)
         const int cl = f - 3;
         if (cl >= c0 && cl < c1) {
 #pragma unroll
-            for (int v = 0; v < 4; ++v) A.lamA[comp[v] * A.np + base + (long)cl * sd] += compose_hi_lo(acc[v][0], 0.0f);
+            for (int v = 0; v < 4; ++v)
+                A.lamA[comp[v] * A.np + base + (long)cl * sd] = r.lam[v][tid] + compose_hi_lo(acc[v][0], 0.0f);
         }
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
@@ -965,11 +992,15 @@ __global__ void __launch_bounds__(256) rev_gather_cells_kernel(RevArgs A)
 // neighbouring tiles: sum_partials32_kernel adds the partials of a face in a
 // fixed order.
 struct Rev32Args {
-    const float *lamL, *lamLt;        // padded cell adjoints; lamL null in stage 2
+    // cell adjoints, lamL null in stage 2: padded, for x faces the copies with y
+    // fastest (the lanes run along y: from the padded arrays every lane reads
+    // a sector of its own: 1.07 and 0.66 ms a stage against 0.44 and 0.40 of
+    // the other directions on 256x128x128, now the same)
+    const float *lamL, *lamLt;
     const float *ihd, *ih1, *ih2;     // inverse cell widths along d, t1, t2 (padded index)
     float *part;                      // per tile: 8 x SQ_H x SQ_W face-box adjoints
     int n1, n2, nf, nd, d, t1, t2;
-    long np, sd, s1, s2, base;        // padded strides along d, t1, t2; index of cell (0, 0, 0)
+    long np, sd, s1, s2, base;        // of the cell adjoints: strides of a component, along d, t1, t2; index of cell (0, 0, 0)
     Phys<float> ph;
     Scalars *scal;
 };
@@ -1016,20 +1047,19 @@ __global__ void __launch_bounds__(256, 2) rev_tile32_kernel(const __grid_constan
         // RA: per face, the 4 Gauss points
         const int a = ta * TX + tx, b = tb * TY + ty;
         if (a < A.n1 && b < A.n2) {
-            const bool hasl = f >= 1, hasr = f < A.nd;
             const long ir = A.base + (long)f * A.sd + (long)a * A.s1 + (long)b * A.s2, il = ir - A.sd;
-            const bool okc = in_bounds(il, A.np) && in_bounds(ir, A.np);
+            const bool hasl = f >= 1 && in_bounds(il, A.np), hasr = f < A.nd && in_bounds(ir, A.np);
             const float ihl = hasl ? A.ihd[f - 1 + G] : 0.0f, ihr = hasr ? A.ihd[f + G] : 0.0f;
             float sF0[4] = {0, 0, 0, 0}, sF1[4] = {0, 0, 0, 0};
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
                 const long o = gc[v] * A.np;
-                const float ll = (hasl && okc) ? A.lamLt[o + il] : 0.0f;
-                const float lr = (hasr && okc) ? A.lamLt[o + ir] : 0.0f;
+                const float ll = hasl ? A.lamLt[o + il] : 0.0f;
+                const float lr = hasr ? A.lamLt[o + ir] : 0.0f;
                 sF1[v] = 0.25f * (-ll * ihl + lr * ihr);
                 if (needF0) {
-                    const float ml = (hasl && okc) ? A.lamL[o + il] : 0.0f;
-                    const float mr = (hasr && okc) ? A.lamL[o + ir] : 0.0f;
+                    const float ml = hasl ? A.lamL[o + il] : 0.0f;
+                    const float mr = hasr ? A.lamL[o + ir] : 0.0f;
                     sF0[v] = 0.25f * (-ml * ihl + mr * ihr);
                 }
             }
@@ -1362,23 +1392,46 @@ struct UpdFactors {
     double l1, l2, t1, t2;   // lamL = l1 lamWs + l2 lamP, lamLt = t1 lamWs + t2 lamP
 };
 
-template <typename T, int STAGE>
+// XT: behind lamL and lamLt also their interior cells with y fastest
+// (Rev32Args), through a shared tile; 8 y values fill a sector.
+template <typename T, int STAGE, bool XT>
 __global__ void __launch_bounds__(256) rev_update_kernel(const double *lamWs, const double *lamP, double *lamW, T *lamL,
                                                          T *lamLt, UpdFactors k, long np, int nx, int ny, int P0, int P1)
 {
-    const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y;
-    if (i >= nx || j >= ny) return;
-    const long l = lin(P0, P1, i, j, blockIdx.z);
+    __shared__ T tile[XT ? (STAGE == 1 ? 8 : 4) : 1][XT ? TX : 1][XT ? TY + 1 : 1];
+    const int i = blockIdx.x * TX + threadIdx.x, j = blockIdx.y * TY + threadIdx.y;
+    if (i < nx && j < ny) {
+        const long l = lin(P0, P1, i, j, blockIdx.z);
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        const long o = v * np + l;
-        if (STAGE == 2) {
-            lamLt[o] = T(k.t2 * lamP[o]);
-        } else {
-            const double ws = lamWs[o], p = lamP[o];
-            lamW[o] = ws + p;
-            lamL[o] = T(k.l1 * ws + k.l2 * p);
-            lamLt[o] = T(k.t1 * ws + k.t2 * p);
+        for (int v = 0; v < 4; ++v) {
+            const long o = v * np + l;
+            const double p = lamP[o];
+            T Lt;
+            if (STAGE == 2) {
+                Lt = T(k.t2 * p);
+            } else {
+                const double ws = lamWs[o];
+                lamW[o] = ws + p;
+                const T L = T(k.l1 * ws + k.l2 * p);
+                Lt = T(k.t1 * ws + k.t2 * p);
+                lamL[o] = L;
+                if (XT) tile[4 + v][threadIdx.x][threadIdx.y] = L;
+            }
+            lamLt[o] = Lt;
+            if (XT) tile[v][threadIdx.x][threadIdx.y] = Lt;
+        }
+    }
+    if constexpr (XT) {
+        __syncthreads();
+        const int t = threadIdx.y * TX + threadIdx.x, ti = t / TY, tj = t % TY;
+        const int x = blockIdx.x * TX + ti, y = blockIdx.y * TY + tj;
+        if (x < nx && y < ny) {
+            const long n = (long)nx * ny * gridDim.z, o = ((long)blockIdx.z * nx + x) * ny + y;
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                lamLt[4 * np + v * n + o] = tile[v][ti][tj];
+                if (STAGE == 1) lamL[4 * np + v * n + o] = tile[4 + v][ti][tj];
+            }
         }
     }
 }
@@ -1743,6 +1796,25 @@ void spatial_adjoint(const Ctx &c, const AdjWork &w, const double *Aw, void *con
     }
 }
 
+// Cells of a line that a thread of rev_face_cells32_kernel owns: the least
+// number of faces walked one after the other, ceil(blocks / resident) segments
+// of cells + 5 faces and about one of start, for nb blocks per segment.
+int rev_cells(long nb, int ncells, int resident)
+{
+    int best = ncells;
+    double cost = -1.0;
+    for (int S = 1; S == 1 || (ncells + S - 1) / S >= 4; ++S) {
+        const int cells = (ncells + S - 1) / S;
+        const long blocks = nb * ((ncells + cells - 1) / cells);
+        const double t = (double)((blocks + resident - 1) / resident) * (cells + 6);
+        if (cost < 0.0 || t < cost) {
+            cost = t;
+            best = cells;
+        }
+    }
+    return best;
+}
+
 // S^T of an FP32C grid through the fused reverse: per direction the forward
 // face boxes from the FP32 working array A32 (as the forward read it), RA-RC
 // in one pass over the tiles, the partials added per face, then RD on the
@@ -1754,13 +1826,18 @@ void spatial_adjoint_fused32(const Ctx &cw, const AdjWork &w, const float *A32, 
     const Phys<float> ph = make_phys<float>(c);
     const dim3 blk(TX, TY);
     const size_t smem = rev_tile32_smem_bytes();
-    static int grid_blocks = 0;
-    if (!grid_blocks) {
-        int per = 0;
+    struct Resident {
+        int tile, cells;
+    };
+    static const Resident resident = [smem] {   // blocks of each kernel on the device at once
+        int t = 0, r = 0;
         cudaFuncSetAttribute(rev_tile32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, rev_tile32_kernel, TX * TY, smem);
-        grid_blocks = (per > 0 ? per : 1) * sm_count();
-    }
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&t, rev_tile32_kernel, TX * TY, smem);
+        cudaFuncSetAttribute(rev_face_cells32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)rev_cells_smem_bytes());
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, rev_face_cells32_kernel, 256, rev_cells_smem_bytes());
+        return Resident{std::max(t, 1) * sm_count(), std::max(r, 1) * sm_count()};
+    }();
     for (int d = 0; d < 3; ++d) {
         const int t1 = tan1(d), t2 = tan2(d);
         launch_face_state32(c, d, A32);
@@ -1784,10 +1861,19 @@ void spatial_adjoint_fused32(const Ctx &cw, const AdjWork &w, const float *A32, 
         Q.s2 = stride[t2];
         Q.base = G * (stride[0] + stride[1] + stride[2]);
         Q.np = c.np;
+        if (d == 0) {   // y fastest, then x, then z, interior cells
+            Q.lamL = lamL ? lamL + 4 * c.np : nullptr;
+            Q.lamLt = lamLt + 4 * c.np;
+            Q.sd = c.n[1];
+            Q.s1 = 1;
+            Q.s2 = (long)c.n[0] * c.n[1];
+            Q.base = 0;
+            Q.np = (long)c.n[0] * c.n[1] * c.n[2];
+        }
         Q.ph = ph;
         Q.scal = w.sc;
         const long ntiles = (long)((Q.n1 + TX - 1) / TX) * ((Q.n2 + TY - 1) / TY) * Q.nf;
-        const int grid = (int)(ntiles < grid_blocks ? ntiles : grid_blocks);
+        const int grid = (int)(ntiles < resident.tile ? ntiles : resident.tile);
         rev_tile32_kernel<<<grid, blk, smem, c.stream>>>(c.tmap[d], Q);
         sum_partials32_kernel<<<dim3((Q.n1 + 4 + TX - 1) / TX, (Q.n2 + 4 + TY - 1) / TY, Q.nf), blk, 0, c.stream>>>(
             w.part, (float *)w.lamFQ, c.nfq, c.e1p[d], Q.n1, Q.n2);
@@ -1817,11 +1903,10 @@ void spatial_adjoint_fused32(const Ctx &cw, const AdjWork &w, const float *A32, 
         R.n2 = c.n[t2];
         R.np = c.np;
         R.ph = make_phys<double>(c);
-        const int nf = c.n[d] + 1;
-        const dim3 gfs((R.n1 + 4 + 31) / 32, (R.n2 + 4 + 7) / 8, (nf + kRevMarch - 1) / kRevMarch);
-        (void)gfs;
-        rev_face_cells32_kernel<<<dim3((R.n1 + 4 + 31) / 32, (R.n2 + 4 + 7) / 8,
-                                       (R.nd + 2 * G + kRevCells - 1) / kRevCells), blk, 0, c.stream>>>(R);
+        const long nb = ((long)(R.n1 + 4) * (R.n2 + 4) + 255) / 256;
+        const int cells = rev_cells(nb, R.nd + 2 * G, resident.cells);
+        rev_face_cells32_kernel<<<dim3((unsigned)nb, (R.nd + 2 * G + cells - 1) / cells), 256, rev_cells_smem_bytes(),
+                                  c.stream>>>(R, cells);
     }
 }
 
@@ -2046,12 +2131,16 @@ void adjoint_reverse(const Ctx &c, const AdjWork &w, const RotorDev *rot, const 
     // stage 2: W' = P + dt^2/3 Lt(W*)
     const bool f32 = w.gp_bytes == 4;
     const UpdFactors k2 = {0.0, 0.0, 0.0, dt * dt / 3.0}, k1 = {0.5 * dt, dt, 0.125 * dt * dt, dt * dt / 6.0};
-    if (f32)
-        rev_update_kernel<float, 2><<<gcell, blk, 0, c.stream>>>(nullptr, w.lamP, nullptr, nullptr, (float *)w.lamLt, k2,
-                                                                 c.np, c.n[0], c.n[1], c.P[0], c.P[1]);
+    const bool xt = w.A0f != nullptr;   // the fused FP32 reverse
+    if (xt)
+        rev_update_kernel<float, 2, true><<<gcell, blk, 0, c.stream>>>(nullptr, w.lamP, nullptr, nullptr, (float *)w.lamLt,
+                                                                       k2, c.np, c.n[0], c.n[1], c.P[0], c.P[1]);
+    else if (f32)
+        rev_update_kernel<float, 2, false><<<gcell, blk, 0, c.stream>>>(nullptr, w.lamP, nullptr, nullptr, (float *)w.lamLt,
+                                                                        k2, c.np, c.n[0], c.n[1], c.P[0], c.P[1]);
     else
-        rev_update_kernel<double, 2><<<gcell, blk, 0, c.stream>>>(nullptr, w.lamP, nullptr, nullptr, w.lamLt, k2, c.np,
-                                                                  c.n[0], c.n[1], c.P[0], c.P[1]);
+        rev_update_kernel<double, 2, false><<<gcell, blk, 0, c.stream>>>(nullptr, w.lamP, nullptr, nullptr, w.lamLt, k2,
+                                                                         c.np, c.n[0], c.n[1], c.P[0], c.P[1]);
     cudaMemsetAsync(w.lamA, 0, bytes4, c.stream);
     if (w.A0f)
         spatial_adjoint_fused32(c, w, w.Wsf, nullptr, (const float *)w.lamLt);
@@ -2059,12 +2148,17 @@ void adjoint_reverse(const Ctx &c, const AdjWork &w, const RotorDev *rot, const 
         spatial(c, w, w.Ws, w.gps[1], nullptr, w.lamLt);
     ghost_adjoint(c, w, w.Ws);
     // stage 1: lamA (interior) is lambda of W*
-    if (f32)
-        rev_update_kernel<float, 1><<<gcell, blk, 0, c.stream>>>(w.lamA, w.lamP, w.lamW, (float *)w.lamL, (float *)w.lamLt,
-                                                                 k1, c.np, c.n[0], c.n[1], c.P[0], c.P[1]);
+    if (xt)
+        rev_update_kernel<float, 1, true><<<gcell, blk, 0, c.stream>>>(w.lamA, w.lamP, w.lamW, (float *)w.lamL,
+                                                                       (float *)w.lamLt, k1, c.np, c.n[0], c.n[1], c.P[0],
+                                                                       c.P[1]);
+    else if (f32)
+        rev_update_kernel<float, 1, false><<<gcell, blk, 0, c.stream>>>(w.lamA, w.lamP, w.lamW, (float *)w.lamL,
+                                                                        (float *)w.lamLt, k1, c.np, c.n[0], c.n[1], c.P[0],
+                                                                        c.P[1]);
     else
-        rev_update_kernel<double, 1><<<gcell, blk, 0, c.stream>>>(w.lamA, w.lamP, w.lamW, w.lamL, w.lamLt, k1, c.np,
-                                                                  c.n[0], c.n[1], c.P[0], c.P[1]);
+        rev_update_kernel<double, 1, false><<<gcell, blk, 0, c.stream>>>(w.lamA, w.lamP, w.lamW, w.lamL, w.lamLt, k1, c.np,
+                                                                         c.n[0], c.n[1], c.P[0], c.P[1]);
     cudaMemsetAsync(w.lamA, 0, bytes4, c.stream);
     if (w.A0f)
         spatial_adjoint_fused32(c, w, w.A0f, (const float *)w.lamL, (const float *)w.lamLt);
