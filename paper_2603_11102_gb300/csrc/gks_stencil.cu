@@ -220,10 +220,30 @@ struct FaceEqArgs {
     Phys<C> ph;      // in the compute type
 };
 
-// Faces per thread of the marching face-state kernels: FP32 (packed) and
-// FP64 / double-single (the longer march halves the FP32 kernel's window
-// warm-up at the same speed of the march itself).
-constexpr int kMarch32 = 32, kMarch = 16;
+// Blocks of the face-state kernels (ALL: of the launch of all directions):
+// threads, blocks that fit on an SM, and how few of them keep it as busy. FP32
+// with 64, 128, 256 threads: 1.87, 1.83, 1.89 ms a step of 384x256x256;
+// double-single with 64 and 256 1.07 and 1.00 ms on 96^3, 0.076 and 0.108 in the
+// launch of all directions of 32^3, whose few blocks spread better when small.
+// FP64: 12 warps at 168 registers are what the FP64 pipe's latency needs (16 at
+// 128 registers spill, 3.42 against 3.14 ms).
+template <typename C, bool ALL>
+constexpr int kEqThreads = ALL || std::is_same<C, double>::value ? 64 : std::is_same<C, dsf>::value ? 256 : 128;
+template <typename C, bool ALL>
+constexpr int kEqBlocks = std::is_same<C, float>::value ? (ALL ? 8 : 6) : std::is_same<C, dsf>::value ? (ALL ? 8 : 2) : 6;
+template <typename C, bool ALL>
+constexpr int kEqBusy = std::is_same<C, float>::value ? (ALL ? 1 : 6) : std::is_same<C, dsf>::value ? (ALL ? 6 : 2) : 5;
+
+// A block takes consecutive positions of the extended face plane, t1 fastest,
+// whatever its width: 32 x 8 blocks leave a fifth of the lanes idle on the
+// 132 x 132 positions of a 128^3 grid and half of them on 36 x 36.
+__device__ __forceinline__ bool face_position(unsigned p, int n1, int n2, int &a, int &b)
+{
+    const unsigned r = p / (unsigned)(n1 + 4);
+    a = (int)(p - r * (unsigned)(n1 + 4)) - 2;
+    b = (int)r - 2;
+    return b < n2 + 2;
+}
 
 // Marching variant: each thread walks K consecutive faces along d at one
 // tangential position of the extended face box, with the differences around
@@ -232,12 +252,11 @@ constexpr int kMarch32 = 32, kMarch = 16;
 // right-face value of cell f-1 and the left-face value of cell f. Launched
 // for FP64 grids in FP64 arithmetic; FP32 grids and double-single arithmetic
 // take the packed variants below, which march the same way.
-__device__ __forceinline__ void face_eq_march(const FaceEqArgs<double, double> &A, int3 blk)
+__device__ __forceinline__ void face_eq_march(const FaceEqArgs<double, double> &A, int2 blk)
 {
-    const int a = (int)(blk.x * 32 + threadIdx.x) - 2;
-    const int b = (int)(blk.y * 8 + threadIdx.y) - 2;
-    const int f0 = blk.z * A.K;
-    if (a >= A.n1 + 2 || b >= A.n2 + 2 || f0 >= A.nf) return;
+    int a, b;
+    const int f0 = blk.y * A.K;
+    if (!face_position((unsigned)blk.x * blockDim.x + threadIdx.x, A.n1, A.n2, a, b) || f0 >= A.nf) return;
     const int f1 = min(f0 + A.K, A.nf);
     const long base = (long)(a + G) * A.s1 + (long)(b + G) * A.s2;   // cell index along d = -G
     // cells f0-3 .. f1+1 are read, faces f0 .. f1-1 written
@@ -292,17 +311,17 @@ __device__ __forceinline__ void face_eq_march(const FaceEqArgs<double, double> &
 //
 // SEG (the x faces, whose cells are consecutive along the march but a row
 // apart across t1): a warp's lanes are 4 consecutive march segments of K
-// faces times 8 rows along t1, so that the rows a warp walks (8 per
-// component instead of 32) stay in L1 for the K faces that reuse each sector;
-// a store of the face box still writes 4 whole sectors (8 rows of 4
-// segments).
+// faces times 8 positions, so that the rows a warp walks (8 per component
+// instead of 32) stay in L1 for the K faces that reuse each sector; a store
+// of the face box still writes 4 whole sectors (8 rows of 4 segments).
 template <bool SEG>
-__device__ __forceinline__ void face_eq_f2(const FaceEqArgs<float, float> &A, int3 blk)
+__device__ __forceinline__ void face_eq_f2(const FaceEqArgs<float, float> &A, int2 blk)
 {
-    const int a = SEG ? (int)(blk.x * 8 + (threadIdx.x & 7)) - 2 : (int)(blk.x * 32 + threadIdx.x) - 2;
-    const int b = (int)(blk.y * 8 + threadIdx.y) - 2;
-    const int f0 = SEG ? (int)(blk.z * 4 + (threadIdx.x >> 3)) * A.K : blk.z * A.K;
-    if (a >= A.n1 + 2 || b >= A.n2 + 2 || f0 >= A.nf) return;
+    const int t = threadIdx.x;
+    int a, b;
+    const int f0 = SEG ? (blk.y * 4 + ((t >> 3) & 3)) * A.K : blk.y * A.K;
+    if (!face_position((unsigned)blk.x * (SEG ? blockDim.x / 4 : blockDim.x) + (SEG ? (t >> 5) * 8 + (t & 7) : t), A.n1, A.n2, a, b) || f0 >= A.nf)
+        return;
     const int f1 = min(f0 + A.K, A.nf);
     const long base = (long)(a + G) * A.s1 + (long)(b + G) * A.s2;   // cell index along d = -G
     // cells f0-3 .. f1+1 are read, faces f0 .. f1-1 written
@@ -359,12 +378,11 @@ __device__ __forceinline__ void face_eq_f2(const FaceEqArgs<float, float> &A, in
 // half-space terms of the left and right states as one pair, the normal
 // slopes paired like the components. Every lane takes the operations of the
 // scalar double-single kernel, so the face boxes have the same bits.
-__device__ __forceinline__ void face_eq_ds2(const FaceEqArgs<double, dsf> &A, int3 blk)
+__device__ __forceinline__ void face_eq_ds2(const FaceEqArgs<double, dsf> &A, int2 blk)
 {
-    const int a = (int)(blk.x * 32 + threadIdx.x) - 2;
-    const int b = (int)(blk.y * 8 + threadIdx.y) - 2;
-    const int f0 = blk.z * A.K;
-    if (a >= A.n1 + 2 || b >= A.n2 + 2 || f0 >= A.nf) return;
+    int a, b;
+    const int f0 = blk.y * A.K;
+    if (!face_position((unsigned)blk.x * blockDim.x + threadIdx.x, A.n1, A.n2, a, b) || f0 >= A.nf) return;
     const int f1 = min(f0 + A.K, A.nf);
     const long base = (long)(a + G) * A.s1 + (long)(b + G) * A.s2;   // cell index along d = -G
     // cells f0-3 .. f1+1 are read, faces f0 .. f1-1 written
@@ -421,28 +439,71 @@ __device__ __forceinline__ void face_eq_ds2(const FaceEqArgs<double, dsf> &A, in
     }
 }
 
-// Blocks of the face-state launch of one direction: FP32 x faces (unit stride
-// along the normal) by march segments of at most 8 faces, 4 per warp.
-template <typename R, typename C>
-dim3 face_eq_blocks(FaceEqArgs<R, C> &E, int d)
+// Blocks of a face plane with `threads` threads (FP32 x faces: 4 segments a
+// warp, a quarter of the positions).
+inline int face_eq_plane(bool seg, int threads, int n1, int n2)
 {
-    if (std::is_same<C, float>::value && d == 0) {
-        E.K = std::min(E.K, 8);
-        return dim3((E.n1 + 4 + 7) / 8, (E.n2 + 4 + 7) / 8, (E.nf + 4 * E.K - 1) / (4 * E.K));
+    const int per = seg ? threads / 4 : threads;
+    return (int)(((long)(n1 + 4) * (n2 + 4) + per - 1) / per);
+}
+// Blocks of the face-state launch of one direction, along the plane and the march.
+template <typename R, typename C, bool ALL>
+dim3 face_eq_blocks(const FaceEqArgs<R, C> &E, int d)
+{
+    const bool seg = std::is_same<C, float>::value && d == 0;
+    const int k = seg ? 4 * E.K : E.K;
+    return dim3(face_eq_plane(seg, kEqThreads<C, ALL>, E.n1, E.n2), (E.nf + k - 1) / k);
+}
+
+// Faces per thread of the marching face-state kernels, for the directions of
+// one launch: of all lengths of the march that cut the faces into equal
+// segments, the one with the least work on the busiest SM, K faces and about
+// one to start the window for each of its blocks; fewer blocks than fit, and a
+// last wave of fewer than kEqBusy, take as long as those. (Halving a fixed
+// length until the launch had two blocks to an SM left 680 FP64 blocks of
+// 128^3 on 152 SMs.) The x segments of FP32 grids are 4 or 8 faces: whole
+// sectors, 4 of them a line; 9 faces, which fill the blocks better, took 0.39
+// against 0.36 ms a step of 256x128x128. Face state of a step with this rule and
+// face_position, before and now: FP64 128^3 8.94 -> 6.61 ms and 32^3 0.349 ->
+// 0.181, double-single 96^3 1.41 -> 1.00, FP32C 384x256x256 1.896 -> 1.830,
+// 256x128x128 0.360 -> 0.347, 128^3 0.210 -> 0.203, 32^3 0.0187 -> 0.0165.
+template <typename R, typename C, bool ALL>
+void march_faces(FaceEqArgs<R, C> *E, const int *dir, int nd)
+{
+    constexpr bool F32 = std::is_same<C, float>::value;
+    constexpr long fit = kEqBlocks<C, ALL>, busy = kEqBusy<C, ALL>;
+    const int sms = sm_count();
+    long best = -1;
+    for (int K = 4; K <= 128; ++K) {
+        long blocks = 0;
+        int most = 0, k[3];
+        for (int i = 0; i < nd; ++i) {
+            const bool seg = F32 && dir[i] == 0;
+            const int per = seg ? 4 : 1, Ks = seg ? (K < 8 ? 4 : 8) : K;
+            const int S = (E[i].nf + per * Ks - 1) / (per * Ks);
+            k[i] = seg ? Ks : (E[i].nf + S - 1) / S;
+            blocks += (long)face_eq_plane(seg, kEqThreads<C, ALL>, E[i].n1, E[i].n2) * S;
+            most = std::max(most, k[i]);
+        }
+        const long m = (blocks + sms - 1) / sms, last = m % fit;   // of the busiest SM, in its last wave
+        const long cost = (m <= fit ? fit : m - last + (last ? std::max(last, busy) : 0)) * (most + (F32 && !ALL && dir[0] == 0 ? 2 : 1));
+        if (best < 0 || cost < best) {
+            best = cost;
+            for (int i = 0; i < nd; ++i) E[i].K = k[i];
+        }
     }
-    return dim3((E.n1 + 4 + 31) / 32, (E.n2 + 4 + 7) / 8, (E.nf + E.K - 1) / E.K);
 }
 
 template <bool SEG>
-__global__ void __launch_bounds__(256, 3) face_eq_f2_kernel(FaceEqArgs<float, float> A)
+__global__ void __launch_bounds__(kEqThreads<float, false>, kEqBlocks<float, false>) face_eq_f2_kernel(FaceEqArgs<float, float> A)
 {
-    face_eq_f2<SEG>(A, make_int3(blockIdx.x, blockIdx.y, blockIdx.z));
+    face_eq_f2<SEG>(A, make_int2(blockIdx.x, blockIdx.y));
 }
 template <typename C>
-__global__ void __launch_bounds__(256, std::is_same<C, dsf>::value ? 2 : 1)
+__global__ void __launch_bounds__(kEqThreads<C, false>, kEqBlocks<C, false>)
     face_eq_kernel(const __grid_constant__ FaceEqArgs<double, C> A)
 {
-    const int3 blk = make_int3(blockIdx.x, blockIdx.y, blockIdx.z);
+    const int2 blk = make_int2(blockIdx.x, blockIdx.y);
     if constexpr (std::is_same<C, dsf>::value)
         face_eq_ds2(A, blk);
     else
@@ -452,14 +513,15 @@ __global__ void __launch_bounds__(256, std::is_same<C, dsf>::value ? 2 : 1)
 template <typename R, typename C>
 void launch_face_eq(FaceEqArgs<R, C> E, int d, cudaStream_t stream)
 {
-    const dim3 g = face_eq_blocks(E, d), blk(TX, TY);
+    march_faces<R, C, false>(&E, &d, 1);
+    const dim3 g = face_eq_blocks<R, C, false>(E, d);
     if constexpr (std::is_same<C, float>::value) {
         if (d == 0)
-            face_eq_f2_kernel<true><<<g, blk, 0, stream>>>(E);
+            face_eq_f2_kernel<true><<<g, kEqThreads<C, false>, 0, stream>>>(E);
         else
-            face_eq_f2_kernel<false><<<g, blk, 0, stream>>>(E);
+            face_eq_f2_kernel<false><<<g, kEqThreads<C, false>, 0, stream>>>(E);
     } else {
-        face_eq_kernel<C><<<g, blk, 0, stream>>>(E);
+        face_eq_kernel<C><<<g, kEqThreads<C, false>, 0, stream>>>(E);
     }
 }
 
@@ -468,17 +530,16 @@ void launch_face_eq(FaceEqArgs<R, C> E, int d, cudaStream_t stream)
 template <typename R, typename C>
 struct FaceEq3 {
     FaceEqArgs<R, C> d[3];
-    int gx[3], gy[3], first[4];   // blocks along t1 and t2 of each direction, its first block
+    int gx[3], first[4];   // blocks of a face plane of each direction, its first block
 };
 template <typename R, typename C>
-__global__ void __launch_bounds__(256, std::is_same<C, double>::value ? 1 : 2)
+__global__ void __launch_bounds__(kEqThreads<C, true>, kEqBlocks<C, true>)
     face_eq_all_kernel(const __grid_constant__ FaceEq3<R, C> E)
 {
     int b = blockIdx.x;
     const int d = b < E.first[1] ? 0 : (b < E.first[2] ? 1 : 2);
     b -= E.first[d];
-    const int r = b / E.gx[d];
-    const int3 blk = make_int3(b - r * E.gx[d], r % E.gy[d], r / E.gy[d]);
+    const int2 blk = make_int2(b % E.gx[d], b / E.gx[d]);
     if constexpr (std::is_same<C, float>::value) {
         if (d == 0)
             face_eq_f2<true>(E.d[0], blk);
@@ -1415,21 +1476,6 @@ __global__ void __launch_bounds__(256) update_kernel(const __grid_constant__ Upd
         U.scal->t = U.scal->t + dt;
 }
 
-// Faces per thread of the marching face-state kernel: k0 (kMarch32 or
-// kMarch), halved (down to 4) while the launch would have fewer than
-// min_per_sm blocks per SM, so that a smaller grid spreads its march over
-// more resident blocks (each halving adds one WENO5 pair per thread to warm
-// the window up). The packed FP32 kernel (3 blocks per SM) asks for 9, three
-// waves: measured on 128^3, 192^3 and 384x256x256 grids this picked the
-// fastest of 8, 16 and 32 faces each time (0.045, 0.122, 0.383 ms per
-// launch). The FP64 kernels ask for 2.
-int march_faces(long blocks_xy, int nf, int k0, int min_per_sm)
-{
-    int K = k0;
-    while (K > 4 && blocks_xy * ((nf + K - 1) / K) < (long)min_per_sm * sm_count()) K /= 2;
-    return K;
-}
-
 template <typename K>
 int persistent_grid(K kernel, size_t smem)
 {
@@ -1501,9 +1547,7 @@ FaceEqArgs<R, C> face_eq_args(const Ctx &c, int d, const R *w, const Phys<C> &ph
     E.c2 = 1 + t2;
     E.ph = ph;
     E.nf = c.n[d] + 1;
-    constexpr bool F32 = std::is_same<C, float>::value;
-    E.K = march_faces((long)((E.n1 + 4 + 31) / 32) * ((E.n2 + 4 + 7) / 8), E.nf, F32 ? kMarch32 : kMarch,
-                      F32 ? 9 : 2);
+    E.K = 1;
     return E;
 }
 
@@ -1630,22 +1674,17 @@ void stage_impl(const Ctx &c)
     if (c.small) {
         // all directions at once: their face boxes have buffers of their own
         FaceEq3<R, C> E;
-        long blocks = 0;
-        for (int d = 0; d < 3; ++d) {
-            E.d[d] = face_eq_args<R, C>(c, d, w, ph);
-            blocks += (long)((E.d[d].n1 + 4 + 31) / 32) * ((E.d[d].n2 + 4 + 7) / 8);
-        }
+        const int dirs[3] = {0, 1, 2};
+        for (int d = 0; d < 3; ++d) E.d[d] = face_eq_args<R, C>(c, d, w, ph);
+        march_faces<R, C, true>(E.d, dirs, 3);
         E.first[0] = 0;
         for (int d = 0; d < 3; ++d) {
-            constexpr bool F32 = std::is_same<C, float>::value;
-            E.d[d].K = march_faces(blocks, E.d[d].nf, F32 ? kMarch32 : kMarch, F32 ? 9 : 2);
-            const dim3 g = face_eq_blocks(E.d[d], d);
+            const dim3 g = face_eq_blocks<R, C, true>(E.d[d], d);
             E.gx[d] = g.x;
-            E.gy[d] = g.y;
-            E.first[d + 1] = E.first[d] + g.x * g.y * g.z;
+            E.first[d + 1] = E.first[d] + g.x * g.y;
         }
         mark(c, K_FACE_EQ, 1);
-        face_eq_all_kernel<R, C><<<E.first[3], dim3(TX, TY), 0, c.stream>>>(E);
+        face_eq_all_kernel<R, C><<<E.first[3], kEqThreads<C, true>, 0, c.stream>>>(E);
         mark(c, K_FACE_EQ, 0);
         FluxMaps<3> maps;
         FluxLaunch<R, C, 3> F;
