@@ -817,69 +817,86 @@ __device__ __forceinline__ void sts4(dsf *p, const dsf q[4])
     reinterpret_cast<float4 *>(p)[1] = make_float4(q[2].hi, q[2].lo, q[3].hi, q[3].lo);
 }
 
-static_assert(TX * TY == 256 && SQ_H == 12 && TX == 32, "t1-pass task split assumes 32 x 8 tiles");
+static_assert(TX * TY == 256 && TY == 8 && SQ_H == 12 && TX == 32, "t1-pass task split assumes 32 x 8 tiles");
 
-// t1 pass of one tile of H rows (with the tangential halo): values and
-// t1-derivatives of Q0, values of the normal slope, at the two t1 Gauss
-// points, for every row of the tile. 64 H equal tasks (Q0 or slope,
-// component, row, group of 4 columns), H / 4 per thread: a task reads 8
-// consecutive values of its row and writes 4 columns; the lanes of a warp
-// share the kind and the component (8 H is a multiple of 32).
-template <typename R, typename C, int H = SQ_H>
-__device__ __forceinline__ void tile_t1_pass(const R *sq, C *st, int tid)
+// Physical row of row r (0 <= r < 2 SQ_H) of a tile's t1 results, a ring of
+// SQ_H rows.
+__device__ __forceinline__ int ring_row(int r) { return r < SQ_H ? r : r - SQ_H; }
+
+// One task of the t1 pass: a group of 4 columns of row r of a face-box tile,
+// values and t1-derivatives of Q0 (kind 0) or values of the normal slope of
+// component v at the two t1 Gauss points, into row rp of st. It reads 8
+// consecutive values and writes 4 columns.
+template <typename R, typename C>
+__device__ __forceinline__ void t1_task(const R *sq, C *st, int kind, int v, int r, int rp, int cg)
 {
-    static_assert(H % 4 == 0, "a warp's tasks share kind and component");
-    constexpr int NQ = 32 * H, NV = 8 * H, ROWS = H * TX;
+    constexpr int ROWS = SQ_H * TX;
+    C q[8];
+    lds8(sq + ((kind * 4 + v) * SQ_H + r) * SQ_W + 4 * cg, q);
+    C *o = st + rp * TX + 4 * cg;
+    if constexpr (std::is_same<C, dsf>::value) {
+        dsf x[4][4];
+        if (kind == 0) {
+            dsf D[7];
 #pragma unroll
-    for (int j = 0; j < H / 4; ++j) {
-        const int task = tid + j * 256;
-        const int kind = task >= NQ, rem = task - kind * NQ, v = rem / NV, rc = rem - v * NV;
-        const int r = rc >> 3, cg = rc & 7;
-        C q[8];
-        lds8(sq + ((kind * 4 + v) * H + r) * SQ_W + 4 * cg, q);
-        C *o = st + r * TX + 4 * cg;
-        if constexpr (std::is_same<C, dsf>::value) {
-            dsf x[4][4];
-            if (kind == 0) {
-                dsf D[7];
+            for (int i = 0; i < 7; ++i) D[i] = q[i + 1] - q[i];
 #pragma unroll
-                for (int i = 0; i < 7; ++i) D[i] = q[i + 1] - q[i];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    dsf2 val, der;
-                    ds_val_der<false>(q[i + 2], D + i, val, der);
-                    x[0][i] = val.lane(0);
-                    x[1][i] = val.lane(1);
-                    x[2][i] = der.lane(0);
-                    x[3][i] = der.lane(1);
-                }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) sts4(o + (v * 4 + k) * ROWS, x[k]);
-            } else {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const dsf2 val = ds_val_direct<false>(q + i);
-                    x[0][i] = val.lane(0);
-                    x[1][i] = val.lane(1);
-                }
-                sts4(o + (16 + v * 2 + 0) * ROWS, x[0]);
-                sts4(o + (16 + v * 2 + 1) * ROWS, x[1]);
+            for (int i = 0; i < 4; ++i) {
+                dsf2 val, der;
+                ds_val_der<false>(q[i + 2], D + i, val, der);
+                x[0][i] = val.lane(0);
+                x[1][i] = val.lane(1);
+                x[2][i] = der.lane(0);
+                x[3][i] = der.lane(1);
             }
-        } else if (kind == 0) {
-            C vm[4], vp[4], dm[4], dp[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) tan_val_der(q[i], q[i + 1], q[i + 2], q[i + 3], q[i + 4], vm[i], vp[i], dm[i], dp[i]);
-            sts4(o + (v * 4 + 0) * ROWS, vm);
-            sts4(o + (v * 4 + 1) * ROWS, vp);
-            sts4(o + (v * 4 + 2) * ROWS, dm);
-            sts4(o + (v * 4 + 3) * ROWS, dp);
+            for (int k = 0; k < 4; ++k) sts4(o + (v * 4 + k) * ROWS, x[k]);
         } else {
-            C vm[4], vp[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) tan_val_direct(q[i], q[i + 1], q[i + 2], q[i + 3], q[i + 4], vm[i], vp[i]);
-            sts4(o + (16 + v * 2 + 0) * ROWS, vm);
-            sts4(o + (16 + v * 2 + 1) * ROWS, vp);
+            for (int i = 0; i < 4; ++i) {
+                const dsf2 val = ds_val_direct<false>(q + i);
+                x[0][i] = val.lane(0);
+                x[1][i] = val.lane(1);
+            }
+            sts4(o + (16 + v * 2 + 0) * ROWS, x[0]);
+            sts4(o + (16 + v * 2 + 1) * ROWS, x[1]);
         }
+    } else if (kind == 0) {
+        C vm[4], vp[4], dm[4], dp[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) tan_val_der(q[i], q[i + 1], q[i + 2], q[i + 3], q[i + 4], vm[i], vp[i], dm[i], dp[i]);
+        sts4(o + (v * 4 + 0) * ROWS, vm);
+        sts4(o + (v * 4 + 1) * ROWS, vp);
+        sts4(o + (v * 4 + 2) * ROWS, dm);
+        sts4(o + (v * 4 + 3) * ROWS, dp);
+    } else {
+        C vm[4], vp[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) tan_val_direct(q[i], q[i + 1], q[i + 2], q[i + 3], q[i + 4], vm[i], vp[i]);
+        sts4(o + (16 + v * 2 + 0) * ROWS, vm);
+        sts4(o + (16 + v * 2 + 1) * ROWS, vp);
+    }
+}
+
+// t1 pass of the last H rows of a face-box tile into the ring of rows, whose
+// first tile row stands at `off`: 64 H equal tasks, H / 4 per thread; the
+// lanes of a warp share the kind and the component and take 4 rows. The
+// double-single task is long and not unrolled (one copy for every H).
+template <typename R, typename C>
+__device__ __forceinline__ void tile_t1_pass(const R *sq, C *st, int tid, int H, int off)
+{
+    const int per = H >> 2, lane = tid & 31;
+    auto round = [&](int j) {
+        const int wt = (tid >> 5) + 8 * j, kv = H == TY ? wt >> 1 : wt / 3, r = SQ_H - H + 4 * (wt - kv * per) + (lane >> 3);
+        t1_task(sq, st, kv >> 2, kv & 3, r, ring_row(r + off), lane & 7);
+    };
+    if constexpr (std::is_same<C, dsf>::value) {
+#pragma unroll 1
+        for (int j = 0; j < per; ++j) round(j);
+    } else {
+        round(0);
+        round(1);
+        if (H == SQ_H) round(2);
     }
 }
 

@@ -594,27 +594,28 @@ __device__ __forceinline__ dsf face_avg_neg(dsf s) { return scale_pow2(s, -0.25f
 // slope at the two t2 Gauss points -g, +g (k = 0, 1); the density's slopes
 // negated, as gk_flux takes them.
 template <int V>
-__device__ __forceinline__ void t2_pass(const double *st, int m, int tx, int ty, double q[2], double dn[2], double d1[2],
+__device__ __forceinline__ void t2_pass(const double *st, int m, const int ro[5], double q[2], double dn[2], double d1[2],
                                         double d2[2])
 {
     using R = double;
     constexpr bool NEG = V == 0;
-    const R *x = st + (V * 4 + m) * ST_ROWS + ty * TX + tx;
-    const R *y = st + (V * 4 + 2 + m) * ST_ROWS + ty * TX + tx;
-    const R *z = st + (16 + V * 2 + m) * ST_ROWS + ty * TX + tx;
-    tan_val_der<R, NEG>(x[0], x[TX], x[2 * TX], x[3 * TX], x[4 * TX], q[0], q[1], d2[0], d2[1]);
-    tan_val_direct<R, NEG>(y[0], y[TX], y[2 * TX], y[3 * TX], y[4 * TX], d1[0], d1[1]);
-    tan_val_direct<R, NEG>(z[0], z[TX], z[2 * TX], z[3 * TX], z[4 * TX], dn[0], dn[1]);
+    const R *x = st + (V * 4 + m) * ST_ROWS;
+    const R *y = st + (V * 4 + 2 + m) * ST_ROWS;
+    const R *z = st + (16 + V * 2 + m) * ST_ROWS;
+    tan_val_der<R, NEG>(x[ro[0]], x[ro[1]], x[ro[2]], x[ro[3]], x[ro[4]], q[0], q[1], d2[0], d2[1]);
+    tan_val_direct<R, NEG>(y[ro[0]], y[ro[1]], y[ro[2]], y[ro[3]], y[ro[4]], d1[0], d1[1]);
+    tan_val_direct<R, NEG>(z[ro[0]], z[ro[1]], z[ro[2]], z[ro[3]], z[ro[4]], dn[0], dn[1]);
 }
 
 // t2 pass at each t1 Gauss point m, then the flux at (m, -g), (m, +g): the
-// sums of F0 and of -F1 over the 4 Gauss points of face (tx, ty) of the tile.
+// sums of F0 and of -F1 over the 4 Gauss points of a face, whose 5 rows of t1
+// results stand at st + ro[i].
 // GP (the recorded steps of the adjoint) with gp set: the inputs of Gauss
 // point g = 2m + n (Q0 with its density as rho; normal slope, t1 and t2
 // slopes; 4 components each) go to gp[(16 g + k) ngp + face], as double or
 // (gp32) rounded to float.
 template <bool NEED_F0, bool GP = false>
-__device__ __forceinline__ void tile_gauss_flux(const FluxPhys<double> &ph, const double *st, int tx, int ty, double ih1,
+__device__ __forceinline__ void tile_gauss_flux(const FluxPhys<double> &ph, const double *st, const int ro[5], double ih1,
                                                 double ih2, double acc0[4], double acc1[4], void *gp = nullptr,
                                                 int gp32 = 0, long ngp = 0, long face = 0)
 {
@@ -623,10 +624,10 @@ __device__ __forceinline__ void tile_gauss_flux(const FluxPhys<double> &ph, cons
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
         double t[4][4][2];   // [Q0, normal slope, t1 slope, t2 slope][component][t2 Gauss point]
-        t2_pass<0>(st, m, tx, ty, t[0][0], t[1][0], t[2][0], t[3][0]);
-        t2_pass<1>(st, m, tx, ty, t[0][1], t[1][1], t[2][1], t[3][1]);
-        t2_pass<2>(st, m, tx, ty, t[0][2], t[1][2], t[2][2], t[3][2]);
-        t2_pass<3>(st, m, tx, ty, t[0][3], t[1][3], t[2][3], t[3][3]);
+        t2_pass<0>(st, m, ro, t[0][0], t[1][0], t[2][0], t[3][0]);
+        t2_pass<1>(st, m, ro, t[0][1], t[1][1], t[2][1], t[3][1]);
+        t2_pass<2>(st, m, ro, t[0][2], t[1][2], t[2][2], t[3][2]);
+        t2_pass<3>(st, m, ro, t[0][3], t[1][3], t[2][3], t[3][3]);
         if constexpr (GP) {
             if (gp) {
 #pragma unroll
@@ -691,37 +692,37 @@ __device__ __forceinline__ void tile_gauss_flux_f2(const FluxPhys<f2> &ph, const
 // same t2 pass, the flux at the two t2 Gauss points of each t1 Gauss point
 // as one evaluation on packed double-single pairs.
 template <int V>
-__device__ __forceinline__ void t2_pass_ds2(const dsf *st, int m, int tx, int ty, dsf2 &q, dsf2 &dn, dsf2 &d1, dsf2 &d2)
+__device__ __forceinline__ void t2_pass_ds2(const dsf *st, int m, const int ro[5], dsf2 &q, dsf2 &dn, dsf2 &d1, dsf2 &d2)
 {
     constexpr bool NEG = V == 0;
-    const dsf *x = st + (V * 4 + m) * ST_ROWS + ty * TX + tx;
-    const dsf *y = st + (V * 4 + 2 + m) * ST_ROWS + ty * TX + tx;
-    const dsf *z = st + (16 + V * 2 + m) * ST_ROWS + ty * TX + tx;
+    const dsf *x = st + (V * 4 + m) * ST_ROWS;
+    const dsf *y = st + (V * 4 + 2 + m) * ST_ROWS;
+    const dsf *z = st + (16 + V * 2 + m) * ST_ROWS;
     dsf p[5], D[4];
 #pragma unroll
-    for (int i = 0; i < 5; ++i) p[i] = x[i * TX];
+    for (int i = 0; i < 5; ++i) p[i] = x[ro[i]];
 #pragma unroll
     for (int i = 0; i < 4; ++i) D[i] = p[i + 1] - p[i];
     ds_val_der<NEG>(p[2], D, q, d2);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) p[i] = y[i * TX];
+    for (int i = 0; i < 5; ++i) p[i] = y[ro[i]];
     d1 = ds_val_direct<NEG>(p);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) p[i] = z[i * TX];
+    for (int i = 0; i < 5; ++i) p[i] = z[ro[i]];
     dn = ds_val_direct<NEG>(p);
 }
 template <bool NEED_F0>
-__device__ __forceinline__ void tile_gauss_flux_ds2(const FluxPhys<dsf2> &ph, const dsf *st, int tx, int ty, dsf ih1,
+__device__ __forceinline__ void tile_gauss_flux_ds2(const FluxPhys<dsf2> &ph, const dsf *st, const int ro[5], dsf ih1,
                                                     dsf ih2, dsf acc0[4], dsf acc1[4])
 {
     dsf2 s0[4], s1[4];   // the t2 Gauss points -g, +g in the lanes
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
         dsf2 Qv[4], Dn[4], D1[4], D2[4];
-        t2_pass_ds2<0>(st, m, tx, ty, Qv[0], Dn[0], D1[0], D2[0]);
-        t2_pass_ds2<1>(st, m, tx, ty, Qv[1], Dn[1], D1[1], D2[1]);
-        t2_pass_ds2<2>(st, m, tx, ty, Qv[2], Dn[2], D1[2], D2[2]);
-        t2_pass_ds2<3>(st, m, tx, ty, Qv[3], Dn[3], D1[3], D2[3]);
+        t2_pass_ds2<0>(st, m, ro, Qv[0], Dn[0], D1[0], D2[0]);
+        t2_pass_ds2<1>(st, m, ro, Qv[1], Dn[1], D1[1], D2[1]);
+        t2_pass_ds2<2>(st, m, ro, Qv[2], Dn[2], D1[2], D2[2]);
+        t2_pass_ds2<3>(st, m, ro, Qv[3], Dn[3], D1[3], D2[3]);
         dsf2 F0[4], F1[4];
         gk_flux<dsf2, NEED_F0>(ph, Qv, Dn, D1, D2, dsf2(ih1), dsf2(ih2), F0, F1);
 #pragma unroll
@@ -737,10 +738,15 @@ __device__ __forceinline__ void tile_gauss_flux_ds2(const FluxPhys<dsf2> &ph, co
     }
 }
 
-// Persistent: each block walks tiles blockIdx.x, +gridDim.x, ...; the face
+// Persistent: each block takes a run of consecutive tiles, t2 fastest; the face
 // box of a tile is dead once its t1 pass is in shared memory, so the next
 // tile's face box is fetched by TMA into the same buffer while the Gauss
 // points of the current one are computed (one buffer: more blocks per SM).
+// A tile that follows its neighbour along t2 finds its first 4 rows of t1
+// results there (the rows are a ring of SQ_H, turned by TY a tile) and passes
+// only the 8 others, a third less of the t1 operations in kernels that the FP64
+// pipe (85 % busy) or the issue of double-single bounds: x and y fluxes of a step
+// of 128^3 FP64 11.2 -> 10.4 ms, of 96^3 double-single 1.22 -> 1.13 ms.
 struct TilePos {
     int t, d, f, a0, b0;   // tile, direction, face plane, first face along t1 and t2
 };
@@ -756,7 +762,9 @@ __global__ void __launch_bounds__(256, std::is_same<C, dsf>::value ? 2 : 1)
     C *st = reinterpret_cast<C *>(sq + SQ_N);
     uint64_t *bar = reinterpret_cast<uint64_t *>(st + ST_N);
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
-    const int ntiles = F.first[ND];
+    // runs of equal length, the first blocks (one to an SM) one tile more
+    const int run = F.first[ND] / (int)gridDim.x, more = F.first[ND] % (int)gridDim.x, blk = blockIdx.x;
+    const int t0 = blk * run + min(blk, more), tend = t0 + run + (blk < more);
     const uint32_t bytes = (uint32_t)(SQ_N * sizeof(R));
     auto tile = [&](int t) {
         TilePos p;
@@ -764,14 +772,14 @@ __global__ void __launch_bounds__(256, std::is_same<C, dsf>::value ? 2 : 1)
         p.d = ND == 1 ? 0 : (t < F.first[1] ? 0 : (t < F.first[ND - 1] ? 1 : ND - 1));
         const FluxArgs<R, C> &A = F.A[p.d];
         const int NA = (A.n1 + TX - 1) / TX, NB = (A.n2 + TY - 1) / TY;
-        const int l = t - F.first[p.d], r = l / NA;
-        p.a0 = (l - r * NA) * TX;
-        p.f = r / NB;
-        p.b0 = (r - p.f * NB) * TY;
+        const int l = t - F.first[p.d], r = l / NB;
+        p.b0 = (l - r * NB) * TY;
+        p.f = r / NA;
+        p.a0 = (r - p.f * NA) * TX;
         return p;
     };
     auto load = [&](const TilePos &p) {
-        if (tid == 0 && p.t < ntiles)
+        if (tid == 0 && p.t < tend)
             tma_load_tile(&maps.d[p.d], sq, &bar[0], p.a0, p.b0, p.f, bytes);
     };
     if (tid == 0) {
@@ -779,17 +787,20 @@ __global__ void __launch_bounds__(256, std::is_same<C, dsf>::value ? 2 : 1)
         mbar_fence_init();
     }
     __syncthreads();
-    TilePos cur = tile(blockIdx.x);
+    TilePos cur = tile(t0);
     load(cur);
-    for (int k = 0; cur.t < ntiles; ++k) {
-        const TilePos nxt = tile(cur.t + gridDim.x);
+    int off = 0;   // ring row of the tile's first row
+    for (int k = 0; cur.t < tend; ++k) {
+        const TilePos nxt = tile(cur.t + 1);
         const FluxArgs<R, C> &A = F.A[cur.d];
         const bool ok = mbar_wait(&bar[0], (uint32_t)(k & 1));
         if (__syncthreads_or(!ok)) {
             if (tid == 0) atomicOr(&A.scal->flags, FLAG_TIMEOUT);
             return;
         }
-        tile_t1_pass(sq, st, tid);
+        const bool next_to = k > 0 && cur.b0 > 0;   // the last tile's neighbour
+        off = next_to ? ring_row(off + TY) : 0;
+        tile_t1_pass(sq, st, tid, next_to ? TY : SQ_H, off);
         __syncthreads();
         // the face box is free: fetch the next tile's while this one's Gauss
         // points are computed
@@ -800,11 +811,14 @@ __global__ void __launch_bounds__(256, std::is_same<C, dsf>::value ? 2 : 1)
         if (a < A.n1 && b < A.n2) {
             const C ih1 = cvt<C>(__ldg(A.ih1 + a + G)), ih2 = cvt<C>(__ldg(A.ih2 + b + G));
             C acc0[4], acc1[4];
+            int ro[5];
+#pragma unroll
+            for (int i = 0; i < 5; ++i) ro[i] = ring_row(ty + i + off) * TX + tx;
             const long o = ((long)cur.f * A.n2 + b) * A.n1 + a;
             if constexpr (std::is_same<C, dsf>::value)
-                tile_gauss_flux_ds2<NEED_F0>(flux_phys_ds2(A.ph), st, tx, ty, ih1, ih2, acc0, acc1);
+                tile_gauss_flux_ds2<NEED_F0>(flux_phys_ds2(A.ph), st, ro, ih1, ih2, acc0, acc1);
             else
-                tile_gauss_flux<NEED_F0, GP>(flux_phys(A.ph), st, tx, ty, ih1, ih2, acc0, acc1, A.gp, A.gp32, A.ngp,
+                tile_gauss_flux<NEED_F0, GP>(flux_phys(A.ph), st, ro, ih1, ih2, acc0, acc1, A.gp, A.gp32, A.ngp,
                                              o);
 #pragma unroll
             for (int v = 0; v < 4; ++v) {

@@ -51,6 +51,20 @@ def test_face_kernels_at_tile_and_segment_edges(gks, n):
         g.close()
 
 
+@pytest.mark.parametrize("precision", ["fp64", "fp64ds"])
+@pytest.mark.parametrize("n", [(40, 50, 61), (33, 71, 45)], ids=lambda n: "%dx%dx%d" % n)
+def test_flux_tile_runs(gks, n, precision):
+    # several tiles to a block: runs that start inside a row of tiles along t2
+    # or pass from one row, plane or direction to the next
+    w = smooth_workload(n, [(2, 4), (0, 0), (1, 2)], seed=sum(n))
+    o = oracle_from_workload(w)
+    o.step(2)
+    g = grid(gks, w, precision)
+    g.step(2)
+    assert rel_linf(g.get_state(), o.get_state()) <= TOL[precision]
+    g.close()
+
+
 def raw_state(g):
     """The stored component arrays of a grid, (arrays, P2, P1, P0)."""
     import torch
