@@ -458,9 +458,9 @@ __global__ void __launch_bounds__(256) rev_t2_kernel(RevArgs A)
 template <typename T>
 __global__ void __launch_bounds__(256) rev_t1_kernel(RevArgs A)
 {
-    const int ap = (int)(blockIdx.x * 32 + threadIdx.x) - 2, bp = (int)(blockIdx.y * 8 + threadIdx.y) - 2;
-    const int f = blockIdx.z;
-    if (ap >= A.n1 + 2 || bp >= A.n2 + 2) return;
+    int ap, bp;
+    const int f = blockIdx.y;
+    if (!face_position(blockIdx.x * 256u + threadIdx.x, A.n1, A.n2, ap, bp)) return;
     T lq[4] = {0, 0, 0, 0}, ln[4] = {0, 0, 0, 0};
     const T *lr = (const T *)A.lamR;
     const int alo = ap - 2 < 0 ? 0 : ap - 2, ahi = ap + 2 > A.n1 - 1 ? A.n1 - 1 : ap + 2;
@@ -500,9 +500,9 @@ __global__ void __launch_bounds__(256) rev_face_state_kernel(RevArgs A)
     using T = double;
     const double *lamFQ = (const double *)A.lamFQ;
     double *lamC = (double *)A.lamC;
-    const int a = (int)(blockIdx.x * 32 + threadIdx.x) - 2, b = (int)(blockIdx.y * 8 + threadIdx.y) - 2;
-    const int nf = A.nd + 1, f0 = blockIdx.z * kRevMarch;
-    if (a >= A.n1 + 2 || b >= A.n2 + 2 || f0 >= nf) return;
+    int a, b;
+    const int nf = A.nd + 1, f0 = blockIdx.y * kRevMarch;
+    if (!face_position(blockIdx.x * 256u + threadIdx.x, A.n1, A.n2, a, b) || f0 >= nf) return;
     const int f1 = min(f0 + kRevMarch, nf);
     const long stride[3] = {1, (long)A.P[0], (long)A.P[0] * A.P[1]};
     const long sd = stride[A.d];
@@ -661,9 +661,9 @@ __global__ void __launch_bounds__(256) rev_face_state32_kernel(RevArgs A)
 {
     const float *lamFQ = (const float *)A.lamFQ;
     float *lamC = (float *)A.lamC;
-    const int a = (int)(blockIdx.x * 32 + threadIdx.x) - 2, b = (int)(blockIdx.y * 8 + threadIdx.y) - 2;
-    const int nf = A.nd + 1, f0 = blockIdx.z * kRevMarch;
-    if (a >= A.n1 + 2 || b >= A.n2 + 2 || f0 >= nf) return;
+    int a, b;
+    const int nf = A.nd + 1, f0 = blockIdx.y * kRevMarch;
+    if (!face_position(blockIdx.x * 256u + threadIdx.x, A.n1, A.n2, a, b) || f0 >= nf) return;
     const int f1 = min(f0 + kRevMarch, nf);
     const long stride[3] = {1, (long)A.P[0], (long)A.P[0] * A.P[1]};
     const long sd = stride[A.d];
@@ -797,11 +797,10 @@ __global__ void __launch_bounds__(256, 2) rev_face_cells32_kernel(RevArgs A, int
     RevSlot *ring = reinterpret_cast<RevSlot *>(smem_raw);
     const float *lamFQ = (const float *)A.lamFQ;
     const int tid = threadIdx.x;
-    const long pos = blockIdx.x * 256L + tid;
-    const int a = (int)(pos % (A.n1 + 4)) - 2, b = (int)(pos / (A.n1 + 4)) - 2;
+    int a, b;
     const int nf = A.nd + 1;
     const int c0 = (int)blockIdx.y * cells - G, c1 = min(c0 + cells, A.nd + G);
-    if (b >= A.n2 + 2 || c0 >= A.nd + G) return;
+    if (!face_position(blockIdx.x * 256u + tid, A.n1, A.n2, a, b) || c0 >= A.nd + G) return;
     const int fs = max(0, c0 - 2), fe = min(nf - 1, c1 + 2);   // faces [fs, fe]
     if (fs > fe) return;
     // padded strides by axis (selects, not an indexed local array)
@@ -957,9 +956,9 @@ template <typename T>
 __global__ void __launch_bounds__(256) rev_gather_cells_kernel(RevArgs A)
 {
     const T *lamC = (const T *)A.lamC;
-    const int a = (int)(blockIdx.x * 32 + threadIdx.x) - 2, b = (int)(blockIdx.y * 8 + threadIdx.y) - 2;
-    const int c = (int)blockIdx.z - G;
-    if (a >= A.n1 + 2 || b >= A.n2 + 2) return;
+    int a, b;
+    const int c = (int)blockIdx.y - G;
+    if (!face_position(blockIdx.x * 256u + threadIdx.x, A.n1, A.n2, a, b)) return;
     const int comp[4] = {0, 1 + A.d, 1 + A.t1, 1 + A.t2};
     T acc[4] = {0, 0, 0, 0};
     const int flo = c - 2 < 0 ? 0 : c - 2, fhi = c + 3 > A.nd ? A.nd : c + 3;
@@ -1734,6 +1733,12 @@ __global__ void alm_sample_add_serial_kernel(AlmAdjArgs A, const double *ptc, co
         }
 }
 
+// Blocks of 256 consecutive positions of an extended face plane (face_position):
+// the FP64 grids' t1, face-state and gather reverses on 68 x 68 positions had 32 x 8
+// blocks half idle (gradient of 128x64x64 9.17 -> 8.88 ms). The partial sums
+// keep the tiles' own 32 x 8 blocks, whose reads are aligned to them.
+unsigned plane_blocks(int n1, int n2) { return (unsigned)(((long)(n1 + 4) * (n2 + 4) + 255) / 256); }
+
 // S^T: adjoint of the spatial operator of working array Aw (ghost-filled),
 // for lamL (may be null) and lamLt; result accumulated into w.lamA.
 template <typename T>
@@ -1785,14 +1790,14 @@ void spatial_adjoint(const Ctx &c, const AdjWork &w, const double *Aw, void *con
         const int nf = c.n[d] + 1;
         rev_flux_kernel<T><<<dim3((R.n1 + 31) / 32, (R.n2 + kRevFluxB - 1) / kRevFluxB, nf), blk, 0, c.stream>>>(R);
         rev_t2_kernel<T><<<dim3((R.n1 + 31) / 32, (R.n2 + 4 + kRevT2 - 1) / kRevT2, nf), blk, 0, c.stream>>>(R);
-        rev_t1_kernel<T><<<dim3((R.n1 + 4 + 31) / 32, (R.n2 + 4 + 7) / 8, nf), blk, 0, c.stream>>>(R);
-        const dim3 gfs((R.n1 + 4 + 31) / 32, (R.n2 + 4 + 7) / 8, (nf + kRevMarch - 1) / kRevMarch);
+        const unsigned plane = plane_blocks(R.n1, R.n2);
+        rev_t1_kernel<T><<<dim3(plane, nf), 256, 0, c.stream>>>(R);
+        const dim3 gfs(plane, (nf + kRevMarch - 1) / kRevMarch);
         if (f32)
-            rev_face_state32_kernel<<<gfs, blk, 0, c.stream>>>(R);
+            rev_face_state32_kernel<<<gfs, 256, 0, c.stream>>>(R);
         else
-            rev_face_state_kernel<<<gfs, blk, 0, c.stream>>>(R);
-        rev_gather_cells_kernel<T><<<dim3((R.n1 + 4 + 31) / 32, (R.n2 + 4 + 7) / 8, R.nd + 2 * G), blk, 0,
-                                     c.stream>>>(R);
+            rev_face_state_kernel<<<gfs, 256, 0, c.stream>>>(R);
+        rev_gather_cells_kernel<T><<<dim3(plane, R.nd + 2 * G), 256, 0, c.stream>>>(R);
     }
 }
 
@@ -1903,9 +1908,9 @@ void spatial_adjoint_fused32(const Ctx &cw, const AdjWork &w, const float *A32, 
         R.n2 = c.n[t2];
         R.np = c.np;
         R.ph = make_phys<double>(c);
-        const long nb = ((long)(R.n1 + 4) * (R.n2 + 4) + 255) / 256;
-        const int cells = rev_cells(nb, R.nd + 2 * G, resident.cells);
-        rev_face_cells32_kernel<<<dim3((unsigned)nb, (R.nd + 2 * G + cells - 1) / cells), 256, rev_cells_smem_bytes(),
+        const unsigned plane = plane_blocks(R.n1, R.n2);
+        const int cells = rev_cells(plane, R.nd + 2 * G, resident.cells);
+        rev_face_cells32_kernel<<<dim3(plane, (R.nd + 2 * G + cells - 1) / cells), 256, rev_cells_smem_bytes(),
                                   c.stream>>>(R, cells);
     }
 }

@@ -770,6 +770,17 @@ __device__ __forceinline__ void ds_val_der(dsf c, const dsf D[4], dsf2 &val, dsf
     der = d.value();
 }
 
+// A block takes consecutive positions of the extended face plane, t1 fastest,
+// whatever its width: 32 x 8 blocks leave a fifth of the lanes idle on the
+// 132 x 132 positions of a 128^3 grid and half of them on 36 x 36.
+__device__ __forceinline__ bool face_position(unsigned p, int n1, int n2, int &a, int &b)
+{
+    const unsigned r = p / (unsigned)(n1 + 4);
+    a = (int)(p - r * (unsigned)(n1 + 4)) - 2;
+    b = (int)r - 2;
+    return b < n2 + 2;
+}
+
 constexpr int TX = 32, TY = 8;              // face tile
 constexpr int SQ_W = TX + 4, SQ_H = TY + 4; // tile with the tangential halo
 constexpr int SQ_N = 8 * SQ_H * SQ_W;

@@ -234,17 +234,6 @@ constexpr int kEqBlocks = std::is_same<C, float>::value ? (ALL ? 8 : 6) : std::i
 template <typename C, bool ALL>
 constexpr int kEqBusy = std::is_same<C, float>::value ? (ALL ? 1 : 6) : std::is_same<C, dsf>::value ? (ALL ? 6 : 2) : 5;
 
-// A block takes consecutive positions of the extended face plane, t1 fastest,
-// whatever its width: 32 x 8 blocks leave a fifth of the lanes idle on the
-// 132 x 132 positions of a 128^3 grid and half of them on 36 x 36.
-__device__ __forceinline__ bool face_position(unsigned p, int n1, int n2, int &a, int &b)
-{
-    const unsigned r = p / (unsigned)(n1 + 4);
-    a = (int)(p - r * (unsigned)(n1 + 4)) - 2;
-    b = (int)r - 2;
-    return b < n2 + 2;
-}
-
 // Marching variant: each thread walks K consecutive faces along d at one
 // tangential position of the extended face box, with the differences around
 // the current cell in registers (WenoMarch). Per cell it forms both face
