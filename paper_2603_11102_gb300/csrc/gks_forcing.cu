@@ -256,10 +256,10 @@ __device__ __forceinline__ void add_comp(float &hi, float &lo, float d)
 // Gaussian, Eq. (Gaussian)). 8 lanes share a cell, each taking every 8th point
 // in order, and their sums meet in a fixed shuffle tree (a box of 20,000 cells
 // is 75 blocks with a thread per cell: half the SMs idle and each thread
-// walking 150 points; 36 -> 20 us in FP32, 0.39 -> 0.05 ms in FP64 on a
-// 256x96x96 grid, whose points all took the FP64 distance). The blade screen and the distances
-// are formed in FP32 on hub-relative coordinates, staged in shared memory
-// (error below 2e-6 relative in r^2). FP32C grids: the weights in FP32; only a
+// walking 150 points; 36 -> 20 us in FP32, in FP64 on a 256x96x96 grid, whose
+// points all took the FP64 distance, 0.42 -> 0.13 ms with the loads). The blade
+// screen and the distances are formed in FP32 on hub-relative coordinates,
+// staged in shared memory (error below 2e-6 relative in r^2). FP32C grids: the weights in FP32; only a
 // point whose r^2 lies within 1e-5 of the cut takes the FP64 distance. FP64
 // grids: every point that passes the FP32 screen with that margin takes the
 // FP64 distance and weight. Either way the support is decided exactly as in
