@@ -422,8 +422,8 @@ int gks_step_reverse(gks_grid *g, void *d_tape, void *d_scratch, const double *d
 
 /* Kernel accounting of the library's own kernels. Every kernel launch is
  * counted per group (0 prep, 1 ghost, 2 cfl, 3 face_eq, 4 face_flux: x and
- * y faces, 5 flux_update: z faces fused with the stage update, 6 alm, 7 ibm,
- * 8 misc); with timing enabled each launch is also
+ * y faces, on small grids all faces, 5 flux_update: z faces and the stage
+ * update, 6 alm, 7 ibm, 8 misc); with timing enabled each launch is also
  * bracketed by CUDA events on the grid's stream and its duration summed.
  * gks_profile_enable sets timing on or off and clears the counters;
  * gks_profile_read synchronises, fills out and clears the counters. With

@@ -2036,6 +2036,7 @@ size_t adjoint_scratch_carve(const Ctx &c, long npts_total, void *base, AdjWork 
     w->lamA = k.take(np4);
     w->lamW = k.take(np4);
     w->lamP = k.take(np4);
+    // FP32C: np4 floats, then their interior cells with y fastest (rev_update_kernel)
     w->lamL = k.take(np4);
     w->lamLt = k.take(np4);
     long nR = 0, maxsurf = 0;
