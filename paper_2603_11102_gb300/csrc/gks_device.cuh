@@ -124,11 +124,10 @@ __device__ __forceinline__ void weno5_pair(const R q[5], R &right, R &left)
 // erf(z), exp(-z^2) - 1 and exp(-z^2) of the half-space moments, z =
 // sqrt(lambda) U. For |z| <= 1/2 (|U| up to 7 U_ref at Ma 0.1), with t = z^2:
 //   erf z = z E(t),  exp(-t) - 1 = -t X(-t),
-// E and X as polynomials of least deviation on 0 <= t <= 1/4 (Chebyshev fits
-// of the two Maclaurin series): degree 4 in FP32 (within 1.5e-9 and 2.4e-9,
-// relative) and degree 8 in FP64 and double-single (within 4.3e-18 and
-// 7.3e-18), 4 and 8 multiply-adds less per pair than the truncated series of
-// the same accuracy. exp = 1 + expm1. Beyond 1/2 the library functions.
+// E and X in FP64 and double-single as polynomials of least deviation on 0 <=
+// t <= 1/4 (Chebyshev fits of the two Maclaurin series), of degree 8 (within
+// 4.3e-18 and 7.3e-18), 8 multiply-adds less per pair than the truncated series
+// of the same accuracy. exp = 1 + expm1. Beyond 1/2 the library functions.
 template <typename T>
 __device__ __forceinline__ void half_space_polys(T t, T x, T &E, T &X)
 {
@@ -146,19 +145,22 @@ __device__ __forceinline__ void half_space_polys(T t, T x, T &E, T &X)
         X = fma(X, x, T(cx[k]));
     }
 }
+// FP32: the truncated Maclaurin series themselves (n = 0..6 and 1..7, first
+// dropped terms below 4e-10 and 2e-9 relative). Shorter polynomials of the same
+// accuracy round differently, and the FP32C gradients follow (WenoWindow).
 template <typename T>
-__device__ __forceinline__ void half_space_polys32(T t, T x, T &E, T &X)
+__device__ __forceinline__ void half_space_series32(T t, T x, T &E, T &X)
 {
-    constexpr double ce[5] = {0.0047190825672188138798, -0.026757732735015515622, 0.11282831428465861874,
-                              -0.37612609007469802928, 1.1283791656017914552};
-    constexpr double cx[5] = {0.0075136062215127308948, 0.04149065410396734984, 0.16665108206608517899,
-                              0.49999951482098960754, 0.99999999757585578433};
+    constexpr double k = 1.1283791670955126;   // 2 / sqrt(pi)
+    constexpr double ce[7] = {k / (720.0 * 13.0), -k / (120.0 * 11.0), k / (24.0 * 9.0), -k / (6.0 * 7.0),
+                              k / (2.0 * 5.0), -k / 3.0, k};
+    constexpr double cx[7] = {1.0 / 5040.0, 1.0 / 720.0, 1.0 / 120.0, 1.0 / 24.0, 1.0 / 6.0, 0.5, 1.0};
     E = T(ce[0]);
     X = T(cx[0]);
 #pragma unroll
-    for (int k = 1; k < 5; ++k) {
-        E = fma(E, t, T(ce[k]));
-        X = fma(X, x, T(cx[k]));
+    for (int i = 1; i < 7; ++i) {
+        E = fma(E, t, T(ce[i]));
+        X = fma(X, x, T(cx[i]));
     }
 }
 __device__ __forceinline__ void half_space_terms(double z, double &e, double &m1, double &ex)
@@ -181,7 +183,7 @@ __device__ __forceinline__ void half_space_terms(float z, float &e, float &m1, f
     const float t = __fmul_rn(z, z), x = -t;
     if (fabsf(z) <= 0.5f) {
         float E, X;
-        half_space_polys32(t, x, E, X);
+        half_space_series32(t, x, E, X);
         e = __fmul_rn(E, z);
         m1 = __fmul_rn(X, x);
         ex = __fadd_rn(1.0f, m1);
@@ -459,7 +461,7 @@ __device__ __forceinline__ void face_equilibrium_ds2(const Phys<dsf> &ph, const 
 // ---- FP32 face state on packed pairs ----
 
 // Approximate reciprocal per lane (1 ulp; one instruction: the arguments, a
-// density or a sum of squared smoothness indicators of at least 1e-23, are
+// density or a sum of squared smoothness indicators of at least 1e-24, are
 // never subnormal, so the flush of subnormal inputs changes nothing).
 __device__ __forceinline__ float rcp_approx(float x)
 {
@@ -468,7 +470,6 @@ __device__ __forceinline__ float rcp_approx(float x)
     return r;
 }
 __device__ __forceinline__ f2 wrcp(f2 x) { return f2(rcp_approx(x.v.x), rcp_approx(x.v.y)); }
-__device__ __forceinline__ f2 wnrcp(f2 x) { return f2(rcp_approx(-x.v.x), rcp_approx(-x.v.y)); }
 
 // half_space_terms of two FP32 arguments: the polynomials of both lanes as
 // pairs when both lie in |z| <= 1/2 (the same operations per lane as the
@@ -478,7 +479,7 @@ __device__ __forceinline__ void half_space_terms(f2 z, f2 &e, f2 &m1, f2 &ex)
     if (fabsf(z.v.x) <= 0.5f && fabsf(z.v.y) <= 0.5f) {
         const f2 t = z * z, x = t * f2(-1.0f);
         f2 E, X;
-        half_space_polys32(t, x, E, X);
+        half_space_series32(t, x, E, X);
         e = E * z;
         m1 = X * x;
         ex = f2(1.0f) + m1;
@@ -500,11 +501,10 @@ __device__ __forceinline__ void half_space_terms(f2 z, f2 &e, f2 &m1, f2 &ex)
 // D_{i-1/2} + D_{i+1/2} and S_{i+1} - 2 D_{i+1/2}. A cell that enters the
 // march brings one new difference of each order and one new square, where
 // the 5-cell form redoes them for every cell: 33 operations per cell and
-// component against 53 (FP32 pairs) and 81 (FP64). The FP64 face state is
-// bound by the FP64 pipe and follows the count (6 launches of a 96^3 step:
-// 7.92 -> 4.67 ms), the double-single one too (2.38 -> 1.66 ms); the FP32 one
-// waits on its loads as well (a 384x256x256 step: 2.27 -> 2.15 ms). Written
-// without a product that feeds an addition, so that no contraction is left to
+// component against 81. The FP64 face state is bound by the FP64 pipe and
+// follows the count (6 launches of a 96^3 step: 7.92 -> 4.67 ms), the
+// double-single one too (2.38 -> 1.66 ms). Written without a product that
+// feeds an addition, so that no contraction is left to
 // the compiler and a face's bits do not depend on its position in the march.
 template <typename T>
 struct WenoMarch {
@@ -565,12 +565,6 @@ struct WenoMarch {
     // r = cr - nr / dr, l = cl + nl / dl
     static __device__ __forceinline__ void sub_quotients(T nr, T dr, T cr, T &r, T nl, T dl, T cl, T &l);
 };
-template <>
-__device__ __forceinline__ void WenoMarch<f2>::sub_quotients(f2 nr, f2 dr, f2 cr, f2 &r, f2 nl, f2 dl, f2 cl, f2 &l)
-{
-    r = fma(nr, wnrcp(dr), cr);
-    l = fma(nl, wrcp(dl), cl);
-}
 // One FP64 division for both faces (the denominators are sums of 8th powers
 // of differences above 1e-23; where their product overflows, each by itself).
 template <>
@@ -597,6 +591,81 @@ __device__ __forceinline__ void WenoMarch<dsf2>::sub_quotients(dsf2 nr, dsf2 dr,
     r = cr - nr / dr;
     l = cl + nl / dl;
 }
+
+// weno5_pair of two components at once, every multiply-add fused explicitly
+// and the constant factors folded into the candidates:
+//  - the indicators are those of weno5_pair divided by 13/12 (the weights
+//    depend on their ratios only): s_k = (eps 12/13 + t_k^2 + (3/13) u_k^2)^2,
+//    with u_0 = t_0 + 2 (c - b) and u_2 = t_2 + 2 (c - d);
+//  - the right-face weights times 10 s0 s1 s2 / 3 are s1 s2 / 3, 2 s0 s2 and
+//    s0 s1 (mirrored for the left face), so with the candidates P_k = the
+//    integer-coefficient ones divided by 18, 3 and 6 the face value is
+//    (s12 P0 + s02 P1 + s01 P2) / (s12 / 3 + 2 s02 + s01).
+__device__ __forceinline__ void weno5_pair2(const f2 q[5], f2 &right, f2 &left)
+{
+    const f2 m2(-2.0f), two(2.0f), eps(float(12e-6 / 13.0)), k(float(3.0 / 13.0));
+    const f2 a = q[0], b = q[1], c = q[2], d = q[3], e = q[4];
+    f2 t = fma(b, m2, a) + c, u = fma(c - b, two, t);
+    f2 s0 = fma(t, t, fma(u * k, u, eps));
+    t = fma(c, m2, b) + d;
+    u = b - d;
+    f2 s1 = fma(t, t, fma(u * k, u, eps));
+    t = fma(d, m2, c) + e;
+    u = fma(c - d, two, t);
+    f2 s2 = fma(t, t, fma(u * k, u, eps));
+    s0 = s0 * s0;
+    s1 = s1 * s1;
+    s2 = s2 * s2;
+    const f2 s02 = s0 * s2, s01 = s0 * s1, s12 = s1 * s2;
+    const f2 third(float(1.0 / 3.0));
+    const f2 c3 = c * third, c53 = c * f2(float(5.0 / 3.0)), c1118 = c * f2(float(11.0 / 18.0));
+    const f2 k19(float(1.0 / 9.0)), k718(float(-7.0 / 18.0)), k23(float(2.0 / 3.0)), km13(float(-1.0 / 3.0));
+    const f2 k56(float(5.0 / 6.0)), km16(float(-1.0 / 6.0));
+    {
+        // right face: candidates on (a,b,c), (b,c,d), (c,d,e)
+        const f2 P0 = fma(a, k19, fma(b, k718, c1118));
+        const f2 P1 = fma(b, km13, fma(d, k23, c53));
+        const f2 P2 = fma(e, km16, fma(d, k56, c3));
+        right = fma(s12, P0, fma(s02, P1, s01 * P2)) * wrcp(fma(s12, third, fma(s02, two, s01)));
+    }
+    {
+        // left face: the mirrored candidates with indicators s2, s1, s0
+        const f2 P0 = fma(e, k19, fma(d, k718, c1118));
+        const f2 P1 = fma(d, km13, fma(b, k23, c53));
+        const f2 P2 = fma(a, km16, fma(b, k56, c3));
+        left = fma(s01, P0, fma(s02, P1, s12 * P2)) * wrcp(fma(s01, third, fma(s02, two, s12)));
+    }
+}
+
+// The 5-cell window of a march of FP32 component pairs, with WenoMarch's
+// interface. The differences of WenoMarch, 33 operations per cell and
+// component against 53, are hardly faster here, where the march waits on its
+// loads (face state of a 384x256x256 step 1.84 ms against 1.83 with the window,
+// of 128^3 0.206 against 0.214), and every value of an FP32C state then rounds
+// differently, and with it the gradients: the FP32 rounding of the face values
+// is seen through the curvature of the weights, 4e-6 of the root mean square of
+// an inflow-speed gradient, a sum that nearly cancels. The rounding of this
+// path is part of its results (tests/test_gpu_fp32c_rounding.py).
+struct WenoWindow {
+    f2 w[5];   // cells i - 2 .. i + 2; before a push the first 4 are i - 2 .. i + 1
+
+    __device__ __forceinline__ void start(f2 q0, f2 q1, f2 q2, f2 q3)
+    {
+        w[0] = q0; w[1] = q1; w[2] = q2; w[3] = q3;
+    }
+    // 12 x the normal slope times the centre distance at the face between i - 1 and i
+    __device__ __forceinline__ f2 slope12() const
+    {
+        return fma(w[3] - w[0], f2(-1.0f), (w[2] - w[1]) * f2(15.0f));
+    }
+    __device__ __forceinline__ void push(f2 e, f2 &right, f2 &left)
+    {
+        w[4] = e;
+        weno5_pair2(w, right, left);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[k] = w[k + 1];
+    }
+};
 
 // face_equilibrium with the components paired as (rho, m_n) and (m_t1, m_t2)
 // (index 0 and 1 of L, R and Q0) and the half-space terms of the left and
@@ -661,7 +730,6 @@ __device__ __forceinline__ FluxPhys<dsf2> flux_phys_ds2(const Phys<dsf> &p)
 }
 // rho and 1 / rho; FP64 grids store rho whole (off = 0)
 __device__ __forceinline__ f2 whole_rho(f2 off, f2 q) { return off + q; }
-__device__ __forceinline__ float whole_rho(float off, float q) { return __fadd_rn(off, q); }
 __device__ __forceinline__ double whole_rho(double, double q) { return q; }
 __device__ __forceinline__ dsf2 whole_rho(dsf2, dsf2 q) { return q; }
 __device__ __forceinline__ double inverse(double a) { return 1.0 / a; }
@@ -923,22 +991,6 @@ __device__ __forceinline__ void tile_t1_pass(const R *sq, C *st, int tid, int H,
 // The face state of a 384x256x256 step took 2.15 ms with 8 separate stores
 // and takes 1.90 ms with 4 paired ones.
 
-// tan_val_der of a component pair, with the operations of the marching flux
-// kernel (the same bits): E -+ O and Do -+ De with the last terms fused.
-__device__ __forceinline__ void pair_t1(const f2 q[5], f2 &vm, f2 &vp, f2 &dm, f2 &dp)
-{
-    constexpr float o1 = float(0.20046884346862007), o2 = float(0.028065638085606807);
-    constexpr float e1 = float(0.41697519441472974), e2 = float(0.032075014954979206);
-    const f2 d1 = fma(q[2], f2(-2.0f), q[3] + q[1]), d2 = fma(q[2], f2(-2.0f), q[4] + q[0]);
-    const f2 a1 = q[3] - q[1], a2 = q[4] - q[0];
-    const f2 E = fma(d1, f2(float(1.0 / 1080.0)), fma(d2, f2(float(-1.0 / 4320.0)), q[2]));
-    const f2 D = fma(a1, f2(float(2.0 / 3.0)), a2 * f2(float(-1.0 / 12.0)));
-    vm = fma(a1, f2(-o1), fma(a2, f2(o2), E));
-    vp = fma(a1, f2(o1), fma(a2, f2(-o2), E));
-    dm = fma(d1, f2(-e1), fma(d2, f2(e2), D));
-    dp = fma(d1, f2(e1), fma(d2, f2(-e2), D));
-}
-
 // t1 pass of a face-box tile of H rows: 64 H equal tasks (pair, row, group of
 // 2 columns), H / 4 per thread: 6 pairs in by 128-bit loads, 2 columns out by
 // one 128-bit store per array (consecutive lanes, consecutive 16 bytes: no
@@ -963,7 +1015,8 @@ __device__ __forceinline__ void tile_t1_pass_f2(const float2 *sq, float2 *st, in
         f2 v[4][2];
         if (p < 2) {
 #pragma unroll
-            for (int i = 0; i < 2; ++i) pair_t1(q + i, v[0][i], v[1][i], v[2][i], v[3][i]);
+            for (int i = 0; i < 2; ++i)
+                tan_val_der(q[i], q[i + 1], q[i + 2], q[i + 3], q[i + 4], v[0][i], v[1][i], v[2][i], v[3][i]);
             o += 4 * p * ROWS;
         } else {
 #pragma unroll

@@ -2,8 +2,8 @@
 //
 // Per stage and per direction d (x, y, z):
 //   face_eq      one thread per tangential position of the extended face box,
-//                marching along d with the differences around a cell in
-//                registers: WENO5-JS (Sec. 2, Jiang-Shu) left/right states
+//                marching along d with the differences around a cell (FP32C:
+//                the 5 cells) in registers: WENO5-JS (Sec. 2, Jiang-Shu) left/right states
 //                from one paired evaluation per cell, the equilibrium state
 //                Q0 from the half Maxwellians (u>0 from the left, u<0 from
 //                the right), and the quartic normal slope of Q0.
@@ -322,7 +322,7 @@ __device__ __forceinline__ void face_eq_f2(const FaceEqArgs<float, float> &A, in
                           A.w + (long)A.c2 * A.np + base};
     float2 *fq = reinterpret_cast<float2 *>(A.fq);   // component pairs (see tile_t1_pass_f2)
     // cells f0-3 .. f0 start the march at cell f0-1, cell f0+1 completes it
-    WenoMarch<f2> w[2];
+    WenoWindow w[2];
     f2 Qprev[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
@@ -341,7 +341,7 @@ __device__ __forceinline__ void face_eq_f2(const FaceEqArgs<float, float> &A, in
     for (int v = 0; v < 4; ++v) nxt[v] = __ldg(pc[v] + (long)(f0 + 2 + G) * A.sd);
 #pragma unroll 2
     for (int f = f0; f < f1; ++f) {
-        const f2 ihf(A.ihf[f]);
+        const f2 s(A.ihf[f] * float(1.0 / 12.0));
         const long o = ((long)f * (A.n2 + 4) + (b + 2)) * A.e1p + (a + 2);
         const f2 e[2] = {f2(nxt[0], nxt[1]), f2(nxt[2], nxt[3])};
         if (f + 1 < f1) {
@@ -352,7 +352,7 @@ __device__ __forceinline__ void face_eq_f2(const FaceEqArgs<float, float> &A, in
         f2 Ql[2], Qr[2], Q0[2];
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-            fq[(2 + q) * A.nfq + o] = (w[q].slope() * ihf).v;
+            fq[(2 + q) * A.nfq + o] = (w[q].slope12() * s).v;
             Ql[q] = Qprev[q];
             w[q].push(e[q], Qprev[q], Qr[q]);
         }
@@ -868,10 +868,13 @@ __device__ __forceinline__ void march_row(const float2 *box, int lane, MarchWin 
             const float d1 = __fmaf_rn(q[2], -2.0f, __fadd_rn(q[3], q[1]));
             const float d2 = __fmaf_rn(q[2], -2.0f, __fadd_rn(q[4], q[0]));
             const float a1 = __fsub_rn(q[3], q[1]), a2 = __fsub_rn(q[4], q[0]);
+            // tan_val_der with the two Gauss points in the lanes
             const float E = __fmaf_rn(d1, float(1.0 / 1080.0), __fmaf_rn(d2, float(-1.0 / 4320.0), q[2]));
-            const float D = __fmaf_rn(a1, float(2.0 / 3.0), __fmul_rn(a2, float(-1.0 / 12.0)));
-            w.v[2 * P + c][J] = fma(f2(a1), f2(-o1, o1), fma(f2(a2), f2(o2, -o2), f2(E)));
-            w.d[2 * P + c][J] = fma(f2(d1), f2(-e1, e1), fma(f2(d2), f2(e2, -e2), f2(D)));
+            const float O = __fmaf_rn(a1, o1, __fmul_rn(a2, -o2));
+            const float Do = __fmaf_rn(a1, float(2.0 / 3.0), __fmul_rn(a2, float(-1.0 / 12.0)));
+            const float De = __fmaf_rn(d1, e1, __fmul_rn(d2, -e2));
+            w.v[2 * P + c][J] = fma(f2(O), f2(-1.0f, 1.0f), f2(E));
+            w.d[2 * P + c][J] = fma(f2(De), f2(-1.0f, 1.0f), f2(Do));
         }
 #pragma unroll
         for (int k = 0; k < 5; ++k) x[k] = box[((2 + P) * RB + J) * SQ_W + lane + k];
