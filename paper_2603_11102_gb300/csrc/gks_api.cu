@@ -564,6 +564,7 @@ int gks_add_actuator_lines(gks_grid *g, const gks_rotor_desc *d, int *id)
     r.rmax = rmax;
     rmax = fmax(fabs(rmax), fabs(rmin));
     const double cut = 3.0 * d->eps;
+    r.screen = (float)fmax(1e-5, 5e-7 * (rmax / cut + 2.0));
     if (cell_range(c, 0, d->hub[0] - cut, d->hub[0] + cut, r.box[0]) ||
         cell_range(c, 1, d->hub[1] - rmax - cut, d->hub[1] + rmax + cut, r.box[1]) ||
         cell_range(c, 2, d->hub[2] - rmax - cut, d->hub[2] + rmax + cut, r.box[2]))

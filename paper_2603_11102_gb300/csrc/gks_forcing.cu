@@ -259,11 +259,14 @@ __device__ __forceinline__ void add_comp(float &hi, float &lo, float d)
 // walking 150 points; 36 -> 20 us in FP32, in FP64 on a 256x96x96 grid, whose
 // points all took the FP64 distance, 0.42 -> 0.13 ms with the loads). The blade
 // screen and the distances are formed in FP32 on hub-relative coordinates,
-// staged in shared memory (error below 2e-6 relative in r^2). FP32C grids: the weights in FP32; only a
-// point whose r^2 lies within 1e-5 of the cut takes the FP64 distance. FP64
-// grids: every point that passes the FP32 screen with that margin takes the
-// FP64 distance and weight. Either way the support is decided exactly as in
-// FP64.
+// staged in shared memory. Rounded to 2^-24 of up to R + 3 eps, they leave an
+// error of 2^-24 (4 R / (3 eps) + 12) in r^2 relative to the cut's: the margin
+// `screen` is twice that, 1e-5 at least (up to R/eps = 54), and ten times as
+// wide for the blade, whose nearest point has the rounding of its direction
+// too. FP32C grids: the weights in FP32; only a point whose r^2 lies within the
+// margin of the cut takes the FP64 distance. FP64 grids: every point that passes
+// the FP32 screen with that margin takes the FP64 distance and weight. Either
+// way the support is decided exactly as in FP64.
 constexpr int kSpreadPts = 256;   // points staged at a time
 
 template <typename R>
@@ -283,7 +286,8 @@ __global__ void __launch_bounds__(256) alm_spread_kernel(Lattice L, void *S, Rot
     const double cut = 3.0 * r.eps;
     const int npts = r.nb * r.np;
     const float pc[3] = {(float)(xc[0] - r.hub[0]), (float)(xc[1] - r.hub[1]), (float)(xc[2] - r.hub[2])};
-    const float c2 = (float)(cut * cut), c2lo = c2 * (1.0f - 1e-5f), c2hi = c2 * (1.0f + 1e-5f);
+    const float c2 = (float)(cut * cut), c2lo = c2 * (1.0f - r.screen), c2hi = c2 * (1.0f + r.screen);
+    const float c2blade = c2 * (1.0f + 10.0f * r.screen);
     const float rmin = (float)r.rmin, rmax = (float)r.rmax;
     // every point of blade b lies on the segment hub + s e_r, s in [rmin,
     // rmax]; a cell farther than 3 eps from it gets nothing of the blade
@@ -293,7 +297,7 @@ __global__ void __launch_bounds__(256) alm_spread_kernel(Lattice L, void *S, Rot
         float sp = pc[1] * e2 - pc[2] * e1;
         sp = fminf(fmaxf(sp, rmin), rmax);
         const float qy = pc[1] - sp * e2, qz = pc[2] + sp * e1;
-        if (on && pc[0] * pc[0] + qy * qy + qz * qz <= c2 * 1.0001f) near |= 1u << b;
+        if (on && pc[0] * pc[0] + qy * qy + qz * qz <= c2blade) near |= 1u << b;
     }
     R f[3] = {R(0), R(0), R(0)};
     bool any = false;

@@ -138,6 +138,7 @@ struct RotorDev {
     double tip_g[2];    // g1 of the tip factor: axial, tangential
     double hub[3], omega, az0, radius, eps, rho_inf, uref;
     double rmin, rmax;  // smallest and largest point radius
+    float screen;       // relative margin of the projection's FP32 r^2 against the cut (alm_spread_kernel)
     double *r, *chord, *twist, *width, *scale;  // device arrays
     double *X;          // 3 nb np positions of the last step
     float *Xr;          // the same relative to the hub, FP32 (projection screen)
