@@ -77,9 +77,12 @@ __device__ __forceinline__ long lin(const int P0, const int P1, int i, int j, in
 
 // ------------------------------------------------------ reverse building blocks
 
-__device__ __forceinline__ float rev_inverse(float a) { return rcp_approx(a); }
+// Reciprocals of the reverse, correctly rounded in FP32 too (the forward's
+// approximate one is off by an ulp and flushes what lies above 2^126 to zero;
+// it is worth 0.9 % of the gradient of 256x128x128).
+__device__ __forceinline__ float rev_inverse(float a) { return __frcp_rn(a); }
 __device__ __forceinline__ double rev_inverse(double a) { return 1.0 / a; }
-__device__ __forceinline__ f2 rev_inverse(f2 a) { return wrcp(a); }
+__device__ __forceinline__ f2 rev_inverse(f2 a) { return f2(__frcp_rn(a.v.x), __frcp_rn(a.v.y)); }
 
 // Adjoint of dev::gk_flux: given the adjoints of F0 (if needF0) and F1, the
 // adjoints of its inputs (index-space tangential slopes, density slopes as
@@ -608,8 +611,8 @@ struct Weno32 {
         s01 = s0 * s1;
         s12 = s1 * s2;
         const float w = 18.0f * (s0 * s2);
-        ir = rcp_approx(fmaf(3.0f, s12, fmaf(9.0f, s01, w)));
-        il = rcp_approx(fmaf(3.0f, s01, fmaf(9.0f, s12, w)));
+        ir = rev_inverse(fmaf(3.0f, s12, fmaf(9.0f, s01, w)));
+        il = rev_inverse(fmaf(3.0f, s01, fmaf(9.0f, s12, w)));
         a = s12 * Tm;
         b = s01 * Tp;
     }
