@@ -217,11 +217,12 @@ def time_oracle(w, steps, warmup):
 
 def source_hash(group="face_flux"):
     """Hash of the source a kernel group's measured figures depend on: the
-    device header and the group's section of gks_stencil.cu."""
+    device headers and the group's section of gks_stencil.cu."""
     csrc = os.path.join(ROOT, "paper_2603_11102_gb300", "csrc")
     h = hashlib.sha256()
-    with open(os.path.join(csrc, "gks_device.cuh"), "rb") as fh:
-        h.update(fh.read())
+    for header in ("gks_device.cuh", "gks_ds.cuh"):
+        with open(os.path.join(csrc, header), "rb") as fh:
+            h.update(fh.read())
     with open(os.path.join(csrc, "gks_stencil.cu")) as fh:
         text = fh.read()
     first, last = SECTIONS[group]
