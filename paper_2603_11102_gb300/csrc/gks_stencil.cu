@@ -1961,13 +1961,14 @@ __global__ void __launch_bounds__(256) diag_partial_kernel(const void *S, long n
                 const double w = hz[k0 + k + G], m2 = fma(q[1], q[1], fma(q[2], q[2], q[3] * q[3]));
                 const int hw = __double2hiint(q[0]), e = ((hw >> 20) & 0x7ff) - 896;
                 double u;
-                if (e >= 27 && e <= 227) {
+                if (e > 52 && e <= 227) {
                     // the top 24 bits of rho as a float, the rest as its low part
+                    // (a normal float down to 2^-74)
                     const float f = __uint_as_float((hw & 0x80000000u) | ((unsigned int)e << 23) | ((hw & 0xfffffu) << 3) |
                                                     ((unsigned int)__double2loint(q[0]) >> 29));
                     const float g = __fmul_rn(__uint2float_rn((unsigned int)__double2loint(q[0]) & 0x1fffffffu),
-                                              __uint_as_float((unsigned int)(e > 52 ? e - 52 : 0) << 23));
-                    u = quotient(m2, q[0], rcp_ds(f, e > 52 ? copysignf(g, f) : 0.0f));
+                                              __uint_as_float((unsigned int)(e - 52) << 23));
+                    u = quotient(m2, q[0], rcp_ds(f, copysignf(g, f)));
                 } else {
                     u = m2 / q[0];
                 }
