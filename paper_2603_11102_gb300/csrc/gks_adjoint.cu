@@ -1002,7 +1002,8 @@ struct Rev32Args {
     const float *ihd, *ih1, *ih2;     // inverse cell widths along d, t1, t2 (padded index)
     float *part;                      // per tile: 8 x SQ_H x SQ_W face-box adjoints
     int n1, n2, nf, nd, d, t1, t2;
-    long np, sd, s1, s2, base;        // of the cell adjoints: strides of a component, along d, t1, t2; index of cell (0, 0, 0)
+    // of the cell adjoints: strides of a component, along d, t1, t2; index of cell (0, 0, 0)
+    long np, sd, s1, s2, base;
     Phys<float> ph;
     Scalars *scal;
 };
@@ -1043,7 +1044,7 @@ __global__ void __launch_bounds__(256, 2) rev_tile32_kernel(const __grid_constan
             if (tid == 0) atomicOr(&A.scal->flags, FLAG_TIMEOUT);
             return;
         }
-        tile_t1_pass_f2<SQ_H>(reinterpret_cast<const float2 *>(sq), reinterpret_cast<float2 *>(st), tid);
+        tile_t1_pass_f2(reinterpret_cast<const float2 *>(sq), reinterpret_cast<float2 *>(st), tid);
         __syncthreads();
 
         // RA: per face, the 4 Gauss points
@@ -1068,8 +1069,8 @@ __global__ void __launch_bounds__(256, 2) rev_tile32_kernel(const __grid_constan
             const float ih1 = A.ih1[a + G], ih2 = A.ih2[b + G];
 #pragma unroll
             for (int m = 0; m < 2; ++m) {
-                f2 q2[1][4], n2[1][4], a2[1][4], b2[1][4];
-                t2_pass_f2<SQ_H, 1, false>(reinterpret_cast<const float2 *>(st), m, tx, ty, q2, n2, a2, b2);
+                f2 q2[4], n2[4], a2[4], b2[4];
+                t2_pass_f2<false>(reinterpret_cast<const float2 *>(st), m, tx, ty, q2, n2, a2, b2);
                 // the flux reverse at the two t2 Gauss points as one evaluation on
                 // packed FP32 pairs (the points in the lanes)
                 {
@@ -1086,7 +1087,7 @@ __global__ void __launch_bounds__(256, 2) rev_tile32_kernel(const __grid_constan
                     p2.off = f2(A.ph.off);
                     p2.sqlam = f2(A.ph.sqlam);
                     p2.kE = f2(A.ph.kE);
-                    gk_flux_rev<f2>(p2, q2[0], n2[0], a2[0], b2[0], f2(ih1), f2(ih2), s0, s1, needF0, qb, Dnb, D1b, D2b);
+                    gk_flux_rev<f2>(p2, q2, n2, a2, b2, f2(ih1), f2(ih2), s0, s1, needF0, qb, Dnb, D1b, D2b);
 #pragma unroll
                     for (int nn = 0; nn < 2; ++nn) {
                         float *gp = ga + (16 * (2 * m + nn)) * (TX * TY) + tid;

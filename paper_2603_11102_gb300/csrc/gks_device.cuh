@@ -34,12 +34,6 @@ Phys<R> make_phys(const Ctx &c)
     return p;
 }
 
-// Division in the working type: IEEE division in FP64; the two-instruction
-// approximate division (2 ulp) in FP32, whose error is far below the FP32
-// rounding of the stencil itself.
-__device__ __forceinline__ double wdiv(double a, double b) { return a / b; }
-__device__ __forceinline__ float wdiv(float a, float b) { return __fdividef(a, b); }
-
 // |U|^2 of a cell for the CFL time step, with every operation rounded
 // explicitly so that each kernel that forms it gets the same bits: FP32C from
 // hi + lo in FP32, FP64 from the state. max_u2 keeps a NaN.
@@ -50,7 +44,6 @@ __device__ __forceinline__ float cell_u2f(const float h[4], const float l[4])
     const float m2 = __fadd_rn(__fadd_rn(__fmul_rn(a, a), __fmul_rn(b, b)), __fmul_rn(c, c));
     return __fdiv_rn(m2, __fmul_rn(r, r));
 }
-__device__ __forceinline__ double cell_u2(const float h[4], const float l[4]) { return (double)cell_u2f(h, l); }
 __device__ __forceinline__ double cell_u2(const double w[4])
 {
     const double m2 = __dadd_rn(__dadd_rn(__dmul_rn(w[1], w[1]), __dmul_rn(w[2], w[2])), __dmul_rn(w[3], w[3]));
@@ -109,7 +102,7 @@ __device__ __forceinline__ void weno5_pair(const R q[5], R &right, R &left)
         const R p1 = -b + R(5) * c + R(2) * d;
         const R p2 = R(2) * c + R(5) * d - e;
         const R w2 = R(3) * s01;
-        right = wdiv(s12 * p0 + w02 * p1 + w2 * p2, R(6) * (s12 + w02 + w2));
+        right = (s12 * p0 + w02 * p1 + w2 * p2) / (R(6) * (s12 + w02 + w2));
     }
     // left face: candidates on (e,d,c), (d,c,b), (c,b,a) with indicators s2, s1, s0
     {
@@ -117,7 +110,7 @@ __device__ __forceinline__ void weno5_pair(const R q[5], R &right, R &left)
         const R p1 = -d + R(5) * c + R(2) * b;
         const R p2 = R(2) * c + R(5) * b - a;
         const R w2 = R(3) * s12;
-        left = wdiv(s01 * p0 + w02 * p1 + w2 * p2, R(6) * (s01 + w02 + w2));
+        left = (s01 * p0 + w02 * p1 + w2 * p2) / (R(6) * (s01 + w02 + w2));
     }
 }
 
@@ -254,33 +247,6 @@ __device__ __forceinline__ void face_equilibrium(const Phys<double> &ph, const d
 //   O  = (25 sqrt3 / 216) a1 - (7 sqrt3 / 432) a2,
 //   Do = (2/3) a1 - (1/12) a2,
 //   De = (13 sqrt3 / 54)(s1 - 2 q0) - (sqrt3 / 54)(s2 - 2 q0).
-template <typename R>
-__device__ __forceinline__ void tan_val(R qm2, R qm1, R q0, R qp1, R qp2, R &vm, R &vp)
-{
-    const R d1 = fma(q0, R(-2.0), qp1 + qm1), d2 = fma(q0, R(-2.0), qp2 + qm2);
-    const R a1 = qp1 - qm1, a2 = qp2 - qm2;
-    const R E = fma(d1, R(1.0 / 1080.0), fma(d2, R(-1.0 / 4320.0), q0));
-    const R O = R(0.20046884346862007) * a1 - R(0.028065638085606807) * a2;
-    vm = E - O;
-    vp = E + O;
-}
-
-// The same values as tan_val as two 5-weight dot products (all on the FMA
-// pipe). Used for rows that vanish identically in a uniform state (normal
-// slopes, tangential derivatives), where the weights not summing exactly to
-// one in floating point is harmless. NEG: the negated values (the density
-// slopes as gk_flux takes them), from negated weights.
-template <typename R, bool NEG = false>
-__device__ __forceinline__ void tan_val_direct(R qm2, R qm1, R q0, R qp1, R qp2, R &vm, R &vp)
-{
-    constexpr double s = NEG ? -1.0 : 1.0;
-    const R w0 = R(s * (-1.0 / 4320.0 + 0.028065638085606807)), w1 = R(s * (1.0 / 1080.0 - 0.20046884346862007));
-    const R w2 = R(s * 719.0 / 720.0);
-    const R w3 = R(s * (1.0 / 1080.0 + 0.20046884346862007)), w4 = R(s * (-1.0 / 4320.0 - 0.028065638085606807));
-    vp = fma(w4, qp2, fma(w3, qp1, fma(w2, q0, fma(w1, qm1, w0 * qm2))));
-    vm = fma(w0, qp2, fma(w1, qp1, fma(w2, q0, fma(w3, qm1, w4 * qm2))));
-}
-
 // NEG: the derivatives negated.
 template <typename R, bool NEG = false>
 __device__ __forceinline__ void tan_val_der(R qm2, R qm1, R q0, R qp1, R qp2, R &vm, R &vp, R &dm,
@@ -297,6 +263,22 @@ __device__ __forceinline__ void tan_val_der(R qm2, R qm1, R q0, R qp1, R qp2, R 
     vp = E + O;
     dm = Do - De;
     dp = Do + De;
+}
+
+// The values alone as two 5-weight dot products (all on the FMA pipe). Used
+// for rows that vanish identically in a uniform state (normal slopes,
+// tangential derivatives), where the weights not summing exactly to one in
+// floating point is harmless. NEG: the negated values (the density slopes as
+// gk_flux takes them), from negated weights.
+template <typename R, bool NEG = false>
+__device__ __forceinline__ void tan_val_direct(R qm2, R qm1, R q0, R qp1, R qp2, R &vm, R &vp)
+{
+    constexpr double s = NEG ? -1.0 : 1.0;
+    const R w0 = R(s * (-1.0 / 4320.0 + 0.028065638085606807)), w1 = R(s * (1.0 / 1080.0 - 0.20046884346862007));
+    const R w2 = R(s * 719.0 / 720.0);
+    const R w3 = R(s * (1.0 / 1080.0 + 0.20046884346862007)), w4 = R(s * (-1.0 / 4320.0 - 0.028065638085606807));
+    vp = fma(w4, qp2, fma(w3, qp1, fma(w2, q0, fma(w1, qm1, w0 * qm2))));
+    vm = fma(w0, qp2, fma(w1, qp1, fma(w2, q0, fma(w3, qm1, w4 * qm2))));
 }
 
 // ---- Packed FP32 pairs ----
@@ -325,10 +307,6 @@ __device__ __forceinline__ f2 operator-(f2 a, f2 b) { return fma(b, f2(-1.0f), a
 __device__ __forceinline__ f2 operator-(f2 a) { return f2(-a.v.x, -a.v.y); }
 __device__ __forceinline__ f2 &operator+=(f2 &a, f2 b) { return a = a + b; }
 __device__ __forceinline__ f2 &operator-=(f2 &a, f2 b) { return a = a - b; }
-// IEEE division per lane (the scalar FP32 path's a / b)
-__device__ __forceinline__ f2 operator/(f2 a, f2 b) { return f2(__fdiv_rn(a.v.x, b.v.x), __fdiv_rn(a.v.y, b.v.y)); }
-// the two-instruction approximate division of the scalar FP32 path, per lane
-__device__ __forceinline__ f2 wdiv(f2 a, f2 b) { return f2(__fdividef(a.v.x, b.v.x), __fdividef(a.v.y, b.v.y)); }
 
 // Two double-single values side by side (hi and lo parts as packed pairs):
 // every operation is lane by lane the double-single operation of gks_ds.cuh
@@ -398,7 +376,6 @@ __device__ __forceinline__ dsf2 operator/(dsf2 a, dsf2 b)
     return fast_two_sum(q1, q2);
 }
 __device__ __forceinline__ dsf2 &operator+=(dsf2 &a, dsf2 b) { return a = a + b; }
-__device__ __forceinline__ dsf2 wdiv(dsf2 a, dsf2 b) { return a / b; }
 
 __device__ __forceinline__ dsf2 &operator*=(dsf2 &a, dsf2 b) { return a = a * b; }
 // a b + c with the product left unnormalised (exact high product, its error
@@ -446,7 +423,7 @@ __device__ __forceinline__ void face_equilibrium_ds2(const Phys<dsf> &ph, const 
 {
     // lanes (left, right) of rho and m_n
     const dsf2 r(L[0].lane(0), R[0].lane(0));
-    const dsf2 U = wdiv(dsf2(L[0].lane(1), R[0].lane(1)), r);
+    const dsf2 U = dsf2(L[0].lane(1), R[0].lane(1)) / r;
     dsf2 e, m1, x;
     half_space_terms(dsf2(ph.sqlam) * U, e, m1, x);
     const dsf Pl = dsf(0.5) + scale_pow2(e.lane(0), 0.5f);   // <u^0>_{u>0} of the left state
@@ -857,12 +834,6 @@ constexpr int ST_N = 24 * ST_ROWS;
 
 // 8 consecutive values of a shared-memory row from a 16-byte aligned address,
 // and 4 consecutive values to one.
-__device__ __forceinline__ void lds8(const float *p, float q[8])
-{
-    const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 4);
-    q[0] = a.x; q[1] = a.y; q[2] = a.z; q[3] = a.w;
-    q[4] = b.x; q[5] = b.y; q[6] = b.z; q[7] = b.w;
-}
 __device__ __forceinline__ void lds8(const double *p, double q[8])
 {
 #pragma unroll
@@ -871,10 +842,6 @@ __device__ __forceinline__ void lds8(const double *p, double q[8])
         q[2 * i] = a.x;
         q[2 * i + 1] = a.y;
     }
-}
-__device__ __forceinline__ void sts4(float *p, const float q[4])
-{
-    *reinterpret_cast<float4 *>(p) = make_float4(q[0], q[1], q[2], q[3]);
 }
 __device__ __forceinline__ void sts4(double *p, const double q[4])
 {
@@ -991,19 +958,18 @@ __device__ __forceinline__ void tile_t1_pass(const R *sq, C *st, int tid, int H,
 // The face state of a 384x256x256 step took 2.15 ms with 8 separate stores
 // and takes 1.90 ms with 4 paired ones.
 
-// t1 pass of a face-box tile of H rows: 64 H equal tasks (pair, row, group of
-// 2 columns), H / 4 per thread: 6 pairs in by 128-bit loads, 2 columns out by
+// t1 pass of a face-box tile: 64 SQ_H equal tasks (pair, row, group of 2
+// columns), SQ_H / 4 per thread: 6 pairs in by 128-bit loads, 2 columns out by
 // one 128-bit store per array (consecutive lanes, consecutive 16 bytes: no
 // bank conflict; groups of 4 columns would store 32 bytes apart).
-template <int H>
 __device__ __forceinline__ void tile_t1_pass_f2(const float2 *sq, float2 *st, int tid)
 {
-    static_assert(H % 4 == 0, "a warp's tasks share the pair");
-    constexpr int NV = 16 * H, ROWS = H * TX;
+    static_assert(SQ_H % 4 == 0, "a warp's tasks share the pair");
+    constexpr int NV = 16 * SQ_H, ROWS = SQ_H * TX;
 #pragma unroll
-    for (int j = 0; j < H / 4; ++j) {
+    for (int j = 0; j < SQ_H / 4; ++j) {
         const int task = tid + j * 256, p = task / NV, rem = task - p * NV, r = rem >> 4, cg = rem & 15;
-        const float4 *in = reinterpret_cast<const float4 *>(sq + (p * H + r) * SQ_W + 2 * cg);
+        const float4 *in = reinterpret_cast<const float4 *>(sq + (p * SQ_H + r) * SQ_W + 2 * cg);
         f2 q[6];
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
@@ -1064,47 +1030,35 @@ __device__ __forceinline__ void pair_val_der(const f2 p[5], f2 &x0, f2 &x1, f2 &
     d1 = f2(__fsub_rn(Do.v.y, De.v.y), __fadd_rn(Do.v.y, De.v.y));
 }
 
-// The t2 pass of the NE faces (tx, r0 + e) of a tile of H rows at t1 Gauss
-// point m: values and t2 slopes of Q0, values of the t1 slopes and of the
-// normal slope at the two t2 Gauss points (the lanes), each row read once
-// over the 4 + NE rows that the faces' stencils cover. NEG: the density's
-// slopes negated, as gk_flux takes them.
-template <int H, int NE, bool NEG>
-__device__ __forceinline__ void t2_pass_f2(const float2 *st, int m, int tx, int r0, f2 q[NE][4], f2 dn[NE][4],
-                                           f2 d1[NE][4], f2 d2[NE][4])
+// The t2 pass of face (tx, ty) of a tile at t1 Gauss point m: values and t2
+// slopes of Q0, values of the t1 slopes and of the normal slope at the two t2
+// Gauss points (the lanes). NEG: the density's slopes negated, as gk_flux takes
+// them.
+template <bool NEG>
+__device__ __forceinline__ void t2_pass_f2(const float2 *st, int m, int tx, int ty, f2 q[4], f2 dn[4], f2 d1[4], f2 d2[4])
 {
-    constexpr int ROWS = H * TX;
-    const float2 *s = st + r0 * TX + tx;
+    const float2 *s = st + ty * TX + tx;
+    f2 p[5];
 #pragma unroll
     for (int P = 0; P < 2; ++P) {
-        f2 p[4 + NE];
 #pragma unroll
-        for (int i = 0; i < 4 + NE; ++i) p[i] = f2(s[(4 * P + m) * ROWS + i * TX]);
+        for (int i = 0; i < 5; ++i) p[i] = f2(s[(4 * P + m) * ST_ROWS + i * TX]);
+        if (P == 0)
+            pair_val_der<NEG>(p, q[0], q[1], d2[0], d2[1]);
+        else
+            pair_val_der<false>(p, q[2], q[3], d2[2], d2[3]);
 #pragma unroll
-        for (int e = 0; e < NE; ++e) {
-            if (P == 0)
-                pair_val_der<NEG>(p + e, q[e][0], q[e][1], d2[e][0], d2[e][1]);
-            else
-                pair_val_der<false>(p + e, q[e][2], q[e][3], d2[e][2], d2[e][3]);
-        }
+        for (int i = 0; i < 5; ++i) p[i] = f2(s[(4 * P + 2 + m) * ST_ROWS + i * TX]);
+        if (P == 0)
+            pair_val_direct<NEG>(p, d1[0], d1[1]);
+        else
+            pair_val_direct<false>(p, d1[2], d1[3]);
 #pragma unroll
-        for (int i = 0; i < 4 + NE; ++i) p[i] = f2(s[(4 * P + 2 + m) * ROWS + i * TX]);
-#pragma unroll
-        for (int e = 0; e < NE; ++e) {
-            if (P == 0)
-                pair_val_direct<NEG>(p + e, d1[e][0], d1[e][1]);
-            else
-                pair_val_direct<false>(p + e, d1[e][2], d1[e][3]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4 + NE; ++i) p[i] = f2(s[(8 + 2 * P + m) * ROWS + i * TX]);
-#pragma unroll
-        for (int e = 0; e < NE; ++e) {
-            if (P == 0)
-                pair_val_direct<NEG>(p + e, dn[e][0], dn[e][1]);
-            else
-                pair_val_direct<false>(p + e, dn[e][2], dn[e][3]);
-        }
+        for (int i = 0; i < 5; ++i) p[i] = f2(s[(8 + 2 * P + m) * ST_ROWS + i * TX]);
+        if (P == 0)
+            pair_val_direct<NEG>(p, dn[0], dn[1]);
+        else
+            pair_val_direct<false>(p, dn[2], dn[3]);
     }
 }
 
@@ -1113,7 +1067,6 @@ constexpr size_t flux_smem_bytes()
 {
     return (size_t)(SQ_N + ST_N) * sizeof(R) + 2 * sizeof(unsigned long long);
 }
-
 
 // ---- TMA and mbarrier helpers (sm_90+ PTX) ----
 

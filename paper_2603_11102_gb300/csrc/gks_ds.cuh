@@ -163,7 +163,6 @@ __device__ __forceinline__ dsf fma(dsf a, dsf b, dsf c)
     const dsf r = fast_two_sum(s.hi, __fadd_rn(s.lo, t.hi));
     return dsf(r.hi, __fadd_rn(r.lo, t.lo));
 }
-__device__ __forceinline__ dsf wdiv(dsf a, dsf b) { return a / b; }
 // exact scaling by a power of two
 __device__ __forceinline__ dsf scale_pow2(dsf a, float p) { return dsf(__fmul_rn(a.hi, p), __fmul_rn(a.lo, p)); }
 

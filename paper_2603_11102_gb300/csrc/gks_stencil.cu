@@ -3,27 +3,28 @@
 // Per stage and per direction d (x, y, z):
 //   face_eq      one thread per tangential position of the extended face box,
 //                marching along d with the differences around a cell (FP32C:
-//                the 5 cells) in registers: WENO5-JS (Sec. 2, Jiang-Shu) left/right states
-//                from one paired evaluation per cell, the equilibrium state
-//                Q0 from the half Maxwellians (u>0 from the left, u<0 from
-//                the right), and the quartic normal slope of Q0.
-//   face_flux    (x, y) linear quartic reconstruction of Q0 and its normal
-//                slope to the 2x2 Gauss points (Sec. 2, Eq. (x_example)) and
-//                the gas-kinetic flux F0 and its time derivative F1 at each
-//                point (Sec. 2, Eq. (flux); Appendix), averaged with weights
-//                1/4 and stored per face. FP32C: warps marching along t2 with
-//                the t1-pass rows in registers; FP64 and double-single:
-//                persistent blocks on 32x8 face tiles loaded by TMA, the t1
-//                pass in shared memory. The flux of FP32 and double-single
-//                arithmetic runs at two Gauss points at once on packed pairs.
-//   flux_update  FP32C: the z-face flux, walking z per tile column, fused with
-//                the divergence (Eq. (finite)) and the two-stage fourth-order
-//                combination of every cell; FP64: the z-face flux like the
-//                others, then the update over the stored fluxes. Stage 2 also
-//                prepares the next step (FP32 input, max |U|^2 for the CFL
-//                step).
+//                the 5 cells) in registers: WENO5-JS (Sec. 2, Jiang-Shu)
+//                left/right states from one paired evaluation per cell, the
+//                equilibrium state Q0 from the half Maxwellians (u>0 from the
+//                left, u<0 from the right), and the quartic normal slope of Q0.
+//   face_flux    (large FP32C grids: x and y) linear quartic reconstruction of
+//                Q0 and its normal slope to the 2x2 Gauss points (Sec. 2, Eq.
+//                (x_example)) and the gas-kinetic flux F0 and its time
+//                derivative F1 at each point (Sec. 2, Eq. (flux); Appendix),
+//                averaged with weights 1/4 and stored per face. FP32C: warps
+//                marching along t2 with the t1-pass rows in registers; FP64 and
+//                double-single: persistent blocks on 32x8 face tiles loaded by
+//                TMA, the t1 pass in shared memory. The flux of FP32 and
+//                double-single arithmetic runs at two Gauss points at once on
+//                packed pairs.
+//   flux_update  large FP32C grids: the z-face flux, walking z per tile column,
+//                fused with the divergence (Eq. (finite)) and the two-stage
+//                fourth-order combination of every cell; the others: the
+//                update over the stored fluxes of all three directions. Stage
+//                2 also prepares the next step (FP32 input, max |U|^2 for the
+//                CFL step).
 // Small grids run the three directions of face_eq and of face_flux as one
-// launch each and the update over stored fluxes.
+// launch each.
 //
 // All arithmetic runs in the working type R: double for GKS_FP64, float for
 // GKS_FP32C. The reconstruction works on rho - off (off = rho_ref in FP32C,
@@ -309,8 +310,8 @@ __device__ __forceinline__ void face_eq_f2(const FaceEqArgs<float, float> &A, in
     const int t = threadIdx.x;
     int a, b;
     const int f0 = SEG ? (blk.y * 4 + ((t >> 3) & 3)) * A.K : blk.y * A.K;
-    if (!face_position((unsigned)blk.x * (SEG ? blockDim.x / 4 : blockDim.x) + (SEG ? (t >> 5) * 8 + (t & 7) : t), A.n1, A.n2, a, b) || f0 >= A.nf)
-        return;
+    const unsigned pos = SEG ? blk.x * (blockDim.x / 4) + (t >> 5) * 8 + (t & 7) : blk.x * blockDim.x + t;
+    if (!face_position(pos, A.n1, A.n2, a, b) || f0 >= A.nf) return;
     const int f1 = min(f0 + A.K, A.nf);
     const long base = (long)(a + G) * A.s1 + (long)(b + G) * A.s2;   // cell index along d = -G
     // cells f0-3 .. f1+1 are read, faces f0 .. f1-1 written
@@ -365,8 +366,7 @@ __device__ __forceinline__ void face_eq_f2(const FaceEqArgs<float, float> &A, in
 // face_eq_march for FP64 grids in double-single arithmetic on packed
 // pairs: WENO5 of the components paired as (rho, m_n) and (m_t1, m_t2), the
 // half-space terms of the left and right states as one pair, the normal
-// slopes paired like the components. Every lane takes the operations of the
-// scalar double-single kernel, so the face boxes have the same bits.
+// slopes paired like the components.
 __device__ __forceinline__ void face_eq_ds2(const FaceEqArgs<double, dsf> &A, int2 blk)
 {
     int a, b;
@@ -475,7 +475,8 @@ void march_faces(FaceEqArgs<R, C> *E, const int *dir, int nd)
             most = std::max(most, k[i]);
         }
         const long m = (blocks + sms - 1) / sms, last = m % fit;   // of the busiest SM, in its last wave
-        const long cost = (m <= fit ? fit : m - last + (last ? std::max(last, busy) : 0)) * (most + (F32 && !ALL && dir[0] == 0 ? 2 : 1));
+        const long waves = m <= fit ? fit : m - last + (last ? std::max(last, busy) : 0);
+        const long cost = waves * (most + (F32 && !ALL && dir[0] == 0 ? 2 : 1));
         if (best < 0 || cost < best) {
             best = cost;
             for (int i = 0; i < nd; ++i) E[i].K = k[i];
@@ -484,7 +485,8 @@ void march_faces(FaceEqArgs<R, C> *E, const int *dir, int nd)
 }
 
 template <bool SEG>
-__global__ void __launch_bounds__(kEqThreads<float, false>, kEqBlocks<float, false>) face_eq_f2_kernel(FaceEqArgs<float, float> A)
+__global__ void __launch_bounds__(kEqThreads<float, false>, kEqBlocks<float, false>)
+    face_eq_f2_kernel(FaceEqArgs<float, float> A)
 {
     face_eq_f2<SEG>(A, make_int2(blockIdx.x, blockIdx.y));
 }
@@ -661,10 +663,10 @@ __device__ __forceinline__ void tile_gauss_flux_f2(const FluxPhys<f2> &ph, const
 {
 #pragma unroll
     for (int m = 0; m < 2; ++m) {
-        f2 Qv[1][4], Dn[1][4], D1[1][4], D2[1][4];   // the two t2 Gauss points -g, +g in the lanes
-        t2_pass_f2<SQ_H, 1, true>(st, m, tx, ty, Qv, Dn, D1, D2);
+        f2 Qv[4], Dn[4], D1[4], D2[4];   // the two t2 Gauss points -g, +g in the lanes
+        t2_pass_f2<true>(st, m, tx, ty, Qv, Dn, D1, D2);
         f2 F0[4], F1[4];
-        gk_flux<f2, NEED_F0>(ph, Qv[0], Dn[0], D1[0], D2[0], f2(ih1), f2(ih2), F0, F1);
+        gk_flux<f2, NEED_F0>(ph, Qv, Dn, D1, D2, f2(ih1), f2(ih2), F0, F1);
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             if (NEED_F0) {
@@ -1028,8 +1030,9 @@ __global__ void __launch_bounds__(32 * kMarchWarps, 1)
 // Rows per march segment: S segments of L = ceil(n2 / S) rows; the busiest
 // warp's rows are least (the priming rows of a segment cost their t1 pass,
 // about one face together), over up to 64 segments. On large grids this picks
-// long segments with even rounds of the warps, on 32^3 single rows (1056
-// items for 1216 warps).
+// long segments with even rounds of the warps (128^3: 19 rows, 3612 items for
+// 3 x 1216 warps), in the launch of all directions of 32^3, with a third of the
+// warps for each, 3 rows (363 items for 405 warps).
 int march_segment(int na, int nf, int n2, int warps)
 {
     double best = -1.0;
@@ -1317,7 +1320,7 @@ __global__ void __launch_bounds__(256, 2)
             __syncthreads();
             return;
         }
-        tile_t1_pass_f2<SQ_H>(sq, st, tid);
+        tile_t1_pass_f2(sq, st, tid);
         __syncthreads();
         // the face box is free: fetch the next tile's during this one's flux
         if (tid == 0 && nxt.it < nitems) {
