@@ -40,9 +40,9 @@ from paper_2603_11102_gb300 import workloads as WL  # noqa: E402
 # the current kernel source is committed (profiles/flops.txt, ncu counts of
 # the FFMA, FADD and FMUL instructions executed).
 FLOPS_ESTIMATE = {
-    # WENO5 of 4 variables on differences (both faces of a cell, 50 each),
+    # WENO5 of 4 variables on the 5-cell window (both faces of a cell, 85 each),
     # half-space equilibrium (~98 with its two series), normal slope (4 x 5)
-    "face_eq": 4 * 50 + 98 + 20,
+    "face_eq": 4 * 85 + 98 + 20,
     # t1 pass (4 x (25 + 17) per row, 1.1 rows a face), t2 pass (2 x 4 x 63), 4 fluxes, average
     "face_flux_stage1": 185 + 504 + 4 * 101 + 8,
     "face_flux_stage2": 185 + 504 + 4 * 82 + 4,

@@ -786,8 +786,8 @@ __global__ void __launch_bounds__(256) rev_face_state32_kernel(RevArgs A)
 // extended face plane are dealt out to the threads in one row (a block of 32 x 8
 // leaves a quarter of the threads of 132 x 132 positions idle), and a line is
 // cut so that the blocks fill whole waves (rev_cells; 918 blocks on 304 places
-// took 4 waves): 0.37 -> 0.22 ms for the y and z faces of 256x128x128, 0.48 ->
-// 0.37 ms for the x faces, whose cells lie a row apart across the lanes.
+// took 4 waves): 0.37 -> 0.24 ms for the y and z faces of 256x128x128, 0.48 ->
+// 0.35 ms for the x faces, whose cells lie a row apart across the lanes.
 struct RevSlot {
     double lam[4][256];
     float q[8][256], w[4][256];

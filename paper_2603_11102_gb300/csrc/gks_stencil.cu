@@ -223,7 +223,7 @@ struct FaceEqArgs {
 
 // Blocks of the face-state kernels (ALL: of the launch of all directions):
 // threads, blocks that fit on an SM, and how few of them keep it as busy. FP32
-// with 64, 128, 256 threads: 1.87, 1.83, 1.89 ms a step of 384x256x256;
+// with 64, 128, 256 threads: 1.82, 1.82, 1.88 ms a step of 384x256x256;
 // double-single with 64 and 256 1.07 and 1.00 ms on 96^3, 0.076 and 0.108 in the
 // launch of all directions of 32^3, whose few blocks spread better when small.
 // FP64: 12 warps at 168 registers are what the FP64 pipe's latency needs (16 at
@@ -454,8 +454,9 @@ dim3 face_eq_blocks(const FaceEqArgs<R, C> &E, int d)
 // sectors, 4 of them a line; 9 faces, which fill the blocks better, took 0.39
 // against 0.36 ms a step of 256x128x128. Face state of a step with this rule and
 // face_position, before and now: FP64 128^3 8.94 -> 6.61 ms and 32^3 0.349 ->
-// 0.181, double-single 96^3 1.41 -> 1.00, FP32C 384x256x256 1.896 -> 1.830,
-// 256x128x128 0.360 -> 0.347, 128^3 0.210 -> 0.203, 32^3 0.0187 -> 0.0165.
+// 0.181, double-single 96^3 1.41 -> 1.00. FP32C waits on its loads and takes the
+// halved length as well: 1.82 and 1.82 ms on 384x256x256, 0.359 and 0.356 on
+// 256x128x128, 0.207 and 0.214 on 128^3.
 template <typename R, typename C, bool ALL>
 void march_faces(FaceEqArgs<R, C> *E, const int *dir, int nd)
 {
